@@ -173,6 +173,106 @@ void parallel_for(int n, F fn) {
     if (!e.empty()) throw ArgError(e);
 }
 
+// FP64 SYRK on the tensor cores: batches of consecutive subdomains whose digits of X (16 bytes per value) fit
+// `budget` bytes (one subdomain at least), the tiles of each batch in groups of subdomains whose digits stay in L2
+// (most expensive tile first within a group), and the pieces of X to cut.
+void plan_syrk_oz(feti_ctx* c, size_t budget) {
+  constexpr double kGroupBytes = 64e6;  // of digits, about half of L2
+  constexpr int kUnits = 2048;          // (piece, column) units per CTA of the cutting kernel
+  const int ns = c->nsub;
+  auto xsize = [&](int i) { return (size_t)c->bps[c->subs[i].bp].Xsize; };
+  // chunks of every 128 x 128 tile of a plan (shared by the subdomains of that plan)
+  std::vector<std::vector<int>> chunks(c->bps.size());
+  for (size_t b = 0; b < c->bps.size(); ++b) {
+    auto& B = c->bps[b];
+    auto& P = c->pats[c->bp_pat[b]];
+    const int nt = B.nb2 * (B.nb2 + 1) / 2;
+    std::vector<int> np;
+    for (int t = 0; t < nt; ++t) {
+      np.clear();
+      for (int k = B.t2_off[t]; k < B.t2_off[t + 1]; ++k) np.push_back((P.sn_w[B.t2_sn[k]] + 7) / 8);
+      chunks[b].push_back(syrk_oz_chunks(np.data(), (int)np.size()));
+    }
+  }
+  std::vector<int4> items, ditems;
+  c->oz_batches.clear();
+  size_t most = 0;
+  for (int i = 0; i < ns;) {
+    OzBatch o{};
+    o.sub0 = i;
+    o.x0 = c->info[i].X;
+    o.item0 = (int)items.size();
+    o.ditem0 = (int)ditems.size();
+    size_t bytes = 0;
+    while (i < ns && (o.nsub == 0 || bytes + 16 * xsize(i) <= budget)) {
+      // one group of subdomains
+      std::vector<int4> grp;
+      double gb = 0;
+      while (i < ns && gb < kGroupBytes && (o.nsub == 0 || bytes + 16 * xsize(i) <= budget)) {
+        auto& B = c->bps[c->subs[i].bp];
+        auto& P = c->pats[c->subs[i].pat];
+        for (int bi = 0; bi < B.nb2; ++bi)
+          for (int bj = 0; bj <= std::min(2 * bi + 1, B.nb - 1); ++bj) {
+            const int t = bi * (bi + 1) / 2 + bj / 2;
+            grp.push_back(make_int4(i, bi | bj << 16, chunks[c->subs[i].bp][t], t));
+          }
+        for (int s : B.act) {
+          const int units = (P.sn_w[s] + 7) / 8 * (B.je[s] - B.jb[s]);
+          for (int u = 0; u < units; u += kUnits) ditems.push_back(make_int4(i, s, u, std::min(kUnits, units - u)));
+        }
+        o.m_max = std::max(o.m_max, c->subs[i].m);
+        bytes += 16 * xsize(i);
+        gb += 16.0 * xsize(i);
+        ++o.nsub;
+        ++i;
+      }
+      std::stable_sort(grp.begin(), grp.end(), [](const int4& a, const int4& b) { return a.z > b.z; });
+      items.insert(items.end(), grp.begin(), grp.end());
+    }
+    o.nitems = (int)items.size() - o.item0;
+    o.nditems = (int)ditems.size() - o.ditem0;
+    c->oz_batches.push_back(o);
+    most = std::max(most, bytes);
+  }
+  dfree(c, c->d_oz_items);
+  dfree(c, c->d_oz_ditems);
+  c->d_oz_items = c->d_oz_ditems = nullptr;
+  c->d_oz_items = upload(c, items);
+  c->d_oz_ditems = upload(c, ditems);
+  CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
+  c->xd_bytes = most;
+}
+
+// The digit buffer: as many subdomains at a time as a fifth of the free memory holds (16 GB at most), fewer if the
+// allocator refuses; false when not even one subdomain fits (the FP64-pipe kernel takes over).
+bool reserve_syrk_oz(feti_ctx* c) {
+  if (c->d_XD) return true;
+  if (!c->oz_batches.empty()) {  // released after the previous assembly (recompute_X)
+    try {
+      c->d_XD = dalloc(c, c->xd_bytes);
+      return true;
+    } catch (std::bad_alloc&) {
+    }
+  }
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  size_t want = 0;
+  for (int i = 0; i < c->nsub; ++i) want += 16 * (size_t)c->bps[c->subs[i].bp].Xsize;
+  const size_t budget = std::min(want, std::min<size_t>((size_t)16 << 30, free_b / 5));
+  for (size_t b : {budget, (size_t)0}) {
+    try {
+      plan_syrk_oz(c, b);
+      c->d_XD = dalloc(c, c->xd_bytes);
+      if (!c->d_oz_ex) c->d_oz_ex = (int*)dalloc(c, (size_t)std::max<int64_t>(c->ncols, 1) * sizeof(int));
+      return true;
+    } catch (std::bad_alloc&) {
+      dfree(c, c->d_XD);
+      c->d_XD = nullptr;
+    }
+  }
+  return false;
+}
+
 void build(feti_ctx* c) {
   using clk = std::chrono::steady_clock;
   auto t0 = clk::now();
@@ -1042,6 +1142,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
                 tcmode, tf32_out,
                 ctx->d_status, s2, 0, ctx->d_X2, ctx->d_L32, split ? 1 : 0);
   };
+  // FP64: the SYRK by exact slicing on the tensor cores
+  const bool oz = !ctx->fp32 && ctx->opt.assembly_route != 2 && ctx->stats.syrk_flops > 0 && reserve_syrk_oz(ctx);
   // the numeric phase as one sequence of launches (recorded once into a CUDA graph, see below); r2: the
   // TRSM-path route (F_i = B_i P^T L^{-T} X_i in host-driven batches, not captured)
   auto enqueue = [&](cudaStream_t s2, unsigned evf, bool r2) {
@@ -1146,7 +1248,12 @@ feti_status feti_assemble(feti_ctx* ctx) {
       run_syrk(ctx->syrk_variant);
       ctx->stats.syrk_variant = ctx->syrk_variant;
     } else {
-      launch_syrk_f64(ctx->P, ctx->d_syrk_items, ctx->nsyrk, (const double*)ctx->d_X, (double*)ctx->d_F,
+      if (oz)
+        for (const auto& b : ctx->oz_batches)
+          launch_syrk_oz(ctx->P, (const double*)ctx->d_X, b, ctx->d_oz_ditems, ctx->d_oz_items, ctx->d_XD,
+                         ctx->d_oz_ex, (double*)ctx->d_F, ctx->nsm, ctx->d_status, s2);
+      else
+        launch_syrk_f64(ctx->P, ctx->d_syrk_items, ctx->nsyrk, (const double*)ctx->d_X, (double*)ctx->d_F,
                       std::min(ctx->nsyrk, ctx->nsm * 8), s2);
     }
     if (ctx->precond_kind == 2) {
@@ -1159,6 +1266,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
   };
   // Cholesky, pruned TRSM, unit-lower scaling, SYRK (+ lumped values, or the Dirichlet factorisation and tiles)
   ctx->stats.launches += 4 + (ctx->precond_kind == 1 ? 1 : ctx->precond_kind == 2 ? 2 : 0);
+  if (oz) ctx->stats.launches += 3 * (int64_t)ctx->oz_batches.size() - 1;
   const int want = ctx->opt.assembly_route;
   if (want == 2 || (want == 3 && ctx->route_tuned && ctx->route == 2)) {
     ctx->route = 2;
@@ -1169,7 +1277,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     }
     enqueue(st, cudaEventRecordDefault, true);
     CK(cudaGetLastError());
-  } else if (ctx->asm_exec && ctx->asm_X == ctx->d_X && ctx->asm_X2 == ctx->d_X2) {
+  } else if (ctx->asm_exec && ctx->asm_X == ctx->d_X && ctx->asm_X2 == ctx->d_X2 && ctx->asm_XD == ctx->d_XD) {
     CK(cudaGraphLaunch(ctx->asm_exec, st));
   } else {
     ctx->route = want == 1 ? 1 : 0;
@@ -1213,6 +1321,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       if (e != cudaSuccess) throw CudaError(std::string("assembly graph: ") + cudaGetErrorString(e));
       ctx->asm_X = ctx->d_X;
       ctx->asm_X2 = ctx->d_X2;
+      ctx->asm_XD = ctx->d_XD;
     }
   }
   CK(cudaGetLastError());
@@ -1231,6 +1340,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
     ctx->d_X = nullptr;
     dfree(ctx, ctx->d_X2);
     ctx->d_X2 = nullptr;
+    dfree(ctx, ctx->d_XD);
+    ctx->d_XD = nullptr;
   }
   float a, b, cc, d;
   CK(cudaEventElapsedTime(&a, ctx->ev[0], ctx->ev[1]));

@@ -230,6 +230,14 @@ struct AdjBatch {
 };
 constexpr int kBuildCols = 512;  // columns of V_Y per item of the adjoint's X_u W product
 
+// A run of consecutive subdomains whose digits of X fit the digit buffer together (FP64 SYRK on the tensor cores).
+struct OzBatch {
+  int sub0, nsub, m_max;
+  int item0, nitems;    // tiles (syrk_oz items)
+  int ditem0, nditems;  // pieces of X blocks to cut
+  int64_t x0;           // first X element
+};
+
 // flags of the numeric Cholesky (kern_factor.cu)
 enum : int { kCholNoReg = 1, kCholStopRoot = 2, kCholSkipBig = 4 };
 

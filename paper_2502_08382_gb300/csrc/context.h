@@ -95,6 +95,13 @@ struct feti_ctx {
   bool syrk_tuned = false;
   int* d_impl_order = nullptr;
   int2* d_syrk_items = nullptr;
+  // FP64 SYRK on the tensor cores: batches of subdomains, their tiles and X pieces, digits and column exponents
+  std::vector<feti::OzBatch> oz_batches;
+  int4* d_oz_items = nullptr;
+  int4* d_oz_ditems = nullptr;
+  void* d_XD = nullptr;
+  size_t xd_bytes = 0;
+  int* d_oz_ex = nullptr;
   feti::TileDesc* d_tdesc = nullptr;
   struct ApplyCand {
     int variant, grid;  // tile-kernel variant (load batch) and grid
@@ -162,6 +169,7 @@ struct feti_ctx {
   cudaGraphExec_t asm_exec = nullptr;  // the numeric assembly (Cholesky, TRSM, scaling, SYRK), replayed on st
   void* asm_X = nullptr;             // the X buffers the assembly graph was captured with
   void* asm_X2 = nullptr;
+  void* asm_XD = nullptr;
   uint16_t* d_X2 = nullptr;          // bf16 hi/lo copy of X (split-bf16 SYRK operands)
   float* d_L32 = nullptr;            // FP32 copy of L for the mixed TRSM
   cudaGraphExec_t pcg_exec = nullptr;  // captured chunk of iterations (replayed on st)

@@ -42,6 +42,11 @@ void launch_syrk_tc(const DevPlan& P, const int2* items, int nitems, const float
 size_t syrk_tc_smem(int split);
 void launch_syrk_f64(const DevPlan& P, const int2* items, int nitems, const double* X, double* F, int grid,
                      cudaStream_t st);
+void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const int4* ditems, const int4* items,
+                    void* XD, int* EX, double* F, int nsm, int* status, cudaStream_t st);
+// chunks of the tile whose contributing supernodes have np[0 .. n) 8-row pieces (the loaders' batching)
+int syrk_oz_chunks(const int* np, int n);
+
 // ev_tiles0/1: optional events recorded just before / after the F-streaming kernel
 void launch_apply(const DevPlan& P, bool fp32, const TileDesc* desc, int ntiles, const void* F, const int* qmap,
                   int64_t ncols, const double* p, void* pg, void* rowpart, void* colpart, const int2* blocks,
