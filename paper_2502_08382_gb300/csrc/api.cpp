@@ -1189,7 +1189,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     run_chol(ctx->chol_pick, ctx->P, 0, 0, true);
     CK(cudaEventRecordWithFlags(ctx->ev[1], s2, evf));
     if (r2) {
-      launch_unit_scale(ctx->P, ctx->nsub, ctx->P.dinv, s2);
+      launch_unit_scale(ctx->P, ctx->nsub, ctx->nmax, ctx->P.dinv, s2);
       CK(cudaEventRecordWithFlags(ctx->ev[2], s2, evf));
       trsm_path_entry(ctx);
       CK(cudaEventRecordWithFlags(ctx->ev[3], s2, evf));
@@ -1220,7 +1220,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     }
     run_trsm(ctx->trsm_cands[ctx->trsm_pick], s2);
     // the implicit solves take L in unit-lower form; the TRSM above was its last user as L
-    launch_unit_scale(ctx->P, ctx->nsub, ctx->P.dinv, s2);
+    launch_unit_scale(ctx->P, ctx->nsub, ctx->nmax, ctx->P.dinv, s2);
     CK(cudaEventRecordWithFlags(ctx->ev[2], s2, evf));
     if (ctx->fp32) {
       auto run_syrk = [&](int variant) {
