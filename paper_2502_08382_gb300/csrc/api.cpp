@@ -932,7 +932,7 @@ void build(feti_ctx* c) {
     D.task_nbig = upload(c, nbig);
     c->P2.task_nbig = D.task_nbig;
     c->d_tdone = (int*)dalloc(c, (size_t)std::max(base, 1) * sizeof(int));
-    // the tensor-core Cholesky's items: the large tasks, children first; its scratch per CTA: the bf16 slices and
+    // the tensor-core Cholesky's items: the large tasks, children first; its scratch per cluster: the bf16 digits and
     // a row exponent for every row of the largest such front
     {
       int fmax = 0;
@@ -946,9 +946,12 @@ void build(feti_ctx* c) {
       c->n_tc_items = (int)tci.size();
       if (c->n_tc_items > 0) {
         c->d_tc_items = upload(c, tci);
-        c->grid_tc = std::min(c->nsm, std::min(c->n_tc_items, c->grid_chol));
+        int nbig_sub = 0;
+        for (int i = 0; i < ns; ++i) nbig_sub += c->pats[c->subs[i].pat].has_big ? 1 : 0;
+        c->tc_cluster = chol_tc_cluster(nbig_sub, c->nsm);
+        c->grid_tc = std::max(1, std::min(c->nsm / c->tc_cluster, std::min(c->n_tc_items, c->grid_chol)));
         c->slice_stride = chol_tc_scratch(fmax);
-        c->d_slices = (uint16_t*)dalloc(c, (size_t)c->grid_tc * c->slice_stride * 2);
+        c->d_slices = (char*)dalloc(c, (size_t)c->grid_tc * c->slice_stride);
       }
     }
     // nothing to split: the whole-subdomain items only
@@ -1167,7 +1170,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
         CK(cudaMemsetAsync(ctx->d_tdone, 0, (size_t)std::max(ctx->ntask_total, 1) * sizeof(int), s2));
         launch_chol_tc(P, ctx->d_tc_items, ctx->n_tc_items, ctx->d_queue + qslot + 1, ctx->d_tdone, ctx->d_hand,
                        ctx->d_ws, ctx->ws_stride, ctx->chol_front, ctx->d_slices, ctx->slice_stride, ctx->grid_tc,
-                       ctx->d_status, s2, flags);
+                       ctx->tc_cluster, ctx->d_status, s2, flags);
       }
     };
     if (!ctx->chol_tuned) {

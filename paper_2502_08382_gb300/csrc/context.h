@@ -86,8 +86,8 @@ struct feti_ctx {
   int* d_tdone = nullptr;            // per global task: child tasks finished
   double* d_hand = nullptr;          // hand-over slots of split subtree roots
   int4* d_tc_items = nullptr;        // the large fronts' tasks (the tensor-core Cholesky's items)
-  int n_tc_items = 0, grid_tc = 0;
-  uint16_t* d_slices = nullptr;      // its per-CTA scratch (bf16 slices and row exponents)
+  int n_tc_items = 0, grid_tc = 0, tc_cluster = 1;  // items, clusters and CTAs per cluster
+  char* d_slices = nullptr;          // its per-cluster scratch (bf16 digits and row exponents)
   int64_t slice_stride = 0;
   int2* d_l16_items = nullptr;       // (subdomain, supernode) of the panels with a row-major hi/lo copy
   int n_l16 = 0;

@@ -1,0 +1,686 @@
+// Tensor-core Cholesky of the large fronts (P.sn_big: the fronts at least big_f wide and their ancestors, the top of
+// each supernodal tree), after chol_kernel has done everything below them.
+//
+// A front's w own columns go in blocks of 128, and inside a block in steps of 32:
+//   pivot   the 32 x 32 block's factor L_bb and inverse on the FP64 pipe (eight warps);
+//   panel   the rows below, X = A L_bb^{-T}, on the tensor cores (K = 32, N = 32);
+//   block   the block's later columns, C -= X X^T, on the tensor cores (K = 32);
+// after the block the rest of the front takes C -= X X^T with K = 128.  All products run by exact slicing of FP64
+// into bf16 digits (oz.cuh); a product costs one FP64 addition per entry of C, the rest of the epilogue (sums of the
+// accumulators, normalisation, rounding to nearest) is integer arithmetic, because one FP64 instruction of a warp
+// takes 64 clocks of its scheduler here.
+//
+// A cluster of C CTAs (1, 2, 4 or 8; one CTA per SM) takes one front at a time: every CTA repeats the pivot, the rows
+// of the panel and the tiles of the updates are dealt out, and barriers between the phases order the accesses (all
+// shared data is in global memory).  C is as large as keeps the CTAs within the SMs (chol_tc_cluster).
+//
+// Measured (the kernel alone; before: 9 slices of 7 bits, 45 MMAs of N = 32 per 16-deep step, one CTA per front, the
+// panel on the FP64 pipe): 64 uneven 3D heat subdomains 50.3 -> 11.8 ms (C = 2), 27 elasticity subdomains of 12^3
+// 59.0 -> 11.4 ms (C = 4), 64 of them 66.0 -> 19.9 ms (C = 2), 125 uneven 3D heat subdomains 40.8 -> 6.0 ms (C = 1).
+// What bounds it now: on wide fronts the staging of the digits (96 KB from L2 per 2304 clocks of MMA), on fronts of a
+// few hundred rows the pivot blocks (16 k clocks of FP64 work for 32 columns) and the barriers between the phases.
+//
+// The digits are written pre-swizzled (64-byte swizzle, 8-row atoms): [digit][32-deep chunk][row][64 bytes], so any
+// 8-row-aligned run of rows of one digit and chunk is a ready operand, loaded by one bulk copy.  Tiles are 128 rows x
+// 64 columns: a stage holds the 8 A digits and the digits of two blocks of 32 B columns, each with its own set of
+// accumulators (256 TMEM columns), so one set is drained while the other is filled.  Warp 0 issues the MMAs, warp 1
+// the copies, warps 4-11 run the epilogue; all twelve do the rest.  Every mbarrier wait is bounded; a CTA that gives
+// up keeps to the cluster's barriers and skips its work.
+#include <algorithm>
+#include <cuda_bf16.h>
+
+#include "chol_common.cuh"
+#include "common.cuh"
+#include "kernels.h"
+#include "oz.cuh"
+
+namespace feti {
+namespace {
+
+constexpr int kCT = 384;                                    // threads per CTA
+constexpr int kCM = 128, kCH = 32;                          // rows of a tile, columns of one B block
+constexpr int kCA = kCM * 64, kCB = kCH * 64;               // bytes of one digit of A / of a B block (one chunk)
+constexpr int kCStage = kDig * (kCA + 2 * kCB);             // 96 KB
+constexpr int kCStages = 2;
+constexpr int kCBlk = 128;                                  // columns per block
+constexpr int kCDyn = 1024 + kCStages * kCStage + kDig * kCB;  // + the digits of L_bb^{-1}
+
+struct PivotSmem {
+  double D[kNB][kNB + 1];   // the block, then L_bb
+  double M[kNB][kNB + 1];   // L_bb^{-1}
+  double col[2][kNB];       // the pivot column below the pivot (double-buffered)
+  double cols[2][kNB];      // the same times the reciprocal pivot, which stands in the other places
+};
+static_assert(sizeof(PivotSmem) <= kCStage, "the pivot's buffers alias the stage ring");
+
+__device__ __forceinline__ uint32_t cl_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cl_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// barrier of all threads of the cluster; orders their global accesses (generic and bulk copies)
+__device__ __forceinline__ void cl_sync() {
+  __syncwarp();
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+struct CtState {
+  uint8_t* ring;
+  uint8_t* bpan;      // digits of L_bb^{-1}
+  uint64_t *full, *empty, *accf, *acce, *drain;
+  volatile int* abort;
+  uint32_t tmem;
+  uint32_t chunks;    // chunks staged so far (stage and phase)
+  uint32_t units;     // 32-column units multiplied so far (accumulator set and phase)
+};
+
+// the value 2^ex (2^32 hi + lo) rounded to nearest, by integer arithmetic
+__device__ __forceinline__ double dig_value(long long hi, long long lo, int ex) {
+  hi += lo >> 32;
+  uint32_t l = (uint32_t)lo;
+  const bool neg = hi < 0;
+  if (neg) {
+    hi = ~hi + (l == 0);
+    l = -l;
+  }
+  unsigned long long h = (unsigned long long)hi;
+  if (h == 0) {
+    h = l;
+    l = 0;
+    ex -= 32;
+  }
+  const int lz = __clzll((long long)h);
+  const unsigned long long x = (unsigned long long)l << 32;
+  const unsigned long long m = lz < 64 ? (h << lz) | (lz ? x >> (64 - lz) : 0ULL) : 0ULL;
+  const unsigned long long mant = (m >> 11) + ((m >> 10) & 1);  // 53 bits, 2^52 <= mant <= 2^53
+  const int e = 95 - lz + ex;                                   // value = mant 2^(e - 52)
+  unsigned long long b = ((unsigned long long)(e + 1022) << 52) + mant;
+  if (h == 0 || e < -1021) b = 0;
+  if (h != 0 && e > 1022) b = 0x7FF0000000000000ULL;
+  return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ULL : 0ULL)));
+}
+
+// Digits of the rows [r0, r1) (multiples of 8) of the column-major A (ld, K <= 128 columns): row exponents EX and the
+// digits in the layout above (npad rows; rows >= n are zero).  Four lanes per row, eight of its columns each.
+template <int NCK>
+__device__ __forceinline__ void dig_rows(const double* A, int64_t ld, int n, int K, int r0, int r1, char* SL, int nck,
+                                         int npad, int* EX, int warp, int nwarps) {
+  const int lane = threadIdx.x % 32, q = lane & 3;
+  for (int rb = r0 + warp * 8; rb < r1; rb += nwarps * 8) {
+    const int i = rb + (lane >> 2);
+    double v[NCK][8];
+    uint32_t mx = 0;
+#pragma unroll
+    for (int c = 0; c < NCK; ++c)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = c * 32 + q * 8 + e;
+        v[c][e] = (i < n && k < K) ? __ldcg(A + (int64_t)k * ld + i) : 0.0;
+        mx = max(mx, (uint32_t)__double2hiint(v[c][e]) & 0x7fffffffu);
+      }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const int ex = dig_exponent(mx);
+    if (q == 0) EX[i] = ex;
+    const int64_t o = (int64_t)i * 64 + ((q ^ ((i >> 1) & 3)) << 4);
+#pragma unroll
+    for (int c = 0; c < NCK; ++c) {
+      if (c >= nck) break;
+      uint64_t w[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[c][e], ex);
+#pragma unroll
+      for (int p = 0; p < kDig; ++p)
+        *reinterpret_cast<uint4*>(SL + ((int64_t)(p * nck + c) * npad) * 64 + o) =
+            make_uint4(dig_pair(w[0], w[1], p), dig_pair(w[2], w[3], p), dig_pair(w[4], w[5], p),
+                       dig_pair(w[6], w[7], p));
+    }
+  }
+}
+
+// One phase of products on the tensor cores.  Tiles t = first, first + step, ... < ntile:
+//  PANEL   tile t is row block t of A (digits SA, one chunk); Out[row, j] = (A L_bb^{-T})[row, j] for j < ncol, written
+//          to Ls columns kb + j (row i0 + row of the front); exponents of L_bb^{-1} in EXB.
+//  update  tile t is (row block tm, 64-column block tn): C -= A A^T for the columns [i0, ce) on and below the diagonal,
+//          C in Ls (columns < w) or W; n = rows of A.
+template <bool PANEL>
+__device__ __forceinline__ void dig_product(CtState& st, const char* SA, const int* EX, const int* EXB, int n, int nck,
+                                            int first, int step, int ntile, int ntn, double* Ls, int64_t f, int w,
+                                            double* W, int r, int i0, int kb, int ncol) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int npad = (n + kCM - 1) / kCM * kCM;
+  const int64_t digA = (int64_t)nck * npad * 64;  // bytes between digits
+  const uint32_t ring = smem_u32(st.ring);
+  // tile t: row block tm holds min(2 (tm + 1), ntn) column blocks
+  auto tile_of = [&](int t, int& tm, int& tn) {
+    if (PANEL) {
+      tm = t;
+      tn = 0;
+      return;
+    }
+    tm = 0;
+    const int nfull = (ntn + 1) / 2;  // row blocks before this one have fewer column blocks
+    // sum_{m < tm} 2 (m + 1) = tm (tm + 1)
+    tm = (int)((sqrtf(4.f * t + 1.f) - 1.f) * 0.5f);
+    while ((tm + 1) * (tm + 2) <= t) ++tm;
+    while (tm * (tm + 1) > t) --tm;
+    if (tm >= nfull - 1) {
+      const int base = (nfull - 1) * nfull;  // tiles of the first nfull - 1 row blocks
+      const int q = t - base;
+      const int c0 = min(2 * nfull, ntn);
+      tm = nfull - 1 + q / c0;
+      tn = q % c0;
+      return;
+    }
+    tn = t - tm * (tm + 1);
+  };
+  const int mine = first < ntile ? (ntile - first + step - 1) / step : 0;
+  const uint32_t nu = PANEL ? 1 : 2;  // units (32-column blocks) per tile
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();  // the ring's generic use is over
+  const bool live = !*st.abort;
+  if (live && warp == 1 && lane == 0) {
+    // ---- copies
+    bool ok = true;
+    uint32_t cg = st.chunks;
+    for (int q = 0; q < mine && ok; ++q) {
+      int tm, tn;
+      tile_of(first + q * step, tm, tn);
+      for (int c = 0; c < nck && ok; ++c, ++cg) {
+        const uint32_t s = cg % kCStages;
+        if (cg >= kCStages) ok = dig_wait(smem_u32(&st.empty[s]), ((cg / kCStages) - 1) & 1, st.abort);
+        if (!ok) break;
+        const uint32_t sA = ring + s * kCStage, sB = sA + kDig * kCA, bar = smem_u32(&st.full[s]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                     "r"(PANEL ? kDig * kCA : kCStage)
+                     : "memory");
+        const char* a0 = SA + ((int64_t)c * npad + (int64_t)tm * kCM) * 64;
+        const char* b0 = SA + ((int64_t)c * npad + (int64_t)tn * 64) * 64;
+#pragma unroll 1
+        for (int p = 0; p < kDig; ++p) {
+          bulk_copy(sA + p * kCA, a0 + p * digA, kCA, bar);
+          if (!PANEL) {
+            bulk_copy(sB + p * kCB, b0 + p * digA, kCB, bar);
+            bulk_copy(sB + (kDig + p) * kCB, b0 + p * digA + kCB, kCB, bar);
+          }
+        }
+      }
+    }
+    if (!ok) {
+      // the copies in flight land (bounded) before the block goes on
+      for (uint32_t k = cg > kCStages ? cg - kCStages : 0; k < cg; ++k)
+        mbar_wait(smem_u32(&st.full[k % kCStages]), (k / kCStages) & 1);
+    }
+  } else if (live && warp == 0 && lane == 0) {
+    // ---- MMAs
+    bool ok = true, issued = false;
+    uint32_t cg = st.chunks, un = st.units;
+    for (int q = 0; q < mine && ok; ++q, un += nu) {
+      for (int c = 0; c < nck && ok; ++c, ++cg) {
+        const uint32_t s = cg % kCStages;
+        ok = dig_wait(smem_u32(&st.full[s]), (cg / kCStages) & 1, st.abort);
+        const uint32_t sA = ring + s * kCStage, sB = PANEL ? smem_u32(st.bpan) : sA + kDig * kCA;
+        for (uint32_t h = 0; h < nu && ok; ++h) {
+          const uint32_t u = un + h, set = u & 1;
+          if (c == 0 && u >= 2) ok = dig_wait(smem_u32(&st.acce[set]), ((u >> 1) - 1) & 1, st.abort);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+          for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+            for (int p = 0; p < kDig; ++p)
+              mma_f16(st.tmem + set * 256 + p * kCH, sw64_desc(sA + p * kCA + kk * 32),
+                      sw64_desc(sB + h * (kDig * kCB) + kk * 32), idesc_m128(1u, (uint32_t)(kCH * (kDig - p))),
+                      (c == 0 && kk == 0 && p == 0) ? 0u : 1u);
+          issued = true;
+          if (c == nck - 1) mma_commit(smem_u32(&st.accf[set]));
+        }
+        if (ok) mma_commit(smem_u32(&st.empty[s]));
+      }
+    }
+    if (!ok && issued) {  // nothing is issued after this: every MMA is done before TMEM is released
+      mma_commit(smem_u32(st.drain));
+      mbar_wait(smem_u32(st.drain), 0);
+    }
+  } else if (live && warp >= 4) {
+    // ---- epilogue: TMEM lane quarter warp % 4, 16 columns of the unit
+    const int quarter = warp % 4, ch = (warp - 4) / 4;
+    uint32_t un = st.units;
+    int ok = 1;
+    for (int q = 0; q < mine && ok; ++q) {
+      int tm, tn;
+      tile_of(first + q * step, tm, tn);
+      const int ri = tm * kCM + quarter * 32 + lane, gi = i0 + ri;  // row of A / of the front
+      const int ei = ri < n ? __ldcg(EX + ri) : 0;
+      for (uint32_t h = 0; h < nu && ok; ++h, ++un) {
+        const uint32_t set = un & 1;
+        const int cb = tn * 64 + h * kCH + ch * 16;  // first column (relative to i0, or to kb)
+        // the C entries this thread subtracts from, loaded while the tile is multiplied
+        double* base = nullptr;
+        int64_t ld = 0;
+        int nc = 0;
+        double cv[16];
+        if (PANEL) {
+          base = Ls + (int64_t)(kb + cb) * f + gi;
+          ld = f;
+          nc = ri < n ? min(16, ncol - cb) : 0;
+        } else {
+          nc = ri < n ? min(16, min(ncol, ri + 1) - cb) : 0;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int gj = i0 + cb + e;
+            cv[e] = e < nc ? __ldcg(gj < w ? Ls + (int64_t)gj * f + gi : W + (int64_t)(gj - w) * r + (gi - w)) : 0.0;
+          }
+        }
+        if (lane == 0) ok = dig_wait(smem_u32(&st.accf[set]), (un >> 1) & 1, st.abort) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t t0 = st.tmem + ((uint32_t)(quarter * 32) << 16) + set * 256 + ch * 16;
+#pragma unroll
+        for (int e0 = 0; e0 < 16; e0 += 4) {
+          uint32_t a[4][kDig];
+#pragma unroll
+          for (int d = 0; d < kDig; ++d) tmem_ld4(t0 + d * kCH + e0, a[0][d], a[1][d], a[2][d], a[3][d]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (e0 == 12) {  // the set's last columns are in registers: hand it back
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&st.acce[set]);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int c = e0 + e;
+            if (c < nc) {
+              long long hi = 0, lo = 0;
+              dig_sum(a[e], hi, lo);
+              const int ej = PANEL ? EXB[cb + c] : __ldcg(EX + cb + c);
+              double t = dig_value(hi, lo, ei + ej - 68);
+              if (ei == kExpBad || ej == kExpBad) t = __longlong_as_double(0x7FF8000000000000LL);
+              if (PANEL) {
+                base[c * ld] = t;
+              } else {
+                const int gj = i0 + cb + c;
+                if (gj < w) Ls[(int64_t)gj * f + gi] = cv[c] - t;
+                else W[(int64_t)(gj - w) * r + (gi - w)] = cv[c] - t;
+              }
+            }
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (live) {
+    st.chunks += (uint32_t)(mine * nck);
+    st.units += (uint32_t)mine * nu;
+  }
+}
+
+// L_bb and L_bb^{-1} of the nbk x nbk block in sm.D by the CTA's first eight warps: lane = row, warp v holds columns
+// v, v + 8, v + 16, v + 24 of the block (from the diagonal on) and of the inverse (up to the diagonal).  Elimination of
+// [A | I]: step k subtracts column k (times the row k of the inverse part, whose rows are scaled by the reciprocal
+// pivots at the end).  L_bb goes to sm.D, its inverse to sm.M.
+__device__ __forceinline__ void pivot_block(PivotSmem& sm, int nbk, int* bad) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (warp >= 8) return;
+  double a[4], m[4], rsl = 1.0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int j = warp + 8 * u;
+    a[u] = sm.D[lane][j];
+    m[u] = lane == j ? 1.0 : 0.0;
+  }
+  for (int k = 0; k < nbk; ++k) {
+    double *col = sm.col[k & 1], *cols = sm.cols[k & 1];
+    const int ku = k >> 3;
+    if ((k & 7) == warp) {
+      double v = 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u == ku) v = a[u];
+      double d = __shfl_sync(0xffffffffu, v, k);
+      if (!(d > 0.0)) {  // not positive: reported, replaced by 1 so that the sweep stays finite
+        if (lane == 0) *bad = 1;
+        d = 1.0;
+        if (lane == k) v = 1.0;
+      }
+      const double rs = rsqrt(d);
+      v *= rs;  // lane k: the pivot d / sqrt(d)
+      if (lane >= k) sm.D[lane][k] = v;
+      col[lane] = lane > k ? v : 0.0;
+      cols[lane] = lane > k ? v * rs : rs;
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    const double l = col[lane], ls = lane > k ? cols[lane] : 0.0;
+    if (lane == k) rsl = cols[k];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = warp + 8 * u;
+      if (j > k && j < nbk) a[u] = fma(-l, col[j], a[u]);
+      if (j <= k) m[u] = fma(-ls, __shfl_sync(0xffffffffu, m[u], k), m[u]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int j = warp + 8 * u;
+    sm.M[lane][j] = (lane < nbk && j < nbk && lane >= j) ? m[u] * rsl : 0.0;
+  }
+}
+
+// The digits of L_bb^{-1} (rows j < 32, K = 32) into the panel's B operand in shared memory, and its row exponents.
+__device__ __forceinline__ void dig_inverse(const PivotSmem& sm, uint8_t* bpan, int* EXB) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, q = lane & 3;
+  if (warp >= 4) return;
+  const int i = warp * 8 + (lane >> 2);
+  double v[8];
+  uint32_t mx = 0;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    v[e] = sm.M[i][q * 8 + e];
+    mx = max(mx, (uint32_t)__double2hiint(v[e]) & 0x7fffffffu);
+  }
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  const int ex = dig_exponent(mx);
+  if (q == 0) EXB[i] = ex;
+  uint64_t w[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[e], ex);
+#pragma unroll
+  for (int p = 0; p < kDig; ++p)
+    *reinterpret_cast<uint4*>(bpan + p * kCB + i * 64 + ((q ^ ((i >> 1) & 3)) << 4)) =
+        make_uint4(dig_pair(w[0], w[1], p), dig_pair(w[2], w[3], p), dig_pair(w[4], w[5], p),
+                   dig_pair(w[6], w[7], p));
+}
+
+// Assemble a front in global memory: the f x w panel Ls (column-major, in the factor's storage) and the r x r bottom
+// block W, from the K entries, the fixing-DOF penalty rho and the children's update blocks (stack or hand-over slots),
+// the work dealt to all threads of the cluster.
+__device__ __forceinline__ void assemble_cluster(const DevPlan& P, const SubInfo& S, int s, const double* K, double* L,
+                                                 double rho, double* W, const double* stack, const double* hand,
+                                                 int gtid, int gthreads) {
+  const int gs = S.sn0 + s;
+  const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
+  double* Ls = L + P.Lofs[gs];
+  for (int64_t idx = gtid; idx < (int64_t)f * w; idx += gthreads) Ls[idx] = 0.0;
+  for (int64_t idx = gtid; idx < (int64_t)r * r; idx += gthreads) W[idx] = 0.0;
+  cl_sync();
+  for (int64_t k = P.kmap_off[gs] + gtid; k < P.kmap_off[gs + 1]; k += gthreads) L[P.kmap_dst[k]] = K[P.kmap_src[k]];
+  cl_sync();
+  for (int k = gtid; k < S.nfix; k += gthreads)
+    if (P.fix_sn[S.fix0 + k] == s) {
+      double* d = L + P.fix_pos[S.fix0 + k];
+      *d = __ldcg(d) + rho;
+    }
+  for (int c = P.ch_off[gs]; c < P.ch_off[gs + 1]; ++c) {
+    const int gc = S.sn0 + P.ch_list[c];
+    const int rc = P.sn_r[gc];
+    const double* U = child_update(P, gc, stack, nullptr, hand);
+    const int* rl = P.rel + P.rel_off[gc];
+    cl_sync();
+    // four elements per thread and step, their loads issued before their read-modify-writes (distinct targets)
+    const int64_t n = (int64_t)rc * rc;
+    for (int64_t base = gtid; base < n; base += 4 * (int64_t)gthreads) {
+      double* dst[4];
+      double v[4], cur[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t idx = base + (int64_t)u * gthreads;
+        dst[u] = nullptr;
+        if (idx < n) {
+          const int b = (int)(idx / rc), a = (int)(idx - (int64_t)b * rc);
+          if (a >= b) {
+            const int ra = rl[a], rb = rl[b];
+            v[u] = __ldcg(U + idx);
+            dst[u] = rb < w ? Ls + (int64_t)rb * f + ra : W + (int64_t)(rb - w) * r + (ra - w);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) cur[u] = dst[u] ? __ldcg(dst[u]) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (dst[u]) *dst[u] = cur[u] + v[u];
+    }
+  }
+  cl_sync();
+}
+
+// Items: one task of the plan's split (subdomain, task, global task id, parent's global task id), children before
+// parents.  The fronts' children outside the large set handed their update blocks over (chol_kernel ran first); a
+// large child task's block comes from its hand-over slot after a bounded wait on the task's counter of finished large
+// children (tdone), others through the cluster's stack.  Flags as in chol_kernel.
+__global__ void __launch_bounds__(kCT, 1)
+    chol_tc_kernel(DevPlan P, const int4* items, int nitems, int* queue, int* tdone, double* hand_all, double* ws,
+                   int64_t ws_stride, int64_t front_sz, char* scratch, int64_t scratch_stride, int flags,
+                   int* status) {
+  extern __shared__ uint8_t ct_raw[];
+  uint8_t* ring = ct_raw + ((1024u - (smem_u32(ct_raw) & 1023u)) & 1023u);
+  PivotSmem& sm = *reinterpret_cast<PivotSmem*>(ring);
+  __shared__ uint64_t full[kCStages], empty[kCStages], accf[2], acce[2], drain;
+  __shared__ uint32_t tmem_s;
+  __shared__ volatile int abort_s;
+  __shared__ int bad, item_s, EXB[kNB];
+  __shared__ double red[kCT / 32];
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  const int rank = (int)cl_rank(), C = (int)cl_size(), cluster = blockIdx.x / C;
+  const int gtid = rank * kCT + tid, gthreads = C * kCT;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int k = 0; k < kCStages; ++k) {
+      mbar_init(&full[k], 1);
+      mbar_init(&empty[k], 1);
+    }
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(&accf[k], 1);
+      mbar_init(&acce[k], 8);
+    }
+    mbar_init(&drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    abort_s = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  CtState st{};
+  st.ring = ring;
+  st.bpan = ring + kCStages * kCStage;
+  st.full = full;
+  st.empty = empty;
+  st.accf = accf;
+  st.acce = acce;
+  st.drain = &drain;
+  st.abort = &abort_s;
+  st.tmem = tmem_s;
+  double* W = ws + (int64_t)cluster * ws_stride;
+  double* stack = W + front_sz;
+  char* SL = scratch + (int64_t)cluster * scratch_stride;
+  for (;;) {
+    cl_sync();
+    if (rank == 0 && tid == 0) {
+      int it = atomicAdd(queue, 1);
+      if (it < nitems && P.task_nbig[items[it].z] > 0) {
+        // the large child tasks were taken before this one and are running: wait for them (bounded)
+        const int4 item = items[it];
+        int ok = 0;
+        for (int i = 0; i < (1 << 26); ++i) {
+          if (*(volatile int*)(tdone + item.z) >= P.task_nbig[item.z]) {
+            ok = 1;
+            break;
+          }
+          __nanosleep(64);
+        }
+        __threadfence();
+        if (!ok) {
+          atomicOr(status, kStatTimeout);
+          if (item.w >= 0) atomicAdd(tdone + item.w, 1);  // no cascade of waits above a failure
+          it = -1;
+        }
+      }
+      for (int c = 0; c < C; ++c)
+        asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.s32 [a], %2;\n\t}" ::"r"(
+                         smem_u32(&item_s)),
+                     "r"(c), "r"(it)
+                     : "memory");
+    }
+    if (tid == 0) bad = 0;
+    cl_sync();
+    const int it = item_s;
+    if (it >= nitems) break;
+    if (it < 0) continue;
+    const int4 item = items[it];
+    const int si = item.x, task = item.y;
+    const SubInfo S = P.sub[si];
+    const double* K = P.Kval + S.Kval;
+    double* L = P.L + S.L;
+    double* hand = hand_all + S.hbase;
+    double mx = 0.0;  // rho = max diag K_i, as in chol_kernel
+    for (int i = tid; i < S.n; i += kCT) mx = fmax(mx, K[P.diag_src[S.diag0 + i]]);
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();
+    double rho = red[0];
+    for (int k = 1; k < kCT / 32; ++k) rho = fmax(rho, red[k]);
+    if (flags & kCholNoReg) rho = 0.0;
+    for (int s = 0; s < S.nsn; ++s) {
+      const int gs = S.sn0 + s;
+      if (!P.sn_big[gs] || P.sn_task[gs] != task) continue;
+      const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
+      double* Ls = L + P.Lofs[gs];
+      assemble_cluster(P, S, s, K, L, rho, W, stack, hand, gtid, gthreads);
+      if (!((flags & kCholStopRoot) && s == S.nsn - 1)) {
+        for (int kB = 0; kB < w; kB += kCBlk) {
+          const int kE = min(w, kB + kCBlk);
+          for (int kb = kB; kb < kE; kb += kNB) {
+            const int ke = min(kE, kb + kNB), nbk = ke - kb, n = f - ke;
+            const int npad = (n + kCM - 1) / kCM * kCM, ntm = npad / kCM;
+            char *S1 = SL, *S2 = SL + (int64_t)npad * 512;  // the panel's digits before and after the solve
+            int* EX1 = reinterpret_cast<int*>(SL + (int64_t)npad * 1024);
+            int* EX2 = EX1 + npad;
+            // the pivot block (every CTA), and the digits of this CTA's panel rows
+            for (int idx = tid; idx < kNB * kNB; idx += kCT) {
+              const int i = idx % kNB, j = idx / kNB;
+              sm.D[i][j] = (i < nbk && j <= i) ? __ldcg(Ls + (int64_t)(kb + j) * f + kb + i) : 0.0;
+            }
+            __syncthreads();
+            pivot_block(sm, nbk, &bad);
+            // warps 8-11 start on the panel rows while the others factor the block
+            if (warp >= 8)
+              for (int tm = rank; tm < ntm; tm += C)
+                dig_rows<1>(Ls + (int64_t)kb * f + ke, f, n, nbk, tm * kCM, tm * kCM + kCM, S1, 1, npad, EX1,
+                            warp - 8, 4);
+            __syncthreads();
+            dig_inverse(sm, st.bpan, EXB);
+            double lb[3];
+            for (int u = 0; u < 3; ++u) {
+              const int idx = tid + u * kCT;
+              lb[u] = idx < kNB * kNB ? sm.D[idx % kNB][idx / kNB] : 0.0;
+            }
+            dig_product<true>(st, S1, EX1, EXB, n, 1, rank, C, ntm, 1, Ls, f, w, W, r, ke, kb, nbk);
+            if (ke < kE)
+              for (int tm = rank; tm < ntm; tm += C)
+                dig_rows<1>(Ls + (int64_t)kb * f + ke, f, n, nbk, tm * kCM, tm * kCM + kCM, S2, 1, npad, EX2, warp,
+                            kCT / 32);
+            cl_sync();
+            if (rank == 0)  // every CTA has read the block
+              for (int u = 0; u < 3; ++u) {
+                const int idx = tid + u * kCT, i = idx % kNB, j = idx / kNB;
+                if (idx < kNB * kNB && i < nbk && j <= i) Ls[(int64_t)(kb + j) * f + kb + i] = lb[u];
+              }
+            if (ke < kE) {
+              const int ntn = (kE - ke + 63) / 64;
+              int ntile = 0;
+              for (int tm = 0; tm < ntm; ++tm) ntile += min(2 * (tm + 1), ntn);
+              dig_product<false>(st, S2, EX2, nullptr, n, 1, rank, C, ntile, ntn, Ls, f, w, W, r, ke, 0, kE - ke);
+              cl_sync();
+            }
+          }
+          if (kE < f) {
+            const int n = f - kE, K2 = kE - kB, nck = (K2 + 31) / 32;
+            const int npad = (n + kCM - 1) / kCM * kCM, ntm = npad / kCM, ntn = (n + 63) / 64;
+            int* EX = reinterpret_cast<int*>(SL + (int64_t)npad * 64 * kDig * nck);
+            for (int q = (rank * (kCT / 32) + warp) * 8; q < npad; q += C * (kCT / 32) * 8)
+              dig_rows<4>(Ls + (int64_t)kB * f + kE, f, n, K2, q, q + 8, SL, nck, npad, EX, 0, 1);
+            cl_sync();
+            int ntile = 0;
+            for (int tm = 0; tm < ntm; ++tm) ntile += min(2 * (tm + 1), ntn);
+            dig_product<false>(st, SL, EX, nullptr, n, nck, rank, C, ntile, ntn, Ls, f, w, W, r, kE, 0, n);
+            cl_sync();
+          }
+        }
+      }
+      cl_sync();
+      if (P.sn_parent[gs] >= 0) {
+        double* Uout = P.sn_hoff[gs] >= 0 ? hand + P.sn_hoff[gs] : stack + P.upd_ofs[gs];
+        for (int64_t idx = gtid; idx < (int64_t)r * r; idx += gthreads) Uout[idx] = __ldcg(W + idx);
+      }
+      cl_sync();
+    }
+    if (tid == 0 && bad) atomicOr(status, kStatNotSPD);
+    if (rank == 0 && tid == 0 && item.w >= 0) {
+      __threadfence();  // the task's factor panels and hand-over block (ordered by the barrier above) before the count
+      atomicAdd(tdone + item.w, 1);
+    }
+  }
+  if (tid == 0 && abort_s) atomicOr(status, kStatTimeout);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(st.tmem), "r"(512));
+  }
+}
+
+}  // namespace
+
+// CTAs per cluster for nsub subdomains with large fronts on nsm SMs
+int chol_tc_cluster(int nsub, int nsm) {
+  int c = 1;
+  while (c < 8 && 2 * c * nsub <= nsm) c *= 2;
+  return c;  // 8 is the portable limit
+}
+
+void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue, int* tdone, double* hand,
+                    double* ws, int64_t ws_stride, int64_t front_sz, void* scratch, int64_t scratch_stride,
+                    int clusters, int cluster, int* status, cudaStream_t st, int flags) {
+  if (nitems <= 0) return;
+  cudaFuncSetAttribute(chol_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCDyn);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(std::min(clusters, nitems) * cluster));
+  cfg.blockDim = dim3(kCT);
+  cfg.dynamicSmemBytes = kCDyn;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, chol_tc_kernel, P, items, nitems, queue, tdone, hand, ws, ws_stride, front_sz,
+                     (char*)scratch, scratch_stride, flags, status);
+}
+
+int64_t chol_tc_scratch(int fmax) {
+  const int64_t npad = (fmax + kCM - 1) / kCM * kCM;
+  return (npad * (2 * kDig * kCBlk + 8) + 127) / 128 * 128;
+}
+
+}  // namespace feti

@@ -14,6 +14,7 @@
 
 #include <cuda_bf16.h>
 
+#include "chol_common.cuh"
 #include "common.cuh"
 #include "kernels.h"
 #include "symbolic.h"
@@ -21,14 +22,6 @@
 
 namespace feti {
 namespace {
-
-__device__ __forceinline__ int pop_item(int* queue) {
-  __shared__ int item;
-  __syncthreads();
-  if (threadIdx.x == 0) item = atomicAdd(queue, 1);
-  __syncthreads();
-  return item;
-}
 
 // acc[u][v] += sum_k A[k][r0 + 16u] * B[k][c0 + 16v] for u < NU, v < NV
 // (skipping v > u on diagonal tiles).  NU / NV are warp-uniform counts of
@@ -178,7 +171,6 @@ __device__ void factor_front(Smem& sm, double* Ls, int f, int w, double* W, int 
     for (int ti = 0; ti < T; ++ti) {
       for (int tj = 0; tj <= ti; ++tj) {
         const int ri = i0 + ti * kT, cj = i0 + tj * kT;
-        if (cj >= ce) break;
         for (int idx = tid; idx < nbk * kT; idx += kThreads) {
           int x = idx % kT, k = idx / kT;
           const double* col = Ls + (int64_t)(kb + k) * f;
@@ -196,7 +188,7 @@ __device__ void factor_front(Smem& sm, double* Ls, int f, int w, double* W, int 
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             int j = cj + tx + 16 * v;
-            if (u < nu && v < nv && i < f && j <= i && j < ce) {
+            if (u < nu && v < nv && i < f && j <= i) {
               double* p = (j < w) ? Ls + (int64_t)j * f + i : W + (int64_t)(j - w) * r + (i - w);
               *p -= acc[u][v];
             }
@@ -228,14 +220,6 @@ template <int TEAM>
 __device__ __forceinline__ void team_sync() {
   if constexpr (TEAM == 32) __syncwarp();
   else __syncthreads();
-}
-
-// Update block of child gc: a small child's lives in the CTA's small region, a split root's (a child factored
-// by another task) in its hand-over slot, others on the stack.
-__device__ __forceinline__ const double* child_update(const DevPlan& P, int gc, const double* stack,
-                                                      const double* smallreg, const double* hand) {
-  if (hand && P.sn_hoff[gc] >= 0) return hand + P.sn_hoff[gc];
-  return P.sn_small[gc] ? smallreg + P.usm_ofs[gc] : stack + P.upd_ofs[gc];
 }
 
 // Assemble front gs (K entries, rho on fixing DOFs, children's update blocks),
@@ -518,441 +502,6 @@ __global__ void __launch_bounds__(kThreads, 4) chol_kernel(DevPlan P, const int4
         atomicAdd(tdone + item.w, 1);
       }
     }
-  }
-}
-
-// ---------------------------------------------------------------- tensor-core Cholesky of the large fronts
-//
-// The fronts at least big_f wide and their ancestors (the top of each supernodal tree) are factored by
-// chol_tc_kernel after chol_kernel has done everything below them.  A front's w own columns go in blocks of
-// 128: the block's columns are eliminated on the FP64 pipe (32-column steps, their updates applied to the
-// block's own columns only), and then the trailing matrix C = front[kE:, kE:] (its lower triangle, in Ls and W)
-// takes the block's rank-128 update C -= A A^T, A = Ls[kE:, kB:kE], on the tensor cores by exact slicing of
-// FP64 into bf16 integers (the Ozaki scheme): each row i of A is scaled by a power of two 2^(e_i - 6) with
-// e_i the largest exponent in the row, and its 63 leading fixed-point bits are cut into 9 signed 7-bit
-// integers s_p (p = 0 most significant), each exact in bf16, so A_ik = 2^(e_i - 6) sum_p s_p,ik 2^(-7p) up to
-// 2^(e_i - 62).  The products of slices p, q (p + q <= 8, 45 pairs) are summed over K = 128 on the tensor cores
-// with FP32 accumulation, one TMEM accumulator per d = p + q <= 7 (the d = 8 products into the d = 7 one, their
-// B slices scaled by 2^-7).  For d <= 6 every partial sum is an integer below (d + 1) 128 127^2 < 2^24, so those
-// FP32 sums are exact; the d = 7 one lies 2^-49 below the leading scale.  The epilogue combines them,
-// sum_k A_ik A_jk = 2^(e_i + e_j - 40) (sum_{d <= 4} acc_d 2^(7 (4 - d)) + sum_{d >= 5} acc_d 2^(7 (4 - d))),
-// the first sum exactly in 64-bit integers, the small rest in FP32 (its rounding below 2^-53 of K sigma_i sigma_j,
-// sigma = 2^(e + 1)), and applies C_ij -= that with one FP64 FMA.  The dropped pairs (p + q >= 9) and the cut
-// bits add below K 2^(e_i + e_j - 58): the whole error stays below K 2^-52 sigma_i sigma_j, inside FP64's own
-// normwise bound for the same dot product (tests/test_slicing_model.py checks the model on the host).
-constexpr int kOzS = 9;                              // slices of 7 bits
-constexpr int kOzAcc = 8;  // accumulators: d = 0 .. 6, and d = 7 with the d = 8 products (B slices scaled by 2^-7)
-constexpr int kOzK = 128;                            // columns of one panel block (K of one update)
-constexpr int kOzKC = 32;                            // K per stage: one 64-byte swizzled row per operand row
-constexpr int kOzN = 32;                             // C tile: 128 rows x 32 columns (9 accumulators x 32 TMEM columns)
-constexpr int kOzM = 128;                            // rows of a C tile (the MMA M)
-constexpr int kOzOpA = kOzM * 64, kOzOpB = kOzN * 64;
-constexpr int kOzStage = kOzS * (kOzOpA + 2 * kOzOpB);  // 108 KB: A slices, B slices, B slices x 2^-7 of a chunk
-constexpr int kOzStages = 2;
-constexpr int kOzSetCols = kOzAcc * kOzN;               // TMEM columns of one accumulator set (two sets)
-constexpr int kCholTcDyn = 1024 + kOzStages * kOzStage;
-static_assert(sizeof(Smem) <= kOzStages * kOzStage, "the FP64 steps' buffers alias the stage ring");
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(taddr));
-}
-
-// Layout of the slices in the per-CTA scratch: for slice p (p >= 9: slice p - 9 times 2^-7) and 32-deep chunk c,
-// the rows one after another
-// (npad = rows rounded up to 128), each row 32 bf16 = 64 bytes with its four 16-byte pieces already in the
-// 64-byte swizzle of an 8-row atom (piece q of row r at q ^ ((r >> 1) & 3)): any 8-row-aligned run of rows of
-// one (p, c) is a ready MMA operand, loaded by one bulk copy.
-__device__ __forceinline__ int64_t oz_row(int p, int c, int npad, int r) {
-  return ((int64_t)(p * (kOzK / kOzKC) + c) * npad + r) * kOzKC;
-}
-
-// Slices of A = Ls[i0 + i, kb0 + k] (i < n = f - i0, k < K = ke0 - kb0 <= 128; zero for k >= K and for the
-// padding rows): row exponent EX[i] and the slices in the layout above.  A warp takes 32 rows (lane = row: the
-// loads of one column are contiguous).
-__device__ void oz_slice(const double* Ls, int f, int i0, int kb0, int ke0, uint16_t* SL, int* EX) {
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int n = f - i0, K = ke0 - kb0, npad = (n + kOzM - 1) / kOzM * kOzM;
-  const int nch = (K + kOzKC - 1) / kOzKC;  // the chunks the update reads
-  for (int rb = warp * 32; rb < npad; rb += kThreads) {
-    const int i = rb + lane;
-    const bool ok = i < n;
-    int e = -1074;
-    for (int k = 0; k < K; ++k) {
-      const double x = ok ? Ls[(int64_t)(kb0 + k) * f + i0 + i] : 0.0;
-      const int be = (int)((__double_as_longlong(x) >> 52) & 0x7FF);
-      if (be) e = max(e, be - 1023);
-    }
-    if (ok) EX[i] = e;
-    for (int kc = 0; kc < nch * kOzKC; kc += 8) {
-      uint32_t pk[kOzS][4], pks[kOzS][4];
-#pragma unroll
-      for (int kk = 0; kk < 8; kk += 2) {
-        int sv[2][kOzS];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = kc + kk + h;
-          const double x = (ok && k < K) ? Ls[(int64_t)(kb0 + k) * f + i0 + i] : 0.0;
-          const long long b = __double_as_longlong(x);
-          const int be = (int)((b >> 52) & 0x7FF);
-          unsigned long long F = 0;
-          if (be) {
-            const unsigned long long m = (unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | (1ULL << 52);
-            const int sh = (be - 1023) - e + 10;  // <= 10: F < 2^63
-            F = sh >= 0 ? (m << sh) : (sh > -64 ? (m >> -sh) : 0ULL);
-          }
-          const bool neg = b < 0;
-#pragma unroll
-          for (int p = 0; p < kOzS; ++p) {
-            const int v = (int)((F >> (56 - 7 * p)) & 127ULL);
-            sv[h][p] = neg ? -v : v;
-          }
-        }
-#pragma unroll
-        for (int p = 0; p < kOzS; ++p) {
-          const uint32_t lo = __bfloat16_as_ushort(__float2bfloat16_rn((float)sv[0][p]));
-          const uint32_t hi = __bfloat16_as_ushort(__float2bfloat16_rn((float)sv[1][p]));
-          pk[p][kk / 2] = lo | (hi << 16);
-          // the same integer times 2^-7 (exact in bf16): the B operand of the d = 8 products
-          const uint32_t los = __bfloat16_as_ushort(__float2bfloat16_rn((float)sv[0][p] * 0x1p-7f));
-          const uint32_t his = __bfloat16_as_ushort(__float2bfloat16_rn((float)sv[1][p] * 0x1p-7f));
-          pks[p][kk / 2] = los | (his << 16);
-        }
-      }
-      const int c = kc / kOzKC, q = (kc % kOzKC) / 8;
-#pragma unroll
-      for (int p = 0; p < kOzS; ++p) {
-        const int64_t o = ((q ^ ((i >> 1) & 3)) * 8);
-        *reinterpret_cast<uint4*>(SL + oz_row(p, c, npad, i) + o) = make_uint4(pk[p][0], pk[p][1], pk[p][2], pk[p][3]);
-        *reinterpret_cast<uint4*>(SL + oz_row(kOzS + p, c, npad, i) + o) =
-            make_uint4(pks[p][0], pks[p][1], pks[p][2], pks[p][3]);
-      }
-    }
-  }
-}
-
-// the row exponents follow the slices of an n-row A
-__device__ __forceinline__ int* oz_ex(uint16_t* SL, int n) {
-  const int npad = (n + kOzM - 1) / kOzM * kOzM;
-  return reinterpret_cast<int*>(SL + oz_row(2 * kOzS, 0, npad, 0));
-}
-
-__device__ __forceinline__ void oz_expect(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void oz_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-// C -= A A^T on the lower triangle of the trailing matrix (rows [i0, f), columns [i0, ce); columns < w in Ls,
-// the others in W) from the slices.  Tiles of 128 rows x 32 columns with a column block not right of the row
-// block.  Warp 0 (one thread) loads each 32-deep chunk with 27 bulk copies (A slices, B slices, scaled B slices)
-// completing on the stage's "full" mbarrier and, one chunk behind, issues its 45 x 2 MMAs (slice pair p, q into
-// accumulator min(p + q, 7) of the tile's accumulator set: TMEM columns 256 (tile mod 2) + 32 accumulator) and
-// commits them to the stage's "empty" mbarrier, and after a tile's last chunk to the set's "accumulators full"
-// mbarrier.  Warps 4-7 combine the accumulators of each tile (epilogue above) while warp 0 already multiplies
-// the next tile into the other set, and release the set on its "accumulators empty" mbarrier (one arrival per
-// warp).  tcnt counts the CTA's tiles (the sets' phases).  Every wait is bounded.
-__device__ bool oz_update(uint8_t* ring, uint64_t* gbar, uint64_t* fbar, uint64_t* afull, uint64_t* aempty,
-                          uint32_t tmem, uint32_t& g, uint32_t& tcnt, int* abort_flag, const uint16_t* SL,
-                          const int* EX, int n, int K, double* Ls, int f, int w, double* W, int r, int i0, int ce) {
-  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  volatile int* abortv = abort_flag;
-  const int ntm = (n + kOzM - 1) / kOzM, npad = ntm * kOzM;
-  const int nce = ce - i0;               // columns of C
-  constexpr int kTnPerTm = kOzM / kOzN;  // column blocks per row block
-  int ntile = 0;  // tiles (tm, tn) with a column block not right of the row block: tn < (tm + 1) kTnPerTm
-  const int ntnmax = (nce + kOzN - 1) / kOzN;
-  for (int tm = 0; tm < ntm; ++tm) ntile += min((tm + 1) * kTnPerTm, ntnmax);
-  const int nck = (K + kOzKC - 1) / kOzKC;
-  const int total = ntile * nck;
-  if (total == 0) return true;
-  const uint32_t sb0 = smem_u32(ring);
-  const uint32_t g0 = g, t0 = tcnt;
-  constexpr uint32_t idesc = idesc_m128(1u, (uint32_t)kOzN);
-  auto tile_of = [&](int t, int& tm, int& tn) {
-    tm = 0;
-    for (;;) {
-      const int c = min((tm + 1) * kTnPerTm, ntnmax);
-      if (t < c) break;
-      t -= c;
-      ++tm;
-    }
-    tn = t;
-  };
-  __syncthreads();  // the slices are written and the ring's earlier generic use is over
-  if (warp == 0) {
-    if (lane == 0) {
-      int last_load = -1, last_mma = -1;
-      auto load = [&](int q) {  // the 27 bulk copies of chunk q into its stage
-        last_load = q;
-        const uint32_t st = (g0 + q) % kOzStages, sbase = sb0 + st * kOzStage;
-        const uint32_t full = smem_u32(&fbar[st]);
-        const int ck = q % nck;
-        int tm, tn;
-        tile_of(q / nck, tm, tn);
-        oz_expect(full, (uint32_t)kOzStage);
-#pragma unroll 1
-        for (int p = 0; p < kOzS; ++p) {
-          oz_bulk(sbase + p * kOzOpA, SL + oz_row(p, ck, npad, tm * kOzM), kOzOpA, full);
-          oz_bulk(sbase + kOzS * kOzOpA + p * kOzOpB, SL + oz_row(p, ck, npad, tn * kOzN), kOzOpB, full);
-          oz_bulk(sbase + kOzS * (kOzOpA + kOzOpB) + p * kOzOpB, SL + oz_row(kOzS + p, ck, npad, tn * kOzN), kOzOpB,
-                  full);
-        }
-      };
-      asm volatile("fence.proxy.async.global;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bool ok = true;
-      load(0);
-      for (int j = 0; j < total && ok; ++j) {
-        const int ck = j % nck, tile = j / nck;
-        const uint32_t st = (g0 + j) % kOzStages, tg = t0 + tile, set = tg & 1;
-        const int q = j + 1;  // the next chunk: its stage is free once the MMAs of the chunk that used it are done
-        if (q < total) {
-          if (q >= kOzStages) {
-            const uint32_t gp = g0 + q - kOzStages;
-            ok = mbar_wait(smem_u32(&gbar[gp % kOzStages]), (gp / kOzStages) & 1);
-          }
-          if (ok) load(q);
-        }
-        // a tile's first chunk: its accumulator set is free once the epilogue of the tile two before is done
-        if (ok && ck == 0 && tg >= 2) ok = mbar_wait(smem_u32(&aempty[set]), ((tg >> 1) - 1) & 1);
-        if (ok) ok = mbar_wait(smem_u32(&fbar[st]), ((g0 + j) / kOzStages) & 1);
-        if (ok && *abortv) ok = false;
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sA = sb0 + st * kOzStage, sB = sA + kOzS * kOzOpA, sBs = sB + kOzS * kOzOpB;
-        const uint32_t acc0 = tmem + set * kOzSetCols;
-#pragma unroll 1
-        for (int p = 0; p < kOzS; ++p)
-#pragma unroll 1
-          for (int qq = 0; qq < kOzS - p; ++qq) {
-            const bool d8 = p + qq == kOzAcc;  // the d = 8 pairs go into accumulator 7 with B scaled by 2^-7
-            const uint32_t acc = acc0 + (uint32_t)((d8 ? kOzAcc - 1 : p + qq) * kOzN);
-            const uint32_t bq = (d8 ? sBs : sB) + qq * kOzOpB;
-#pragma unroll
-            for (int kk = 0; kk < kOzKC / 16; ++kk)
-              mma_f16(acc, sw64_desc(sA + p * kOzOpA + kk * 32), sw64_desc(bq + kk * 32), idesc,
-                      (ck > 0 || p > 0 || kk > 0 || d8) ? 1u : 0u);
-          }
-        mma_commit(smem_u32(&gbar[st]));
-        if (ck == nck - 1) mma_commit(smem_u32(&afull[set]));
-        last_mma = j;
-      }
-      if (!ok) {
-        *abortv = 1;
-        // wait (bounded) for the last copies and MMAs issued
-        if (last_mma >= 0) {
-          const uint32_t gq = g0 + last_mma;
-          mbar_wait(smem_u32(&gbar[gq % kOzStages]), (gq / kOzStages) & 1);
-        }
-        if (last_load > last_mma) {
-          const uint32_t gq = g0 + last_load;
-          mbar_wait(smem_u32(&fbar[gq % kOzStages]), (gq / kOzStages) & 1);
-        }
-      }
-    }
-    __syncwarp();
-  } else if (warp >= 4) {
-    const int q4 = warp % 4;  // TMEM lane quarter: rows q4 * 32 .. + 31 of the tile
-    for (int tile = 0; tile < ntile; ++tile) {
-      const uint32_t tg = t0 + tile, set = tg & 1;
-      int ok = 1;
-      if (lane == 0) ok = !*abortv && mbar_wait(smem_u32(&afull[set]), (tg >> 1) & 1);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
-        if (lane == 0) *abortv = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int tm, tn;
-      tile_of(tile, tm, tn);
-      const int ri = tm * kOzM + q4 * 32 + lane;  // row of C (relative to i0)
-      const int gi = i0 + ri;
-      const int ei = ri < n ? EX[ri] : 0;
-#pragma unroll 1
-      for (int cg = 0; cg < kOzN / 8; ++cg) {
-        const int cbase = tn * kOzN + cg * 8;  // first column of this group (relative to i0)
-        uint32_t a[kOzAcc][8];
-#pragma unroll
-        for (int d = 0; d < kOzAcc; ++d)
-          tmem_ld8(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(set * kOzSetCols + d * kOzN + cg * 8), a[d]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (ri < n) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int cj = cbase + e, gj = i0 + cj;
-            if (cj < nce && gj <= gi) {
-              long long I = 0;
-#pragma unroll
-              for (int d = 0; d <= 4; ++d)
-                I += (long long)__float2int_rn(__uint_as_float(a[d][e])) << (7 * (4 - d));
-              float small = 0.f;  // sum_{d >= 5} acc_d 2^(-7 (d - 4)), Horner from the smallest
-#pragma unroll
-              for (int d = kOzAcc - 1; d >= 5; --d) small = (small + __uint_as_float(a[d][e])) * 0x1p-7f;
-              const double t = (double)I + (double)small;
-              const int ex = ei + EX[cj] - 40;
-              const double sc = ex >= -1022 ? __longlong_as_double((long long)(ex + 1023) << 52) : 0.0;
-              double* pc = gj < w ? Ls + (int64_t)gj * f + gi : W + (int64_t)(gj - w) * r + (gi - w);
-              *pc = fma(-t, sc, *pc);
-            }
-          }
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&aempty[set])) : "memory");
-    }
-  }
-  __syncthreads();  // every role has finished this update
-  g = g0 + total;
-  tcnt = t0 + ntile;
-  return !*abortv;
-}
-
-// The large fronts (P.sn_big), one task of the plan's split per item (subdomain, task, global task id, parent's
-// global task id), children before parents; one CTA per SM (the stage ring takes 217 KB of shared memory and
-// the two accumulator sets all 512 TMEM columns), all resident.  The fronts' children outside the set
-// handed their update blocks over (chol_kernel ran first); a large child task's block comes from its hand-over
-// slot after a bounded wait on the task's counter of finished large children (tdone), others through the
-// CTA's stack as in chol_kernel.  The same flags as chol_kernel.
-__global__ void __launch_bounds__(kThreads, 1) chol_tc_kernel(DevPlan P, const int4* items, int nitems, int* queue,
-                                                            int* tdone, double* hand_all, double* ws,
-                                                            int64_t ws_stride, int64_t front_sz, uint16_t* slices,
-                                                            int64_t slice_stride, int flags, int* status) {
-  extern __shared__ uint8_t oz_raw[];
-  uint8_t* ring = oz_raw + ((1024u - (smem_u32(oz_raw) & 1023u)) & 1023u);
-  Smem& sm = *reinterpret_cast<Smem*>(ring);  // the FP64 steps' buffers (never in use with the ring)
-  __shared__ uint64_t gbar[kOzStages], fbar[kOzStages];  // per stage: MMAs done ("empty"), copies landed ("full")
-  __shared__ uint64_t afull[2], aempty[2];  // per accumulator set: tile multiplied / epilogue done
-  __shared__ uint32_t tmem_s;
-  __shared__ int abort_s, bad;
-  __shared__ double red[kThreads / 32];
-  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
-                 "r"(512));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    for (int k = 0; k < kOzStages; ++k) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&gbar[k])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&fbar[k])));
-    }
-    for (int k = 0; k < 2; ++k) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&afull[k])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&aempty[k])));  // the 4 epilogue warps
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    abort_s = 0;
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_s;
-  uint32_t g = 0, tcnt = 0;
-  double* W = ws + (int64_t)blockIdx.x * ws_stride;
-  double* stack = W + front_sz;
-  uint16_t* SL = slices + (int64_t)blockIdx.x * slice_stride;
-  for (;;) {
-    const int it = pop_item(queue);
-    if (it >= nitems) break;
-    const int4 item = items[it];
-    const int si = item.x, task = item.y;
-    const SubInfo S = P.sub[si];
-    const double* K = P.Kval + S.Kval;
-    double* L = P.L + S.L;
-    double* hand = hand_all + S.hbase;
-    if (tid == 0) {
-      bad = 0;
-      // the large child tasks were taken before this one and are running: wait for them (bounded)
-      int ok = 1;
-      if (P.task_nbig[item.z] > 0) {
-        ok = 0;
-        for (int i = 0; i < (1 << 26); ++i) {
-          if (*(volatile int*)(tdone + item.z) >= P.task_nbig[item.z]) {
-            ok = 1;
-            break;
-          }
-          __nanosleep(64);
-        }
-      }
-      __threadfence();
-      if (!ok) {
-        atomicOr(status, kStatTimeout);
-        bad = 2;
-        if (item.w >= 0) atomicAdd(tdone + item.w, 1);  // no cascade of waits above a failure
-      }
-    }
-    __syncthreads();
-    if (bad == 2) continue;
-    double mx = 0.0;  // rho = max diag K_i, as in chol_kernel
-    for (int i = tid; i < S.n; i += kThreads) mx = fmax(mx, K[P.diag_src[S.diag0 + i]]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) red[warp] = mx;
-    __syncthreads();
-    double rho = red[0];
-    for (int k = 1; k < kThreads / 32; ++k) rho = fmax(rho, red[k]);
-    if (flags & kCholNoReg) rho = 0.0;
-    __syncthreads();
-    for (int s = 0; s < S.nsn && !abort_s; ++s) {
-      const int gs = S.sn0 + s;
-      if (!P.sn_big[gs] || P.sn_task[gs] != task) continue;
-      const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
-      double* Ls = L + P.Lofs[gs];
-      assemble_tiled(P, S, s, K, L, rho, W, stack, nullptr, hand);
-      __syncthreads();
-      if (!((flags & kCholStopRoot) && s == S.nsn - 1)) {
-        bool okf = true;
-        for (int kB = 0; kB < w && okf; kB += kOzK) {
-          const int kE = min(w, kB + kOzK);
-          // the block's 32-column steps: the pivot block and the panel below it on the FP64 pipe, the rank-32
-          // update of the block's later columns on the tensor cores
-          for (int kb = kB; kb < kE && okf; kb += kNB) {
-            const int ke = min(kE, kb + kNB);
-            factor_front(sm, Ls, f, w, W, r, &bad, kb, ke, ke);
-            __syncthreads();
-            if (ke < kE) {
-              int* EX = oz_ex(SL, f - ke);
-              oz_slice(Ls, f, ke, kb, ke, SL, EX);
-              okf = oz_update(ring, gbar, fbar, afull, aempty, tmem, g, tcnt, &abort_s, SL, EX, f - ke, ke - kb, Ls, f,
-                              w, W, r, ke, kE);
-            }
-          }
-          // the rank-128 update of the rest of the front
-          if (okf && kE < f) {
-            int* EX = oz_ex(SL, f - kE);
-            oz_slice(Ls, f, kE, kB, kE, SL, EX);
-            okf = oz_update(ring, gbar, fbar, afull, aempty, tmem, g, tcnt, &abort_s, SL, EX, f - kE, kE - kB, Ls, f,
-                            w, W, r, kE, f);
-          }
-        }
-      }
-      __syncthreads();
-      if (P.sn_parent[gs] >= 0) {
-        double* Uout = P.sn_hoff[gs] >= 0 ? hand + P.sn_hoff[gs] : stack + P.upd_ofs[gs];
-        for (int64_t idx = tid; idx < (int64_t)r * r; idx += kThreads) Uout[idx] = W[idx];
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      if (bad) atomicOr(status, kStatNotSPD);
-      if (item.w >= 0 && !abort_s) {
-        __threadfence();  // the task's factor panels and hand-over block before the count
-        atomicAdd(tdone + item.w, 1);
-      }
-    }
-    if (abort_s) break;
-  }
-  if (tid == 0 && abort_s) atomicOr(status, kStatTimeout);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
   }
 }
 
@@ -1746,21 +1295,6 @@ void launch_chol(const DevPlan& P, const int4* items, int nitems, int use_tasks,
   cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   chol_kernel<<<grid, kThreads, smem, st>>>(P, items, nitems, use_tasks, queue, tdone, hand, ws, ws_stride, front_sz,
                                             stack_sz, flags, status);
-}
-
-void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue, int* tdone, double* hand,
-                    double* ws, int64_t ws_stride, int64_t front_sz, uint16_t* slices, int64_t slice_stride, int grid,
-                    int* status, cudaStream_t st, int flags) {
-  if (nitems <= 0) return;
-  cudaFuncSetAttribute(chol_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholTcDyn);
-  chol_tc_kernel<<<std::min(grid, nitems), kThreads, kCholTcDyn, st>>>(P, items, nitems, queue, tdone, hand, ws,
-                                                                       ws_stride, front_sz, slices, slice_stride,
-                                                                       flags, status);
-}
-
-int64_t chol_tc_scratch(int fmax) {
-  const int64_t npad = (fmax + kOzM - 1) / kOzM * kOzM;
-  return (npad * (2 * kOzS * kOzK + 2) + 127) / 128 * 128;
 }
 
 int chol_ctas_per_sm() {
