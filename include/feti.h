@@ -128,13 +128,13 @@ typedef struct {
                                  SMs.  The factor is the same bit for bit either way */
   int32_t syrk_kernel;        /* split-bf16 SYRK kernel: 0 = autotuned at the first feti_assemble; 1, 2, 3 =
                                  feti_stats.syrk_variant 0, 1, 2 (the same F bit for bit) */
-  int32_t chol_tc;            /* 0 = the rank-32 and rank-128 updates of the fronts at least 384 wide run on
+  int32_t chol_tc;            /* 0 = the rank-32 and rank-128 updates of the fronts at least 256 wide run on
                                  the tensor cores by exact slicing of FP64 into bf16 integers (integer partial
                                  sums exact in FP32; error below FP64's own normwise bound); 1 = all of the
                                  Cholesky on the FP64 pipe */
   int32_t chol_tc_front;      /* with chol_tc = 0: the narrowest front (w + r) taken by the tensor-core kernel,
-                                 with all its ancestors (0 = 384, the fastest measured on the 3D elasticity
-                                 workload; values below 128 act as 128) */
+                                 with all its ancestors (0 = 256, within 3% of the fastest measured on 3D
+                                 elasticity and uneven 3D heat; at least 128) */
 } feti_options;
 
 typedef struct {

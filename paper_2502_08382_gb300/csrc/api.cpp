@@ -353,11 +353,18 @@ void build(feti_ctx* c) {
     for (auto& sh : c->subs) total += c->pats[sh.pat].chol_flops;
     const double slots = (double)std::max(1, nsm * chol_ctas_per_sm());
     const double target = total / (4.0 * slots);
-    // fronts at least 384 wide (and their ancestors) go to the tensor-core Cholesky unless switched off
+    // fronts at least 256 wide (and their ancestors) go to the tensor-core Cholesky unless switched off.  Whole
+    // factorisation with 192 / 256 / 384: 27 elasticity subdomains of 12^3 15.7 / 15.1 / 17.0 ms, 64 of them 28.1 /
+    // 26.7 / 29.0, 216 of them 85.2 / 82.1 / 81.8; 64 uneven 3D heat subdomains 23.6 / 27.3 / 32.4, 125 of them 24.1 /
+    // 18.9 / 22.1
     if (c->opt.chol_tc < 0 || c->opt.chol_tc > 1) throw ArgError("bad chol_tc (0 tensor cores for large fronts, 1 off)");
     if (c->opt.chol_tc_front < 0) throw ArgError("bad chol_tc_front (0 default, else the narrowest front)");
-    const int big_f = c->opt.chol_tc == 1 ? 0 : (c->opt.chol_tc_front > 0 ? std::max(c->opt.chol_tc_front, 128) : 384);
+    const int big_f = c->opt.chol_tc == 1 ? 0 : (c->opt.chol_tc_front > 0 ? std::max(c->opt.chol_tc_front, 128) : 256);
     for (auto& P : c->pats) plan_tasks(P, target, big_f);
+    // what chol_kernel does (everything outside the large set) is cut by the same rule on its own flops
+    double small = 0;
+    for (auto& sh : c->subs) small += c->pats[sh.pat].sub_flops;
+    for (auto& P : c->pats) plan_tasks(P, target, big_f, small / (4.0 * slots));
   }
   c->stats.t_symbolic_ms = std::chrono::duration<double, std::milli>(clk::now() - t0).count();
   c->stats.npatterns = (int)c->pats.size();
@@ -467,6 +474,7 @@ void build(feti_ctx* c) {
   std::vector<int2> l16_items;
   int fixo = 0, alo = 0;
   double chol = 0, trsm = 0, syrk = 0, syrke = 0, implb = 0;
+  int64_t sub_cf = 0, sub_chol = 0;
   int64_t max_chol = 0, max_rhs = 0, max_cf = 0, max_rf = 0, max_usm = 0;
   size_t esz = c->fp32 ? 4 : 8;
   double apply_bytes = 0, stored_bytes = 0;
@@ -569,6 +577,8 @@ void build(feti_ctx* c) {
     max_chol = std::max(max_chol, P.chol_stack);
     max_usm = std::max(max_usm, P.usm_size);
     max_cf = std::max(max_cf, P.chol_front);
+    sub_cf = std::max(sub_cf, P.sub_front);
+    sub_chol = std::max(sub_chol, P.sub_stack);
     max_rhs = std::max(max_rhs, B.rhs_stack);
     max_rf = std::max(max_rf, B.rhs_front);
     apply_bytes += (double)esz * s.m * (s.m + 1) / 2.0 + (double)s.m * (4 + 8 + 8);
@@ -766,6 +776,14 @@ void build(feti_ctx* c) {
     c->grid_trsm32 = std::max(1, std::min(c->grid_trsm32, c->grid_trsm));
   }
   int gw = std::max(c->grid_chol, c->grid_trsm);
+  c->grid_ws = gw;
+  // chol_kernel needs the fronts and stacks outside the large set only: as many CTAs as fit the same workspace (its
+  // tasks outnumber the subdomains; with one CTA per subdomain 64 subdomains left half the SMs idle)
+  c->sub_front = sub_cf;
+  c->sub_stack = sub_chol;
+  c->sub_stride = std::max<int64_t>((sub_cf + sub_chol + max_usm + 31) / 32 * 32, 32);
+  c->grid_chol = (int)std::max<int64_t>(
+      c->grid_chol, std::min<int64_t>((int64_t)c->nsm * chol_ctas_per_sm(), (int64_t)gw * c->ws_stride / c->sub_stride));
 
   // ---- device uploads
   DevPlan& D = c->P;
@@ -949,7 +967,7 @@ void build(feti_ctx* c) {
         int nbig_sub = 0;
         for (int i = 0; i < ns; ++i) nbig_sub += c->pats[c->subs[i].pat].has_big ? 1 : 0;
         c->tc_cluster = chol_tc_cluster(nbig_sub, c->nsm);
-        c->grid_tc = std::max(1, std::min(c->nsm / c->tc_cluster, std::min(c->n_tc_items, c->grid_chol)));
+        c->grid_tc = std::max(1, std::min(c->nsm / c->tc_cluster, std::min(c->n_tc_items, c->grid_ws)));
         c->slice_stride = chol_tc_scratch(fmax);
         c->d_slices = (char*)dalloc(c, (size_t)c->grid_tc * c->slice_stride);
       }
@@ -1161,7 +1179,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       if (v) CK(cudaMemsetAsync(ctx->d_tdone, 0, (size_t)std::max(ctx->ntask_total, 1) * sizeof(int), s2));
       const int fl = flags | (ctx->n_tc_items > 0 ? kCholSkipBig : 0);
       launch_chol(P, ctx->d_chol_items[v], ctx->chol_nitems[v], v, ctx->d_queue + qslot, ctx->d_tdone, ctx->d_hand,
-                  ctx->d_ws, ctx->ws_stride, ctx->chol_front, ctx->chol_stack,
+                  ctx->d_ws, ctx->sub_stride, ctx->sub_front, ctx->sub_stack,
                   std::min(ctx->grid_chol, ctx->chol_nitems[v]), ctx->d_status, s2, fl);
       if (ctx->n_tc_items > 0) {
         // the large fronts on the tensor cores, after everything below them

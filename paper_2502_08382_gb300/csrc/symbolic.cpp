@@ -645,7 +645,8 @@ void analyse_pattern(int n, const int64_t* rp, const int32_t* col, const double*
   }
 }
 
-void plan_tasks(PatternPlan& P, double target, int big_f) {
+void plan_tasks(PatternPlan& P, double target, int big_f, double target_small) {
+  if (target_small <= 0) target_small = target;
   const int ns = P.nsn;
   std::vector<double> own(ns, 0.0), sub(ns, 0.0);
   for (int s = 0; s < ns; ++s) {
@@ -686,7 +687,7 @@ void plan_tasks(PatternPlan& P, double target, int big_f) {
     if (p < 0) {
       P.sn_task[s] = 0;
     } else if ((P.sn_big[p] && !P.sn_big[s]) ||
-               (target > 0 && !P.sn_small[s] && sub[s] > target && P.sn_r[s] > 0)) {
+               (target > 0 && !P.sn_small[s] && sub[s] > (P.sn_big[s] ? target : target_small) && P.sn_r[s] > 0)) {
       const int t = (int)P.task_parent.size();
       P.task_parent.push_back(P.sn_task[p]);
       P.task_cost.push_back(0.0);
@@ -712,6 +713,25 @@ void plan_tasks(PatternPlan& P, double target, int big_f) {
   // tasks are numbered parents first, so heights follow from the highest numbers down
   for (int t = P.ntask - 1; t >= 1; --t)
     P.task_height[P.task_parent[t]] = std::max(P.task_height[P.task_parent[t]], P.task_height[t] + 1);
+  // the update stack of the supernodes outside the large set: each maximal subtree of them starts an empty one (its
+  // root hands its block over), so chol_kernel's CTAs need far less workspace than a whole tree's stack
+  P.sub_stack = P.sub_front = 0;
+  P.sub_flops = 0;
+  std::vector<int64_t> size(ns, 0);
+  int64_t top = 0;
+  for (int s = 0; s < ns; ++s) {  // postorder: a subtree's supernodes are consecutive
+    if (P.sn_big[s]) continue;
+    int64_t base = top;
+    for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) base -= size[P.ch_list[k]];
+    const int64_t rr = (int64_t)P.sn_r[s] * P.sn_r[s];
+    size[s] = P.sn_parent[s] >= 0 ? rr : 0;
+    P.upd_stack_ofs[s] = base;
+    top = base + size[s];
+    P.sub_stack = std::max(P.sub_stack, top);
+    P.sub_front = std::max(P.sub_front, rr);
+    P.sub_flops += own[s];
+    if (P.sn_parent[s] < 0 || P.sn_big[P.sn_parent[s]]) top = 0;
+  }
 }
 
 void plan_rhs(const PatternPlan& P, int m, const int32_t* B_dof, BPlan& Bp) {

@@ -71,13 +71,16 @@ struct PatternPlan {
   bool has_big = false;
   std::vector<int> task_big;       // 1: the task's supernodes are large (the tensor-core Cholesky's)
   std::vector<int> task_nbig;      // large child tasks
+  int64_t sub_stack = 0, sub_front = 0;  // doubles of update stack / front of the supernodes outside the large set
+  double sub_flops = 0;            // their Cholesky flops
 };
 
 // Cut the pattern's supernodal tree into Cholesky tasks: a child subtree whose flops exceed `target` becomes
 // a task of its own (recursively), so that one large subdomain can be factored by several CTAs.  big_f > 0:
 // the fronts at least big_f wide and their ancestors (the tensor-core Cholesky's work) form tasks of their own,
-// cut by the same rule, and every other child of that set starts a task.
-void plan_tasks(PatternPlan& P, double target, int big_f = 0);
+// cut by the same rule, and every other child of that set starts a task.  target_small > 0: the target outside the
+// large set.  Also lays the update stack of the supernodes outside the large set out anew (upd_stack_ofs).
+void plan_tasks(PatternPlan& P, double target, int big_f = 0, double target_small = 0);
 
 struct BPlan {
   int m = 0, m_pad = 0, nb = 0;
