@@ -1040,10 +1040,11 @@ void build(feti_ctx* c) {
     CK(cudaMallocHost((void**)&c->h_ctrl, sizeof(PcgCtrl)));
     launch_build_G(D, c->d_colsub, qo, c->d_R, c->d_G6, c->st);
     CK(cudaGetLastError());
-    size_t sm = implicit_smem(c->nmax, c->impl_maxf);
+    c->impl_wide = implicit_wide(ns, c->nsm, c->nmax, c->impl_maxf);
+    size_t sm = implicit_smem(c->nmax, c->impl_maxf, c->impl_wide);
     if (sm > 227 * 1024) throw ArgError("subdomain too large for the shared-memory implicit solve");
     c->impl_smem = sm;
-    c->grid_impl = std::min(ns, c->nsm * implicit_occupancy(sm));
+    c->grid_impl = std::min(ns, c->nsm * implicit_occupancy(sm, c->impl_wide));
     c->ustride = std::max<int64_t>((max_usize + 31) / 32 * 32, 32);
     c->d_uws = (double*)dalloc(c, (size_t)c->grid_impl * c->ustride * 8);
   }
@@ -1211,6 +1212,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     CK(cudaEventRecordWithFlags(ctx->ev[1], s2, evf));
     if (r2) {
       launch_unit_scale(ctx->P, ctx->nsub, ctx->nmax, ctx->P.dinv, s2);
+      if (ctx->impl_wide) launch_inv_blocks(ctx->P, ctx->nsub, s2);
       CK(cudaEventRecordWithFlags(ctx->ev[2], s2, evf));
       trsm_path_entry(ctx);
       CK(cudaEventRecordWithFlags(ctx->ev[3], s2, evf));
@@ -1242,6 +1244,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     run_trsm(ctx->trsm_cands[ctx->trsm_pick], s2);
     // the implicit solves take L in unit-lower form; the TRSM above was its last user as L
     launch_unit_scale(ctx->P, ctx->nsub, ctx->nmax, ctx->P.dinv, s2);
+    if (ctx->impl_wide) launch_inv_blocks(ctx->P, ctx->nsub, s2);
     CK(cudaEventRecordWithFlags(ctx->ev[2], s2, evf));
     if (ctx->fp32) {
       auto run_syrk = [&](int variant) {

@@ -125,6 +125,7 @@ struct feti_ctx {
   int grid_chol = 0, grid_trsm = 0, grid_impl = 0;
   int grid_trsm32 = 0;  // CTAs of the mixed-precision TRSM (its occupancy with the tensor-core stage ring)
   size_t impl_smem = 0;
+  bool impl_wide = false;   // one 1024-thread CTA per subdomain
   double* d_uws = nullptr;  // update vectors of the implicit solve, ustride doubles per CTA
   int64_t ustride = 0;
   int impl_maxf = 0;

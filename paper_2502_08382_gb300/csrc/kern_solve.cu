@@ -132,23 +132,31 @@ __device__ __forceinline__ void bwd_warp(const DevPlan& P, const SubInfo& S, int
   __syncwarp();
 }
 
-// Whole CTA: forward step of a large supernode on the shared front vector.
+// Barrier of the 256 threads that share a supernode: the CTA, or team `team` of a wide CTA.
+template <bool TEAM>
+__device__ __forceinline__ void cta_sync(int team) {
+  if constexpr (TEAM) asm volatile("bar.sync %0, 256;" ::"r"(team + 1) : "memory");
+  else __syncthreads();
+}
+
+// 256 threads: forward step of a large supernode on the shared front vector.
 // 32 x 32 unit-lower diagonal blocks are staged in shared memory and solved
 // by warp 0; all threads apply the block's columns to the rest of the front.
+template <bool TEAM = false>
 __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int gs, const double* d2,
-                                        double* ubuf, double* y, double* sf, double (*sm_blk)[kW + 1], int tid) {
+                                        double* ubuf, double* y, double* sf, double (*sm_blk)[kW + 1], int tid, int team = 0) {
   const int warp = tid / 32, lane = tid % 32;
   const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f_ = w + r;
   const double* Ls = P.L + S.L + P.Lofs[gs];
   for (int i = tid; i < f_; i += kThreads) sf[i] = i < w ? y[c0 + i] : 0.0;
-  __syncthreads();
+  cta_sync<TEAM>(team);
   for (int c = P.ch_off[gs]; c < P.ch_off[gs + 1]; ++c) {
     const int gc = S.sn0 + P.ch_list[c];
     const int rc = P.sn_r[gc];
     const double* U = ubuf + P.uofs[gc];
     const int* rl = P.rel + P.rel_off[gc];
     for (int k = tid; k < rc; k += kThreads) sf[rl[k]] += U[k];
-    __syncthreads();
+    cta_sync<TEAM>(team);
   }
   for (int kb = 0; kb < w; kb += kW) {
     const int nbk = min(kW, w - kb);
@@ -156,7 +164,7 @@ __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int 
       const int k = idx / kW, i = idx % kW;  // column k, row i of the block
       if (i < nbk) sm_blk[i][k] = (i >= k) ? Ls[(int64_t)(kb + k) * f_ + kb + i] : 0.0;
     }
-    __syncthreads();
+    cta_sync<TEAM>(team);
     if (warp == 0) {
       double yi = lane < nbk ? sf[kb + lane] : 0.0;
       for (int k = 0; k < nbk; ++k) {
@@ -165,7 +173,7 @@ __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int 
       }
       if (lane < nbk) sf[kb + lane] = yi;
     }
-    __syncthreads();
+    cta_sync<TEAM>(team);
     // rows in pairs (i, i + kThreads) per thread, so that each group of column loads has twice the bytes in
     // flight; a last unpaired row alone.  Every row's sum runs over k in the same order either way.
     int i = kb + nbk + tid;
@@ -187,30 +195,31 @@ __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int 
       for (int k = 0; k < nbk; ++k) acc = fma(Ls[(int64_t)(kb + k) * f_ + i], sf[kb + k], acc);
       sf[i] -= acc;
     }
-    __syncthreads();
+    cta_sync<TEAM>(team);
   }
   double* Us = ubuf + P.uofs[gs];
   for (int i = tid; i < f_; i += kThreads) {
     if (i < w) y[c0 + i] = sf[i] * d2[c0 + i];
     else Us[i - w] = sf[i];
   }
-  __syncthreads();
+  cta_sync<TEAM>(team);
 }
 
-// Whole CTA: backward step of a large supernode (x_rows already final).  The
+// 256 threads: backward step of a large supernode (x_rows already final).  The
 // entries x_rows are gathered into sf first; then each warp takes kBC own
 // columns at a time, so their column loads are in flight together (the dot
 // product of each column runs over the rows in the same order as with one
 // column per warp, and is reduced the same way).
 constexpr int kBC = 4;
+template <bool TEAM = false>
 __device__ __forceinline__ void bwd_cta(const DevPlan& P, const SubInfo& S, int gs, double* y, double* sf,
-                                        double (*sm_blk)[kW + 1], int tid) {
+                                        double (*sm_blk)[kW + 1], int tid, int team = 0) {
   const int warp = tid / 32, lane = tid % 32;
   const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f_ = w + r;
   const double* Ls = P.L + S.L + P.Lofs[gs];
   const int* rows = P.rows + P.sn_rows[gs];
   for (int k = tid; k < r; k += kThreads) sf[k] = y[rows[k]];
-  __syncthreads();
+  cta_sync<TEAM>(team);
   for (int l0 = warp * kBC; l0 < w; l0 += (kThreads / 32) * kBC) {
     if (l0 + kBC <= w) {
       double acc[kBC];
@@ -244,7 +253,7 @@ __device__ __forceinline__ void bwd_cta(const DevPlan& P, const SubInfo& S, int 
       }
     }
   }
-  __syncthreads();
+  cta_sync<TEAM>(team);
   for (int kb = ((w - 1) / kW) * kW; kb >= 0; kb -= kW) {
     const int nbk = min(kW, w - kb);
     if (nbk == kW) {
@@ -282,7 +291,7 @@ __device__ __forceinline__ void bwd_cta(const DevPlan& P, const SubInfo& S, int 
       const int k = idx / kW, i = idx % kW;
       if (i < nbk) sm_blk[i][k] = (i >= k) ? Ls[(int64_t)(kb + k) * f_ + kb + i] : 0.0;
     }
-    __syncthreads();
+    cta_sync<TEAM>(team);
     if (warp == 0) {
       double yi = lane < nbk ? y[c0 + kb + lane] : 0.0;
       for (int k = nbk - 1; k >= 0; --k) {
@@ -291,44 +300,272 @@ __device__ __forceinline__ void bwd_cta(const DevPlan& P, const SubInfo& S, int 
       }
       if (lane < nbk) y[c0 + kb + lane] = yi;
     }
+    cta_sync<TEAM>(team);
+  }
+}
+
+// ---------------------------------------------------------------- one wide CTA per subdomain
+//
+// With at most one subdomain per SM the 256-thread CTA above leaves the SM waiting: each 32-column block of a large
+// supernode was a 32-step chain in one warp, then a few column loads in flight per thread.  The wide CTA (1024
+// threads) applies the block's inverse instead (inv_block_kernel keeps it above the diagonal of the block, where the
+// panel holds nothing), splits the 32 columns of each update over four groups of threads, so that all of a block's
+// loads are in flight at once, and issues the first of them before the block's own entries are solved.  FP64
+// instructions are the scarce resource (64 clocks of a scheduler each): dot products run on eight lanes per column,
+// which needs three additions per four columns to reduce.  Supernodes of moderate size (kTeamF, kTeamW) spend most of
+// their time in chains of index loads, so the wide CTA's four teams of 256 threads take one each, side by side.
+// Measured per application (before: 256 threads per subdomain): 64 elasticity subdomains of 12^3 5.7 -> 2.7 ms, 125
+// uneven 3D heat subdomains 9.0 -> 4.75 ms (its largest subdomain sets it: two sweeps of 3.5 M entries on one SM's
+// FP64 pipe take 1.8 ms).
+constexpr int kWide = 1024;
+constexpr int kTeamF = 512, kTeamW = 64;  // largest front and width a team takes
+constexpr int kWR = 512;  // rows of an update pass (two per thread of a group)
+struct WideSmem {
+  double blk[2][kW][kW + 1];  // inverses of the unit-lower diagonal blocks (strictly lower part)
+  double dp[4][kW];           // partial products of a block
+};
+// dynamic shared memory behind the front vector: the warps' fronts (and the wide updates' partial sums) and WideSmem,
+// or the four teams' fronts and diagonal blocks
+constexpr int kWideBuf = kWide / 32 * kWF + (int)(sizeof(WideSmem) / 8);
+static_assert(4 * (kTeamF + kW * (kW + 1)) <= kWideBuf, "the teams' buffers fit");
+
+// (i, k) of the inverse of the unit-lower block kb, k < i, stands at row k of column i
+__device__ __forceinline__ void wide_stage(const double* Ls, int f_, int kb, int nbk, double (*blk)[kW + 1], int t,
+                                           int nt) {
+  for (int idx = t; idx < kW * kW; idx += nt) {
+    const int k = idx % kW, i = idx / kW;
+    blk[i][k] = (i < nbk && k < i) ? Ls[(int64_t)(kb + i) * f_ + kb + k] : 0.0;
+  }
+}
+
+__device__ __forceinline__ void fwd_wide(const DevPlan& P, const SubInfo& S, int gs, const double* d2, double* ubuf,
+                                         double* y, double* sf, double* part, WideSmem& ws, int tid) {
+  const int warp = tid / 32, lane = tid % 32, g = tid / 256, t = tid % 256;
+  const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f_ = w + r;
+  const double* Ls = P.L + S.L + P.Lofs[gs];
+  wide_stage(Ls, f_, 0, min(kW, w), ws.blk[0], tid, kWide);
+  for (int i = tid; i < f_; i += kWide) sf[i] = i < w ? y[c0 + i] : 0.0;
+  __syncthreads();
+  for (int c = P.ch_off[gs]; c < P.ch_off[gs + 1]; ++c) {
+    const int gc = S.sn0 + P.ch_list[c];
+    const int rc = P.sn_r[gc];
+    const double* U = ubuf + P.uofs[gc];
+    const int* rl = P.rel + P.rel_off[gc];
+    for (int k = tid; k < rc; k += kWide) sf[rl[k]] += U[k];
     __syncthreads();
+  }
+  // the own rows, block by block
+  for (int kb = 0, cur = 0; kb < w; kb += kW, cur ^= 1) {
+    const int nbk = min(kW, w - kb);
+    const int k0 = 8 * g, r0 = kb + nbk;
+    const bool upd = r0 < w;  // then the block is full
+    // the first rows' columns, in flight while the block is solved
+    double l[8];
+    if (upd) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) l[e] = r0 + t < w ? Ls[(int64_t)(kb + k0 + e) * f_ + r0 + t] : 0.0;
+    }
+    if (warp < 4) {
+      double p = 0.0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        p = fma(ws.blk[cur][lane][8 * warp + e], 8 * warp + e < nbk ? sf[kb + 8 * warp + e] : 0.0, p);
+      ws.dp[warp][lane] = p;
+    } else if (kb + kW < w) {
+      wide_stage(Ls, f_, kb + kW, min(kW, w - kb - kW), ws.blk[cur ^ 1], tid - 128, kWide - 128);
+    }
+    __syncthreads();
+    if (warp == 0 && lane < nbk)
+      sf[kb + lane] += (ws.dp[0][lane] + ws.dp[1][lane]) + (ws.dp[2][lane] + ws.dp[3][lane]);
+    __syncthreads();
+    if (!upd) break;
+    for (int i0 = r0, h = 0; i0 < w; i0 += 256, ++h) {
+      double* pt = part + (h & 1) * 1024;
+      const int i = i0 + t;
+      if (h > 0) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) l[e] = i < w ? Ls[(int64_t)(kb + k0 + e) * f_ + i] : 0.0;
+      }
+      if (i0 + (t & ~31) < w) {
+        double acc = 0.0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc = fma(l[e], sf[kb + k0 + e], acc);
+        pt[g * 256 + t] = acc;
+      }
+      __syncthreads();
+      if (tid < 256 && i < w) sf[i] -= (pt[t] + pt[256 + t]) + (pt[512 + t] + pt[768 + t]);
+    }
+    __syncthreads();
+  }
+  // the rows below: each group of threads a quarter of the columns, nothing to wait for
+  {
+    const int kq = (w + 3) / 4, k0 = min(w, g * kq), k1 = min(w, k0 + kq);
+    int h = 0;
+    for (int i0 = w; i0 < f_; i0 += kWR, ++h) {
+      double* pt = part + (h & 1) * 4 * kWR;
+      const int i = i0 + t;
+      double acc = 0.0, acc2 = 0.0;
+      if (i0 + 256 + (t & ~31) < f_) {
+        const int i2 = min(i + 256, f_ - 1);
+#pragma unroll 8
+        for (int k = k0; k < k1; ++k) {
+          const double* col = Ls + (int64_t)k * f_;
+          const double z = sf[k];
+          acc = fma(col[i], z, acc);
+          acc2 = fma(col[i2], z, acc2);
+        }
+      } else if (i0 + (t & ~31) < f_) {
+        const int i1 = min(i, f_ - 1);
+#pragma unroll 8
+        for (int k = k0; k < k1; ++k) acc = fma(Ls[(int64_t)k * f_ + i1], sf[k], acc);
+      }
+      pt[g * kWR + t] = acc;
+      pt[g * kWR + 256 + t] = acc2;
+      __syncthreads();
+      if (tid < kWR && i0 + tid < f_)
+        sf[i0 + tid] -= (pt[tid] + pt[kWR + tid]) + (pt[2 * kWR + tid] + pt[3 * kWR + tid]);
+    }
+    __syncthreads();
+  }
+  double* Us = ubuf + P.uofs[gs];
+  for (int i = tid; i < f_; i += kWide) {
+    if (i < w) y[c0 + i] = sf[i] * d2[c0 + i];
+    else Us[i - w] = sf[i];
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ double sum8(double a) {
+  a += __shfl_xor_sync(0xffffffffu, a, 4);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  return a;
+}
+
+__device__ __forceinline__ void bwd_wide(const DevPlan& P, const SubInfo& S, int gs, double* y, double* sf,
+                                         WideSmem& ws, int tid) {
+  const int warp = tid / 32, lane = tid % 32, c4 = lane / 8, l8 = lane % 8;
+  const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f_ = w + r;
+  const double* Ls = P.L + S.L + P.Lofs[gs];
+  const int* rows = P.rows + P.sn_rows[gs];
+  for (int k = tid; k < r; k += kWide) sf[k] = y[rows[k]];
+  const int kl = ((w - 1) / kW) * kW;
+  wide_stage(Ls, f_, kl, w - kl, ws.blk[0], tid, kWide);
+  __syncthreads();
+  // the rows below: each warp four columns at a time
+  for (int l0 = 4 * warp; l0 < w; l0 += 4 * (kWide / 32)) {
+    const int l = l0 + c4;
+    const double* col = Ls + (int64_t)min(l, w - 1) * f_ + w;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int k = l8; k < r; k += 8) acc = fma(col[k], sf[k], acc);
+    acc = sum8(acc);
+    if (l8 == 0 && l < w) y[c0 + l] -= acc;
+  }
+  __syncthreads();
+  for (int kb = kl, cur = 0; kb >= 0; kb -= kW, cur ^= 1) {
+    const int nbk = min(kW, w - kb);
+    // the supernode's own rows below the block: columns kb + 4 (warp % 8) + c4, a quarter of the rows per warp
+    {
+      const int l = min(kb + 4 * (warp % 8) + c4, w - 1);
+      const double* col = Ls + (int64_t)l * f_;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int i = kb + nbk + 8 * (warp / 8) + l8; i < w; i += 32) acc = fma(col[i], y[c0 + i], acc);
+      acc = sum8(acc);
+      if (l8 == 0) ws.dp[warp / 8][4 * (warp % 8) + c4] = acc;
+    }
+    __syncthreads();
+    double v = 0.0;
+    if (warp < 4) {
+      if (lane < nbk)
+        v = y[c0 + kb + lane] - ((ws.dp[0][lane] + ws.dp[1][lane]) + (ws.dp[2][lane] + ws.dp[3][lane]));
+      double p = 0.0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        p = fma(ws.blk[cur][8 * warp + e][lane], __shfl_sync(0xffffffffu, v, 8 * warp + e), p);
+      __syncwarp();
+      asm volatile("bar.sync 2, 128;" ::: "memory");  // the four warps have read dp
+      ws.dp[warp][lane] = p;
+    } else if (kb > 0) {
+      wide_stage(Ls, f_, kb - kW, kW, ws.blk[cur ^ 1], tid - 128, kWide - 128);
+    }
+    __syncthreads();
+    if (warp == 0 && lane < nbk)
+      y[c0 + kb + lane] = v + ((ws.dp[0][lane] + ws.dp[1][lane]) + (ws.dp[2][lane] + ws.dp[3][lane]));
+    __syncthreads();
+  }
+}
+
+// Inverses of the unit-lower 32 x 32 diagonal blocks of the supernodes that the wide solves take, kept above the
+// diagonal of their own block ((i, k), k < i, at row k of column i).  One warp per block, lane = column.
+__global__ void __launch_bounds__(128) inv_block_kernel(DevPlan P, int nsub) {
+  __shared__ double B[4][kW][kW + 1];
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  double(*D)[kW + 1] = B[warp];
+  for (int si = blockIdx.y; si < nsub; si += gridDim.y) {
+    const SubInfo& S = P.sub[si];
+    for (int s = blockIdx.x; s < S.nsn; s += gridDim.x) {
+      const int gs = S.sn0 + s;
+      const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
+      if (w <= 32 && f_ <= kWF) continue;
+      double* Ls = P.L + S.L + P.Lofs[gs];
+      for (int kb = kW * warp; kb < w; kb += 4 * kW) {
+        const int nbk = min(kW, w - kb);
+        for (int k = 0; k < kW; ++k)
+          D[lane][k] = (lane < nbk && k < lane) ? Ls[(int64_t)(kb + k) * f_ + kb + lane] : 0.0;
+        __syncwarp();
+        double m[kW];
+#pragma unroll
+        for (int i = 0; i < kW; ++i) {
+          double a = i == lane ? 1.0 : 0.0;
+#pragma unroll
+          for (int k = 0; k < i; ++k) a = fma(-D[i][k], m[k], a);
+          m[i] = a;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 1; i < kW; ++i)
+          if (i < nbk && lane < i) Ls[(int64_t)(kb + i) * f_ + kb + lane] = m[i];
+      }
+    }
   }
 }
 
 // MODE 0: qi = B L^-T L^-1 P B^T p        (implicit apply, eq. 11)
 // MODE 1: qi = B K_reg^{-1} f             (d = B K^+ f - c, eq. 7)
 // MODE 2: u  = K_reg^{-1} (f - B^T lambda) (eq. 5 without R alpha)
-// MODE 3: column j of Z = K_reg^{-1} B^T for one subdomain (items = its
-//         sorted columns; `nsub` is the column count, order[0] the subdomain);
-//         written to u as Z[dof * m + B-row of column j] (original DOF order)
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 4) implicit_kernel(DevPlan P, const int* order, int nsub, int* queue,
-                                                             const double* p, const double* f, double* qi,
-                                                             double* u, double* uws, int64_t ustride, int nmax,
-                                                             int maxf) {
-  extern __shared__ double y[];  // [nmax] subdomain vector, [maxf] front, [8 kWF] warp fronts
-  __shared__ double sm_blk[kW][kW + 1];
+// NT: threads of the CTA (256, or the wide 1024).
+template <int MODE, int NT>
+__global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
+    implicit_kernel(DevPlan P, const int* order, int nsub, int* queue, const double* p, const double* f, double* qi,
+                    double* u, double* uws, int64_t ustride, int nmax, int maxf) {
+  // [nmax] subdomain vector, [maxf] front, [NT / 32 kWF] warp fronts (the wide updates' partial sums), wide: WideSmem
+  extern __shared__ double y[];
+  __shared__ __align__(16) uint8_t blk_raw[NT == kWide ? 16 : sizeof(double) * kW * (kW + 1)];
+  double(*sm_blk)[kW + 1] = reinterpret_cast<double(*)[kW + 1]>(blk_raw);
+  static_assert(kWide / 32 * kWF >= 2 * 4 * kWR, "the partial sums fit the warp fronts");
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   double* sfront = y + nmax;
   double* wbuf = sfront + maxf;
+  WideSmem& wsm = *reinterpret_cast<WideSmem*>(wbuf + NT / 32 * kWF);  // NT == kWide
   double* ubuf = uws + (int64_t)blockIdx.x * ustride;
   for (;;) {
     const int itx = pop_item_s(queue);
     if (itx >= nsub) return;
-    const int si = MODE == 3 ? order[0] : order[itx];
+    const int si = order[itx];
     const SubInfo& S = P.sub[si];
     const int n = S.n;
     const double* d2 = P.dinv + S.dof;  // 1 / L_jj^2 (unit-lower form)
-    for (int k = tid; k < n; k += kThreads) y[k] = 0.0;
+    for (int k = tid; k < n; k += NT) y[k] = 0.0;
     __syncthreads();
-    if (MODE == 3 && tid == 0) y[P.spos[S.col0 + itx]] = P.qsign[S.qcol + itx];
     if (MODE == 1 || MODE == 2)
-      for (int k = tid; k < n; k += kThreads) y[P.iperm[S.diag0 + k]] = f[S.dof + k];
+      for (int k = tid; k < n; k += NT) y[P.iperm[S.diag0 + k]] = f[S.dof + k];
     __syncthreads();
     if (MODE == 0 || MODE == 2) {
       // B^T p: columns sharing a DOF are adjacent in sorted order; the first of a run sums it
       const int* sp = P.spos + S.col0;
-      for (int j = tid; j < S.m; j += kThreads) {
+      for (int j = tid; j < S.m; j += NT) {
         if (j > 0 && sp[j - 1] == sp[j]) continue;
         double s = 0.0;
         for (int jj = j; jj < S.m && sp[jj] == sp[j]; ++jj) s += P.qsign[S.qcol + jj] * p[P.qmap[S.qcol + jj]];
@@ -347,47 +584,72 @@ __global__ void __launch_bounds__(kThreads, 4) implicit_kernel(DevPlan P, const 
     const int* lsn = P.lvl_sn;
     for (int l = 0; l < S.nlev; ++l) {
       const int lo = lvo[l], hi = lvo[l + 1];
-      for (int it = lo + warp; it < hi; it += kThreads / 32) {
+      for (int it = lo + warp; it < hi; it += NT / 32) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w > 32 || f_ > kWF) continue;
         fwd_warp(P, S, gs, d2, ubuf, y, wbuf + warp * kWF, lane);
       }
       __syncthreads();
+      if constexpr (NT == kWide) {
+        double* tbuf = wbuf + (tid / 256) * (kTeamF + kW * (kW + 1));
+        int q = 0;
+        for (int it = lo; it < hi; ++it) {
+          const int gs = S.sn0 + lsn[it];
+          const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
+          if ((w <= 32 && f_ <= kWF) || w > kTeamW || f_ > kTeamF) continue;
+          if ((q++ & 3) != tid / 256) continue;
+          fwd_cta<true>(P, S, gs, d2, ubuf, y, tbuf, reinterpret_cast<double(*)[kW + 1]>(tbuf + kTeamF), tid % 256, tid / 256);
+        }
+        __syncthreads();
+      }
       for (int it = lo; it < hi; ++it) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w <= 32 && f_ <= kWF) continue;
-        fwd_cta(P, S, gs, d2, ubuf, y, sfront, sm_blk, tid);
+        if (NT == kWide && w <= kTeamW && f_ <= kTeamF) continue;
+        if constexpr (NT == kWide) fwd_wide(P, S, gs, d2, ubuf, y, sfront, wbuf, wsm, tid);
+        else fwd_cta(P, S, gs, d2, ubuf, y, sfront, sm_blk, tid);
       }
     }
     // backward substitution L^T x = z, level by level from the roots; every
     // supernode reads only ancestors' entries of x and writes its own columns
     for (int l = S.nlev - 1; l >= 0; --l) {
       const int lo = lvo[l], hi = lvo[l + 1];
-      for (int it = lo + warp; it < hi; it += kThreads / 32) {
+      for (int it = lo + warp; it < hi; it += NT / 32) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w > 32 || f_ > kWF) continue;
         bwd_warp(P, S, gs, y, wbuf + warp * kWF, lane);
       }
       __syncthreads();
+      if constexpr (NT == kWide) {
+        double* tbuf = wbuf + (tid / 256) * (kTeamF + kW * (kW + 1));
+        int q = 0;
+        for (int it = lo; it < hi; ++it) {
+          const int gs = S.sn0 + lsn[it];
+          const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
+          if ((w <= 32 && f_ <= kWF) || w > kTeamW || f_ > kTeamF) continue;
+          if ((q++ & 3) != tid / 256) continue;
+          bwd_cta<true>(P, S, gs, y, tbuf, reinterpret_cast<double(*)[kW + 1]>(tbuf + kTeamF), tid % 256, tid / 256);
+        }
+        __syncthreads();
+      }
       for (int it = lo; it < hi; ++it) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w <= 32 && f_ <= kWF) continue;
-        bwd_cta(P, S, gs, y, sfront, sm_blk, tid);
+        if (NT == kWide && w <= kTeamW && f_ <= kTeamF) continue;
+        if constexpr (NT == kWide) bwd_wide(P, S, gs, y, sfront, wsm, tid);
+        else bwd_cta(P, S, gs, y, sfront, sm_blk, tid);
       }
     }
     __syncthreads();
     if (MODE == 0 || MODE == 1) {
-      for (int j = tid; j < S.m_pad; j += kThreads)
+      for (int j = tid; j < S.m_pad; j += NT)
         qi[S.qcol + j] = j < S.m ? P.qsign[S.qcol + j] * y[P.spos[S.col0 + j]] : 0.0;
-    } else if (MODE == 2) {
-      for (int k = tid; k < n; k += kThreads) u[S.dof + k] = y[P.iperm[S.diag0 + k]];
     } else {
-      const int col = P.colperm[S.qcol + itx];  // B row of this sorted column
-      for (int k = tid; k < n; k += kThreads) u[(int64_t)k * S.m + col] = y[P.iperm[S.diag0 + k]];
+      for (int k = tid; k < n; k += NT) u[S.dof + k] = y[P.iperm[S.diag0 + k]];
     }
     __syncthreads();
   }
@@ -665,28 +927,40 @@ inline int grid_for(int64_t n, int per = 256, int cap = 152 * 16) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, cap));
 }
 
-size_t implicit_smem(int nmax, int maxf) { return ((size_t)nmax + maxf + (kThreads / 32) * kWF) * 8; }
+size_t implicit_smem(int nmax, int maxf, bool wide) {
+  return ((size_t)nmax + maxf + (wide ? kWideBuf : kThreads / 32 * kWF)) * 8;
+}
 
-void launch_implicit(int mode, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
+// The wide CTA takes one subdomain per SM; with more subdomains than SMs several 256-thread CTAs per SM hide one
+// another's latency better.
+bool implicit_wide(int nsub, int nsm, int nmax, int maxf) {
+  return nsub <= nsm && implicit_smem(nmax, maxf, true) + 1024 <= 227 * 1024;
+}
+
+template <int MODE>
+static void launch_implicit_mode(bool wide, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
+                                 const double* f, double* qi, double* u, double* uws, int64_t ustride, int nmax,
+                                 int maxf, int grid, size_t smem, cudaStream_t st) {
+  if (wide) {
+    cudaFuncSetAttribute(implicit_kernel<MODE, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    implicit_kernel<MODE, kWide><<<grid, kWide, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
+                                                            maxf);
+  } else {
+    cudaFuncSetAttribute(implicit_kernel<MODE, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    implicit_kernel<MODE, kThreads><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride,
+                                                                  nmax, maxf);
+  }
+}
+
+void launch_implicit(int mode, bool wide, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
                      const double* f, double* qi, double* u, double* uws, int64_t ustride, int nmax, int maxf,
                      int grid, size_t smem, cudaStream_t st) {
-  if (mode == 3) {
-    cudaFuncSetAttribute(implicit_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<3><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
-                                                        maxf);
-  } else if (mode == 0) {
-    cudaFuncSetAttribute(implicit_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<0><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
-                                                        maxf);
-  } else if (mode == 1) {
-    cudaFuncSetAttribute(implicit_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<1><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
-                                                        maxf);
-  } else {
-    cudaFuncSetAttribute(implicit_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<2><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
-                                                        maxf);
-  }
+  auto fn = mode == 0 ? launch_implicit_mode<0> : mode == 1 ? launch_implicit_mode<1> : launch_implicit_mode<2>;
+  fn(wide, P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf, grid, smem, st);
+}
+
+void launch_inv_blocks(const DevPlan& P, int nsub, cudaStream_t st) {
+  inv_block_kernel<<<dim3(32, (unsigned)std::min(nsub, 65535)), 128, 0, st>>>(P, nsub);
 }
 
 void launch_unit_scale(const DevPlan& P, int nsub, int nmax, double* d2, cudaStream_t st) {
@@ -695,10 +969,11 @@ void launch_unit_scale(const DevPlan& P, int nsub, int nmax, double* d2, cudaStr
   unit_scale_kernel<<<dim3((unsigned)gx, (unsigned)std::min(nsub, 65535)), 256, 0, st>>>(P, nsub, d2);
 }
 
-int implicit_occupancy(size_t smem) {
+int implicit_occupancy(size_t smem, bool wide) {
+  if (wide) return 1;
   int nb = 0;
-  cudaFuncSetAttribute(implicit_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, implicit_kernel<0>, kThreads, smem);
+  cudaFuncSetAttribute(implicit_kernel<0, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, implicit_kernel<0, kThreads>, kThreads, smem);
   return std::max(nb, 1);
 }
 
