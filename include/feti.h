@@ -134,7 +134,7 @@ typedef struct {
                                  Cholesky on the FP64 pipe */
   int32_t chol_tc_front;      /* with chol_tc = 0: the narrowest front (w + r) taken by the tensor-core kernel,
                                  with all its ancestors (0 = 256, within 3% of the fastest measured on 3D
-                                 elasticity and uneven 3D heat; at least 128) */
+                                 elasticity and uneven 3D heat; values below 128 act as 128) */
 } feti_options;
 
 typedef struct {

@@ -273,6 +273,64 @@ bool reserve_syrk_oz(feti_ctx* c) {
   return false;
 }
 
+// Buffers and work lists of the FP64 forward solve of the large fronts on the tensor cores; false where there are no
+// such fronts or the digits take more than a third of the free memory (trsm_kernel then solves everything).
+bool reserve_trsm_oz(feti_ctx* c) {
+  if (c->tx_planned && (!c->tx_on || c->d_LD)) return c->tx_on;
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  const bool first = !c->tx_planned;
+  c->tx_planned = true;
+  c->tx_on = false;
+  if (c->ld_bytes == 0 || c->ld_bytes + c->th_bytes > free_b / 3) return false;
+  try {
+    if (first) {
+      std::vector<int4> di;
+      int64_t n256 = 0;
+      for (int i = 0; i < c->nsub; ++i) {
+        auto& P = c->pats[c->subs[i].pat];
+        auto& B = c->bps[c->subs[i].bp];
+        int64_t ofs = 0;
+        for (int s = 0; s < P.nsn; ++s) {
+          if (!P.sn_big[s]) continue;
+          for (int kB = 0; kB < P.sn_w[s]; kB += 128) {
+            if (B.je[s] > B.jb[s]) di.push_back(make_int4(i, s, kB, (int)(ofs / 512)));
+            ofs += trsm_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
+          }
+        }
+        if (P.has_big) n256 += (c->subs[i].m + 255) / 256;
+      }
+      c->tx_cw = n256 >= 2 * (int64_t)c->nsm ? 256 : 128;
+      std::vector<int> order;
+      for (int i = 0; i < c->nsub; ++i)
+        if (c->pats[c->subs[i].pat].has_big && c->subs[i].m > 0) order.push_back(i);
+      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return c->bps[c->subs[a].bp].trsm_flops > c->bps[c->subs[b].bp].trsm_flops;
+      });
+      std::vector<int2> it;
+      for (int i : order)
+        for (int ca = 0; ca < c->subs[i].m; ca += c->tx_cw) it.push_back(make_int2(i, ca));
+      c->n_tx_ditems = (int)di.size();
+      c->n_tx_items = (int)it.size();
+      if (it.empty() || di.empty()) return false;
+      c->tx_grid = std::min(c->nsm, c->n_tx_items);
+      c->d_tx_ditems = upload(c, di);
+      c->d_tx_items = upload(c, it);
+      c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * (c->tx_front + c->tx_stack) * c->tx_cw * 8);
+      c->d_txscr = (char*)dalloc(c, (size_t)c->tx_grid * trsm_oz_scratch(c->tx_cw));
+      CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
+    }
+    if (!c->d_txscr) return false;
+    c->d_LD = dalloc(c, c->ld_bytes);
+    c->d_th = (double*)dalloc(c, std::max<size_t>(c->th_bytes, 8));
+    c->tx_on = true;
+  } catch (std::bad_alloc&) {
+    dfree(c, c->d_LD);
+    c->d_LD = nullptr;
+  }
+  return c->tx_on;
+}
+
 void build(feti_ctx* c) {
   using clk = std::chrono::steady_clock;
   auto t0 = clk::now();
@@ -379,6 +437,8 @@ void build(feti_ctx* c) {
   // or more) get a row-major bf16 hi/lo copy of their panel, pat_lh elements per pattern
   std::vector<int64_t> pat_lh(c->pats.size(), 0), pat_di(c->pats.size(), 0);
   auto lh_big = [&](const PatternPlan& P, int s) { return c->fp32 && (P.sn_r[s] >= 128 || P.sn_w[s] >= 256); };
+  // FP64: the large fronts' digits and update blocks (kern_trsm_oz.cu)
+  std::vector<int64_t> ld_ofs, tx_ofs, th_ofs, pat_ld(c->pats.size(), 0), bp_th(c->bps.size(), 0);
   std::vector<int> lvl_off, lvl_sn, pat_lvl0(c->pats.size());
   int64_t max_usize = 0;
   std::vector<int> pat_sn0(c->pats.size());
@@ -410,6 +470,25 @@ void build(feti_ctx* c) {
         pat_di[p] += (int64_t)((P.sn_w[s] + 127) / 128) * 4 * 32 * 32;
       }
       uofs.push_back(P.uofs[s]);
+    }
+    if (!c->fp32) {
+      // the digits of each 128-column block, and an update stack of the large supernodes alone
+      std::vector<int64_t> size(P.nsn, 0);
+      int64_t top = 0;
+      for (int s = 0; s < P.nsn; ++s) {  // postorder
+        ld_ofs.push_back(P.sn_big[s] ? pat_ld[p] / 512 : -1);
+        int64_t base = top;
+        if (P.sn_big[s]) {
+          for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) base -= size[P.ch_list[k]];
+          for (int kB = 0; kB < P.sn_w[s]; kB += 128) pat_ld[p] += trsm_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
+          const int64_t rp = (P.sn_r[s] + 7) & ~7;
+          size[s] = P.sn_parent[s] >= 0 ? rp : 0;
+          c->tx_front = std::max(c->tx_front, rp);
+          top = base + size[s];
+          c->tx_stack = std::max(c->tx_stack, top);
+        }
+        tx_ofs.push_back(base);
+      }
     }
     pat_lvl0[p] = (int)lvl_off.size();
     {
@@ -448,6 +527,15 @@ void build(feti_ctx* c) {
     jo.insert(jo.end(), B.jo.begin(), B.jo.end());
     Xofs.insert(Xofs.end(), B.Xofs.begin(), B.Xofs.end());
     rhs_ofs.insert(rhs_ofs.end(), B.rhs_stack_ofs.begin(), B.rhs_stack_ofs.end());
+    if (!c->fp32) {
+      auto& P = c->pats[c->bp_pat[b]];
+      for (int s = 0; s < P.nsn; ++s) {
+        const int64_t J = B.je[s] - B.jb[s];
+        const bool slot = !P.sn_big[s] && P.sn_parent[s] >= 0 && P.sn_big[P.sn_parent[s]] && J > 0;
+        th_ofs.push_back(slot ? bp_th[b] : -1);
+        if (slot) bp_th[b] += J * P.sn_r[s];
+      }
+    }
     act.insert(act.end(), B.act.begin(), B.act.end());
     spos.insert(spos.end(), B.spos.begin(), B.spos.end());
     int base = (int)tile_sn.size();
@@ -470,7 +558,7 @@ void build(feti_ctx* c) {
   std::vector<double> eldk, elsc;
   std::vector<double> qsign;
   std::vector<int64_t> fix_pos;
-  int64_t Kofs = 0, Lo = 0, Xo = 0, Fo = 0, qo = 0, dofo = 0, Ro = 0, tpo = 0, hbo = 0, lho = 0, dio = 0;
+  int64_t Kofs = 0, Lo = 0, Xo = 0, Fo = 0, qo = 0, dofo = 0, Ro = 0, tpo = 0, hbo = 0, lho = 0, dio = 0, ldo = 0, tho = 0;
   std::vector<int2> l16_items;
   int fixo = 0, alo = 0;
   double chol = 0, trsm = 0, syrk = 0, syrke = 0, implb = 0;
@@ -521,6 +609,10 @@ void build(feti_ctx* c) {
     hbo += P.hsize;
     I.lh = lho;
     lho += pat_lh[s.pat];
+    I.ld = ldo;
+    ldo += pat_ld[s.pat];
+    I.th = tho;
+    tho += bp_th[s.bp];
     I.di = dio;
     dio += pat_di[s.pat];
     for (int q = 0; q < P.nsn; ++q)
@@ -813,6 +905,11 @@ void build(feti_ctx* c) {
   D.sn_hoff = upload(c, sn_hoff);
   D.lh_ofs = upload(c, lh_ofs);
   D.di_ofs = upload(c, di_ofs);
+  D.ld_ofs = upload(c, ld_ofs);
+  D.tx_ofs = upload(c, tx_ofs);
+  D.th_ofs = upload(c, th_ofs);
+  c->ld_bytes = (size_t)ldo;
+  c->th_bytes = (size_t)tho * 8;
   if (c->fp32) {
     D.LH = (uint16_t*)dalloc(c, (size_t)std::max<int64_t>(lho, 8) * 2);
     D.DI = (float*)dalloc(c, (size_t)std::max<int64_t>(dio, 8) * 4);
@@ -1156,13 +1253,15 @@ feti_status feti_assemble(feti_ctx* ctx) {
   // error is that of its SYRK alone; in the TF32 mode X_i is rounded to TF32 for that SYRK
   const int tcmode = ctx->fp32 ? 2 : 0;
   const int tf32_out = ctx->fp32 && ctx->opt.prec == FETI_PREC_TF32 ? 1 : 0;
+  // FP64: the forward solve of the large fronts by exact slicing on the tensor cores
+  const bool tx = !ctx->fp32 && ctx->opt.assembly_route != 2 && reserve_trsm_oz(ctx);
   ctx->stats.trsm_grid = ctx->fp32 ? ctx->grid_trsm32 : ctx->grid_trsm;
   auto run_trsm = [&](const feti_ctx::TrsmCand& tc, cudaStream_t s2) {
     CK(cudaMemsetAsync(ctx->d_queue + 16, 0, sizeof(int), s2));
     launch_trsm(ctx->P, tc.d_items, tc.nitems, tc.cw, ctx->d_queue + 16, ctx->d_X, ctx->fp32, ctx->d_ws,
                 ctx->ws_stride, ctx->rhs_front, std::min(ctx->fp32 ? ctx->grid_trsm32 : ctx->grid_trsm, tc.nitems),
                 tcmode, tf32_out,
-                ctx->d_status, s2, 0, ctx->d_X2, ctx->d_L32, split ? 1 : 0);
+                ctx->d_status, s2, 0, ctx->d_X2, ctx->d_L32, split ? 1 : 0, tx ? ctx->d_th : nullptr);
   };
   // FP64: the SYRK by exact slicing on the tensor cores
   const bool oz = !ctx->fp32 && ctx->opt.assembly_route != 2 && ctx->stats.syrk_flops > 0 && reserve_syrk_oz(ctx);
@@ -1223,6 +1322,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       launch_l32(ctx->P.L, ctx->d_L32, ctx->stats.L_doubles, ctx->nsm * 8, s2);
       launch_l16(ctx->P, ctx->d_l16_items, ctx->n_l16, ctx->d_L32, ctx->P.LH, ctx->P.DI, ctx->nsm * 6, s2);
     }
+    if (tx) launch_dig_l(ctx->P, ctx->d_tx_ditems, ctx->n_tx_ditems, ctx->d_LD, s2);
     if (!ctx->trsm_tuned) {
       // autotuner: time every work split of the TRSM on this problem (X is the same bitwise for all)
       for (auto& tc : ctx->trsm_cands) {
@@ -1242,6 +1342,13 @@ feti_status feti_assemble(feti_ctx* ctx) {
       CK(cudaEventRecord(ctx->ev[1], s2));
     }
     run_trsm(ctx->trsm_cands[ctx->trsm_pick], s2);
+    if (tx) {
+      CK(cudaMemsetAsync(ctx->d_queue + 17, 0, sizeof(int), s2));
+      launch_trsm_oz(ctx->P, ctx->d_tx_items, ctx->n_tx_items, ctx->tx_cw, ctx->d_queue + 17, ctx->d_LD, ctx->d_th,
+                     (double*)ctx->d_X, ctx->d_txws, (ctx->tx_front + ctx->tx_stack) * ctx->tx_cw,
+                     ctx->tx_front * ctx->tx_cw, ctx->d_txscr, trsm_oz_scratch(ctx->tx_cw), ctx->tx_grid,
+                     ctx->d_status, s2);
+    }
     // the implicit solves take L in unit-lower form; the TRSM above was its last user as L
     launch_unit_scale(ctx->P, ctx->nsub, ctx->nmax, ctx->P.dinv, s2);
     if (ctx->impl_wide) launch_inv_blocks(ctx->P, ctx->nsub, s2);
@@ -1290,6 +1397,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
   };
   // Cholesky, pruned TRSM, unit-lower scaling, SYRK (+ lumped values, or the Dirichlet factorisation and tiles)
   ctx->stats.launches += 4 + (ctx->precond_kind == 1 ? 1 : ctx->precond_kind == 2 ? 2 : 0);
+  if (tx) ctx->stats.launches += 2;
   if (oz) ctx->stats.launches += 3 * (int64_t)ctx->oz_batches.size() - 1;
   const int want = ctx->opt.assembly_route;
   if (want == 2 || (want == 3 && ctx->route_tuned && ctx->route == 2)) {
@@ -1301,7 +1409,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
     }
     enqueue(st, cudaEventRecordDefault, true);
     CK(cudaGetLastError());
-  } else if (ctx->asm_exec && ctx->asm_X == ctx->d_X && ctx->asm_X2 == ctx->d_X2 && ctx->asm_XD == ctx->d_XD) {
+  } else if (ctx->asm_exec && ctx->asm_X == ctx->d_X && ctx->asm_X2 == ctx->d_X2 && ctx->asm_XD == ctx->d_XD &&
+             ctx->asm_LD == ctx->d_LD) {
     CK(cudaGraphLaunch(ctx->asm_exec, st));
   } else {
     ctx->route = want == 1 ? 1 : 0;
@@ -1346,6 +1455,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       ctx->asm_X = ctx->d_X;
       ctx->asm_X2 = ctx->d_X2;
       ctx->asm_XD = ctx->d_XD;
+      ctx->asm_LD = ctx->d_LD;
     }
   }
   CK(cudaGetLastError());
@@ -1366,6 +1476,10 @@ feti_status feti_assemble(feti_ctx* ctx) {
     ctx->d_X2 = nullptr;
     dfree(ctx, ctx->d_XD);
     ctx->d_XD = nullptr;
+    dfree(ctx, ctx->d_LD);
+    ctx->d_LD = nullptr;
+    dfree(ctx, ctx->d_th);
+    ctx->d_th = nullptr;
   }
   float a, b, cc, d;
   CK(cudaEventElapsedTime(&a, ctx->ev[0], ctx->ev[1]));

@@ -42,6 +42,8 @@ struct SubInfo {
   int64_t rpart;     // unused
   int64_t hbase;     // base of this subdomain's Cholesky hand-over slots (doubles)
   int64_t lh;        // base of this subdomain's row-major bf16 hi/lo panels (LH, elements)
+  int64_t ld;        // base of this subdomain's digits of the large panels (LD, bytes)
+  int64_t th;        // base of its update blocks handed from trsm_kernel to trsm_oz_kernel (doubles)
   int64_t di;        // base of this subdomain's inverted 32 x 32 diagonal blocks of the large panels (DI, floats)
 };
 
@@ -79,6 +81,9 @@ struct DevPlan {
   uint16_t* LH;              // row-major bf16 hi/lo copies of the large panels (mixed precision)
   const int64_t* di_ofs;     // [sn] offset of the supernode's inverted diagonal blocks in DI (relative to the
                              // subdomain's di; 4 blocks of 32 x 32 per 128 own rows), -1 where lh_ofs is -1
+  const int64_t* ld_ofs;     // [sn] offset of a large supernode's digits in LD (512 bytes, relative), -1 otherwise
+  const int64_t* tx_ofs;     // [sn] a large supernode's update block on trsm_oz_kernel's stack (doubles per column)
+  const int64_t* th_ofs;     // [bsn] hand-over slot of a supernode below a large one (doubles, relative), -1 otherwise
   float* DI;                 // inverses of the 32 x 32 diagonal blocks of the large panels (FP32)
   double* dinv;              // [dof + j] reciprocal pivots 1 / L_jj (written after the factorisation)
   // bplan tables

@@ -97,6 +97,17 @@ struct feti_ctx {
   bool syrk_tuned = false;
   int* d_impl_order = nullptr;
   int2* d_syrk_items = nullptr;
+  // FP64 forward solve of the large fronts on the tensor cores
+  bool tx_planned = false, tx_on = false;
+  int4* d_tx_ditems = nullptr;       // 128-column blocks of the large panels to cut
+  int2* d_tx_items = nullptr;        // (subdomain, first column) of the solve
+  int n_tx_ditems = 0, n_tx_items = 0, tx_cw = 128, tx_grid = 0;
+  size_t ld_bytes = 0, th_bytes = 0;
+  int64_t tx_front = 0, tx_stack = 0;  // doubles per column
+  void* d_LD = nullptr;              // digits of the large panels
+  double* d_th = nullptr;            // update blocks handed over
+  double* d_txws = nullptr;          // fronts and stacks
+  char* d_txscr = nullptr;           // digits of X per CTA
   // FP64 SYRK on the tensor cores: batches of subdomains, their tiles and X pieces, digits and column exponents
   std::vector<feti::OzBatch> oz_batches;
   int4* d_oz_items = nullptr;
@@ -173,6 +184,7 @@ struct feti_ctx {
   void* asm_X = nullptr;             // the X buffers the assembly graph was captured with
   void* asm_X2 = nullptr;
   void* asm_XD = nullptr;
+  void* asm_LD = nullptr;
   uint16_t* d_X2 = nullptr;          // bf16 hi/lo copy of X (split-bf16 SYRK operands)
   float* d_L32 = nullptr;            // FP32 copy of L for the mixed TRSM
   cudaGraphExec_t pcg_exec = nullptr;  // captured chunk of iterations (replayed on st)

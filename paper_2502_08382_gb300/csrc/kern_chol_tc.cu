@@ -20,29 +20,20 @@
 // What bounds it now: on wide fronts the staging of the digits (96 KB from L2 per 2304 clocks of MMA), on fronts of a
 // few hundred rows the pivot blocks (16 k clocks of FP64 work for 32 columns) and the barriers between the phases.
 //
-// The digits are written pre-swizzled (64-byte swizzle, 8-row atoms): [digit][32-deep chunk][row][64 bytes], so any
-// 8-row-aligned run of rows of one digit and chunk is a ready operand, loaded by one bulk copy.  Tiles are 128 rows x
-// 64 columns: a stage holds the 8 A digits and the digits of two blocks of 32 B columns, each with its own set of
-// accumulators (256 TMEM columns), so one set is drained while the other is filled.  Warp 0 issues the MMAs, warp 1
-// the copies, warps 4-11 run the epilogue; all twelve do the rest.  Every mbarrier wait is bounded; a CTA that gives
-// up keeps to the cluster's barriers and skips its work.
+// The products run on the tiles of oz_engine.cuh.  Every mbarrier wait is bounded; a CTA that gives up keeps to the
+// cluster's barriers and skips its work.
 #include <algorithm>
 #include <cuda_bf16.h>
 
 #include "chol_common.cuh"
 #include "common.cuh"
 #include "kernels.h"
-#include "oz.cuh"
+#include "oz_engine.cuh"
 
 namespace feti {
 namespace {
 
-constexpr int kCT = 384;                                    // threads per CTA
-constexpr int kCM = 128, kCH = 32;                          // rows of a tile, columns of one B block
-constexpr int kCA = kCM * 64, kCB = kCH * 64;               // bytes of one digit of A / of a B block (one chunk)
-constexpr int kCStage = kDig * (kCA + 2 * kCB);             // 96 KB
-constexpr int kCStages = 2;
-constexpr int kCBlk = 128;                                  // columns per block
+constexpr int kCBlk = 128;                                      // columns per block
 constexpr int kCDyn = 1024 + kCStages * kCStage + kDig * kCB;  // + the digits of L_bb^{-1}
 
 struct PivotSmem {
@@ -70,265 +61,71 @@ __device__ __forceinline__ void cl_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
-__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-struct CtState {
-  uint8_t* ring;
-  uint8_t* bpan;      // digits of L_bb^{-1}
-  uint64_t *full, *empty, *accf, *acce, *drain;
-  volatile int* abort;
-  uint32_t tmem;
-  uint32_t chunks;    // chunks staged so far (stage and phase)
-  uint32_t units;     // 32-column units multiplied so far (accumulator set and phase)
+// The panel: Out[row, j] = (A L_bb^{-T})[row, j] for j < ncol to the front's columns kb + j, rows i0 + row.
+struct PanelJob {
+  static constexpr int kUnits = 1;
+  static constexpr bool kBSmem = true;
+  const char* SA;
+  const int *EX, *EXB;
+  int64_t digA, digB;
+  int nck, n, ncol;
+  double* out;  // row 0 of column kb
+  int64_t f;
+  __device__ __forceinline__ void tile(int t, int& tm, int& tn) const {
+    tm = t;
+    tn = 0;
+  }
+  __device__ __forceinline__ const char* a(int tm, int) const { return SA + (int64_t)tm * kCM * 64; }
+  __device__ __forceinline__ const char* b(int, int) const { return nullptr; }
+  __device__ __forceinline__ int begin(int ri) const { return ri < n ? __ldcg(EX + ri) : 0; }
+  __device__ __forceinline__ int load(int ri, int cb, double (&)[16]) const {
+    return ri < n ? min(16, ncol - cb) : 0;
+  }
+  __device__ __forceinline__ int ec(int c) const { return EXB[c]; }
+  __device__ __forceinline__ void store(int ri, int c, double, double t) const { out[(int64_t)c * f + ri] = t; }
 };
 
-// the value 2^ex (2^32 hi + lo) rounded to nearest, by integer arithmetic
-__device__ __forceinline__ double dig_value(long long hi, long long lo, int ex) {
-  hi += lo >> 32;
-  uint32_t l = (uint32_t)lo;
-  const bool neg = hi < 0;
-  if (neg) {
-    hi = ~hi + (l == 0);
-    l = -l;
-  }
-  unsigned long long h = (unsigned long long)hi;
-  if (h == 0) {
-    h = l;
-    l = 0;
-    ex -= 32;
-  }
-  const int lz = __clzll((long long)h);
-  const unsigned long long x = (unsigned long long)l << 32;
-  const unsigned long long m = lz < 64 ? (h << lz) | (lz ? x >> (64 - lz) : 0ULL) : 0ULL;
-  const unsigned long long mant = (m >> 11) + ((m >> 10) & 1);  // 53 bits, 2^52 <= mant <= 2^53
-  const int e = 95 - lz + ex;                                   // value = mant 2^(e - 52)
-  unsigned long long b = ((unsigned long long)(e + 1022) << 52) + mant;
-  if (h == 0 || e < -1021) b = 0;
-  if (h != 0 && e > 1022) b = 0x7FF0000000000000ULL;
-  return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ULL : 0ULL)));
-}
-
-// Digits of the rows [r0, r1) (multiples of 8) of the column-major A (ld, K <= 128 columns): row exponents EX and the
-// digits in the layout above (npad rows; rows >= n are zero).  Four lanes per row, eight of its columns each.
-template <int NCK>
-__device__ __forceinline__ void dig_rows(const double* A, int64_t ld, int n, int K, int r0, int r1, char* SL, int nck,
-                                         int npad, int* EX, int warp, int nwarps) {
-  const int lane = threadIdx.x % 32, q = lane & 3;
-  for (int rb = r0 + warp * 8; rb < r1; rb += nwarps * 8) {
-    const int i = rb + (lane >> 2);
-    double v[NCK][8];
-    uint32_t mx = 0;
-#pragma unroll
-    for (int c = 0; c < NCK; ++c)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = c * 32 + q * 8 + e;
-        v[c][e] = (i < n && k < K) ? __ldcg(A + (int64_t)k * ld + i) : 0.0;
-        mx = max(mx, (uint32_t)__double2hiint(v[c][e]) & 0x7fffffffu);
-      }
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const int ex = dig_exponent(mx);
-    if (q == 0) EX[i] = ex;
-    const int64_t o = (int64_t)i * 64 + ((q ^ ((i >> 1) & 3)) << 4);
-#pragma unroll
-    for (int c = 0; c < NCK; ++c) {
-      if (c >= nck) break;
-      uint64_t w[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[c][e], ex);
-#pragma unroll
-      for (int p = 0; p < kDig; ++p)
-        *reinterpret_cast<uint4*>(SL + ((int64_t)(p * nck + c) * npad) * 64 + o) =
-            make_uint4(dig_pair(w[0], w[1], p), dig_pair(w[2], w[3], p), dig_pair(w[4], w[5], p),
-                       dig_pair(w[6], w[7], p));
-    }
-  }
-}
-
-// One phase of products on the tensor cores.  Tiles t = first, first + step, ... < ntile:
-//  PANEL   tile t is row block t of A (digits SA, one chunk); Out[row, j] = (A L_bb^{-T})[row, j] for j < ncol, written
-//          to Ls columns kb + j (row i0 + row of the front); exponents of L_bb^{-1} in EXB.
-//  update  tile t is (row block tm, 64-column block tn): C -= A A^T for the columns [i0, ce) on and below the diagonal,
-//          C in Ls (columns < w) or W; n = rows of A.
-template <bool PANEL>
-__device__ __forceinline__ void dig_product(CtState& st, const char* SA, const int* EX, const int* EXB, int n, int nck,
-                                            int first, int step, int ntile, int ntn, double* Ls, int64_t f, int w,
-                                            double* W, int r, int i0, int kb, int ncol) {
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int npad = (n + kCM - 1) / kCM * kCM;
-  const int64_t digA = (int64_t)nck * npad * 64;  // bytes between digits
-  const uint32_t ring = smem_u32(st.ring);
-  // tile t: row block tm holds min(2 (tm + 1), ntn) column blocks
-  auto tile_of = [&](int t, int& tm, int& tn) {
-    if (PANEL) {
-      tm = t;
-      tn = 0;
-      return;
-    }
-    tm = 0;
-    const int nfull = (ntn + 1) / 2;  // row blocks before this one have fewer column blocks
+// C -= A A^T for the columns [i0, i0 + ncol) of the front on and below the diagonal, C in Ls (columns < w) or W;
+// n = rows of A, row block tm holds min(2 (tm + 1), ntn) blocks of 64 columns.
+struct UpdateJob {
+  static constexpr int kUnits = 2;
+  static constexpr bool kBSmem = false;
+  const char* SA;
+  const int* EX;
+  int64_t digA, digB;
+  int nck, n, npad, ntn, ncol, i0, w, r;
+  double *Ls, *W;
+  int64_t f;
+  __device__ __forceinline__ void tile(int t, int& tm, int& tn) const {
+    const int nfull = (ntn + 1) / 2;  // the row blocks before this one have fewer column blocks
     // sum_{m < tm} 2 (m + 1) = tm (tm + 1)
     tm = (int)((sqrtf(4.f * t + 1.f) - 1.f) * 0.5f);
     while ((tm + 1) * (tm + 2) <= t) ++tm;
     while (tm * (tm + 1) > t) --tm;
     if (tm >= nfull - 1) {
-      const int base = (nfull - 1) * nfull;  // tiles of the first nfull - 1 row blocks
-      const int q = t - base;
-      const int c0 = min(2 * nfull, ntn);
-      tm = nfull - 1 + q / c0;
-      tn = q % c0;
+      const int q = t - (nfull - 1) * nfull;  // past the tiles of the first nfull - 1 row blocks
+      tm = nfull - 1 + q / ntn;
+      tn = q % ntn;
       return;
     }
     tn = t - tm * (tm + 1);
-  };
-  const int mine = first < ntile ? (ntile - first + step - 1) / step : 0;
-  const uint32_t nu = PANEL ? 1 : 2;  // units (32-column blocks) per tile
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();  // the ring's generic use is over
-  const bool live = !*st.abort;
-  if (live && warp == 1 && lane == 0) {
-    // ---- copies
-    bool ok = true;
-    uint32_t cg = st.chunks;
-    for (int q = 0; q < mine && ok; ++q) {
-      int tm, tn;
-      tile_of(first + q * step, tm, tn);
-      for (int c = 0; c < nck && ok; ++c, ++cg) {
-        const uint32_t s = cg % kCStages;
-        if (cg >= kCStages) ok = dig_wait(smem_u32(&st.empty[s]), ((cg / kCStages) - 1) & 1, st.abort);
-        if (!ok) break;
-        const uint32_t sA = ring + s * kCStage, sB = sA + kDig * kCA, bar = smem_u32(&st.full[s]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                     "r"(PANEL ? kDig * kCA : kCStage)
-                     : "memory");
-        const char* a0 = SA + ((int64_t)c * npad + (int64_t)tm * kCM) * 64;
-        const char* b0 = SA + ((int64_t)c * npad + (int64_t)tn * 64) * 64;
-#pragma unroll 1
-        for (int p = 0; p < kDig; ++p) {
-          bulk_copy(sA + p * kCA, a0 + p * digA, kCA, bar);
-          if (!PANEL) {
-            bulk_copy(sB + p * kCB, b0 + p * digA, kCB, bar);
-            bulk_copy(sB + (kDig + p) * kCB, b0 + p * digA + kCB, kCB, bar);
-          }
-        }
-      }
-    }
-    if (!ok) {
-      // the copies in flight land (bounded) before the block goes on
-      for (uint32_t k = cg > kCStages ? cg - kCStages : 0; k < cg; ++k)
-        mbar_wait(smem_u32(&st.full[k % kCStages]), (k / kCStages) & 1);
-    }
-  } else if (live && warp == 0 && lane == 0) {
-    // ---- MMAs
-    bool ok = true, issued = false;
-    uint32_t cg = st.chunks, un = st.units;
-    for (int q = 0; q < mine && ok; ++q, un += nu) {
-      for (int c = 0; c < nck && ok; ++c, ++cg) {
-        const uint32_t s = cg % kCStages;
-        ok = dig_wait(smem_u32(&st.full[s]), (cg / kCStages) & 1, st.abort);
-        const uint32_t sA = ring + s * kCStage, sB = PANEL ? smem_u32(st.bpan) : sA + kDig * kCA;
-        for (uint32_t h = 0; h < nu && ok; ++h) {
-          const uint32_t u = un + h, set = u & 1;
-          if (c == 0 && u >= 2) ok = dig_wait(smem_u32(&st.acce[set]), ((u >> 1) - 1) & 1, st.abort);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-          for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-            for (int p = 0; p < kDig; ++p)
-              mma_f16(st.tmem + set * 256 + p * kCH, sw64_desc(sA + p * kCA + kk * 32),
-                      sw64_desc(sB + h * (kDig * kCB) + kk * 32), idesc_m128(1u, (uint32_t)(kCH * (kDig - p))),
-                      (c == 0 && kk == 0 && p == 0) ? 0u : 1u);
-          issued = true;
-          if (c == nck - 1) mma_commit(smem_u32(&st.accf[set]));
-        }
-        if (ok) mma_commit(smem_u32(&st.empty[s]));
-      }
-    }
-    if (!ok && issued) {  // nothing is issued after this: every MMA is done before TMEM is released
-      mma_commit(smem_u32(st.drain));
-      mbar_wait(smem_u32(st.drain), 0);
-    }
-  } else if (live && warp >= 4) {
-    // ---- epilogue: TMEM lane quarter warp % 4, 16 columns of the unit
-    const int quarter = warp % 4, ch = (warp - 4) / 4;
-    uint32_t un = st.units;
-    int ok = 1;
-    for (int q = 0; q < mine && ok; ++q) {
-      int tm, tn;
-      tile_of(first + q * step, tm, tn);
-      const int ri = tm * kCM + quarter * 32 + lane, gi = i0 + ri;  // row of A / of the front
-      const int ei = ri < n ? __ldcg(EX + ri) : 0;
-      for (uint32_t h = 0; h < nu && ok; ++h, ++un) {
-        const uint32_t set = un & 1;
-        const int cb = tn * 64 + h * kCH + ch * 16;  // first column (relative to i0, or to kb)
-        // the C entries this thread subtracts from, loaded while the tile is multiplied
-        double* base = nullptr;
-        int64_t ld = 0;
-        int nc = 0;
-        double cv[16];
-        if (PANEL) {
-          base = Ls + (int64_t)(kb + cb) * f + gi;
-          ld = f;
-          nc = ri < n ? min(16, ncol - cb) : 0;
-        } else {
-          nc = ri < n ? min(16, min(ncol, ri + 1) - cb) : 0;
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int gj = i0 + cb + e;
-            cv[e] = e < nc ? __ldcg(gj < w ? Ls + (int64_t)gj * f + gi : W + (int64_t)(gj - w) * r + (gi - w)) : 0.0;
-          }
-        }
-        if (lane == 0) ok = dig_wait(smem_u32(&st.accf[set]), (un >> 1) & 1, st.abort) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t t0 = st.tmem + ((uint32_t)(quarter * 32) << 16) + set * 256 + ch * 16;
-#pragma unroll
-        for (int e0 = 0; e0 < 16; e0 += 4) {
-          uint32_t a[4][kDig];
-#pragma unroll
-          for (int d = 0; d < kDig; ++d) tmem_ld4(t0 + d * kCH + e0, a[0][d], a[1][d], a[2][d], a[3][d]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (e0 == 12) {  // the set's last columns are in registers: hand it back
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&st.acce[set]);
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int c = e0 + e;
-            if (c < nc) {
-              long long hi = 0, lo = 0;
-              dig_sum(a[e], hi, lo);
-              const int ej = PANEL ? EXB[cb + c] : __ldcg(EX + cb + c);
-              double t = dig_value(hi, lo, ei + ej - 68);
-              if (ei == kExpBad || ej == kExpBad) t = __longlong_as_double(0x7FF8000000000000LL);
-              if (PANEL) {
-                base[c * ld] = t;
-              } else {
-                const int gj = i0 + cb + c;
-                if (gj < w) Ls[(int64_t)gj * f + gi] = cv[c] - t;
-                else W[(int64_t)(gj - w) * r + (gi - w)] = cv[c] - t;
-              }
-            }
-          }
-        }
-      }
-    }
   }
-  __syncthreads();
-  if (live) {
-    st.chunks += (uint32_t)(mine * nck);
-    st.units += (uint32_t)mine * nu;
+  __device__ __forceinline__ const char* a(int tm, int c) const { return SA + ((int64_t)c * npad + (int64_t)tm * kCM) * 64; }
+  __device__ __forceinline__ const char* b(int tn, int c) const { return SA + ((int64_t)c * npad + (int64_t)tn * 64) * 64; }
+  __device__ __forceinline__ int begin(int ri) const { return ri < n ? __ldcg(EX + ri) : 0; }
+  __device__ __forceinline__ double* at(int ri, int c) const {
+    const int gi = i0 + ri, gj = i0 + c;
+    return gj < w ? Ls + (int64_t)gj * f + gi : W + (int64_t)(gj - w) * r + (gi - w);
   }
-}
+  __device__ __forceinline__ int load(int ri, int cb, double (&cv)[16]) const {
+    const int nc = ri < n ? min(16, min(ncol, ri + 1) - cb) : 0;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) cv[e] = e < nc ? __ldcg(at(ri, cb + e)) : 0.0;
+    return nc;
+  }
+  __device__ __forceinline__ int ec(int c) const { return __ldcg(EX + c); }
+  __device__ __forceinline__ void store(int ri, int c, double cv, double t) const { *at(ri, c) = cv - t; }
+};
 
 // L_bb and L_bb^{-1} of the nbk x nbk block in sm.D by the CTA's first eight warps: lane = row, warp v holds columns
 // v, v + 8, v + 16, v + 24 of the block (from the diagonal on) and of the inverse (up to the diagonal).  Elimination of
@@ -585,7 +382,7 @@ __global__ void __launch_bounds__(kCT, 1)
             // warps 8-11 start on the panel rows while the others factor the block
             if (warp >= 8)
               for (int tm = rank; tm < ntm; tm += C)
-                dig_rows<1>(Ls + (int64_t)kb * f + ke, f, n, nbk, tm * kCM, tm * kCM + kCM, S1, 1, npad, EX1,
+                dig_rows<1>(ColMajor{Ls + (int64_t)kb * f + ke, f}, n, nbk, tm * kCM, tm * kCM + kCM, S1, 1, npad, EX1,
                             warp - 8, 4);
             __syncthreads();
             dig_inverse(sm, st.bpan, EXB);
@@ -594,11 +391,12 @@ __global__ void __launch_bounds__(kCT, 1)
               const int idx = tid + u * kCT;
               lb[u] = idx < kNB * kNB ? sm.D[idx % kNB][idx / kNB] : 0.0;
             }
-            dig_product<true>(st, S1, EX1, EXB, n, 1, rank, C, ntm, 1, Ls, f, w, W, r, ke, kb, nbk);
+            PanelJob pj{S1, EX1, EXB, (int64_t)npad * 64, 0, 1, n, nbk, Ls + (int64_t)kb * f + ke, f};
+            dig_product(st, pj, rank, C, ntm);
             if (ke < kE)
               for (int tm = rank; tm < ntm; tm += C)
-                dig_rows<1>(Ls + (int64_t)kb * f + ke, f, n, nbk, tm * kCM, tm * kCM + kCM, S2, 1, npad, EX2, warp,
-                            kCT / 32);
+                dig_rows<1>(ColMajor{Ls + (int64_t)kb * f + ke, f}, n, nbk, tm * kCM, tm * kCM + kCM, S2, 1, npad, EX2,
+                            warp, kCT / 32);
             cl_sync();
             if (rank == 0)  // every CTA has read the block
               for (int u = 0; u < 3; ++u) {
@@ -609,7 +407,8 @@ __global__ void __launch_bounds__(kCT, 1)
               const int ntn = (kE - ke + 63) / 64;
               int ntile = 0;
               for (int tm = 0; tm < ntm; ++tm) ntile += min(2 * (tm + 1), ntn);
-              dig_product<false>(st, S2, EX2, nullptr, n, 1, rank, C, ntile, ntn, Ls, f, w, W, r, ke, 0, kE - ke);
+              UpdateJob uj{S2, EX2, (int64_t)npad * 64, (int64_t)npad * 64, 1, n, npad, ntn, kE - ke, ke, w, r, Ls, W, f};
+              dig_product(st, uj, rank, C, ntile);
               cl_sync();
             }
           }
@@ -618,11 +417,13 @@ __global__ void __launch_bounds__(kCT, 1)
             const int npad = (n + kCM - 1) / kCM * kCM, ntm = npad / kCM, ntn = (n + 63) / 64;
             int* EX = reinterpret_cast<int*>(SL + (int64_t)npad * 64 * kDig * nck);
             for (int q = (rank * (kCT / 32) + warp) * 8; q < npad; q += C * (kCT / 32) * 8)
-              dig_rows<4>(Ls + (int64_t)kB * f + kE, f, n, K2, q, q + 8, SL, nck, npad, EX, 0, 1);
+              dig_rows<4>(ColMajor{Ls + (int64_t)kB * f + kE, f}, n, K2, q, q + 8, SL, nck, npad, EX, 0, 1);
             cl_sync();
             int ntile = 0;
             for (int tm = 0; tm < ntm; ++tm) ntile += min(2 * (tm + 1), ntn);
-            dig_product<false>(st, SL, EX, nullptr, n, nck, rank, C, ntile, ntn, Ls, f, w, W, r, kE, 0, n);
+            const int64_t dig = (int64_t)nck * npad * 64;
+            UpdateJob uj{SL, EX, dig, dig, nck, n, npad, ntn, n, kE, w, r, Ls, W, f};
+            dig_product(st, uj, rank, C, ntile);
             cl_sync();
           }
         }

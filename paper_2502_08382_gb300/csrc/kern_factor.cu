@@ -1046,12 +1046,14 @@ __device__ __forceinline__ float round_tf32(float x) {
 // supernode then handles J_s restricted to the block; the restricted ranges nest like J_s itself.
 // X2 (FP32 X only): also write each finished block as bf16 hi/lo halves (hi = bf16(x), lo = bf16(x - hi)),
 // per column wp hi values then wp lo values, for the split-bf16 SYRK.
+// hand (FP64 only): the large fronts are left out, and the update blocks of their children go to their hand-over
+// slots (all columns of J_s, column-major).
 // LT: the factor in the solve's precision (the FP32 copy of L for T = float, L itself for T = double).
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 3)
     trsm_kernel(DevPlan P, const int2* items, int nitems, int cw, int* queue, const T* LT, T* X, T* ws,
                 int64_t ws_stride, int64_t front_sz, int tcmode, int tf32_out, int unit, uint16_t* X2, int x2_out,
-                int* status) {
+                T* hand, int* status) {
   __shared__ uint64_t tc_mbar;
   __shared__ uint64_t tc_gbar[kGS];
   __shared__ uint32_t tc_tmem;
@@ -1105,6 +1107,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     for (int a = 0; a < S.nact; ++a) {
       const int s = P.act[S.act0 + a];
       const int gs = S.sn0 + s, bs = S.bsn0 + s;
+      if (sizeof(T) == 8 && hand && P.sn_big[gs]) continue;  // trsm_oz_kernel's fronts
       const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
       const int wp = (w + 7) & ~7;
       const int jb = max(P.jb[bs], ca), je = min(P.je[bs], cb), jo = max(P.jo[bs], ca);
@@ -1185,6 +1188,8 @@ __global__ void __launch_bounds__(kThreads, 3)
       }
       if (P.sn_parent[gs] >= 0 && !(lho >= 0 && X2s && r > 0)) {
         T* dst = stack + P.rhs_ofs[bs];
+        if (sizeof(T) == 8 && hand && P.th_ofs[bs] >= 0)  // the parent is one of trsm_oz_kernel's fronts
+          dst = hand + S.th + P.th_ofs[bs] + (int64_t)(jb - P.jb[bs]) * r;
         for (int64_t idx = tid; idx < (int64_t)r * J; idx += kThreads) dst[idx] = W2[idx];
       }
       __syncthreads();
@@ -1312,7 +1317,7 @@ static int trsm_smem(bool fp32, int tcmode) {
 
 void launch_trsm(const DevPlan& P, const int2* items, int nitems, int cw, int* queue, void* X, bool fp32,
                  double* ws, int64_t ws_stride, int64_t front_sz, int grid, int tcmode, int tf32_out, int* status,
-                 cudaStream_t st, int unit, uint16_t* X2, const float* L32, int x2_out) {
+                 cudaStream_t st, int unit, uint16_t* X2, const float* L32, int x2_out, double* hand) {
   const int smem = trsm_smem(fp32, tcmode);
   if (fp32) {
     cudaFuncSetAttribute(trsm_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1320,11 +1325,11 @@ void launch_trsm(const DevPlan& P, const int2* items, int nitems, int cw, int* q
                          cudaSharedmemCarveoutMaxShared);
     trsm_kernel<float><<<grid, kThreads, smem, st>>>(P, items, nitems, cw, queue, L32, (float*)X, (float*)ws,
                                                      2 * ws_stride, front_sz, tcmode, tf32_out, 0, X2, x2_out,
-                                                     status);
+                                                     nullptr, status);
   } else {
     cudaFuncSetAttribute(trsm_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     trsm_kernel<double><<<grid, kThreads, smem, st>>>(P, items, nitems, cw, queue, P.L, (double*)X, ws, ws_stride,
-                                                      front_sz, 0, 0, unit, nullptr, 0, status);
+                                                      front_sz, 0, 0, unit, nullptr, 0, hand, status);
   }
 }
 

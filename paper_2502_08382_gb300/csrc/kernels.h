@@ -27,9 +27,11 @@ void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue,
 // per X element): the large fronts (P.lh_ofs >= 0, tcmode 2) use it as GEMM operand; with x2_out every
 // finished block is written to it (the split-bf16 SYRK reads it)
 // L32 (FP32 X only): the FP32 copy of L (launch_l32)
+// hand (FP64 only): leave the large fronts (P.sn_big) out and write the update blocks of their children there
 void launch_trsm(const DevPlan& P, const int2* items, int nitems, int cw, int* queue, void* X, bool fp32,
                  double* ws, int64_t ws_stride, int64_t front_sz, int grid, int tcmode, int tf32_out, int* status,
-                 cudaStream_t st, int unit = 0, uint16_t* X2 = nullptr, const float* L32 = nullptr, int x2_out = 0);
+                 cudaStream_t st, int unit = 0, uint16_t* X2 = nullptr, const float* L32 = nullptr, int x2_out = 0,
+                 double* hand = nullptr);
 int trsm_ctas_per_sm(bool fp32, int tcmode);
 // the row-major bf16 hi/lo copies of the large panels (P.LH) and the inverses of their 32 x 32 diagonal
 // blocks (P.DI) from the FP32 copy of L; items: (subdomain, local supernode) of every panel with P.lh_ofs >= 0
@@ -46,6 +48,15 @@ void launch_syrk_f64(const DevPlan& P, const int2* items, int nitems, const doub
                      cudaStream_t st);
 void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const int4* ditems, const int4* items,
                     void* XD, int* EX, double* F, int nsm, int* status, cudaStream_t st);
+// FP64 forward solve of the large fronts on the tensor cores (kern_trsm_oz.cu): digits of the large panels (items:
+// subdomain, supernode, first column of the 128-column block, its offset / 512), then, after launch_trsm with `hand`,
+// blocks of cw sorted columns (items: subdomain, first column); ws: per CTA front_sz + stack doubles
+int64_t trsm_oz_block_bytes(int w, int r, int kB);
+int64_t trsm_oz_scratch(int cw);
+void launch_dig_l(const DevPlan& P, const int4* items, int nitems, void* LD, cudaStream_t st);
+void launch_trsm_oz(const DevPlan& P, const int2* items, int nitems, int cw, int* queue, const void* LD,
+                    const double* hand, double* X, double* ws, int64_t ws_stride, int64_t front_sz, void* scratch,
+                    int64_t scratch_stride, int grid, int* status, cudaStream_t st);
 // chunks of the tile whose contributing supernodes have np[0 .. n) 8-row pieces (the loaders' batching)
 int syrk_oz_chunks(const int* np, int n);
 
