@@ -186,7 +186,8 @@ def other_rooflines(st, impl_ms, hbm):
 
 # Variant index of the apply autotuner -> kernel name.
 APPLY_KERNELS = ["apply_tiles_kernel<{t}, 4>", "apply_tiles_kernel<{t}, 8>", "apply_tiles_kernel<{t}, 16>",
-                 "apply_ring_kernel<{t}, 4, 3>", "apply_ring_kernel<{t}, 8, 3>", "apply_ring_kernel<{t}, 2, 6>"]
+                 "apply_ring_kernel<{t}, 4, 3>", "apply_ring_kernel<{t}, 8, 3>", "apply_ring_kernel<{t}, 2, 6>",
+                 "apply_dig_kernel"]
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the FP32 apply tile kernels (all variants read the
 # stored F bytes once), from an ncu capture of the kernel as it stands: workload 2 at full size, workload 3 on

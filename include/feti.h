@@ -167,7 +167,8 @@ typedef struct {
   double implicit_ms;         /* CUDA-event time of those applications */
   /* autotuner choice for the apply (after the first feti_assemble) */
   int32_t apply_variant, apply_grid;  /* tile-kernel variant (0-2: register batches of 4, 8, 16 loads;
-                                         3-5: bulk-copy rings of 4x3, 8x3, 2x6 warps x stages) and grid */
+                                         3-5: bulk-copy rings of 4x3, 8x3, 2x6 warps x stages; 6: FP64 tiles
+                                         by digit products) and grid */
   /* autotuner choice for the pruned TRSM (after the first feti_assemble) */
   int32_t trsm_cols;          /* sorted columns per CTA work item (0: a whole subdomain per item) */
   int32_t trsm_grid;          /* persistent CTAs of the TRSM launch */

@@ -524,7 +524,8 @@ void set_tiles_attr() {
 }
 
 // variants of the tile kernel: register pipeline with 4 / 8 / 16-load batches
-// (0, 1, 2), or per-warp bulk-copy rings of W warps x S stages: 4 x 3, 8 x 3, 2 x 6 (3, 4, 5)
+// (0, 1, 2), or per-warp bulk-copy rings of W warps x S stages: 4 x 3, 8 x 3, 2 x 6 (3, 4, 5); FP64 tiles also by
+// digit products, one CTA per tile (6, kern_apply_oz.cu)
 constexpr int kRingW[3] = {4, 8, 2};
 constexpr int kRingS[3] = {3, 3, 6};
 
@@ -559,7 +560,10 @@ void launch_tiles(int variant, int grid, cudaStream_t st, const TileDesc* desc, 
       break;
     case 3: launch_ring<TF, 4, 3>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
     case 4: launch_ring<TF, 8, 3>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
-    default: launch_ring<TF, 2, 6>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
+    case 5: launch_ring<TF, 2, 6>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
+    default:
+      if constexpr (sizeof(TF) == 8) launch_apply_dig(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status);
+      break;
   }
 }
 
@@ -625,9 +629,10 @@ void launch_apply_core(bool fp32, const TileDesc* desc, int ntiles, const void* 
   }
 }
 
-int apply_variants() { return 6; }
+int apply_variants() { return 7; }
 
-int apply_warps_per_cta(int variant) { return variant < 3 ? kApplyThreads / 32 : kRingW[variant - 3]; }
+// warps per CTA, each with tiles of its own (variant 6: the CTA shares one)
+int apply_warps_per_cta(int variant) { return variant < 3 ? kApplyThreads / 32 : variant < 6 ? kRingW[variant - 3] : 1; }
 
 template <typename TF, int W, int S>
 static int occ_ring() {
@@ -647,7 +652,8 @@ static int occ_tiles(int variant) {
     case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, apply_tiles_kernel<TF, 16>, kApplyThreads, 0); break;
     case 3: nb = occ_ring<TF, 4, 3>(); break;
     case 4: nb = occ_ring<TF, 8, 3>(); break;
-    default: nb = occ_ring<TF, 2, 6>(); break;
+    case 5: nb = occ_ring<TF, 2, 6>(); break;
+    default: nb = sizeof(TF) == 8 ? apply_dig_occupancy() : 0; break;
   }
   return nb;
 }

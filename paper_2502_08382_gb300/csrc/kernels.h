@@ -68,6 +68,9 @@ void launch_apply(const DevPlan& P, bool fp32, const TileDesc* desc, int ntiles,
 void launch_apply_core(bool fp32, const TileDesc* desc, int ntiles, const void* F, const void* pg, void* rowpart,
                        void* colpart, int grid, int variant, const int* active, int* status, cudaStream_t st,
                        cudaEvent_t ev_tiles0 = nullptr, cudaEvent_t ev_tiles1 = nullptr, bool ev_external = false);
+void launch_apply_dig(int grid, cudaStream_t st, const TileDesc* desc, int ntiles, const double* F, const double* pg,
+                      double* rowpart, double* colpart, const int* active, int* status);
+int apply_dig_occupancy();
 int apply_variants();
 int apply_max_ctas_per_sm(bool fp32, int variant);
 int apply_warps_per_cta(int variant);

@@ -37,32 +37,6 @@ struct CtState {
   uint32_t units;     // 32-column units multiplied so far (accumulator set and phase)
 };
 
-// the value 2^ex (2^32 hi + lo) rounded to nearest, by integer arithmetic
-__device__ __forceinline__ double dig_value(long long hi, long long lo, int ex) {
-  hi += lo >> 32;
-  uint32_t l = (uint32_t)lo;
-  const bool neg = hi < 0;
-  if (neg) {
-    hi = ~hi + (l == 0);
-    l = -l;
-  }
-  unsigned long long h = (unsigned long long)hi;
-  if (h == 0) {
-    h = l;
-    l = 0;
-    ex -= 32;
-  }
-  const int lz = __clzll((long long)h);
-  const unsigned long long x = (unsigned long long)l << 32;
-  const unsigned long long m = lz < 64 ? (h << lz) | (lz ? x >> (64 - lz) : 0ULL) : 0ULL;
-  const unsigned long long mant = (m >> 11) + ((m >> 10) & 1);  // 53 bits, 2^52 <= mant <= 2^53
-  const int e = 95 - lz + ex;                                   // value = mant 2^(e - 52)
-  unsigned long long b = ((unsigned long long)(e + 1022) << 52) + mant;
-  if (h == 0 || e < -1021) b = 0;
-  if (h != 0 && e > 1022) b = 0x7FF0000000000000ULL;
-  return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ULL : 0ULL)));
-}
-
 // Eight entries of a row (columns k .. k + 7, zero from K on): of a column-major matrix, and of a row-major one whose
 // rows are 16-byte aligned and padded to a multiple of 8.
 struct ColMajor {
