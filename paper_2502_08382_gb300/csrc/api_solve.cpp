@@ -382,6 +382,78 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
   }
 }
 
+// Y = Z W of every entry of an adjoint batch by digit products: groups of (entry, rows) whose digits fit the buffer.
+void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t st,
+                    std::vector<std::vector<DenseEnt>>& keep_ent, std::vector<std::vector<int4>>& keep_it) {
+  std::vector<DenseEnt> ents;
+  std::vector<int4> items;
+  int64_t bytes = 0, nex = 0;
+  auto flush = [&]() {
+    if (ents.empty()) return;
+    if ((int64_t)ents.size() > ctx->adj_ent_cap) {
+      dfree(ctx, ctx->d_adj_ent);
+      ctx->d_adj_ent = (DenseEnt*)dalloc(ctx, ents.size() * sizeof(DenseEnt));
+      ctx->adj_ent_cap = (int64_t)ents.size();
+    }
+    if ((int64_t)items.size() > ctx->adj_dit_cap) {
+      dfree(ctx, ctx->d_adj_dit);
+      ctx->d_adj_dit = (int4*)dalloc(ctx, items.size() * sizeof(int4));
+      ctx->adj_dit_cap = (int64_t)items.size();
+    }
+    if (nex > ctx->adj_dex_cap) {
+      dfree(ctx, ctx->d_adj_dex);
+      ctx->d_adj_dex = (int*)dalloc(ctx, (size_t)nex * sizeof(int));
+      ctx->adj_dex_cap = nex;
+    }
+    keep_ent.push_back(ents);
+    keep_it.push_back(items);
+    CKS(cudaMemcpyAsync(ctx->d_adj_ent, keep_ent.back().data(), ents.size() * sizeof(DenseEnt), cudaMemcpyHostToDevice, st));
+    CKS(cudaMemcpyAsync(ctx->d_adj_dit, keep_it.back().data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+    launch_dense_oz(ctx->d_adj_ent, (int)ents.size(), ctx->d_adj_dit, (int)items.size(), ctx->d_adj_work, ctx->d_adj_dig,
+                    ctx->d_adj_dex, ctx->d_adj_work, ctx->nsm, ctx->d_status, st);
+    ctx->stats.launches += 3;
+    ents.clear();
+    items.clear();
+    bytes = nex = 0;
+  };
+  for (const auto& e : b) {
+    const int64_t q = (e.m + 7) / 8, wb = (int64_t)e.m * q * 128, rb = q * 128, ld = 2 * (int64_t)e.m_pad;
+    const int n = ctx->subs[e.sub].n;
+    for (int r0 = 0; r0 < n;) {
+      int64_t fit = (ctx->adj_dig_bytes - bytes - wb) / rb;
+      if (fit < n - r0) fit = fit / 128 * 128;
+      if (fit <= 0) {
+        flush();
+        fit = (ctx->adj_dig_bytes - wb) / rb;
+        if (fit < n - r0) fit = fit / 128 * 128;
+      }
+      const int rows = (int)std::min<int64_t>(fit, n - r0);
+      DenseEnt d{};
+      d.src_a = e.v_ofs + r0 * ld;
+      d.src_b = e.ws_ofs;
+      d.out = d.src_a + e.m_pad;
+      d.a = bytes;
+      d.b = bytes + rows * rb;
+      d.exa = nex;
+      d.exb = nex + rows;
+      d.ld = ld;
+      d.ldb = e.m_pad;
+      d.rows = rows;
+      d.cols = e.m;
+      d.K = e.m;
+      d.pieces = (int)q;
+      for (int bi = 0; bi < (rows + 127) / 128; ++bi)
+        for (int bj = 0; bj < (e.m + 63) / 64; ++bj)
+          items.push_back(make_int4((int)ents.size(), bi | bj << 16, (int)((q + 3) / 4), 0));
+      ents.push_back(d);
+      bytes += wb + rows * rb;
+      nex += rows + e.m;
+      r0 += rows;
+    }
+  }
+  flush();
+}
+
 // Z_i = P^T L_u^{-T} D^{-2} X_u (and, for the adjoint, Y_i = Z_i W_i) over batches of subdomains whose
 // dense work arrays fit the budget, from X_u = L_u^{-1} P B^T recomputed in FP64 by the pruned forward
 // solve with the unit-lower factor.  W_dev != null: the adjoint, dtheta_e = -sum (dK_e)_ab Y[b,:] . Z[a,:]
@@ -389,14 +461,17 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
 void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStream_t st) {
   const bool adjoint = W_dev != nullptr;
   const int ns = ctx->nsub;
-  if (!ctx->d_Xu) ctx->d_Xu = (double*)dalloc(ctx, (size_t)std::max<int64_t>(ctx->stats.X_elems, 1) * 8);
-  queue_reset(ctx, 40);
-  {
+  // the FP64 assembly's X = L^{-1} P B^T is X_u up to the pivots (X_u = D X); where it is not kept (mixed precision,
+  // recompute_X, the TRSM path) X_u is solved for again
+  const bool haveX = adjoint && !ctx->fp32 && ctx->d_X && ctx->route != 2;
+  if (!haveX && !ctx->d_Xu) ctx->d_Xu = (double*)dalloc(ctx, (size_t)std::max<int64_t>(ctx->stats.X_elems, 1) * 8);
+  if (!haveX) {
+    queue_reset(ctx, 40);
     const auto& tc = ctx->trsm_cands[ctx->trsm_pick];
     launch_trsm(ctx->P, tc.d_items, tc.nitems, tc.cw, ctx->d_queue + 40, ctx->d_Xu, false, ctx->d_ws,
                 ctx->ws_stride, ctx->rhs_front, std::min(ctx->grid_trsm, tc.nitems), 0, 0, ctx->d_status, st, 1);
+    ctx->stats.launches += 1;
   }
-  ctx->stats.launches += 1;
   CKS(cudaGetLastError());
   // batches of subdomains whose dense V (n x 2 m_pad, or n x m_pad for Z alone) and sorted W (m_pad^2) fit
   size_t free_b = 0, total_b = 0;
@@ -404,7 +479,32 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
   const double cap = ctx->opt.adjoint_work_bytes > 0
                          ? (double)ctx->opt.adjoint_work_bytes
                          : std::min<double>(24.0 * (1 << 30), 0.45 * (double)(free_b + ctx->adj_work_bytes));
-  const int64_t budget = std::max<int64_t>((int64_t)(cap / 8), 1);
+  // the adjoint's Y = Z W by digit products on the tensor cores: the digits of W and of as many rows of Z as half the
+  // cap holds (8 GiB at most, the largest subdomain's W and 128 rows at least; the rows' results do not depend on how
+  // many go together); where the allocator refuses, Y is formed as X_u W and solved for with Z
+  bool dense = adjoint;
+  if (dense) {
+    int64_t want = 0, least = 0;
+    for (int i = 0; i < ns; ++i) {
+      if (ctx->subs[i].nelem == 0) continue;
+      const int64_t m = ctx->subs[i].m, q = (m + 7) / 8;
+      want += (m + ctx->subs[i].n) * q * 128;
+      least = std::max(least, (m + 128) * q * 128);
+    }
+    want = std::max(least, std::min(want, (int64_t)std::min(0.5 * cap, 8.0 * (1 << 30))));
+    if (want > ctx->adj_dig_bytes) {
+      dfree(ctx, ctx->d_adj_dig);
+      ctx->d_adj_dig = nullptr;
+      ctx->adj_dig_bytes = 0;
+      try {
+        ctx->d_adj_dig = dalloc(ctx, (size_t)want);
+        ctx->adj_dig_bytes = want;
+      } catch (std::bad_alloc&) {
+        dense = false;
+      }
+    }
+  }
+  const int64_t budget = std::max<int64_t>((int64_t)(cap / 8) - (dense ? ctx->adj_dig_bytes / 8 : 0), 1);
   std::vector<int64_t> woff(ns + 1, 0);
   for (int i = 0; i < ns; ++i) woff[i + 1] = woff[i] + (int64_t)ctx->subs[i].m * ctx->subs[i].m;
   std::vector<std::vector<AdjBatch>> batches;
@@ -465,7 +565,11 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
     ctx->adj_batch_cap = max_nb;
   }
   const int grid = ctx->nsm * 4;
+  std::vector<std::vector<DenseEnt>> keep_ent;  // host sources of the copies in flight
+  std::vector<std::vector<int4>> keep_it;
   for (auto& b : batches) {
+    keep_ent.clear();  // the stream was synchronised at the end of the batch before
+    keep_it.clear();
     const int nb = (int)b.size();
     // work items: the V rows of each (entry, active supernode, 64 own rows) and, for the adjoint, X_u W per
     // kBuildCols columns, largest first; the backward solve per (entry, 64 columns), larger factors first
@@ -484,11 +588,11 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
         const int sn = bp.act[a];
         const int w = pat.sn_w[sn], J = bp.je[sn] - bp.jb[sn];
         for (int k0 = 0; k0 < w; k0 += kT)
-          for (int cg = 0; cg < (adjoint ? mp : 1); cg += kBuildCols)
-            bi.push_back({(double)std::min(kT, w - k0) * J * (adjoint ? std::min(kBuildCols, mp - cg) : 1),
+          for (int cg = 0; cg < (adjoint && !dense ? mp : 1); cg += kBuildCols)
+            bi.push_back({(double)std::min(kT, w - k0) * J * (adjoint && !dense ? std::min(kBuildCols, mp - cg) : 1),
                           make_int4(e, a, k0, cg)});
       }
-      for (int cb = 0; cb < (adjoint ? 2 : 1) * mp / 64; ++cb) si.push_back({pat.nnzL, make_int2(e, cb)});
+      for (int cb = 0; cb < (adjoint && !dense ? 2 : 1) * mp / 64; ++cb) si.push_back({pat.nnzL, make_int2(e, cb)});
     }
     std::stable_sort(bi.begin(), bi.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
     std::stable_sort(si.begin(), si.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
@@ -518,11 +622,12 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
                         (size_t)(l.ws_ofs + (adjoint ? (int64_t)l.m_pad * l.m_pad : 0)) * 8, st));
     if (adjoint) launch_adj_wsort(ctx->d_adj_batch, nb, W_dev, ctx->P.colperm, ctx->d_adj_work, max_mpad, st);
     queue_reset(ctx, 41);
-    launch_adj_build(ctx->P, ctx->d_adj_batch, ctx->d_adj_items4, (int)bv.size(), ctx->d_queue + 41, ctx->d_Xu,
-                     ctx->d_adj_work, std::max(1, std::min<int>(grid, (int)bv.size())), st);
+    launch_adj_build(ctx->P, ctx->d_adj_batch, ctx->d_adj_items4, (int)bv.size(), ctx->d_queue + 41,
+                     haveX ? (const double*)ctx->d_X : ctx->d_Xu, haveX ? 1 : 0, dense ? 1 : 0, ctx->d_adj_work, std::max(1, std::min<int>(grid, (int)bv.size())), st);
     queue_reset(ctx, 42);
     launch_adj_bsolve(ctx->P, ctx->d_adj_batch, ctx->d_adj_items2, (int)sv.size(), ctx->d_queue + 42,
                       ctx->d_adj_work, std::max(1, std::min<int>(grid, (int)sv.size())), st);
+    if (dense) dense_products(ctx, b, st, keep_ent, keep_it);
     if (adjoint)
       launch_adj_contract(ctx->P, ctx->d_adj_batch, nb, max_nel, ctx->d_eldofs, ctx->d_eldk, ctx->d_elsc,
                           ctx->d_adj_work, dtheta_dev, st);
@@ -571,6 +676,9 @@ feti_status feti_adjoint(feti_ctx* ctx, const double* W_dev, double* dtheta_dev)
       dfree(ctx, ctx->d_adj_work);
       ctx->d_adj_work = nullptr;
       ctx->adj_work_bytes = 0;
+      dfree(ctx, ctx->d_adj_dig);
+      ctx->d_adj_dig = nullptr;
+      ctx->adj_dig_bytes = 0;
     }
     return FETI_OK;
   } catch (std::bad_alloc&) {

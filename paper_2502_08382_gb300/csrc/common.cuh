@@ -243,6 +243,14 @@ struct OzBatch {
   int64_t x0;           // first X element
 };
 
+// One dense FP64 product out = A B by exact slicing (launch_dense_oz): A rows x K (ld), B K x cols (ldb), row-major;
+// out has A's ld.  Offsets in doubles of A, B (source) and out, bytes of the digits, entries of the exponents.
+struct DenseEnt {
+  int64_t src_a, src_b, out, a, b;
+  int64_t exa, exb, ld, ldb;
+  int rows, cols, K, pieces;
+};
+
 // flags of the numeric Cholesky (kern_factor.cu)
 enum : int { kCholNoReg = 1, kCholStopRoot = 2, kCholSkipBig = 4 };
 

@@ -201,6 +201,12 @@ struct feti_ctx {
   double* d_Xu = nullptr;          // FP64 X_u = L_u^{-1} P B^T of every subdomain (adjoint)
   double* d_adj_work = nullptr;    // batch work arrays of the adjoint (V and sorted W)
   int64_t adj_work_bytes = 0;
+  void* d_adj_dig = nullptr;       // digits of Z and W (the adjoint's Y = Z W)
+  int64_t adj_dig_bytes = 0;
+  feti::DenseEnt* d_adj_ent = nullptr;
+  int4* d_adj_dit = nullptr;
+  int* d_adj_dex = nullptr;
+  int64_t adj_ent_cap = 0, adj_dit_cap = 0, adj_dex_cap = 0;
   feti::AdjBatch* d_adj_batch = nullptr;
   int64_t adj_batch_cap = 0;
   int4* d_adj_items4 = nullptr;

@@ -6,8 +6,9 @@
 // forward solve X_u = L_u^{-1} P B^T (staircase blocks X_s, w_s x J_s):
 //   Z = P^T L_u^{-T} D^{-2} X_u,   Y = Z W = P^T L_u^{-T} D^{-2} (X_u W),
 //   dL/dtheta_e = -sum_{a,b in e} (dK_e)_ab Y[b,:] . Z[a,:].
-// Forming Y from X_u W (2 nnz(X_u) m flops) and one backward solve is several
-// times cheaper than the dense product Z W (2 n m^2 flops).  The kernels work
+// Y = Z W is a dense product (2 n m^2 flops) on the tensor cores by exact slicing
+// (launch_dense_oz); where its digits do not fit the memory Y comes from X_u W
+// (2 nnz(X_u) m flops) and the backward solve together with Z.  The kernels work
 // on a batch of subdomains whose dense arrays V = [D^{-2} X_u | D^{-2} X_u W]
 // (n x 2 m_pad, row-major, rows in the factor's numbering) fit the buffer:
 //   adj_build_kernel   V_Z rows from X_u, V_Y = X_u W per active supernode
@@ -51,10 +52,12 @@ __global__ void wsort_kernel(const AdjBatch* B, int nb, const double* W, const i
 // One item = (batch entry, active supernode s, 64-row block k0 of its own rows,
 // column group cg of kBuildCols columns):
 //   V_Z[c0 + k][jb + j] = d2[c0 + k] X_s[j][k]            (j < J_s; written by column group 0)
-//   V_Y[c0 + k][c]      = d2[c0 + k] sum_j X_s[j][k] Ws[jb + j][c]
+//   V_Y[c0 + k][c]      = d2[c0 + k] sum_j X_s[j][k] Ws[jb + j][c]   (zcols = 0)
+// scaled: the X given is the assembly's X = D^{-1} X_u, so V_Z = D^{-1} X.
 // computed in 64 x 64 output tiles (4 x 4 per thread) over 32-deep chunks of j.
 __global__ void __launch_bounds__(kAT) adj_build_kernel(DevPlan P, const AdjBatch* B, const int4* items, int nitems,
-                                                       int* queue, const double* Xu, double* work) {
+                                                       int* queue, const double* Xu, int scaled, int zcols,
+                                                       double* work) {
   __shared__ double As[32][kT + 1];  // X chunk: [j][k]
   __shared__ double Bs[32][kT];      // Ws chunk: [j][c]
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -75,12 +78,29 @@ __global__ void __launch_bounds__(kAT) adj_build_kernel(DevPlan P, const AdjBatc
     double* V = work + E.v_ofs;
     const double* Ws = work + E.ws_ofs;
     const int k0 = item.z, nk = min(kT, w - k0);
-    if (item.w == 0)
-      for (int64_t idx = tid; idx < (int64_t)nk * J; idx += kAT) {
-        const int k = (int)(idx % nk), j = (int)(idx / nk);
-        V[(int64_t)(c0 + k0 + k) * ld + jb + j] = d2[c0 + k0 + k] * Xs[(int64_t)j * wp + k0 + k];
+    if (item.w == 0) {
+      double* sc = &Bs[0][0];
+      if (tid < nk) {
+        const double dk = d2[c0 + k0 + tid];
+        sc[tid] = scaled ? sqrt(dk) : dk;
       }
-    const int cend = E.zonly ? 0 : min(mp, item.w + kBuildCols);
+      __syncthreads();
+      // 32 x 32 blocks through shared memory: X is read along k and V written along j
+      for (int kb = 0; kb < nk; kb += 32)
+        for (int j0 = 0; j0 < J; j0 += 32) {
+          for (int idx = tid; idx < 1024; idx += kAT) {
+            const int k = idx % 32, j = idx / 32;
+            if (kb + k < nk && j0 + j < J) As[j][k] = sc[kb + k] * Xs[(int64_t)(j0 + j) * wp + k0 + kb + k];
+          }
+          __syncthreads();
+          for (int idx = tid; idx < 1024; idx += kAT) {
+            const int j = idx % 32, k = idx / 32;
+            if (kb + k < nk && j0 + j < J) V[(int64_t)(c0 + k0 + kb + k) * ld + jb + j0 + j] = As[j][k];
+          }
+          __syncthreads();
+        }
+    }
+    const int cend = E.zonly || zcols ? 0 : min(mp, item.w + kBuildCols);
     for (int cb = item.w; cb < cend; cb += kT) {
       double acc[4][4] = {};
       for (int j0 = 0; j0 < J; j0 += 32) {
@@ -362,8 +382,8 @@ void launch_adj_wsort(const AdjBatch* B, int nb, const double* W, const int* col
 }
 
 void launch_adj_build(const DevPlan& P, const AdjBatch* B, const int4* items, int nitems, int* queue,
-                      const double* Xu, double* work, int grid, cudaStream_t st) {
-  if (nitems > 0) adj_build_kernel<<<grid, kAT, 0, st>>>(P, B, items, nitems, queue, Xu, work);
+                      const double* Xu, int scaled, int zcols, double* work, int grid, cudaStream_t st) {
+  if (nitems > 0) adj_build_kernel<<<grid, kAT, 0, st>>>(P, B, items, nitems, queue, Xu, scaled, zcols, work);
 }
 
 void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, double* work,

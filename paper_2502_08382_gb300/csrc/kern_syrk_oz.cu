@@ -106,10 +106,14 @@ __global__ void __launch_bounds__(256) dig_x_kernel(DevPlan P, const double* X, 
   }
 }
 
-// items: (subdomain, 128-row block | 64-column block << 16, chunks, 128 x 128 tile of the contribution list)
+// SYRK: items (subdomain, 128-row block | 64-column block << 16, chunks, 128 x 128 tile of the contribution list), XD the
+// digits of X, EX the column exponents, out F.
+// DENSE: out = A B^T for the products `ents`; items (product, 128-row block | 64-column block << 16, chunks, 0), XD the
+// digits of A and B per piece of 8 columns (rows contiguous), EX their row exponents.
+template <bool DENSE>
 __global__ void __launch_bounds__(kOThreads, 1)
-    syrk_oz_kernel(DevPlan P, const int4* items, int nitems, const char* XD, int64_t x0, const int* EX, double* F,
-                   int* status) {
+    syrk_oz_kernel(DevPlan P, const DenseEnt* ents, const int4* items, int nitems, const char* XD, int64_t x0,
+                   const int* EX, double* F, int* status) {
   extern __shared__ uint8_t oz_dyn[];
   __shared__ uint64_t full[kOStages], empty[kOStages], accf[2], acce[2], drain;
   __shared__ uint32_t tmem_s;
@@ -146,10 +150,49 @@ __global__ void __launch_bounds__(kOThreads, 1)
     uint32_t cg = 0;  // chunks staged so far
     bool dead = false;
     const int prow = lane & 7, pdig = lane >> 3;  // this lane's row of an 8-row atom, and digits pdig, pdig + 4
+    // one chunk: warp w stages piece w, 24 atoms (16 of A, 4 + 4 of B), digits pdig and pdig + 4
+    auto stage = [&](const char* srcA, int a0, int a1, const char* srcB, int b0, int b1, int ra, int rb) {
+      const uint32_t st = cg % kOStages;
+      if (!dead && cg >= kOStages && !dig_wait(smem_u32(&empty[st]), ((cg / kOStages) - 1) & 1, &s_abort)) dead = true;
+      if (dead) return;
+      const uint32_t sA = smem_u32(smem + st * kOStageBytes), sB = sA + kDig * kOA;
+      const uint32_t so = prow * 64 + ((warp ^ ((prow >> 1) & 3)) << 4);
+#pragma unroll 4
+      for (int at = 0; at < kOM / 8; ++at) {
+        const int j = ra + at * 8 + prow;
+        const bool ok = j >= a0 && j < a1;
+        const char* src = ok ? srcA + (long long)j * 128 + pdig * 16 : XD;
+        const uint32_t dst = sA + pdig * kOA + at * 512 + so;
+        cp_async16(dst, src, ok);
+        cp_async16(dst + 4 * kOA, ok ? src + 64 : XD, ok);
+      }
+#pragma unroll 4
+      for (int at = 0; at < kON / 8; ++at) {
+        const int j = rb + at * 8 + prow;
+        const bool ok = j >= b0 && j < b1;
+        const char* src = ok ? srcB + (long long)j * 128 + pdig * 16 : XD;
+        const uint32_t dst = sB + (at >> 2) * (kDig * kOB) + pdig * kOB + (at & 3) * 512 + so;
+        cp_async16(dst, src, ok);
+        cp_async16(dst + 4 * kOB, ok ? src + 64 : XD, ok);
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(&full[st]);
+    };
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
       const int4 item = items[it];
-      const SubInfo& S = P.sub[item.x];
       const int ra = (item.y & 0xffff) * kOM, rb = (item.y >> 16) * kON;
+      if constexpr (DENSE) {
+        const DenseEnt& e = ents[item.x];
+        for (int ch = 0; ch < item.z; ++ch, ++cg) {
+          const int q = 4 * ch + warp;
+          const bool in = q < e.pieces;
+          stage(XD + e.a + (long long)q * e.rows * 128, 0, in ? e.rows : 0, XD + e.b + (long long)q * e.cols * 128, 0,
+                in ? e.cols : 0, ra, rb);
+        }
+        continue;
+      }
+      const SubInfo& S = P.sub[item.x];
       const int* tl = P.t2_off + S.t20;
       const int cbeg = tl[item.w], cend = tl[item.w + 1];
       for (int c0 = cbeg; c0 < cend; c0 += kOBatch) {
@@ -187,36 +230,8 @@ __global__ void __launch_bounds__(kOThreads, 1)
           if (tid < nw4 - nw) pieces[nw + tid] = Piece{0, 0, 0};
           asm volatile("bar.sync 1, 128;" ::: "memory");
           for (int ch = 0; ch < nw4 / 4; ++ch, ++cg) {
-            const uint32_t st = cg % kOStages;
-            if (!dead && cg >= kOStages && !dig_wait(smem_u32(&empty[st]), ((cg / kOStages) - 1) & 1, &s_abort))
-              dead = true;
-            if (dead) continue;
-            const uint32_t sA = smem_u32(smem + st * kOStageBytes), sB = sA + kDig * kOA;
-            // warp w takes piece w of the chunk: 24 atoms (16 of A, 4 + 4 of B), digits pdig and pdig + 4
             const Piece pc = pieces[ch * 4 + warp];
-            const uint32_t so = prow * 64 + ((warp ^ ((prow >> 1) & 3)) << 4);
-            const char* src0 = XD + pc.base + pdig * 16;
-#pragma unroll 4
-            for (int at = 0; at < kOM / 8; ++at) {
-              const int j = ra + at * 8 + prow;
-              const bool ok = j >= pc.jb && j < pc.je;
-              const char* src = ok ? src0 + (long long)j * 128 : XD;
-              const uint32_t dst = sA + pdig * kOA + at * 512 + so;
-              cp_async16(dst, src, ok);
-              cp_async16(dst + 4 * kOA, ok ? src + 64 : XD, ok);
-            }
-#pragma unroll 4
-            for (int at = 0; at < kON / 8; ++at) {
-              const int j = rb + at * 8 + prow;
-              const bool ok = j >= pc.jb && j < pc.je;
-              const char* src = ok ? src0 + (long long)j * 128 : XD;
-              const uint32_t dst = sB + (at >> 2) * (kDig * kOB) + pdig * kOB + (at & 3) * 512 + so;
-              cp_async16(dst, src, ok);
-              cp_async16(dst + 4 * kOB, ok ? src + 64 : XD, ok);
-            }
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_arrive(&full[st]);
+            stage(XD + pc.base, pc.jb, pc.je, XD + pc.base, pc.jb, pc.je, ra, rb);
           }
           asm volatile("bar.sync 1, 128;" ::: "memory");
         }
@@ -296,6 +311,28 @@ __global__ void __launch_bounds__(kOThreads, 1)
         }
       }
       if (!ok) break;
+      if constexpr (DENSE) {
+        const DenseEnt& e = ents[item.x];
+        const int row = (item.y & 0xffff) * kOM + quarter * 32 + lane, c0 = (item.y >> 16) * kON;
+        if (row < e.rows) {
+          const int ei = EX[e.exa + row];
+          double* out = F + e.out + (int64_t)row * e.ld + c0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const int c = h * kOH + ch * 16 + u;
+              if (c0 + c < e.cols) {
+                const int ej = EX[e.exb + c0 + c];
+                const double t = fma((double)hi[h][u], 4294967296.0, (double)lo[h][u]);
+                out[c] = ei == kExpBad || ej == kExpBad
+                             ? __longlong_as_double(0x7FF8000000000000LL)
+                             : t * dig_pow2(min(ei, 1000) - 34) * dig_pow2(min(ej, 1000) - 34);
+              }
+            }
+        }
+        continue;
+      }
       const SubInfo& S = P.sub[item.x];
       const int row = (item.y & 0xffff) * kOM + quarter * 32 + lane, bj = item.y >> 16;
       const int bi = row / kT, r = row % kT;
@@ -334,19 +371,81 @@ __global__ void __launch_bounds__(kOThreads, 1)
   }
 }
 
+// Row exponents and digits of the dense products' operands: A (rows x K, row-major, ld) and B^T (K x cols, row-major:
+// B's row c is its column c).  blockIdx.y = product.
+__global__ void __launch_bounds__(256) dense_exp_kernel(const DenseEnt* ents, const double* src, int* EX) {
+  const DenseEnt e = ents[blockIdx.y];
+  const int lane = threadIdx.x % 32;
+  for (int i = (blockIdx.x * 256 + threadIdx.x) / 32; i < e.rows; i += gridDim.x * 8) {
+    const double* a = src + e.src_a + (int64_t)i * e.ld;
+    uint32_t mx = 0;
+    for (int k = lane; k < e.K; k += 32) mx = max(mx, (uint32_t)__double2hiint(a[k]) & 0x7fffffffu);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) EX[e.exa + i] = dig_exponent(mx);
+  }
+  for (int c = blockIdx.x * 256 + threadIdx.x; c < e.cols; c += gridDim.x * 256) {
+    const double* b = src + e.src_b + c;
+    uint32_t mx = 0;
+#pragma unroll 8
+    for (int k = 0; k < e.K; ++k) mx = max(mx, (uint32_t)__double2hiint(b[(int64_t)k * e.ldb]) & 0x7fffffffu);
+    EX[e.exb + c] = dig_exponent(mx);
+  }
+}
+
+__device__ __forceinline__ void store_digits(uint4* out, const uint64_t (&c)[8]) {
+#pragma unroll
+  for (int p = 0; p < kDig; ++p)
+    out[p] = make_uint4(dig_pair(c[0], c[1], p), dig_pair(c[2], c[3], p), dig_pair(c[4], c[5], p),
+                        dig_pair(c[6], c[7], p));
+}
+
+__global__ void __launch_bounds__(256) dense_cut_kernel(const DenseEnt* ents, const double* src, const int* EX, char* XD) {
+  const DenseEnt e = ents[blockIdx.y];
+  const int64_t na = (int64_t)e.rows * e.pieces, nb = (int64_t)e.cols * e.pieces;
+  for (int64_t u = blockIdx.x * 256 + threadIdx.x; u < na + nb; u += gridDim.x * 256) {
+    uint64_t c[8];
+    if (u < na) {  // piece fastest: a row's pieces are contiguous
+      const int i = (int)(u / e.pieces), q = (int)(u - (int64_t)i * e.pieces), ex = EX[e.exa + i];
+      const double* a = src + e.src_a + (int64_t)i * e.ld + 8 * q;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) c[k] = dig_cut(8 * q + k < e.K ? a[k] : 0.0, ex);
+      store_digits(reinterpret_cast<uint4*>(XD + e.a + ((int64_t)q * e.rows + i) * 128), c);
+    } else {  // column fastest
+      const int64_t v = u - na;
+      const int q = (int)(v / e.cols), j = (int)(v - (int64_t)q * e.cols), ex = EX[e.exb + j];
+      const double* b = src + e.src_b + (int64_t)8 * q * e.ldb + j;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) c[k] = dig_cut(8 * q + k < e.K ? b[(int64_t)k * e.ldb] : 0.0, ex);
+      store_digits(reinterpret_cast<uint4*>(XD + e.b + ((int64_t)q * e.cols + j) * 128), c);
+    }
+  }
+}
+
 }  // namespace
 
 void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const int4* ditems, const int4* items,
                     void* XD, int* EX, double* F, int nsm, int* status, cudaStream_t st) {
-  cudaFuncSetAttribute(syrk_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kODyn);
+  cudaFuncSetAttribute(syrk_oz_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kODyn);
   if (b.nitems <= 0) return;
   for (int s0 = 0; s0 < b.nsub; s0 += 32768) {
     dim3 g((unsigned)std::max(1, std::min(64, (b.m_max + 7) / 8)), (unsigned)std::min(32768, b.nsub - s0));
     colexp_kernel<<<g, 256, 0, st>>>(P, X, b.sub0 + s0, EX);
   }
   if (b.nditems > 0) dig_x_kernel<<<b.nditems, 256, 0, st>>>(P, X, ditems + b.ditem0, EX, b.x0, (uint4*)XD);
-  syrk_oz_kernel<<<std::min(b.nitems, nsm), kOThreads, kODyn, st>>>(P, items + b.item0, b.nitems, (const char*)XD,
-                                                                   b.x0, EX, F, status);
+  syrk_oz_kernel<false><<<std::min(b.nitems, nsm), kOThreads, kODyn, st>>>(P, nullptr, items + b.item0, b.nitems,
+                                                                          (const char*)XD, b.x0, EX, F, status);
+}
+
+void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const double* src, void* XD, int* EX,
+                     double* out, int nsm, int* status, cudaStream_t st) {
+  if (nent <= 0 || nitems <= 0) return;
+  const dim3 g((unsigned)std::max(1, nsm * 16 / nent), (unsigned)nent);
+  dense_exp_kernel<<<g, 256, 0, st>>>(ents, src, EX);
+  dense_cut_kernel<<<g, 256, 0, st>>>(ents, src, EX, (char*)XD);
+  cudaFuncSetAttribute(syrk_oz_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kODyn);
+  DevPlan P{};
+  syrk_oz_kernel<true><<<std::min(nitems, nsm), kOThreads, kODyn, st>>>(P, ents, items, nitems, (const char*)XD, 0, EX,
+                                                                        out, status);
 }
 
 int syrk_oz_chunks(const int* np, int n) {

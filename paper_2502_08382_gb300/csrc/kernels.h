@@ -48,6 +48,9 @@ void launch_syrk_f64(const DevPlan& P, const int2* items, int nitems, const doub
                      cudaStream_t st);
 void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const int4* ditems, const int4* items,
                     void* XD, int* EX, double* F, int nsm, int* status, cudaStream_t st);
+// dense FP64 products by the same tiles; items (product, 128-row block | 64-column block << 16, 32-deep chunks, 0)
+void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const double* src, void* XD, int* EX,
+                     double* out, int nsm, int* status, cudaStream_t st);
 // FP64 forward solve of the large fronts on the tensor cores (kern_trsm_oz.cu): digits of the large panels (items:
 // subdomain, supernode, first column of the 128-column block, its offset / 512), then, after launch_trsm with `hand`,
 // blocks of cw sorted columns (items: subdomain, first column); ws: per CTA front_sz + stack doubles
@@ -142,7 +145,7 @@ void launch_gemv(const double* A, const double* c, double* z, int D, double alph
 void launch_adj_wsort(const AdjBatch* B, int nb, const double* W, const int* colperm, double* work, int max_mpad,
                       cudaStream_t st);
 void launch_adj_build(const DevPlan& P, const AdjBatch* B, const int4* items, int nitems, int* queue,
-                      const double* Xu, double* work, int grid, cudaStream_t st);
+                      const double* Xu, int scaled, int zcols, double* work, int grid, cudaStream_t st);
 void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, double* work,
                        int grid, cudaStream_t st);
 void launch_adj_contract(const DevPlan& P, const AdjBatch* B, int nb, int max_nelem, const int* eldofs,
