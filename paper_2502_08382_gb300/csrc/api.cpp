@@ -438,6 +438,8 @@ void build(feti_ctx* c) {
   std::vector<int64_t> pat_lh(c->pats.size(), 0), pat_di(c->pats.size(), 0);
   auto lh_big = [&](const PatternPlan& P, int s) { return c->fp32 && (P.sn_r[s] >= 128 || P.sn_w[s] >= 256); };
   // FP64: the large fronts' digits and update blocks (kern_trsm_oz.cu)
+  std::vector<int64_t> lt_ofs;  // the adjoint's backward solve: digits of L^T (kern_bsolve_oz.cu)
+  c->pat_lt.assign(c->pats.size(), 0);
   std::vector<int64_t> ld_ofs, tx_ofs, th_ofs, pat_ld(c->pats.size(), 0), bp_th(c->bps.size(), 0);
   std::vector<int> lvl_off, lvl_sn, pat_lvl0(c->pats.size());
   int64_t max_usize = 0;
@@ -470,6 +472,11 @@ void build(feti_ctx* c) {
         pat_di[p] += (int64_t)((P.sn_w[s] + 127) / 128) * 4 * 32 * 32;
       }
       uofs.push_back(P.uofs[s]);
+    }
+    for (int s = 0; s < P.nsn; ++s) {
+      lt_ofs.push_back(P.sn_big[s] ? c->pat_lt[p] / 512 : -1);
+      for (int kB = 0; P.sn_big[s] && kB < P.sn_w[s]; kB += 128)
+        c->pat_lt[p] += bsolve_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
     }
     if (!c->fp32) {
       // the digits of each 128-column block, and an update stack of the large supernodes alone
@@ -905,6 +912,7 @@ void build(feti_ctx* c) {
   D.sn_hoff = upload(c, sn_hoff);
   D.lh_ofs = upload(c, lh_ofs);
   D.di_ofs = upload(c, di_ofs);
+  D.lt_ofs = upload(c, lt_ofs);
   D.ld_ofs = upload(c, ld_ofs);
   D.tx_ofs = upload(c, tx_ofs);
   D.th_ofs = upload(c, th_ofs);

@@ -564,6 +564,32 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
     ctx->d_adj_batch = (AdjBatch*)dalloc(ctx, (size_t)max_nb * sizeof(AdjBatch));
     ctx->adj_batch_cap = max_nb;
   }
+  // the large fronts' part of the backward solve on the tensor cores, unless their digits find no memory
+  bool boz = dense || !adjoint;
+  if (boz) {
+    int64_t want = 0;
+    for (auto& b : batches) {
+      int64_t t = 0;
+      for (auto& e : b) {
+        e.lt = t;
+        t += ctx->pat_lt[ctx->subs[e.sub].pat];
+      }
+      want = std::max(want, t);
+    }
+    boz = want > 0;
+    try {
+      if (want > ctx->adj_lt_bytes) {
+        dfree(ctx, ctx->d_adj_lt);
+        ctx->d_adj_lt = nullptr;
+        ctx->adj_lt_bytes = 0;
+        ctx->d_adj_lt = dalloc(ctx, (size_t)want);
+        ctx->adj_lt_bytes = want;
+      }
+      if (boz && !ctx->d_adj_bscr) ctx->d_adj_bscr = (char*)dalloc(ctx, (size_t)ctx->nsm * bsolve_oz_scratch());
+    } catch (std::bad_alloc&) {
+      boz = false;
+    }
+  }
   const int grid = ctx->nsm * 4;
   std::vector<std::vector<DenseEnt>> keep_ent;  // host sources of the copies in flight
   std::vector<std::vector<int4>> keep_it;
@@ -624,8 +650,42 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
     queue_reset(ctx, 41);
     launch_adj_build(ctx->P, ctx->d_adj_batch, ctx->d_adj_items4, (int)bv.size(), ctx->d_queue + 41,
                      haveX ? (const double*)ctx->d_X : ctx->d_Xu, haveX ? 1 : 0, dense ? 1 : 0, ctx->d_adj_work, std::max(1, std::min<int>(grid, (int)bv.size())), st);
+    std::vector<int4> lv;
+    std::vector<int2> yv;
+    if (boz) {
+      for (int e = 0; e < nb; ++e) {
+        const auto& pat = ctx->pats[ctx->subs[b[e].sub].pat];
+        int64_t ofs = b[e].lt;
+        for (int s = 0; s < pat.nsn; ++s)
+          for (int kB = 0; pat.sn_big[s] && kB < pat.sn_w[s]; kB += 128) {
+            lv.push_back(make_int4(b[e].sub, s, kB, (int)(ofs / 512)));
+            ofs += bsolve_oz_block_bytes(pat.sn_w[s], pat.sn_r[s], kB);
+          }
+        if (pat.has_big)
+          for (int cb = 0; cb < (b[e].m_pad + 127) / 128; ++cb) yv.push_back(make_int2(e, cb));
+      }
+      if ((int64_t)lv.size() > ctx->adj_lit_cap) {
+        dfree(ctx, ctx->d_adj_lit);
+        ctx->d_adj_lit = (int4*)dalloc(ctx, lv.size() * sizeof(int4));
+        ctx->adj_lit_cap = (int64_t)lv.size();
+      }
+      if ((int64_t)yv.size() > ctx->adj_bit_cap) {
+        dfree(ctx, ctx->d_adj_bit);
+        ctx->d_adj_bit = (int2*)dalloc(ctx, yv.size() * sizeof(int2));
+        ctx->adj_bit_cap = (int64_t)yv.size();
+      }
+      if (!yv.empty()) {
+        CKS(cudaMemcpyAsync(ctx->d_adj_lit, lv.data(), lv.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+        CKS(cudaMemcpyAsync(ctx->d_adj_bit, yv.data(), yv.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+        launch_dig_lt(ctx->P, ctx->d_adj_lit, (int)lv.size(), ctx->d_adj_lt, st);
+        queue_reset(ctx, 43);
+        launch_bsolve_oz(ctx->P, ctx->d_adj_batch, ctx->d_adj_bit, (int)yv.size(), ctx->d_queue + 43, ctx->d_adj_lt,
+                         ctx->d_adj_work, ctx->d_adj_bscr, ctx->nsm, ctx->d_status, st);
+        ctx->stats.launches += 2;
+      }
+    }
     queue_reset(ctx, 42);
-    launch_adj_bsolve(ctx->P, ctx->d_adj_batch, ctx->d_adj_items2, (int)sv.size(), ctx->d_queue + 42,
+    launch_adj_bsolve(ctx->P, ctx->d_adj_batch, ctx->d_adj_items2, (int)sv.size(), ctx->d_queue + 42, boz ? 1 : 0,
                       ctx->d_adj_work, std::max(1, std::min<int>(grid, (int)sv.size())), st);
     if (dense) dense_products(ctx, b, st, keep_ent, keep_it);
     if (adjoint)
@@ -679,6 +739,9 @@ feti_status feti_adjoint(feti_ctx* ctx, const double* W_dev, double* dtheta_dev)
       dfree(ctx, ctx->d_adj_dig);
       ctx->d_adj_dig = nullptr;
       ctx->adj_dig_bytes = 0;
+      dfree(ctx, ctx->d_adj_lt);
+      ctx->d_adj_lt = nullptr;
+      ctx->adj_lt_bytes = 0;
     }
     return FETI_OK;
   } catch (std::bad_alloc&) {

@@ -82,6 +82,7 @@ struct DevPlan {
   const int64_t* di_ofs;     // [sn] offset of the supernode's inverted diagonal blocks in DI (relative to the
                              // subdomain's di; 4 blocks of 32 x 32 per 128 own rows), -1 where lh_ofs is -1
   const int64_t* ld_ofs;     // [sn] offset of a large supernode's digits in LD (512 bytes, relative), -1 otherwise
+  const int64_t* lt_ofs;     // [sn] offset of a large supernode's digits of L^T (512 bytes, relative), -1 otherwise
   const int64_t* tx_ofs;     // [sn] a large supernode's update block on trsm_oz_kernel's stack (doubles per column)
   const int64_t* th_ofs;     // [bsn] hand-over slot of a supernode below a large one (doubles, relative), -1 otherwise
   float* DI;                 // inverses of the 32 x 32 diagonal blocks of the large panels (FP32)
@@ -231,6 +232,7 @@ constexpr int kPcgMaxBlocks = 1184;  // block partials per reduction
 struct AdjBatch {
   int sub, m, m_pad, edofs, nelem;
   int zonly;  // 1: V holds only D^{-2} X_u (row length m_pad), for the TRSM-path assembly of F_i
+  int64_t lt;  // digits of L^T of the large fronts (bytes; bsolve_oz_kernel)
   int64_t qcol, w_src, ws_ofs, v_ofs, el_dofs, el_dk, el_out, dk_stride;
 };
 constexpr int kBuildCols = 512;  // columns of V_Y per item of the adjoint's X_u W product

@@ -201,6 +201,13 @@ struct feti_ctx {
   double* d_Xu = nullptr;          // FP64 X_u = L_u^{-1} P B^T of every subdomain (adjoint)
   double* d_adj_work = nullptr;    // batch work arrays of the adjoint (V and sorted W)
   int64_t adj_work_bytes = 0;
+  std::vector<int64_t> pat_lt;     // per pattern: bytes of the large fronts' digits of L^T
+  void* d_adj_lt = nullptr;        // those digits of one batch, and the backward solve's scratch
+  int64_t adj_lt_bytes = 0;
+  char* d_adj_bscr = nullptr;
+  int4* d_adj_lit = nullptr;
+  int2* d_adj_bit = nullptr;
+  int64_t adj_lit_cap = 0, adj_bit_cap = 0;
   void* d_adj_dig = nullptr;       // digits of Z and W (the adjoint's Y = Z W)
   int64_t adj_dig_bytes = 0;
   feti::DenseEnt* d_adj_ent = nullptr;

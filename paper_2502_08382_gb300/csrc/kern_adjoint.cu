@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kAT) adj_build_kernel(DevPlan P, const AdjBatc
 // as a GEMM over 32-row chunks, then the unit upper-triangular solve with the
 // block's own 32 x 32 triangle (four threads per column, warp reductions).
 __global__ void __launch_bounds__(kAT) adj_bsolve_kernel(DevPlan P, const AdjBatch* B, const int2* items, int nitems,
-                                                        int* queue, double* work) {
+                                                        int* queue, int skip_big, double* work) {
   __shared__ double Lc[32][33];      // L chunk: [k][i]
   __shared__ double Vc[32][kCB];     // V chunk: [i][c]
   __shared__ double Xb[32][kCB];     // the block's rows being solved
@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(kAT) adj_bsolve_kernel(DevPlan P, const AdjBat
     const double* Lsub = P.L + S.L;
     for (int s = S.nsn - 1; s >= 0; --s) {
       const int gs = S.sn0 + s;
+      if (skip_big && P.sn_big[gs]) continue;  // bsolve_oz_kernel's
       const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
       const double* Ls = Lsub + P.Lofs[gs];
       const int* srow = P.rows + P.sn_rows[gs];
@@ -386,9 +387,9 @@ void launch_adj_build(const DevPlan& P, const AdjBatch* B, const int4* items, in
   if (nitems > 0) adj_build_kernel<<<grid, kAT, 0, st>>>(P, B, items, nitems, queue, Xu, scaled, zcols, work);
 }
 
-void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, double* work,
-                       int grid, cudaStream_t st) {
-  if (nitems > 0) adj_bsolve_kernel<<<grid, kAT, 0, st>>>(P, B, items, nitems, queue, work);
+void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue,
+                       int skip_big, double* work, int grid, cudaStream_t st) {
+  if (nitems > 0) adj_bsolve_kernel<<<grid, kAT, 0, st>>>(P, B, items, nitems, queue, skip_big, work);
 }
 
 void launch_adj_contract(const DevPlan& P, const AdjBatch* B, int nb, int max_nelem, const int* eldofs,

@@ -48,6 +48,14 @@ void launch_syrk_f64(const DevPlan& P, const int2* items, int nitems, const doub
                      cudaStream_t st);
 void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const int4* ditems, const int4* items,
                     void* XD, int* EX, double* F, int nsm, int* status, cudaStream_t st);
+// backward solve of the large fronts on the tensor cores (kern_bsolve_oz.cu), before launch_adj_bsolve with skip_big;
+// items: digits (subdomain, supernode, first column of the 128-column block, offset / 512), solve (batch entry, 128-column
+// block); scratch: bsolve_oz_scratch() bytes per CTA
+int64_t bsolve_oz_block_bytes(int w, int r, int kB);
+int64_t bsolve_oz_scratch();
+void launch_dig_lt(const DevPlan& P, const int4* items, int nitems, void* LT, cudaStream_t st);
+void launch_bsolve_oz(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, const void* LT,
+                      double* work, void* scratch, int grid, int* status, cudaStream_t st);
 // dense FP64 products by the same tiles; items (product, 128-row block | 64-column block << 16, 32-deep chunks, 0)
 void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const double* src, void* XD, int* EX,
                      double* out, int nsm, int* status, cudaStream_t st);
@@ -146,7 +154,7 @@ void launch_adj_wsort(const AdjBatch* B, int nb, const double* W, const int* col
                       cudaStream_t st);
 void launch_adj_build(const DevPlan& P, const AdjBatch* B, const int4* items, int nitems, int* queue,
                       const double* Xu, int scaled, int zcols, double* work, int grid, cudaStream_t st);
-void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, double* work,
+void launch_adj_bsolve(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, int skip_big, double* work,
                        int grid, cudaStream_t st);
 void launch_adj_contract(const DevPlan& P, const AdjBatch* B, int nb, int max_nelem, const int* eldofs,
                          const double* eldk, const double* elsc, const double* work, double* g, cudaStream_t st);
