@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kAT) adj_bsolve_kernel(DevPlan P, const AdjBat
       for (int kb = ((w - 1) / 32) * 32; kb >= 0; kb -= 32) {
         const int nbk = min(32, w - kb);
         double acc[8] = {};
+        const int nk = max(0, min(8, nbk - kg * 8));  // this warp's rows of the block
         for (int i0 = kb + nbk; i0 < f; i0 += 32) {
           const int ni = min(32, f - i0);
           __syncthreads();
@@ -183,10 +184,24 @@ __global__ void __launch_bounds__(kAT) adj_bsolve_kernel(DevPlan P, const AdjBat
             Vc[i][cc] = i < ni ? V[(int64_t)rowid[i] * ld + cc] : 0.0;
           }
           __syncthreads();
-          for (int i = 0; i < ni; ++i) {
-            const double v = Vc[i][c];
+          // only the rows the block has (one FP64 instruction of a warp takes 64 clocks of its scheduler): warps
+          // whose rows lie beyond a narrow block go by, the last of its warps takes its rows in pairs
+          if (nk == 8) {
+            for (int i = 0; i < ni; ++i) {
+              const double v = Vc[i][c];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] = fma(Lc[kg * 8 + u][i], v, acc[u]);
+              for (int u = 0; u < 8; ++u) acc[u] = fma(Lc[kg * 8 + u][i], v, acc[u]);
+            }
+          } else if (nk > 0) {
+            for (int i = 0; i < ni; ++i) {
+              const double v = Vc[i][c];
+#pragma unroll
+              for (int u = 0; u < 8; u += 2)
+                if (u < nk) {
+                  acc[u] = fma(Lc[kg * 8 + u][i], v, acc[u]);
+                  acc[u + 1] = fma(Lc[kg * 8 + u + 1][i], v, acc[u + 1]);
+                }
+            }
           }
         }
         __syncthreads();
