@@ -52,6 +52,11 @@ struct feti_ctx {
   feti::DevPlan P{};
   std::vector<feti::DBuf> bufs;
   size_t device_bytes = 0;
+  // pinned staging ring of feti_update_values
+  static constexpr int kSlots = 8;
+  double* h_kslots = nullptr;
+  size_t kslot_len = 0, kslot_next = 0;
+  cudaEvent_t kslot_ev[kSlots] = {};
   // device arrays not in DevPlan
   double* d_Kval = nullptr;
   double* d_L = nullptr;
