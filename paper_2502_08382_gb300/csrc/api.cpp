@@ -1142,7 +1142,7 @@ void build(feti_ctx* c) {
     c->d_part = (double*)dalloc(c, 2 * kPcgMaxBlocks * 8);
     CK(cudaMallocHost((void**)&c->h_sc, 16 * 8));
     c->d_ctrl = (PcgCtrl*)dalloc(c, sizeof(PcgCtrl));
-    CK(cudaMallocHost((void**)&c->h_ctrl, sizeof(PcgCtrl)));
+    CK(cudaMallocHost((void**)&c->h_ctrl, 2 * sizeof(PcgCtrl)));
     launch_build_G(D, c->d_colsub, qo, c->d_R, c->d_G6, c->st);
     CK(cudaGetLastError());
     c->impl_wide = implicit_wide(ns, c->nsm, c->nmax, c->impl_maxf);
@@ -1663,6 +1663,8 @@ void feti_destroy(feti_ctx* ctx) {
   if (ctx->pcg_exec) cudaGraphExecDestroy(ctx->pcg_exec);
   if (ctx->asm_exec) cudaGraphExecDestroy(ctx->asm_exec);
   for (auto e : ctx->pcg_ev) cudaEventDestroy(e);
+  for (auto e : ctx->ctrl_ev)
+    if (e) cudaEventDestroy(e);
   if (ctx->cap_st) cudaStreamDestroy(ctx->cap_st);
   for (auto& b : ctx->bufs) {
     if (ctx->opt.dev_free) ctx->opt.dev_free(b.p, ctx->opt.alloc_ctx);

@@ -122,7 +122,7 @@ void enqueue_precond(feti_ctx* c, int mode, cudaStream_t st) {
     launch_dir_mid(c->fp32, c->d_lamcol, n, c->d_rowpart, c->d_tpart, vec(c, V_U), ctrl, iter, st);
     launch_dir_post(n, c->d_w_off, c->d_w_col, c->d_w_val, vec(c, V_U), v, ctrl, iter, st);
   } else {
-    launch_lumped_apply(n, c->d_w_off, c->d_w_col, c->d_w_val, c->d_m_off, c->d_m_col, c->d_m_val, w, v, ctrl,
+    launch_lumped_apply(n, c->d_w_off, c->d_w_col, c->d_w_val, c->d_m_off, c->d_m_col, c->d_m_val, w, vec(c, V_T), vec(c, V_U), v, ctrl,
                         iter, st);
   }
   if (D > 0) {
@@ -137,7 +137,7 @@ void enqueue_precond(feti_ctx* c, int mode, cudaStream_t st) {
 // nine with the lumped preconditioner; every kernel returns at once if the
 // control block says the iteration has stopped.
 // ev (4 events or null): before the tile kernel, around it, after the gather.
-void enqueue_iteration(feti_ctx* c, double* lam, const cudaEvent_t* ev, cudaStream_t st, bool capture) {
+void enqueue_iteration(feti_ctx* c, double* lam, const cudaEvent_t* ev, cudaStream_t st, bool capture, bool last = false) {
   const unsigned evf = capture ? cudaEventRecordExternal : cudaEventRecordDefault;
   const int n = c->nlam, D = c->dtot;
   const int pre = c->precond ? 1 : 0;
@@ -156,37 +156,40 @@ void enqueue_iteration(feti_ctx* c, double* lam, const cudaEvent_t* ev, cudaStre
     launch_gemv_rows(c->d_Ainv, cvec(c, C_GQ), cvec(c, C_Z), D, ctrl, 0, st);
   }
   launch_pcg_update(c->fp32, c->d_lamg, c->d_c0, c->d_c1, n, c->d_G6, D > 0 ? cvec(c, C_Z) : nullptr, p, qk, d, lam, r,
-                    w, c->d_pg, c->d_part + kPcgMaxBlocks, 0, pre, ctrl, st);
+                    w, c->d_pg, c->d_part + kPcgMaxBlocks, 0, pre, last ? 1 : 0, ctrl, st);
   if (pre) enqueue_precond(c, 0, st);
 }
 
 int iteration_launches(feti_ctx* c) {
-  return (c->dtot > 0 ? 5 : 3) + (c->precond ? (c->dtot > 0 ? 4 : 2) : 0) + (c->precond_kind == 2 ? 3 : 0);
+  return (c->dtot > 0 ? 5 : 3) + (c->precond ? (c->dtot > 0 ? 4 : 2) : 0) + (c->precond_kind == 2 ? 3 : c->precond_kind == 1 ? 2 : 0);
 }
 
 // Capture `chunk` iterations on the private stream into one CUDA graph (once
-// per context and chunk size); replaying it enqueues the whole chunk at once.
+// per context, chunk size and profiling state); replaying it enqueues the whole chunk at once.  Only a profiled chunk
+// records events (four nodes an iteration that the next kernel has to wait for).
 void build_chunk_graph(feti_ctx* c, double* lam, int chunk) {
-  if (c->pcg_exec && c->pcg_chunk == chunk) return;
+  if (c->pcg_exec && c->pcg_chunk == chunk && c->pcg_prof == c->prof) return;
   if (c->pcg_exec) {
     CKS(cudaGraphExecDestroy(c->pcg_exec));
     c->pcg_exec = nullptr;
   }
   if (!c->cap_st) CKS(cudaStreamCreateWithFlags(&c->cap_st, cudaStreamNonBlocking));
-  while ((int)c->pcg_ev.size() < 4 * chunk) {
+  while (c->prof && (int)c->pcg_ev.size() < 4 * chunk) {
     cudaEvent_t e;
     CKS(cudaEventCreate(&e));
     c->pcg_ev.push_back(e);
   }
   cudaGraph_t g = nullptr;
   CKS(cudaStreamBeginCapture(c->cap_st, cudaStreamCaptureModeThreadLocal));
-  for (int k = 0; k < chunk; ++k) enqueue_iteration(c, lam, &c->pcg_ev[4 * k], c->cap_st, true);
+  for (int k = 0; k < chunk; ++k)
+    enqueue_iteration(c, lam, c->prof ? &c->pcg_ev[4 * k] : nullptr, c->cap_st, true, k == chunk - 1);
   cudaError_t e = cudaStreamEndCapture(c->cap_st, &g);
   if (e != cudaSuccess) throw CudaErr(std::string("capture of the PCPG chunk: ") + cudaGetErrorString(e));
   e = cudaGraphInstantiate(&c->pcg_exec, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) throw CudaErr(std::string("instantiation of the PCPG chunk: ") + cudaGetErrorString(e));
   c->pcg_chunk = chunk;
+  c->pcg_prof = c->prof;
 }
 
 // Residual replacement with the FP64 implicit operator (eq. 11): q = F_64 lambda,
@@ -204,10 +207,10 @@ void enqueue_refresh(feti_ctx* c, double* lam, int mode) {
     launch_gemv_rows(c->d_Ainv, cvec(c, C_C), cvec(c, C_Z), D, ctrl, 1, st);
   }
   launch_pcg_update(c->fp32, c->d_lamg, c->d_c0, c->d_c1, n, c->d_G6, D > 0 ? cvec(c, C_Z) : nullptr, p, q, d, lam, r,
-                    w, c->d_pg, c->d_part + kPcgMaxBlocks, mode, c->precond ? 1 : 0, ctrl, st);
+                    w, c->d_pg, c->d_part + kPcgMaxBlocks, mode, c->precond ? 1 : 0, 0, ctrl, st);
   if (c->precond) enqueue_precond(c, mode, st);
   c->stats.launches += (D > 0 ? 3 : 1) + (mode == 2 ? 1 : 0) + (c->precond ? (D > 0 ? 4 : 2) : 0) +
-                       (c->precond_kind == 2 ? 3 : 0);
+                       (c->precond_kind == 2 ? 3 : c->precond_kind == 1 ? 2 : 0);
 }
 
 }  // namespace
@@ -270,6 +273,11 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
     h.maxit = maxit;
     h.active = 1;
     h.restart = ctx->opt.refine_restart ? 1 : 0;
+    // One chunk ahead: the next chunk is enqueued before the host reads the outcome of this one, which the device makes
+    // safe by pausing where the host would step in (drop).  Not with a fixed replacement period, not while profiling
+    // (the chunk's events are read after each), and not where a paused iteration's preconditioned direction is needed.
+    const bool ahead = ctx->opt.refine_every <= 0 && !ctx->prof && (!ctx->precond || h.restart);
+    h.drop = ahead ? ctx->opt.refine_drop : 0.0;
     *ctx->h_ctrl = h;
     CKS(cudaMemcpyAsync(ctx->d_ctrl, ctx->h_ctrl, sizeof(PcgCtrl), cudaMemcpyHostToDevice, st));
     // p_{-1} = q_{-1} = 0 (beta = 0 at the start, but 0 * garbage need not be 0);
@@ -293,6 +301,9 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
         CKS(cudaMemcpyAsync(lam, lambda_dev, (size_t)n * 8, cudaMemcpyDeviceToDevice, st));
       }
       enqueue_refresh(ctx, lam, 1);
+      // the drops count from the cold residual ||w_0||
+      char* cd = reinterpret_cast<char*>(ctx->d_ctrl);
+      CKS(cudaMemcpyAsync(cd + offsetof(PcgCtrl, nw_ref), cd + offsetof(PcgCtrl, nw0), 8, cudaMemcpyDeviceToDevice, st));
     }
     PcgCtrl cur = read_ctrl(ctx);
     const double nw0 = cur.nw0;
@@ -306,17 +317,35 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
     bool conv = cur.conv != 0;
     bool last_refresh = true;  // r holds d - F_64 lambda (true after the start and after a replacement)
     if (!conv) build_chunk_graph(ctx, lam, chunk);
+    if (ahead && !conv && !ctx->ctrl_ev[0])
+      for (auto& e : ctx->ctrl_ev) CKS(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    int enq = 0, seen = 0;  // chunks enqueued and looked at (ahead)
+    auto enqueue_chunk = [&]() {
+      CKS(cudaGraphLaunch(ctx->pcg_exec, st));
+      ctx->stats.launches += (int64_t)chunk * iteration_launches(ctx);
+      CKS(cudaMemcpyAsync(ctx->h_ctrl + (enq & 1), ctx->d_ctrl, sizeof(PcgCtrl), cudaMemcpyDeviceToHost, st));
+      CKS(cudaEventRecord(ctx->ctrl_ev[enq & 1], st));
+      ++enq;
+    };
     while (!conv && cur.it < maxit && !cur.breakdown) {
-      int todo = chunk;
-      if (kref > 0) todo = std::min(todo, std::max(1, kref - (cur.it - it_ref)));
       const int it0 = cur.it;
-      if (todo == chunk) {
-        CKS(cudaGraphLaunch(ctx->pcg_exec, st));
+      if (ahead) {
+        while (enq < seen + 2) enqueue_chunk();
+        CKS(cudaEventSynchronize(ctx->ctrl_ev[seen & 1]));
+        cur = ctx->h_ctrl[seen & 1];
+        ++seen;
       } else {
-        for (int k = 0; k < todo; ++k) enqueue_iteration(ctx, lam, &ctx->pcg_ev[4 * k], st, false);
+        int todo = chunk;
+        if (kref > 0) todo = std::min(todo, std::max(1, kref - (cur.it - it_ref)));
+        if (todo == chunk) {
+          CKS(cudaGraphLaunch(ctx->pcg_exec, st));
+        } else {
+          for (int k = 0; k < todo; ++k)
+            enqueue_iteration(ctx, lam, ctx->prof ? &ctx->pcg_ev[4 * k] : nullptr, st, false);
+        }
+        ctx->stats.launches += (int64_t)todo * iteration_launches(ctx);
+        cur = read_ctrl(ctx);
       }
-      ctx->stats.launches += (int64_t)todo * iteration_launches(ctx);
-      cur = read_ctrl(ctx);
       const int done = cur.it - it0;  // iterations that ran (later ones returned at once)
       if (done > 0) last_refresh = false;
       ctx->stats.apply_calls += done;
@@ -331,11 +360,13 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
       }
       if (cur.breakdown) break;
       const bool due = refine && ((kref > 0 && cur.it - it_ref >= kref) || (drop > 0.0 && cur.nw <= drop * nw_ref) ||
-                                  cur.conv);
+                                  cur.conv || (ahead && !cur.active && cur.it < maxit));
       if (due) {
         // residual replacement (and, after the recursive residual met the stopping rule, its FP64 check)
+        // (the chunk enqueued ahead has returned at once: it stands before the refresh in the stream, paused)
         enqueue_refresh(ctx, lam, 1);
         cur = read_ctrl(ctx);
+        seen = enq;
         last_refresh = true;
         ++nref;
         it_ref = cur.it;

@@ -215,6 +215,8 @@ struct PcgCtrl {
   double tol;     // relative tolerance on ||w|| / ||w_0||
   double floor;   // rounding level of the residual: 64 eps (||d|| + ||F lambda_0||)
   double rel;     // ||w|| / ||w_0||
+  double drop;    // > 0: pause at a chunk's end once nw <= drop * nw_ref (a residual replacement is due)
+  double nw_ref;  // ||w|| at the start or the last residual replacement
   double dd, qq;  // ||d||^2 and ||F lambda_0||^2 (for the floor)
   int active;     // 1 while iterating; kernels of later iterations return when 0
   int it;         // iterations done

@@ -194,6 +194,8 @@ struct feti_ctx {
   float* d_L32 = nullptr;            // FP32 copy of L for the mixed TRSM
   cudaGraphExec_t pcg_exec = nullptr;  // captured chunk of iterations (replayed on st)
   int pcg_chunk = 0;
+  bool pcg_prof = false;             // the captured chunk records events
+  cudaEvent_t ctrl_ev[2] = {nullptr, nullptr};  // control-block copies of chunks enqueued ahead
   std::vector<cudaEvent_t> pcg_ev;  // 4 events per captured iteration (apply timing)
   int* d_dofsub = nullptr;
   // adjoint (element data and dense work buffers, allocated on first use)

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kVT) pcg_update_kernel(const int4* lg, const i
                                                          const double* G6, const double* z, const double* p,
                                                          const double* q, const double* d, double* lam, double* r,
                                                          double* w, TF* pg, double* part, int mode, int pre,
-                                                         PcgCtrl* ctrl) {
+                                                         int last, PcgCtrl* ctrl) {
   __shared__ double red[kVT / 32];
   if (mode == 0 && !ctrl->active) return;
   const double delta = ctrl->delta;
@@ -231,7 +231,11 @@ __global__ void __launch_bounds__(kVT) pcg_update_kernel(const int4* lg, const i
       if (mode == 0) ctrl->it += 1;
       ctrl->rel = ctrl->nw0 > 0.0 ? nw / ctrl->nw0 : 0.0;
       ctrl->conv = (nw <= ctrl->tol * ctrl->nw0 || nw <= ctrl->floor) ? 1 : 0;
-      ctrl->active = (!ctrl->conv && !ctrl->breakdown && ctrl->it < ctrl->maxit) ? 1 : 0;
+      if (mode != 0) ctrl->nw_ref = nw;
+      // last iteration of a chunk: pause where the host will replace the residual, so that a chunk enqueued before the
+      // host has seen this one's outcome returns at once
+      const bool pause = mode == 0 && last && ctrl->drop > 0.0 && nw <= ctrl->drop * ctrl->nw_ref;
+      ctrl->active = (!ctrl->conv && !ctrl->breakdown && ctrl->it < ctrl->maxit && !pause) ? 1 : 0;
       ctrl->cnt_upd = 0;
     }
   }
@@ -254,28 +258,26 @@ __global__ void lumped_values_kernel(int64_t nnz, const int64_t* c_off, const in
   }
 }
 
-// v = W M_core W w, one thread per multiplier a:
-//   v_a = sum_{c in W row a} W_ac sum_{e in M_core row c} m_e sum_{f in W row col_e} W_{col_e f} w_f
-// (W's blocks are a node's few multipliers, so the redundant inner sums are short).
-__global__ void __launch_bounds__(kVT) lumped_apply_kernel(int nlam, const int* woff, const int* wcol,
-                                                           const double* wval, const int* moff, const int* mcol,
-                                                           const double* mval, const double* w, double* v,
-                                                           const PcgCtrl* ctrl, int iteration) {
+// s = M_core t (CSR), eight lanes per row: the middle of v = W M_core W w, whose outer factors are two small products
+// (dir_post_kernel).  One kernel that formed (W w)_col anew for every entry of M_core was a chain of five dependent
+// loads per entry: 70 us per application on 125 uneven 3D heat subdomains (51 k multipliers, 2.6 M entries).
+__global__ void __launch_bounds__(kVT) lumped_core_kernel(int nlam, const int* moff, const int* mcol, const double* mval,
+                                                          const double* t, double* s, const PcgCtrl* ctrl,
+                                                          int iteration) {
   if (iteration && !ctrl->active) return;
-  for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < nlam; a += gridDim.x * blockDim.x) {
+  const int l8 = threadIdx.x & 7;
+  const int rows = (nlam + 3) & ~3;  // whole warps (four rows each) stay together for the shuffles
+  for (int a = (blockIdx.x * blockDim.x + threadIdx.x) / 8; a < rows; a += gridDim.x * blockDim.x / 8) {
     double acc = 0.0;
-    for (int i = woff[a]; i < woff[a + 1]; ++i) {
-      const int c = wcol[i];
-      double sc = 0.0;
-      for (int e = moff[c]; e < moff[c + 1]; ++e) {
-        const int d = mcol[e];
-        double t = 0.0;
-        for (int f = woff[d]; f < woff[d + 1]; ++f) t = fma(wval[f], w[wcol[f]], t);
-        sc = fma(mval[e], t, sc);
-      }
-      acc = fma(wval[i], sc, acc);
+    if (a < nlam) {
+      const int e1 = moff[a + 1];
+#pragma unroll 4
+      for (int e = moff[a] + l8; e < e1; e += 8) acc = fma(mval[e], t[mcol[e]], acc);
     }
-    v[a] = acc;
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (l8 == 0 && a < nlam) s[a] = acc;
   }
 }
 
@@ -399,13 +401,14 @@ void launch_gemv_rows(const double* A, const double* c, double* z, int D, const 
 
 void launch_pcg_update(bool fp32, const int4* lg, const int* c0, const int* c1, int nlam, const double* G6,
                        const double* z, const double* p, const double* q, const double* d, double* lam, double* r,
-                       double* w, void* pg, double* part, int mode, int pre, PcgCtrl* ctrl, cudaStream_t st) {
+                       double* w, void* pg, double* part, int mode, int pre, int last, PcgCtrl* ctrl,
+                       cudaStream_t st) {
   if (fp32)
     pcg_update_kernel<float><<<vgrid(nlam), kVT, 0, st>>>(lg, c0, c1, nlam, G6, z, p, q, d, lam, r, w, (float*)pg,
-                                                          part, mode, pre, ctrl);
+                                                          part, mode, pre, last, ctrl);
   else
     pcg_update_kernel<double><<<vgrid(nlam), kVT, 0, st>>>(lg, c0, c1, nlam, G6, z, p, q, d, lam, r, w, (double*)pg,
-                                                           part, mode, pre, ctrl);
+                                                           part, mode, pre, last, ctrl);
 }
 
 void launch_lumped_values(int64_t nnz, const int64_t* c_off, const int64_t* kidx, const double* sgn,
@@ -415,10 +418,14 @@ void launch_lumped_values(int64_t nnz, const int64_t* c_off, const int64_t* kidx
   lumped_values_kernel<<<g, kVT, 0, st>>>(nnz, c_off, kidx, sgn, Kval, mval);
 }
 
+// v = W M_core W w; t and u: n-vectors of scratch
 void launch_lumped_apply(int nlam, const int* woff, const int* wcol, const double* wval, const int* moff,
-                         const int* mcol, const double* mval, const double* w, double* v, const PcgCtrl* ctrl,
-                         int iteration, cudaStream_t st) {
-  lumped_apply_kernel<<<vgrid(nlam), kVT, 0, st>>>(nlam, woff, wcol, wval, moff, mcol, mval, w, v, ctrl, iteration);
+                         const int* mcol, const double* mval, const double* w, double* t, double* u, double* v,
+                         const PcgCtrl* ctrl, int iteration, cudaStream_t st) {
+  launch_dir_post(nlam, woff, wcol, wval, w, t, ctrl, iteration, st);
+  const int g = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)nlam * 8 + kVT - 1) / kVT, 152 * 16));
+  lumped_core_kernel<<<g, kVT, 0, st>>>(nlam, moff, mcol, mval, t, u, ctrl, iteration);
+  launch_dir_post(nlam, woff, wcol, wval, u, v, ctrl, iteration, st);
 }
 
 void launch_dir_pre(bool fp32, int nlam, const int* woff, const int* wcol, const double* wval, const double* w,

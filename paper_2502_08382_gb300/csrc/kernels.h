@@ -125,12 +125,14 @@ void launch_gemv_rows(const double* A, const double* c, double* z, int D, const 
                       cudaStream_t st);
 void launch_pcg_update(bool fp32, const int4* lg, const int* c0, const int* c1, int nlam, const double* G6,
                        const double* z, const double* p, const double* q, const double* d, double* lam, double* r,
-                       double* w, void* pg, double* part, int mode, int pre, PcgCtrl* ctrl, cudaStream_t st);
+                       double* w, void* pg, double* part, int mode, int pre, int last, PcgCtrl* ctrl,
+                       cudaStream_t st);
+// (last: the chunk's last iteration, see PcgCtrl::drop)
 // lumped preconditioner (kern_pcg.cu)
 void launch_lumped_values(int64_t nnz, const int64_t* c_off, const int64_t* kidx, const double* sgn,
                           const double* Kval, double* mval, cudaStream_t st);
 void launch_lumped_apply(int nlam, const int* woff, const int* wcol, const double* wval, const int* moff,
-                         const int* mcol, const double* mval, const double* w, double* v, const PcgCtrl* ctrl,
+                         const int* mcol, const double* mval, const double* w, double* t, double* u, double* v, const PcgCtrl* ctrl,
                          int iteration, cudaStream_t st);
 // Dirichlet preconditioner (kern_pcg.cu, kern_tiles.cu)
 void launch_schur_tiles(const DevPlan& P, const TileDesc* desc, int ntiles, bool fp32, void* M, int grid,
