@@ -569,7 +569,7 @@ void build(feti_ctx* c) {
   std::vector<int2> l16_items;
   int fixo = 0, alo = 0;
   double chol = 0, trsm = 0, syrk = 0, syrke = 0, implb = 0;
-  int64_t sub_cf = 0, sub_chol = 0;
+  int64_t sub_chol = 0, big_chol = 0;
   int64_t max_chol = 0, max_rhs = 0, max_cf = 0, max_rf = 0, max_usm = 0;
   size_t esz = c->fp32 ? 4 : 8;
   double apply_bytes = 0, stored_bytes = 0;
@@ -676,8 +676,8 @@ void build(feti_ctx* c) {
     max_chol = std::max(max_chol, P.chol_stack);
     max_usm = std::max(max_usm, P.usm_size);
     max_cf = std::max(max_cf, P.chol_front);
-    sub_cf = std::max(sub_cf, P.sub_front);
     sub_chol = std::max(sub_chol, P.sub_stack);
+    big_chol = std::max(big_chol, P.big_stack);
     max_rhs = std::max(max_rhs, B.rhs_stack);
     max_rf = std::max(max_rf, B.rhs_front);
     apply_bytes += (double)esz * s.m * (s.m + 1) / 2.0 + (double)s.m * (4 + 8 + 8);
@@ -859,10 +859,8 @@ void build(feti_ctx* c) {
     // the mixed TRSM holds the tensor-core stage ring in shared memory: fewer resident CTAs
     c->grid_trsm32 = (int)std::min<int64_t>(c->grid_trsm, (int64_t)c->nsm * trsm_ctas_per_sm(true, 2));
   }
-  c->chol_front = max_cf;
   c->rhs_front = max_rf;
-  c->chol_stack = max_chol;
-  c->ws_stride = std::max(max_cf + max_chol + max_usm, max_rf + max_rhs);
+  c->ws_stride = std::max(std::max(max_cf + max_chol, sub_chol) + max_usm, std::max(big_chol, max_rf + max_rhs));
   c->ws_stride = (c->ws_stride + 31) / 32 * 32;
   {
     // the per-CTA workspace (fronts and update stacks) of all persistent CTAs may take at most 40% of the
@@ -876,11 +874,10 @@ void build(feti_ctx* c) {
   }
   int gw = std::max(c->grid_chol, c->grid_trsm);
   c->grid_ws = gw;
-  // chol_kernel needs the fronts and stacks outside the large set only: as many CTAs as fit the same workspace (its
+  // chol_kernel needs the update blocks outside the large set only: as many CTAs as fit the same workspace (its
   // tasks outnumber the subdomains; with one CTA per subdomain 64 subdomains left half the SMs idle)
-  c->sub_front = sub_cf;
   c->sub_stack = sub_chol;
-  c->sub_stride = std::max<int64_t>((sub_cf + sub_chol + max_usm + 31) / 32 * 32, 32);
+  c->sub_stride = std::max<int64_t>((sub_chol + max_usm + 31) / 32 * 32, 32);
   c->grid_chol = (int)std::max<int64_t>(
       c->grid_chol, std::min<int64_t>((int64_t)c->nsm * chol_ctas_per_sm(), (int64_t)gw * c->ws_stride / c->sub_stride));
 
@@ -1298,7 +1295,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       if (v) CK(cudaMemsetAsync(ctx->d_tdone, 0, (size_t)std::max(ctx->ntask_total, 1) * sizeof(int), s2));
       const int fl = flags | (ctx->n_tc_items > 0 ? kCholSkipBig : 0);
       launch_chol(P, ctx->d_chol_items[v], ctx->chol_nitems[v], v, ctx->d_queue + qslot, ctx->d_tdone, ctx->d_hand,
-                  ctx->d_ws, ctx->sub_stride, ctx->sub_front, ctx->sub_stack,
+                  ctx->d_ws, ctx->sub_stride, ctx->sub_stack,
                   std::min(ctx->grid_chol, ctx->chol_nitems[v]), ctx->d_status, s2, fl);
       if (ctx->n_tc_items > 0) {
         // the large fronts on the tensor cores, after everything below them
@@ -1306,7 +1303,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
         CK(cudaMemsetAsync(ctx->d_queue + qslot + 1, 0, sizeof(int), s2));
         CK(cudaMemsetAsync(ctx->d_tdone, 0, (size_t)std::max(ctx->ntask_total, 1) * sizeof(int), s2));
         launch_chol_tc(P, ctx->d_tc_items, ctx->n_tc_items, ctx->d_queue + qslot + 1, ctx->d_tdone, ctx->d_hand,
-                       ctx->d_ws, ctx->ws_stride, ctx->chol_front, ctx->d_slices, ctx->slice_stride, ctx->grid_tc,
+                       ctx->d_ws, ctx->ws_stride, ctx->d_slices, ctx->slice_stride, ctx->grid_tc,
                        ctx->tc_cluster, ctx->d_status, s2, flags);
       }
     };

@@ -65,7 +65,7 @@ struct DevPlan {
   const int* kmap_src;       // relative to the subdomain's K values
   const int* kmap_dst;       // relative to the subdomain's L base
   const int* diag_src;       // relative to the subdomain's K values
-  const int64_t* upd_ofs;    // [sn] relative to the CTA stack
+  const int64_t* upd_ofs;    // [sn] update block in the CTA's (cluster's) workspace, disjoint from its children's
   const int* lvl_off;        // [lvl0 + l] absolute offsets into lvl_sn
   const int* lvl_sn;         // local supernode ids, level by level
   const int64_t* uofs;       // [sn] update-vector offset of the supernode (relative to the CTA workspace)

@@ -64,8 +64,8 @@ struct feti_ctx {
   void* d_F = nullptr;
   double* d_ws = nullptr;
   int grid_ws = 0;            // CTAs' workspaces of ws_stride doubles
-  int64_t sub_stride = 0, sub_front = 0, sub_stack = 0;  // chol_kernel's workspace per CTA (same buffer)
-  int64_t ws_stride = 0, chol_front = 0, rhs_front = 0, chol_stack = 0;
+  int64_t sub_stride = 0, sub_stack = 0;  // chol_kernel's workspace per CTA (same buffer)
+  int64_t ws_stride = 0, rhs_front = 0;
   double* d_trow = nullptr;
   double* d_tpart = nullptr;
   double* d_qi = nullptr;

@@ -15,8 +15,10 @@
 // shared data is in global memory).  C is as large as keeps the CTAs within the SMs (chol_tc_cluster).
 //
 // Measured (the kernel alone; before: 9 slices of 7 bits, 45 MMAs of N = 32 per 16-deep step, one CTA per front, the
-// panel on the FP64 pipe): 64 uneven 3D heat subdomains 50.3 -> 11.8 ms (C = 2), 27 elasticity subdomains of 12^3
-// 59.0 -> 11.4 ms (C = 4), 64 of them 66.0 -> 19.9 ms (C = 2), 125 uneven 3D heat subdomains 40.8 -> 6.0 ms (C = 1).
+// panel on the FP64 pipe, updates copied to the stack): 64 uneven 3D heat subdomains 50.3 -> 13.7 ms (C = 2), 27
+// elasticity subdomains of 12^3 59.0 -> 9.5 ms (C = 4), 64 of them 66.0 -> 15.4 ms (C = 2), 125 uneven 3D heat
+// subdomains 40.8 -> 9.7 ms (C = 1; these fronts were partly chol_kernel's before).  Of this, forming the bottom block
+// in place and assembling by columns took 64 elasticity subdomains from 20.7 to 15.4 ms (assembly and copy were 36%).
 // What bounds it now: on wide fronts the staging of the digits (96 KB from L2 per 2304 clocks of MMA), on fronts of a
 // few hundred rows the pivot blocks (16 k clocks of FP64 work for 32 columns) and the barriers between the phases.
 //
@@ -205,8 +207,9 @@ __device__ __forceinline__ void dig_inverse(const PivotSmem& sm, uint8_t* bpan, 
 }
 
 // Assemble a front in global memory: the f x w panel Ls (column-major, in the factor's storage) and the r x r bottom
-// block W, from the K entries, the fixing-DOF penalty rho and the children's update blocks (stack or hand-over slots),
-// the work dealt to all threads of the cluster.
+// block W (on and below its diagonal), from the K entries, the fixing-DOF penalty rho and the children's update blocks
+// (workspace or hand-over slots), the work dealt to all warps of the cluster by columns: L2 latency bounds it, so a
+// lane has kFly entries of a column in flight, and no warp meets the upper triangle or a division.
 __device__ __forceinline__ void assemble_cluster(const DevPlan& P, const SubInfo& S, int s, const double* K, double* L,
                                                  double rho, double* W, const double* stack, const double* hand,
                                                  int gtid, int gthreads) {
@@ -214,7 +217,10 @@ __device__ __forceinline__ void assemble_cluster(const DevPlan& P, const SubInfo
   const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
   double* Ls = L + P.Lofs[gs];
   for (int64_t idx = gtid; idx < (int64_t)f * w; idx += gthreads) Ls[idx] = 0.0;
-  for (int64_t idx = gtid; idx < (int64_t)r * r; idx += gthreads) W[idx] = 0.0;
+  const int gw = gtid / 32, lane = gtid % 32, nw = gthreads / 32;
+  constexpr int kFly = 8;
+  for (int j = gw; j < r; j += nw)
+    for (int i = j + lane; i < r; i += 32) W[(int64_t)j * r + i] = 0.0;
   cl_sync();
   for (int64_t k = P.kmap_off[gs] + gtid; k < P.kmap_off[gs + 1]; k += gthreads) L[P.kmap_dst[k]] = K[P.kmap_src[k]];
   cl_sync();
@@ -229,29 +235,25 @@ __device__ __forceinline__ void assemble_cluster(const DevPlan& P, const SubInfo
     const double* U = child_update(P, gc, stack, nullptr, hand);
     const int* rl = P.rel + P.rel_off[gc];
     cl_sync();
-    // four elements per thread and step, their loads issued before their read-modify-writes (distinct targets)
-    const int64_t n = (int64_t)rc * rc;
-    for (int64_t base = gtid; base < n; base += 4 * (int64_t)gthreads) {
-      double* dst[4];
-      double v[4], cur[4];
+    for (int b = gw; b < rc; b += nw) {
+      const int rb = rl[b];
+      double* dst = rb < w ? Ls + (int64_t)rb * f : W + (int64_t)(rb - w) * r - w;
+      const double* src = U + (int64_t)b * rc;
+      for (int a0 = b + lane; a0 < rc; a0 += 32 * kFly) {
+        int ra[kFly];
+        double v[kFly], cur[kFly];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int64_t idx = base + (int64_t)u * gthreads;
-        dst[u] = nullptr;
-        if (idx < n) {
-          const int b = (int)(idx / rc), a = (int)(idx - (int64_t)b * rc);
-          if (a >= b) {
-            const int ra = rl[a], rb = rl[b];
-            v[u] = __ldcg(U + idx);
-            dst[u] = rb < w ? Ls + (int64_t)rb * f + ra : W + (int64_t)(rb - w) * r + (ra - w);
-          }
+        for (int u = 0; u < kFly; ++u) {
+          const int a = a0 + 32 * u;
+          ra[u] = a < rc ? rl[a] : -1;
+          v[u] = a < rc ? __ldcg(src + a) : 0.0;
         }
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) cur[u] = ra[u] >= 0 ? __ldcg(dst + ra[u]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < kFly; ++u)
+          if (ra[u] >= 0) dst[ra[u]] = cur[u] + v[u];
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) cur[u] = dst[u] ? __ldcg(dst[u]) : 0.0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (dst[u]) *dst[u] = cur[u] + v[u];
     }
   }
   cl_sync();
@@ -263,8 +265,7 @@ __device__ __forceinline__ void assemble_cluster(const DevPlan& P, const SubInfo
 // children (tdone), others through the cluster's stack.  Flags as in chol_kernel.
 __global__ void __launch_bounds__(kCT, 1)
     chol_tc_kernel(DevPlan P, const int4* items, int nitems, int* queue, int* tdone, double* hand_all, double* ws,
-                   int64_t ws_stride, int64_t front_sz, char* scratch, int64_t scratch_stride, int flags,
-                   int* status) {
+                   int64_t ws_stride, char* scratch, int64_t scratch_stride, int flags, int* status) {
   extern __shared__ uint8_t ct_raw[];
   uint8_t* ring = ct_raw + ((1024u - (smem_u32(ct_raw) & 1023u)) & 1023u);
   PivotSmem& sm = *reinterpret_cast<PivotSmem*>(ring);
@@ -307,8 +308,7 @@ __global__ void __launch_bounds__(kCT, 1)
   st.drain = &drain;
   st.abort = &abort_s;
   st.tmem = tmem_s;
-  double* W = ws + (int64_t)cluster * ws_stride;
-  double* stack = W + front_sz;
+  double* stack = ws + (int64_t)cluster * ws_stride;
   char* SL = scratch + (int64_t)cluster * scratch_stride;
   for (;;) {
     cl_sync();
@@ -362,6 +362,8 @@ __global__ void __launch_bounds__(kCT, 1)
       if (!P.sn_big[gs] || P.sn_task[gs] != task) continue;
       const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
       double* Ls = L + P.Lofs[gs];
+      // the bottom block is formed where the parent reads it
+      double* W = P.sn_hoff[gs] >= 0 ? hand + P.sn_hoff[gs] : stack + P.upd_ofs[gs];
       assemble_cluster(P, S, s, K, L, rho, W, stack, hand, gtid, gthreads);
       if (!((flags & kCholStopRoot) && s == S.nsn - 1)) {
         for (int kB = 0; kB < w; kB += kCBlk) {
@@ -429,11 +431,6 @@ __global__ void __launch_bounds__(kCT, 1)
         }
       }
       cl_sync();
-      if (P.sn_parent[gs] >= 0) {
-        double* Uout = P.sn_hoff[gs] >= 0 ? hand + P.sn_hoff[gs] : stack + P.upd_ofs[gs];
-        for (int64_t idx = gtid; idx < (int64_t)r * r; idx += gthreads) Uout[idx] = __ldcg(W + idx);
-      }
-      cl_sync();
     }
     if (tid == 0 && bad) atomicOr(status, kStatNotSPD);
     if (rank == 0 && tid == 0 && item.w >= 0) {
@@ -460,7 +457,7 @@ int chol_tc_cluster(int nsub, int nsm) {
 }
 
 void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue, int* tdone, double* hand,
-                    double* ws, int64_t ws_stride, int64_t front_sz, void* scratch, int64_t scratch_stride,
+                    double* ws, int64_t ws_stride, void* scratch, int64_t scratch_stride,
                     int clusters, int cluster, int* status, cudaStream_t st, int flags) {
   if (nitems <= 0) return;
   cudaFuncSetAttribute(chol_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCDyn);
@@ -475,7 +472,7 @@ void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue,
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, chol_tc_kernel, P, items, nitems, queue, tdone, hand, ws, ws_stride, front_sz,
+  cudaLaunchKernelEx(&cfg, chol_tc_kernel, P, items, nitems, queue, tdone, hand, ws, ws_stride,
                      (char*)scratch, scratch_stride, flags, status);
 }
 

@@ -116,16 +116,11 @@ __device__ void warp_tri_inverse(const T (*D)[kNB + 1], const T* dinv, T (*Di)[k
 
 // Partial dense factorisation of one front: eliminate the first w columns of
 // the (w+r) x (w+r) symmetric front held as Ls (column-major f x w) and W
-// (column-major r x r, lower part used).  With a column range: eliminate the
-// columns [kB, kE) only and apply their updates to the columns below ce only
-// (the tensor-core Cholesky updates the rest itself).
-__device__ void factor_front(Smem& sm, double* Ls, int f, int w, double* W, int r, int* bad, int kB = 0,
-                             int kE = -1, int ce = -1) {
+// (column-major r x r, lower part used).
+__device__ void factor_front(Smem& sm, double* Ls, int f, int w, double* W, int r, int* bad) {
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, warp = tid / 32;
-  if (kE < 0) kE = w;
-  if (ce < 0) ce = f;
-  for (int kb = kB; kb < kE; kb += kNB) {
-    const int nbk = min(kNB, kE - kb);
+  for (int kb = 0; kb < w; kb += kNB) {
+    const int nbk = min(kNB, w - kb);
     for (int idx = tid; idx < kNB * kNB; idx += kThreads) {
       int i = idx % kNB, j = idx / kNB;
       sm.D[i][j] = (i < nbk && j <= i) ? Ls[(int64_t)(kb + j) * f + kb + i] : 0.0;
@@ -236,8 +231,8 @@ __device__ void packed_front(const DevPlan& P, const SubInfo& S, int s, const do
   for (int e = tid; e < np; e += TEAM) Fp[e] = 0.0;
   team_sync<TEAM>();
   for (int64_t kk = P.kmap_off[gs] + tid; kk < P.kmap_off[gs + 1]; kk += TEAM) {
-    const int64_t rel = P.kmap_dst[kk] - L0;  // column-major f x w panel position
-    Fp[pidx(f, (int)(rel % f), (int)(rel / f))] = K[P.kmap_src[kk]];
+    const uint32_t rel = (uint32_t)(P.kmap_dst[kk] - L0);  // column-major f x w panel position
+    Fp[pidx(f, (int)(rel % (uint32_t)f), (int)(rel / (uint32_t)f))] = K[P.kmap_src[kk]];
   }
   team_sync<TEAM>();
   for (int k = tid; k < S.nfix; k += TEAM)
@@ -251,8 +246,24 @@ __device__ void packed_front(const DevPlan& P, const SubInfo& S, int s, const do
     const double* U = child_update(P, gc, stack, smallreg, hand);
     const int* rl = P.rel + P.rel_off[gc];
     team_sync<TEAM>();
-    for (int b = 0; b < rc; ++b)
-      for (int a = b + tid; a < rc; a += TEAM) Fp[pidx(f, rl[a], rl[b])] += __ldcg(U + (int64_t)b * rc + a);
+    // columns dealt to the warps, four columns of a warp at a time so that their loads are in flight together (an L2
+    // latency per column was most of the time of the middle fronts)
+    constexpr int kW = TEAM / 32;
+    for (int b0 = tid / 32; b0 < rc; b0 += 4 * kW)
+      for (int a = b0 + tid % 32; a < rc; a += 32) {
+        double v[4];
+        int rb[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int b = b0 + u * kW;
+          v[u] = b <= a ? __ldcg(U + (int64_t)b * rc + a) : 0.0;
+          rb[u] = b <= a ? rl[b] : 0;
+        }
+        const int ra = rl[a];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (b0 + u * kW <= a) Fp[pidx(f, ra, rb[u])] += v[u];
+      }
   }
   team_sync<TEAM>();
   // blocked right-looking partial factorisation of the first w columns: one warp
@@ -323,25 +334,25 @@ __device__ void packed_front(const DevPlan& P, const SubInfo& S, int s, const do
     const int row = idx % f, col = idx / f;
     L[L0 + idx] = row >= col ? Fp[pidx(f, row, col)] : 0.0;
   }
-  if (Uout)
-    for (int idx = tid; idx < r * r; idx += TEAM) {
-      const int a = idx % r, b = idx / r;
-      Uout[idx] = a >= b ? Fp[pidx(f, w + a, w + b)] : 0.0;
-    }
+  if (Uout)  // the lower triangle, all that the parent reads
+    for (int b = tid / 32; b < r; b += TEAM / 32)
+      for (int a = b + tid % 32; a < r; a += 32) Uout[b * r + a] = Fp[pidx(f, w + a, w + b)];
   team_sync<TEAM>();
 }
 
 // Assemble a front of the tiled path in global memory: the f x w panel Ls (column-major, in the factor's
-// storage) and the r x r bottom block W, from the K entries, the fixing-DOF penalty rho and the children's update
-// blocks (stack, small region or hand-over slot).
+// storage) and the r x r bottom block W (on and below its diagonal), from the K entries, the fixing-DOF penalty rho
+// and the children's update blocks (stack, small region or hand-over slot), by columns as in packed_front.
 __device__ void assemble_tiled(const DevPlan& P, const SubInfo& S, int s, const double* K, double* L, double rho,
                                double* W, const double* stack, const double* smallreg, const double* hand) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  constexpr int kWarps = kThreads / 32, kFly = 4;
   const int gs = S.sn0 + s;
   const int w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
   double* Ls = L + P.Lofs[gs];
   for (int64_t idx = tid; idx < (int64_t)f * w; idx += kThreads) Ls[idx] = 0.0;
-  for (int64_t idx = tid; idx < (int64_t)r * r; idx += kThreads) W[idx] = 0.0;
+  for (int j = warp; j < r; j += kWarps)
+    for (int i = j + lane; i < r; i += 32) W[(int64_t)j * r + i] = 0.0;
   __syncthreads();
   for (int64_t k = P.kmap_off[gs] + tid; k < P.kmap_off[gs + 1]; k += kThreads)
     L[P.kmap_dst[k]] = K[P.kmap_src[k]];
@@ -354,30 +365,27 @@ __device__ void assemble_tiled(const DevPlan& P, const SubInfo& S, int s, const 
     const double* U = child_update(P, gc, stack, smallreg, hand);
     const int* rl = P.rel + P.rel_off[gc];
     __syncthreads();
-    // four elements per thread and step, their loads issued before their read-modify-writes (distinct
-    // targets: rel is one-to-one)
-    const int64_t n = (int64_t)rc * rc;
-    for (int64_t base = tid; base < n; base += 4 * kThreads) {
-      double* dst[4];
-      double v[4], cur[4];
+    // kFly entries of a column per lane, their loads issued before their read-modify-writes (distinct targets: rel is
+    // one-to-one)
+    for (int b = warp; b < rc; b += kWarps) {
+      const int rb = rl[b];
+      double* dst = rb < w ? Ls + (int64_t)rb * f : W + (int64_t)(rb - w) * r - w;
+      const double* src = U + (int64_t)b * rc;
+      for (int a0 = b + lane; a0 < rc; a0 += 32 * kFly) {
+        int ra[kFly];
+        double v[kFly], cur[kFly];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int64_t idx = base + (int64_t)u * kThreads;
-        dst[u] = nullptr;
-        if (idx < n) {
-          const int b = (int)(idx / rc), a = (int)(idx - (int64_t)b * rc);
-          if (a >= b) {
-            const int ra = rl[a], rb = rl[b];
-            v[u] = __ldcg(U + idx);
-            dst[u] = rb < w ? Ls + (int64_t)rb * f + ra : W + (int64_t)(rb - w) * r + (ra - w);
-          }
+        for (int u = 0; u < kFly; ++u) {
+          const int a = a0 + 32 * u;
+          ra[u] = a < rc ? rl[a] : -1;
+          v[u] = a < rc ? __ldcg(src + a) : 0.0;
         }
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) cur[u] = ra[u] >= 0 ? dst[ra[u]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kFly; ++u)
+          if (ra[u] >= 0) dst[ra[u]] = cur[u] + v[u];
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) cur[u] = dst[u] ? *dst[u] : 0.0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (dst[u]) *dst[u] = cur[u] + v[u];
     }
   }
 }
@@ -398,15 +406,13 @@ __device__ void assemble_tiled(const DevPlan& P, const SubInfo& S, int s, const 
 // parent task.
 __global__ void __launch_bounds__(kThreads, 4) chol_kernel(DevPlan P, const int4* items, int nitems, int use_tasks,
                                                          int* queue, int* tdone, double* hand_all, double* ws,
-                                                         int64_t ws_stride, int64_t front_sz, int64_t stack_sz,
-                                                         int flags, int* status) {
+                                                         int64_t ws_stride, int64_t stack_sz, int flags, int* status) {
   extern __shared__ double dsm[];
   Smem& sm = *reinterpret_cast<Smem*>(dsm);
   __shared__ int bad;
   __shared__ double red[kThreads / 32];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  double* W = ws + (int64_t)blockIdx.x * ws_stride;
-  double* stack = W + front_sz;
+  double* stack = ws + (int64_t)blockIdx.x * ws_stride;
   double* smallreg = stack + stack_sz;
   for (;;) {
     int it = pop_item(queue);
@@ -485,13 +491,11 @@ __global__ void __launch_bounds__(kThreads, 4) chol_kernel(DevPlan P, const int4
         packed_front<kThreads>(P, S, s, K, L, rho, dsm, stack, smallreg, Uout, &bad, tid, factor, hand);
         continue;
       }
+      // the bottom block is formed where the parent reads it (a root has none)
       double* Ls = L + P.Lofs[gs];
-      assemble_tiled(P, S, s, K, L, rho, W, stack, smallreg, hand);
+      assemble_tiled(P, S, s, K, L, rho, Uout, stack, smallreg, hand);
       __syncthreads();
-      if (factor) factor_front(sm, Ls, f, w, W, r, &bad);
-      __syncthreads();
-      if (Uout)
-        for (int64_t idx = tid; idx < (int64_t)r * r; idx += kThreads) Uout[idx] = W[idx];
+      if (factor) factor_front(sm, Ls, f, w, Uout, r, &bad);
       __syncthreads();
     }
     __syncthreads();
@@ -1294,12 +1298,12 @@ void launch_l32(const double* L, float* L32, int64_t n, int grid, cudaStream_t s
 }
 
 void launch_chol(const DevPlan& P, const int4* items, int nitems, int use_tasks, int* queue, int* tdone,
-                 double* hand, double* ws, int64_t ws_stride, int64_t front_sz, int64_t stack_sz, int grid,
-                 int* status, cudaStream_t st, int flags) {
+                 double* hand, double* ws, int64_t ws_stride, int64_t stack_sz, int grid, int* status,
+                 cudaStream_t st, int flags) {
   const int smem = kFrontSmem * 8;
   cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  chol_kernel<<<grid, kThreads, smem, st>>>(P, items, nitems, use_tasks, queue, tdone, hand, ws, ws_stride, front_sz,
-                                            stack_sz, flags, status);
+  chol_kernel<<<grid, kThreads, smem, st>>>(P, items, nitems, use_tasks, queue, tdone, hand, ws, ws_stride, stack_sz,
+                                            flags, status);
 }
 
 int chol_ctas_per_sm() {

@@ -11,8 +11,8 @@ namespace feti {
 // items (subdomain, task, global task id, parent's global task id); use_tasks = 0: whole subdomains.
 // tdone: per global task, child tasks finished (zeroed before the launch); hand: hand-over slots.
 void launch_chol(const DevPlan& P, const int4* items, int nitems, int use_tasks, int* queue, int* tdone,
-                 double* hand, double* ws, int64_t ws_stride, int64_t front_sz, int64_t stack_sz, int grid,
-                 int* status, cudaStream_t st, int flags = 0);
+                 double* hand, double* ws, int64_t ws_stride, int64_t stack_sz, int grid, int* status,
+                 cudaStream_t st, int flags = 0);
 int chol_ctas_per_sm();
 // the large fronts (P.sn_big) after launch_chol with kCholSkipBig: items = the large tasks (subdomain, task, global
 // task, parent's global task) children first, tdone zeroed; `clusters` clusters of `cluster` CTAs, one CTA per SM;
@@ -20,8 +20,8 @@ int chol_ctas_per_sm();
 int64_t chol_tc_scratch(int fmax);
 int chol_tc_cluster(int nsub, int nsm);
 void launch_chol_tc(const DevPlan& P, const int4* items, int nitems, int* queue, int* tdone, double* hand,
-                    double* ws, int64_t ws_stride, int64_t front_sz, void* scratch, int64_t scratch_stride,
-                    int clusters, int cluster, int* status, cudaStream_t st, int flags);
+                    double* ws, int64_t ws_stride, void* scratch, int64_t scratch_stride, int clusters,
+                    int cluster, int* status, cudaStream_t st, int flags);
 // items: (subdomain, first sorted column) pairs, each covering cw columns (cw = 0: all columns)
 // X2 (FP32 X only, may be null): the bf16 hi/lo copy of X (per column: wp hi values, then wp lo values; 2 bf16
 // per X element): the large fronts (P.lh_ofs >= 0, tcmode 2) use it as GEMM operand; with x2_out every

@@ -713,24 +713,38 @@ void plan_tasks(PatternPlan& P, double target, int big_f, double target_small) {
   // tasks are numbered parents first, so heights follow from the highest numbers down
   for (int t = P.ntask - 1; t >= 1; --t)
     P.task_height[P.task_parent[t]] = std::max(P.task_height[P.task_parent[t]], P.task_height[t] + 1);
-  // the update stack of the supernodes outside the large set: each maximal subtree of them starts an empty one (its
-  // root hands its block over), so chol_kernel's CTAs need far less workspace than a whole tree's stack
-  P.sub_stack = P.sub_front = 0;
+  // the update blocks that are neither handed over nor in the small region: placed first-fit (postorder, a block lives
+  // from its own front to its parent's) so that a front's block never overlaps its children's and is formed in place.
+  // The large tasks each start with an empty workspace (a cluster takes one task at a time), the supernodes outside
+  // the large set share one: a maximal subtree of them hands its root's block over, so little of it is ever live.
+  P.sub_stack = P.big_stack = 0;
   P.sub_flops = 0;
-  std::vector<int64_t> size(ns, 0);
-  int64_t top = 0;
-  for (int s = 0; s < ns; ++s) {  // postorder: a subtree's supernodes are consecutive
-    if (P.sn_big[s]) continue;
-    int64_t base = top;
-    for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) base -= size[P.ch_list[k]];
+  std::vector<std::vector<std::pair<int64_t, int>>> live(P.ntask + 1);  // (offset, supernode), ascending
+  for (int s = 0; s < ns; ++s) {
+    auto& lv = live[P.sn_big[s] ? P.sn_task[s] : P.ntask];
     const int64_t rr = (int64_t)P.sn_r[s] * P.sn_r[s];
-    size[s] = P.sn_parent[s] >= 0 ? rr : 0;
-    P.upd_stack_ofs[s] = base;
-    top = base + size[s];
-    P.sub_stack = std::max(P.sub_stack, top);
-    P.sub_front = std::max(P.sub_front, rr);
-    P.sub_flops += own[s];
-    if (P.sn_parent[s] < 0 || P.sn_big[P.sn_parent[s]]) top = 0;
+    if (!P.sn_big[s]) P.sub_flops += own[s];
+    P.upd_stack_ofs[s] = 0;
+    const bool own_block = !P.sn_small[s] && P.sn_hoff[s] < 0 && P.sn_parent[s] >= 0 && rr > 0;
+    if (own_block) {
+      int64_t at = 0;
+      size_t k = 0;
+      for (; k < lv.size() && lv[k].first < at + rr; ++k)
+        at = lv[k].first + (int64_t)P.sn_r[lv[k].second] * P.sn_r[lv[k].second];
+      P.upd_stack_ofs[s] = at;
+      lv.insert(lv.begin() + k, {at, s});
+      int64_t& peak = P.sn_big[s] ? P.big_stack : P.sub_stack;
+      peak = std::max(peak, at + rr);
+    }
+    for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) {
+      const int c = P.ch_list[k];
+      auto& lc = live[P.sn_big[c] ? P.sn_task[c] : P.ntask];
+      for (size_t q = 0; q < lc.size(); ++q)
+        if (lc[q].second == c) {
+          lc.erase(lc.begin() + q);
+          break;
+        }
+    }
   }
 }
 

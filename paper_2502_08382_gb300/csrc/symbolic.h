@@ -71,7 +71,8 @@ struct PatternPlan {
   bool has_big = false;
   std::vector<int> task_big;       // 1: the task's supernodes are large (the tensor-core Cholesky's)
   std::vector<int> task_nbig;      // large child tasks
-  int64_t sub_stack = 0, sub_front = 0;  // doubles of update stack / front of the supernodes outside the large set
+  // doubles of workspace for the update blocks outside and inside the large set (neither handed over nor small)
+  int64_t sub_stack = 0, big_stack = 0;
   double sub_flops = 0;            // their Cholesky flops
 };
 
@@ -79,7 +80,7 @@ struct PatternPlan {
 // a task of its own (recursively), so that one large subdomain can be factored by several CTAs.  big_f > 0:
 // the fronts at least big_f wide and their ancestors (the tensor-core Cholesky's work) form tasks of their own,
 // cut by the same rule, and every other child of that set starts a task.  target_small > 0: the target outside the
-// large set.  Also lays the update stack of the supernodes outside the large set out anew (upd_stack_ofs).
+// large set.  Also lays the update blocks out anew (upd_stack_ofs).
 void plan_tasks(PatternPlan& P, double target, int big_f = 0, double target_small = 0);
 
 struct BPlan {
