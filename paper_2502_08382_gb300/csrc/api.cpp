@@ -234,6 +234,9 @@ void plan_syrk_oz(feti_ctx* c, size_t budget) {
     c->oz_batches.push_back(o);
     most = std::max(most, bytes);
   }
+  // a recorded assembly holds the old lists
+  if (c->asm_exec) CK(cudaGraphExecDestroy(c->asm_exec));
+  c->asm_exec = nullptr;
   dfree(c, c->d_oz_items);
   dfree(c, c->d_oz_ditems);
   c->d_oz_items = c->d_oz_ditems = nullptr;
@@ -268,6 +271,7 @@ bool reserve_syrk_oz(feti_ctx* c) {
     } catch (std::bad_alloc&) {
       dfree(c, c->d_XD);
       c->d_XD = nullptr;
+      c->oz_batches.clear();  // planned anew by the next assembly
     }
   }
   return false;
@@ -1234,11 +1238,20 @@ feti_status feti_update_values(feti_ctx* ctx, int32_t sub, const double* K_val) 
   // updates every subdomain in turn; a copy from pageable memory and a synchronisation each took 40 us a subdomain)
   const size_t n = ctx->subs[sub].col.size();
   if (!ctx->h_kslots) {
+    for (auto& e : ctx->kslot_ev)
+      if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     size_t most = 1;
     for (auto& s : ctx->subs) most = std::max(most, s.col.size());
-    CK(cudaMallocHost((void**)&ctx->h_kslots, most * 8 * feti_ctx::kSlots));
+    if (cudaMallocHost((void**)&ctx->h_kslots, most * 8 * feti_ctx::kSlots) != cudaSuccess) {
+      // no pinned memory left: copied from the caller's array, which must not change until the copy is done
+      (void)cudaGetLastError();
+      ctx->h_kslots = nullptr;
+      CK(cudaMemcpyAsync(ctx->d_Kval + ctx->info[sub].Kval, K_val, n * 8, cudaMemcpyHostToDevice, ctx->st));
+      CK(cudaStreamSynchronize(ctx->st));
+      ctx->assembled = false;
+      return FETI_OK;
+    }
     ctx->kslot_len = most;
-    for (auto& e : ctx->kslot_ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   }
   const int slot = (int)(ctx->kslot_next++ % feti_ctx::kSlots);
   double* h = ctx->h_kslots + (size_t)slot * ctx->kslot_len;
@@ -1426,7 +1439,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     enqueue(st, cudaEventRecordDefault, true);
     CK(cudaGetLastError());
   } else if (ctx->asm_exec && ctx->asm_X == ctx->d_X && ctx->asm_X2 == ctx->d_X2 && ctx->asm_XD == ctx->d_XD &&
-             ctx->asm_LD == ctx->d_LD) {
+             ctx->asm_LD == ctx->d_LD && ctx->asm_th == ctx->d_th) {
     CK(cudaGraphLaunch(ctx->asm_exec, st));
   } else {
     ctx->route = want == 1 ? 1 : 0;
@@ -1472,6 +1485,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
       ctx->asm_X2 = ctx->d_X2;
       ctx->asm_XD = ctx->d_XD;
       ctx->asm_LD = ctx->d_LD;
+      ctx->asm_th = ctx->d_th;
     }
   }
   CK(cudaGetLastError());

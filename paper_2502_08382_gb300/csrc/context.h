@@ -190,6 +190,7 @@ struct feti_ctx {
   void* asm_X2 = nullptr;
   void* asm_XD = nullptr;
   void* asm_LD = nullptr;
+  void* asm_th = nullptr;
   uint16_t* d_X2 = nullptr;          // bf16 hi/lo copy of X (split-bf16 SYRK operands)
   float* d_L32 = nullptr;            // FP32 copy of L for the mixed TRSM
   cudaGraphExec_t pcg_exec = nullptr;  // captured chunk of iterations (replayed on st)
