@@ -320,7 +320,7 @@ bool reserve_trsm_oz(feti_ctx* c) {
       c->tx_grid = std::min(c->nsm, c->n_tx_items);
       c->d_tx_ditems = upload(c, di);
       c->d_tx_items = upload(c, it);
-      c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * (c->tx_front + c->tx_stack) * c->tx_cw * 8);
+      c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * std::max<int64_t>(c->tx_stack, 8) * c->tx_cw * 8);
       c->d_txscr = (char*)dalloc(c, (size_t)c->tx_grid * trsm_oz_scratch(c->tx_cw));
       CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
     }
@@ -483,20 +483,20 @@ void build(feti_ctx* c) {
         c->pat_lt[p] += bsolve_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
     }
     if (!c->fp32) {
-      // the digits of each 128-column block, and an update stack of the large supernodes alone
-      std::vector<int64_t> size(P.nsn, 0);
-      int64_t top = 0;
+      // the digits of each 128-column block, and the update blocks of the large supernodes, each disjoint from its
+      // children's
+      BlockPlaces places;
       for (int s = 0; s < P.nsn; ++s) {  // postorder
         ld_ofs.push_back(P.sn_big[s] ? pat_ld[p] / 512 : -1);
-        int64_t base = top;
+        int64_t base = 0;
         if (P.sn_big[s]) {
-          for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) base -= size[P.ch_list[k]];
           for (int kB = 0; kB < P.sn_w[s]; kB += 128) pat_ld[p] += trsm_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
           const int64_t rp = (P.sn_r[s] + 7) & ~7;
-          size[s] = P.sn_parent[s] >= 0 ? rp : 0;
-          c->tx_front = std::max(c->tx_front, rp);
-          top = base + size[s];
-          c->tx_stack = std::max(c->tx_stack, top);
+          if (P.sn_parent[s] >= 0 && rp > 0) {
+            base = places.take(s, rp);
+            c->tx_stack = std::max(c->tx_stack, base + rp);
+          }
+          for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) places.release(P.ch_list[k]);
         }
         tx_ofs.push_back(base);
       }
@@ -1374,8 +1374,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
     if (tx) {
       CK(cudaMemsetAsync(ctx->d_queue + 17, 0, sizeof(int), s2));
       launch_trsm_oz(ctx->P, ctx->d_tx_items, ctx->n_tx_items, ctx->tx_cw, ctx->d_queue + 17, ctx->d_LD, ctx->d_th,
-                     (double*)ctx->d_X, ctx->d_txws, (ctx->tx_front + ctx->tx_stack) * ctx->tx_cw,
-                     ctx->tx_front * ctx->tx_cw, ctx->d_txscr, trsm_oz_scratch(ctx->tx_cw), ctx->tx_grid,
+                     (double*)ctx->d_X, ctx->d_txws, std::max<int64_t>(ctx->tx_stack, 8) * ctx->tx_cw, ctx->d_txscr, trsm_oz_scratch(ctx->tx_cw), ctx->tx_grid,
                      ctx->d_status, s2);
     }
     // the implicit solves take L in unit-lower form; the TRSM above was its last user as L

@@ -108,7 +108,7 @@ struct feti_ctx {
   int2* d_tx_items = nullptr;        // (subdomain, first column) of the solve
   int n_tx_ditems = 0, n_tx_items = 0, tx_cw = 128, tx_grid = 0;
   size_t ld_bytes = 0, th_bytes = 0;
-  int64_t tx_front = 0, tx_stack = 0;  // doubles per column
+  int64_t tx_stack = 0;  // doubles per column
   void* d_LD = nullptr;              // digits of the large panels
   double* d_th = nullptr;            // update blocks handed over
   double* d_txws = nullptr;          // fronts and stacks

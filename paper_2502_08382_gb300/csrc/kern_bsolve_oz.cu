@@ -156,9 +156,11 @@ struct BackJob {
     }
     return nc;
   }
-  __device__ __forceinline__ int ec(int c) const { return __ldg(EXB + c); }
-  __device__ __forceinline__ void store(int ri, int c, double cv, double t) const {
-    C[(int64_t)c * ld + ri] = SET ? t : cv - t;
+  __device__ __forceinline__ int4 ec4(int c) const { return __ldg(reinterpret_cast<const int4*>(EXB + c)); }
+  __device__ __forceinline__ void store4(int ri, int c, int n4, const double* cv, const double* t) const {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < n4) C[(int64_t)(c + e) * ld + ri] = SET ? t[e] : cv[e] - t[e];
   }
 };
 

@@ -83,8 +83,12 @@ struct PanelJob {
   __device__ __forceinline__ int load(int ri, int cb, double (&)[16]) const {
     return ri < n ? min(16, ncol - cb) : 0;
   }
-  __device__ __forceinline__ int ec(int c) const { return EXB[c]; }
-  __device__ __forceinline__ void store(int ri, int c, double, double t) const { out[(int64_t)c * f + ri] = t; }
+  __device__ __forceinline__ int4 ec4(int c) const { return *reinterpret_cast<const int4*>(EXB + c); }
+  __device__ __forceinline__ void store4(int ri, int c, int n4, const double*, const double* t) const {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < n4) out[(int64_t)(c + e) * f + ri] = t[e];
+  }
 };
 
 // C -= A A^T for the columns [i0, i0 + ncol) of the front on and below the diagonal, C in Ls (columns < w) or W;
@@ -125,8 +129,12 @@ struct UpdateJob {
     for (int e = 0; e < 16; ++e) cv[e] = e < nc ? __ldcg(at(ri, cb + e)) : 0.0;
     return nc;
   }
-  __device__ __forceinline__ int ec(int c) const { return __ldcg(EX + c); }
-  __device__ __forceinline__ void store(int ri, int c, double cv, double t) const { *at(ri, c) = cv - t; }
+  __device__ __forceinline__ int4 ec4(int c) const { return __ldcg(reinterpret_cast<const int4*>(EX + c)); }
+  __device__ __forceinline__ void store4(int ri, int c, int n4, const double* cv, const double* t) const {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (e < n4) *at(ri, c + e) = cv[e] - t[e];
+  }
 };
 
 // L_bb and L_bb^{-1} of the nbk x nbk block in sm.D by the CTA's first eight warps: lane = row, warp v holds columns
@@ -272,7 +280,8 @@ __global__ void __launch_bounds__(kCT, 1)
   __shared__ uint64_t full[kCStages], empty[kCStages], accf[2], acce[2], drain;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
-  __shared__ int bad, item_s, EXB[kNB];
+  __shared__ int bad, item_s;
+  __shared__ __align__(16) int EXB[kNB];
   __shared__ double red[kCT / 32];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int rank = (int)cl_rank(), C = (int)cl_size(), cluster = blockIdx.x / C;

@@ -12,8 +12,8 @@
 //
 // What bounds it: the staging of the digits for wide fronts, the latency of the 32-column steps for narrow ones; two
 // 128-column tiles per item share that latency when there are enough items.  Measured (before: all fronts on the FP64
-// pipe by trsm_kernel): 64 uneven 3D heat subdomains 78.8 ms -> 14.8 + 5.1 (small fronts) + 1.0 (digits of L), 27
-// elasticity subdomains of 12^3 58.6 -> 10.2 + 1.2 + 0.7.
+// pipe by trsm_kernel): 64 uneven 3D heat subdomains 78.8 ms -> 13.7 + 4.9 (small fronts) + 1.0 (digits of L), 27
+// elasticity subdomains of 12^3 58.6 -> 10.0 + 1.3 + 0.7.
 #include <algorithm>
 #include <cuda_bf16.h>
 
@@ -113,10 +113,6 @@ __global__ void __launch_bounds__(256) dig_l_kernel(DevPlan P, const int4* items
               ex + b.ownp, warp, 8);
 }
 
-__device__ __forceinline__ void ld4(const double* p, double* v) {
-  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "l"(p) : "memory");
-  asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "l"(p + 2) : "memory");
-}
 
 // X^T_b = A L_bb^{-T}: rows of the item, the ncol <= 32 columns of the step
 struct SolveJob {
@@ -138,8 +134,17 @@ struct SolveJob {
   __device__ __forceinline__ int load(int ri, int cb, double (&)[16]) const {
     return ri < n ? min(16, ncol - cb) : 0;
   }
-  __device__ __forceinline__ int ec(int c) const { return __ldg(EXB + c); }
-  __device__ __forceinline__ void store(int ri, int c, double, double t) const { X[(int64_t)ri * wp + c] = t; }
+  __device__ __forceinline__ int4 ec4(int c) const { return __ldg(reinterpret_cast<const int4*>(EXB + c)); }
+  __device__ __forceinline__ void store4(int ri, int c, int n4, const double*, const double* t) const {
+    double* p = X + (int64_t)ri * wp + c;
+    if (n4 == 4) {
+      st4(p, t[0], t[1], t[2], t[3]);
+      return;
+    }
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      if (e < n4) p[e] = t[e];
+  }
 };
 
 // C -= X^T L^T: column c of the padded B rows is own column c (c < own) of X, or column c - ownp (< nbot) of the update
@@ -180,20 +185,28 @@ struct RectJob {
     }
     return nc;
   }
-  __device__ __forceinline__ int ec(int c) const { return __ldg(EXB + c); }
-  __device__ __forceinline__ void store(int ri, int c, double cv, double t) const { *at(ri, c) = cv - t; }
+  __device__ __forceinline__ int4 ec4(int c) const { return __ldg(reinterpret_cast<const int4*>(EXB + c)); }
+  __device__ __forceinline__ void store4(int ri, int c, int n4, const double* cv, const double* t) const {
+    double* p = at(ri, c);
+    if (n4 == 4) {
+      st4(p, cv[0] - t[0], cv[1] - t[1], cv[2] - t[2], cv[3] - t[3]);
+      return;
+    }
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      if (e < n4) p[e] = cv[e] - t[e];
+  }
 };
 
 // items: (subdomain, first sorted column), cw columns each (128 or 256)
 __global__ void __launch_bounds__(kCT, 1)
     trsm_oz_kernel(DevPlan P, const int2* items, int nitems, int cw, int* queue, const char* LD, const double* hand,
-                   double* X, double* ws, int64_t ws_stride, int64_t front_sz, char* scratch, int64_t scratch_stride,
-                   int* status) {
+                   double* X, double* ws, int64_t ws_stride, char* scratch, int64_t scratch_stride, int* status) {
   extern __shared__ uint8_t xo_raw[];
   __shared__ uint64_t full[kCStages], empty[kCStages], accf[2], acce[2], drain;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
-  const int tid = threadIdx.x, warp = tid / 32;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
                  "r"(512));
@@ -224,8 +237,7 @@ __global__ void __launch_bounds__(kCT, 1)
   st.drain = &drain;
   st.abort = &abort_s;
   st.tmem = tmem_s;
-  double* W = ws + (int64_t)blockIdx.x * ws_stride;
-  double* stack = W + front_sz;
+  double* stack = ws + (int64_t)blockIdx.x * ws_stride;
   char* SL = scratch + (int64_t)blockIdx.x * scratch_stride;
   char* S2 = SL + (int64_t)cw * 512;
   int* EX1 = reinterpret_cast<int*>(SL + (int64_t)cw * 1024);
@@ -247,8 +259,9 @@ __global__ void __launch_bounds__(kCT, 1)
       const int J = je - jb;
       if (J <= 0) continue;
       double* Xs = Xsub + P.Xofs[bs] + (int64_t)(jb - P.jb[bs]) * wp;
-      for (int64_t idx = tid; idx < (int64_t)wp * J; idx += kCT) Xs[idx] = 0.0;
-      for (int64_t idx = tid; idx < (int64_t)rp * J; idx += kCT) W[idx] = 0.0;
+      double* W = stack + P.tx_ofs[gs] * cw;  // formed where the parent reads it
+      for (int64_t idx = 4 * tid; idx < (int64_t)wp * J; idx += 4 * kCT) st4(Xs + idx, 0.0, 0.0, 0.0, 0.0);
+      for (int64_t idx = 4 * tid; idx < (int64_t)rp * J; idx += 4 * kCT) st4(W + idx, 0.0, 0.0, 0.0, 0.0);
       __syncthreads();
       for (int j = jo + tid; j < je; j += kCT) Xs[(int64_t)(j - jb) * wp + P.spos[S.col0 + j] - c0] = P.qsign[S.qcol + j];
       for (int c = P.ch_off[gs]; c < P.ch_off[gs + 1]; ++c) {
@@ -261,27 +274,28 @@ __global__ void __launch_bounds__(kCT, 1)
         const int ldc = big ? (rc + 7) & ~7 : rc;
         const double* U = big ? stack + P.tx_ofs[gc] * cw : hand + S.th + P.th_ofs[bc] + (int64_t)(jbc - P.jb[bc]) * rc;
         const int* rl = P.rel + P.rel_off[gc];
-        // children own disjoint column ranges; four elements per thread and step, their loads first
-        const int64_t n = (int64_t)rc * Jc;
-        for (int64_t base = tid; base < n; base += 4 * kCT) {
-          double* dst[4];
-          double v[4], cur[4];
+        // children own disjoint column ranges; a column per warp, kFly entries per lane in flight
+        constexpr int kFly = 8;
+        for (int col = warp; col < Jc; col += kCT / 32) {
+          double* Xc = Xs + (int64_t)(coff + col) * wp;
+          double* Wc = W + (int64_t)(coff + col) * rp - w;
+          const double* Uc = U + (int64_t)col * ldc;
+          for (int a0 = lane; a0 < rc; a0 += 32 * kFly) {
+            double* dst[kFly];
+            double v[kFly], cur[kFly];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int64_t idx = base + (int64_t)u * kCT;
-            dst[u] = nullptr;
-            if (idx < n) {
-              const int col = (int)(idx / rc), a2 = (int)(idx - (int64_t)col * rc);
-              const int ra = rl[a2];
-              v[u] = U[(int64_t)col * ldc + a2];
-              dst[u] = ra < w ? Xs + (int64_t)(coff + col) * wp + ra : W + (int64_t)(coff + col) * rp + (ra - w);
+            for (int u = 0; u < kFly; ++u) {
+              const int a2 = a0 + 32 * u;
+              const int ra = a2 < rc ? rl[a2] : 0;
+              v[u] = a2 < rc ? __ldcg(Uc + a2) : 0.0;
+              dst[u] = a2 < rc ? (ra < w ? Xc : Wc) + ra : nullptr;
             }
+#pragma unroll
+            for (int u = 0; u < kFly; ++u) cur[u] = dst[u] ? __ldcg(dst[u]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < kFly; ++u)
+              if (dst[u]) *dst[u] = cur[u] + v[u];
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) cur[u] = dst[u] ? __ldcg(dst[u]) : 0.0;
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (dst[u]) *dst[u] = cur[u] + v[u];
         }
       }
       __syncthreads();
@@ -314,10 +328,6 @@ __global__ void __launch_bounds__(kCT, 1)
         }
         ld += b.end;
       }
-      if (P.sn_parent[gs] >= 0) {
-        double* dst = stack + P.tx_ofs[gs] * cw;
-        for (int64_t idx = tid; idx < (int64_t)rp * J; idx += kCT) dst[idx] = __ldcg(W + idx);
-      }
       __syncthreads();
     }
   }
@@ -341,13 +351,12 @@ void launch_dig_l(const DevPlan& P, const int4* items, int nitems, void* LD, cud
 }
 
 void launch_trsm_oz(const DevPlan& P, const int2* items, int nitems, int cw, int* queue, const void* LD,
-                    const double* hand, double* X, double* ws, int64_t ws_stride, int64_t front_sz, void* scratch,
+                    const double* hand, double* X, double* ws, int64_t ws_stride, void* scratch,
                     int64_t scratch_stride, int grid, int* status, cudaStream_t st) {
   if (nitems <= 0) return;
   cudaFuncSetAttribute(trsm_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kXDyn);
   trsm_oz_kernel<<<std::min(grid, nitems), kCT, kXDyn, st>>>(P, items, nitems, cw, queue, (const char*)LD, hand, X, ws,
-                                                            ws_stride, front_sz, (char*)scratch, scratch_stride,
-                                                            status);
+                                                            ws_stride, (char*)scratch, scratch_stride, status);
 }
 
 }  // namespace feti

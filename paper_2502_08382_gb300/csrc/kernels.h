@@ -66,7 +66,7 @@ int64_t trsm_oz_block_bytes(int w, int r, int kB);
 int64_t trsm_oz_scratch(int cw);
 void launch_dig_l(const DevPlan& P, const int4* items, int nitems, void* LD, cudaStream_t st);
 void launch_trsm_oz(const DevPlan& P, const int2* items, int nitems, int cw, int* queue, const void* LD,
-                    const double* hand, double* X, double* ws, int64_t ws_stride, int64_t front_sz, void* scratch,
+                    const double* hand, double* X, double* ws, int64_t ws_stride, void* scratch,
                     int64_t scratch_stride, int grid, int* status, cudaStream_t st);
 // chunks of the tile whose contributing supernodes have np[0 .. n) 8-row pieces (the loaders' batching)
 int syrk_oz_chunks(const int* np, int n);

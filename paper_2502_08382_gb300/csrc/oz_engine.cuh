@@ -37,8 +37,20 @@ struct CtState {
   uint32_t units;     // 32-column units multiplied so far (accumulator set and phase)
 };
 
-// Eight entries of a row (columns k .. k + 7, zero from K on): of a column-major matrix, and of a row-major one whose
-// rows are 16-byte aligned and padded to a multiple of 8.
+// Four doubles of a row, 32-byte aligned.  A lane has its own row here, so every instruction of a warp meets 32 lines
+// whatever its width: the widest accesses cost the fewest.  (Written and read by the same CTA: plain loads.)
+__device__ __forceinline__ void ld4(const double* p, double* v) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st4(double* p, double a, double b, double c, double d) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+}
+
+// Eight entries of a row (columns k .. k + 7, zero from K on): of a column-major matrix, and of a row-major one of this
+// CTA whose rows are 32-byte aligned and padded to a multiple of 8.
 struct ColMajor {
   const double* A;
   int64_t ld;
@@ -51,13 +63,13 @@ struct RowMajor {
   const double* A;
   int64_t ld;
   __device__ __forceinline__ void get(int i, int k, int K, double (&v)[8]) const {
-    const double2* p = reinterpret_cast<const double2*>(A + (int64_t)i * ld + k);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const double2 x = k < K ? __ldcg(p + e) : make_double2(0.0, 0.0);
-      v[2 * e] = k + 2 * e < K ? x.x : 0.0;
-      v[2 * e + 1] = k + 2 * e + 1 < K ? x.y : 0.0;
+    const double* p = A + (int64_t)i * ld + k;
+    if (k < K) {
+      ld4(p, v);
+      ld4(p + 4, v + 4);
     }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = k + e < K ? v[e] : 0.0;
   }
 };
 
@@ -108,7 +120,8 @@ __device__ __forceinline__ void dig_rows(const SRC& A, int n, int K, int r0, int
 //   nck           32-deep chunks of K
 //   tile(t, tm, tn)
 //   a(tm, c), b(tn, c)   the operands' first digit of chunk c; digA, digB bytes between digits
-//   begin(tm, row), load(row, unit column, C[16]), exponents er() and ec(column), store(row, column, index, C, product)
+//   begin(row)    the row's exponent; load(row, unit column, C[16]) valid columns; ec4(column) four exponents
+//   store4(row, column, count, C, product)   up to four columns (column a multiple of 4)
 template <class JOB>
 __device__ __forceinline__ void dig_product(CtState& st, JOB& job, int first, int step, int ntile) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -207,6 +220,7 @@ __device__ __forceinline__ void dig_product(CtState& st, JOB& job, int first, in
 #pragma unroll
         for (int e0 = 0; e0 < 16; e0 += 4) {
           uint32_t a[4][kDig];
+          const int4 ej4 = e0 < nc ? job.ec4(cb + e0) : make_int4(0, 0, 0, 0);
 #pragma unroll
           for (int d = 0; d < kDig; ++d) tmem_ld4(t0 + d * kCH + e0, a[0][d], a[1][d], a[2][d], a[3][d]);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -215,18 +229,18 @@ __device__ __forceinline__ void dig_product(CtState& st, JOB& job, int first, in
             __syncwarp();
             if (lane == 0) mbar_arrive(&st.acce[set]);
           }
+          double t[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const int c = e0 + e;
-            if (c < nc) {
+            if (e0 + e < nc) {
               long long hi = 0, lo = 0;
               dig_sum(a[e], hi, lo);
-              const int ej = job.ec(cb + c);
-              double t = dig_value(hi, lo, ei + ej - 68);
-              if (ei == kExpBad || ej == kExpBad) t = __longlong_as_double(0x7FF8000000000000LL);
-              job.store(ri, cb + c, cv[c], t);
+              const int ej = e == 0 ? ej4.x : e == 1 ? ej4.y : e == 2 ? ej4.z : ej4.w;
+              t[e] = dig_value(hi, lo, ei + ej - 68);
+              if (ei == kExpBad || ej == kExpBad) t[e] = __longlong_as_double(0x7FF8000000000000LL);
             }
           }
+          if (e0 < nc) job.store4(ri, cb + e0, min(4, nc - e0), cv + e0, t);
         }
       }
     }

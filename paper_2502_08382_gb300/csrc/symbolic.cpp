@@ -719,32 +719,20 @@ void plan_tasks(PatternPlan& P, double target, int big_f, double target_small) {
   // the large set share one: a maximal subtree of them hands its root's block over, so little of it is ever live.
   P.sub_stack = P.big_stack = 0;
   P.sub_flops = 0;
-  std::vector<std::vector<std::pair<int64_t, int>>> live(P.ntask + 1);  // (offset, supernode), ascending
+  std::vector<BlockPlaces> live(P.ntask + 1);
+  auto place = [&](int s) -> BlockPlaces& { return live[P.sn_big[s] ? P.sn_task[s] : P.ntask]; };
   for (int s = 0; s < ns; ++s) {
-    auto& lv = live[P.sn_big[s] ? P.sn_task[s] : P.ntask];
     const int64_t rr = (int64_t)P.sn_r[s] * P.sn_r[s];
     if (!P.sn_big[s]) P.sub_flops += own[s];
     P.upd_stack_ofs[s] = 0;
     const bool own_block = !P.sn_small[s] && P.sn_hoff[s] < 0 && P.sn_parent[s] >= 0 && rr > 0;
     if (own_block) {
-      int64_t at = 0;
-      size_t k = 0;
-      for (; k < lv.size() && lv[k].first < at + rr; ++k)
-        at = lv[k].first + (int64_t)P.sn_r[lv[k].second] * P.sn_r[lv[k].second];
+      const int64_t at = place(s).take(s, rr);
       P.upd_stack_ofs[s] = at;
-      lv.insert(lv.begin() + k, {at, s});
       int64_t& peak = P.sn_big[s] ? P.big_stack : P.sub_stack;
       peak = std::max(peak, at + rr);
     }
-    for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) {
-      const int c = P.ch_list[k];
-      auto& lc = live[P.sn_big[c] ? P.sn_task[c] : P.ntask];
-      for (size_t q = 0; q < lc.size(); ++q)
-        if (lc[q].second == c) {
-          lc.erase(lc.begin() + q);
-          break;
-        }
-    }
+    for (int k = P.ch_off[s]; k < P.ch_off[s + 1]; ++k) place(P.ch_list[k]).release(P.ch_list[k]);
   }
 }
 

@@ -83,6 +83,29 @@ struct PatternPlan {
 // large set.  Also lays the update blocks out anew (upd_stack_ofs).
 void plan_tasks(PatternPlan& P, double target, int big_f = 0, double target_small = 0);
 
+// First-fit places for blocks with a lifetime (take .. release), in one linear workspace.
+struct BlockPlaces {
+  struct Block {
+    int64_t at, size;
+    int id;
+  };
+  std::vector<Block> live;  // ascending, disjoint
+  int64_t take(int id, int64_t size) {
+    int64_t at = 0;
+    size_t k = 0;
+    for (; k < live.size() && live[k].at < at + size; ++k) at = live[k].at + live[k].size;
+    live.insert(live.begin() + k, {at, size, id});
+    return at;
+  }
+  void release(int id) {
+    for (size_t k = 0; k < live.size(); ++k)
+      if (live[k].id == id) {
+        live.erase(live.begin() + k);
+        return;
+      }
+  }
+};
+
 struct BPlan {
   int m = 0, m_pad = 0, nb = 0;
   std::vector<int> colperm;  // sorted column j -> original B row
