@@ -8,6 +8,7 @@
 #include <cstring>
 #include <map>
 #include <numeric>
+#include <queue>
 #include <stdexcept>
 #include <thread>
 #include <unordered_map>
@@ -427,6 +428,41 @@ void build(feti_ctx* c) {
     double small = 0;
     for (auto& sh : c->subs) small += c->pats[sh.pat].sub_flops;
     for (auto& P : c->pats) plan_tasks(P, target, big_f, small / (4.0 * slots));
+    // CTAs per subdomain of the implicit solves, where there is at most one subdomain per SM: the cluster size with
+    // the shortest schedule (largest subdomain first) by the plans' estimates.  Milliseconds per application with
+    // 1 / 2 / 4 / 8: 27 elasticity subdomains of 12^3 2.89 / 1.73 / 1.23 / 1.94, 64 of them 2.97 / 1.79 / 2.44 / 5.0;
+    // 125 uneven 3D heat subdomains 5.26 / 3.12 / 2.13 / 3.6, 8 of 20^3 2.53 / 1.49 / 1.06 / 0.84; 64 2D heat subdomains
+    // of 64^2 0.77 / 0.50 / 0.76 / 1.5, 64 3D ones of 6^3 0.146 / 0.141 / 0.25 / 0.6
+    int nmax = 0, maxf = 0;
+    for (auto& sh : c->subs) nmax = std::max(nmax, sh.n);
+    for (auto& P : c->pats) maxf = std::max(maxf, P.max_f);
+    c->impl_wide = implicit_wide(ns, nsm, nmax, maxf);
+    if (c->impl_wide) {
+      double best = 0;
+      for (int C = 1; C <= 8; C *= 2) {
+        const int ncl = C == 1 ? nsm : implicit_clusters(implicit_smem(nmax, maxf, true), C);
+        if (ncl < 1) break;
+        std::vector<SolveSplit> sp;
+        for (auto& P : c->pats) sp.push_back(plan_solve_split(P, C));
+        std::vector<double> cost;
+        for (auto& sh : c->subs) cost.push_back(sp[sh.pat].cost);
+        std::sort(cost.rbegin(), cost.rend());
+        std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+        for (int k = 0; k < ncl; ++k) load.push(0.0);
+        double t = 0;
+        for (double x : cost) {
+          const double y = load.top() + x;
+          load.pop();
+          load.push(y);
+          t = std::max(t, y);
+        }
+        if (C == 1 || t < 0.95 * best) {
+          best = t;
+          c->impl_cluster = C;
+          c->solve_splits = std::move(sp);
+        }
+      }
+    }
   }
   c->stats.t_symbolic_ms = std::chrono::duration<double, std::milli>(clk::now() - t0).count();
   c->stats.npatterns = (int)c->pats.size();
@@ -445,7 +481,8 @@ void build(feti_ctx* c) {
   std::vector<int64_t> lt_ofs;  // the adjoint's backward solve: digits of L^T (kern_bsolve_oz.cu)
   c->pat_lt.assign(c->pats.size(), 0);
   std::vector<int64_t> ld_ofs, tx_ofs, th_ofs, pat_ld(c->pats.size(), 0), bp_th(c->bps.size(), 0);
-  std::vector<int> lvl_off, lvl_sn, pat_lvl0(c->pats.size());
+  std::vector<int> lvl_off, lvl_sn, pat_lvl0(c->pats.size()), pat_pc0(c->pats.size());
+  std::vector<int4> pieces;
   int64_t max_usize = 0;
   std::vector<int> pat_sn0(c->pats.size());
   std::vector<int64_t> pat_diag0(c->pats.size());
@@ -506,6 +543,16 @@ void build(feti_ctx* c) {
       const int b0 = (int)lvl_sn.size();
       for (int l = 0; l <= P.nlev; ++l) lvl_off.push_back(b0 + P.lvl_off[l]);
       lvl_sn.insert(lvl_sn.end(), P.lvl_sn.begin(), P.lvl_sn.end());
+      pat_pc0[p] = (int)pieces.size();
+      if (c->impl_cluster > 1) {
+        const SolveSplit& sp = c->solve_splits[p];
+        for (int k = 0; k <= c->impl_cluster; ++k) {
+          const int b1 = (int)lvl_sn.size();
+          for (int o : sp.off[k]) lvl_off.push_back(b1 + o);
+          lvl_sn.insert(lvl_sn.end(), sp.own[k].begin(), sp.own[k].end());
+        }
+        for (auto& q : sp.pieces) pieces.push_back(make_int4(q.c0, q.c1, q.rank, 0));
+      }
     }
     max_usize = std::max(max_usize, P.usize);
     c->impl_maxf = std::max(c->impl_maxf, P.max_f);
@@ -602,6 +649,8 @@ void build(feti_ctx* c) {
     I.vr = B.nb > 0 ? s.m - kT * (B.nb - 1) : 0;
     I.nlev = P.nlev;
     I.lvl0 = pat_lvl0[s.pat];
+    I.pc0 = pat_pc0[s.pat];
+    I.npc = c->impl_cluster > 1 ? (int)c->solve_splits[s.pat].pieces.size() : 0;
     I.fix0 = fixo;
     I.alpha0 = alo;
     I.kmapb = 0;
@@ -904,6 +953,7 @@ void build(feti_ctx* c) {
   D.diag_src = upload(c, diag_src);
   D.upd_ofs = upload(c, upd_ofs);
   D.lvl_off = upload(c, lvl_off);
+  D.pieces = upload(c, pieces);
   D.lvl_sn = upload(c, lvl_sn);
   D.uofs = upload(c, uofs);
   D.sn_small = upload(c, sn_small);
@@ -1146,11 +1196,12 @@ void build(feti_ctx* c) {
     CK(cudaMallocHost((void**)&c->h_ctrl, 2 * sizeof(PcgCtrl)));
     launch_build_G(D, c->d_colsub, qo, c->d_R, c->d_G6, c->st);
     CK(cudaGetLastError());
-    c->impl_wide = implicit_wide(ns, c->nsm, c->nmax, c->impl_maxf);
     size_t sm = implicit_smem(c->nmax, c->impl_maxf, c->impl_wide);
     if (sm > 227 * 1024) throw ArgError("subdomain too large for the shared-memory implicit solve");
     c->impl_smem = sm;
-    c->grid_impl = std::min(ns, c->nsm * implicit_occupancy(sm, c->impl_wide));
+    c->grid_impl =
+        c->impl_wide ? std::min(ns, c->impl_cluster > 1 ? implicit_clusters(sm, c->impl_cluster) : c->nsm)
+                     : std::min(ns, c->nsm * implicit_occupancy(sm));
     c->ustride = std::max<int64_t>((max_usize + 31) / 32 * 32, 32);
     c->d_uws = (double*)dalloc(c, (size_t)c->grid_impl * c->ustride * 8);
   }

@@ -45,7 +45,7 @@ void implicit_apply(feti_ctx* c, const double* p, double* q) {
     CKS(cudaEventRecord(ev.a, c->st));
   }
   queue_reset(c, 32);
-  launch_implicit(0, c->impl_wide, c->P, c->d_impl_order, c->nsub, c->d_queue + 32, p, c->d_f, c->d_qi, nullptr, c->d_uws,
+  launch_implicit(0, c->impl_cluster, c->P, c->d_impl_order, c->nsub, c->d_queue + 32, p, c->d_f, c->d_qi, nullptr, c->d_uws,
                   c->ustride, c->nmax, c->impl_maxf, c->grid_impl,
                   c->impl_smem, c->st);
   launch_gather_lambda(c->d_c0, c->d_c1, c->nlam, c->d_qi, q, c->st);
@@ -262,7 +262,7 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
     }
     // d = B K^+ f - c
     queue_reset(ctx, 32);
-    launch_implicit(1, ctx->impl_wide, ctx->P, ctx->d_impl_order, ctx->nsub, ctx->d_queue + 32, nullptr, ctx->d_f, ctx->d_qi,
+    launch_implicit(1, ctx->impl_cluster, ctx->P, ctx->d_impl_order, ctx->nsub, ctx->d_queue + 32, nullptr, ctx->d_f, ctx->d_qi,
                     nullptr, ctx->d_uws, ctx->ustride, ctx->nmax, ctx->impl_maxf, ctx->grid_impl, ctx->impl_smem, st);
     launch_gather_minus_c(ctx->d_c0, ctx->d_c1, n, ctx->d_qi, ctx->d_c, d, st);
     // control block; p = 0 so that the first p = w + beta p (beta = 0) is w_0
@@ -389,7 +389,7 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
     // u = K^+ (f - B^T lambda) + R alpha  (eq. 5)
     if (u_dev) {
       queue_reset(ctx, 32);
-      launch_implicit(2, ctx->impl_wide, ctx->P, ctx->d_impl_order, ctx->nsub, ctx->d_queue + 32, lam, ctx->d_f, nullptr, u_dev,
+      launch_implicit(2, ctx->impl_cluster, ctx->P, ctx->d_impl_order, ctx->nsub, ctx->d_queue + 32, lam, ctx->d_f, nullptr, u_dev,
                       ctx->d_uws, ctx->ustride, ctx->nmax, ctx->impl_maxf, ctx->grid_impl, ctx->impl_smem, st);
       if (D > 0) launch_add_Ralpha(ctx->P, ctx->d_dofsub, ctx->ndof, ctx->d_R, alpha, u_dev, st);
     }

@@ -27,7 +27,9 @@ struct SubInfo {
   int nb2;           // 128-wide blocks
   int vr;            // rows of the last block row (m - kT (nb - 1)); that row stores only these
   int nlev;          // levels of the supernodal tree
-  int lvl0;          // pattern level-offset base (lvl_off, nlev + 1 entries)
+  int lvl0;          // pattern level-offset base (lvl_off, nlev + 1 entries; then one such list per rank of the
+                     // implicit solve's cluster and one for the supernodes that its ranks share)
+  int pc0, npc;      // the ranks' subtrees (pieces)
   int64_t kmapb;     // base of this pattern's kmap entries (kmap_off values are absolute)
   int64_t diag0;     // diag_src base
   int64_t Kval;      // subdomain K values base
@@ -67,6 +69,7 @@ struct DevPlan {
   const int* diag_src;       // relative to the subdomain's K values
   const int64_t* upd_ofs;    // [sn] update block in the CTA's (cluster's) workspace, disjoint from its children's
   const int* lvl_off;        // [lvl0 + l] absolute offsets into lvl_sn
+  const int4* pieces;        // [pc0 + k] columns [x, y) belong to rank z of the implicit solve's cluster
   const int* lvl_sn;         // local supernode ids, level by level
   const int64_t* uofs;       // [sn] update-vector offset of the supernode (relative to the CTA workspace)
   const int* sn_small;       // [sn] 1: small-subtree supernode (warp-factored front)

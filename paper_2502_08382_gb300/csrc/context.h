@@ -46,6 +46,7 @@ struct feti_ctx {
   std::vector<double> c_host;
   std::vector<feti::SubHost> subs;
   std::vector<feti::PatternPlan> pats;
+  std::vector<feti::SolveSplit> solve_splits;  // per pattern, for impl_cluster CTAs
   std::vector<feti::BPlan> bps;
   std::vector<int> bp_pat;
   std::vector<feti::SubInfo> info;
@@ -141,7 +142,8 @@ struct feti_ctx {
   int grid_chol = 0, grid_trsm = 0, grid_impl = 0;
   int grid_trsm32 = 0;  // CTAs of the mixed-precision TRSM (its occupancy with the tensor-core stage ring)
   size_t impl_smem = 0;
-  bool impl_wide = false;   // one 1024-thread CTA per subdomain
+  bool impl_wide = false;   // 1024-thread CTAs,
+  int impl_cluster = 0;     // this many per subdomain (0: 256-thread ones)
   double* d_uws = nullptr;  // update vectors of the implicit solve, ustride doubles per CTA
   int64_t ustride = 0;
   int impl_maxf = 0;

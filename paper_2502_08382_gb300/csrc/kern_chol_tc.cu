@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include "chol_common.cuh"
+#include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.h"
 #include "oz_engine.cuh"
@@ -46,21 +47,10 @@ struct PivotSmem {
 };
 static_assert(sizeof(PivotSmem) <= kCStage, "the pivot's buffers alias the stage ring");
 
-__device__ __forceinline__ uint32_t cl_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cl_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
 // barrier of all threads of the cluster; orders their global accesses (generic and bulk copies)
 __device__ __forceinline__ void cl_sync() {
-  __syncwarp();
   asm volatile("fence.proxy.async.global;" ::: "memory");
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cl_barrier();
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 // The panel: Out[row, j] = (A L_bb^{-T})[row, j] for j < ncol to the front's columns kb + j, rows i0 + row.
@@ -341,11 +331,7 @@ __global__ void __launch_bounds__(kCT, 1)
           it = -1;
         }
       }
-      for (int c = 0; c < C; ++c)
-        asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.s32 [a], %2;\n\t}" ::"r"(
-                         smem_u32(&item_s)),
-                     "r"(c), "r"(it)
-                     : "memory");
+      for (int c = 0; c < C; ++c) cl_store(&item_s, c, it);
     }
     if (tid == 0) bad = 0;
     cl_sync();

@@ -7,6 +7,7 @@
 //    blocked Cholesky and explicit inverse built from 64 x 64 FP64 tile GEMMs;
 //  * the projector P = I - G (G^T G)^{-1} G^T and the PCPG vector updates of
 //    Algorithm 1 (M = I), with dot products reduced in a fixed order.
+#include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -25,6 +26,13 @@ __device__ __forceinline__ int pop_item_s(int* queue) {
 
 constexpr int kWF = 128;  // largest front handled by one warp (needs w <= 32)
 
+// Entry of a child's update vector: another CTA of the cluster may have written it (CL), so not from L1 then.
+template <bool CL>
+__device__ __forceinline__ double ld_upd(const double* p) {
+  if constexpr (CL) return __ldcg(p);
+  else return *p;
+}
+
 // The implicit solves use L in unit-lower form, L = Lu D (D = diag of L),
 // written by unit_scale_kernel after the assembly: the panel holds Lu below
 // the diagonal and zeros on and above it, and d2[j] = 1 / L_jj^2.  Then
@@ -35,6 +43,7 @@ constexpr int kWF = 128;  // largest front handled by one warp (needs w <= 32)
 // l keeps the front entries l + 32 q in registers; per column j, z_j comes
 // from lane j and every front row takes its update in one FMA (the zeros of
 // Lu on and above the diagonal leave the rows <= j unchanged).
+template <bool CL>
 __device__ __forceinline__ void fwd_warp(const DevPlan& P, const SubInfo& S, int gs, const double* d2,
                                          double* ubuf, double* y, double* v, int lane) {
   const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f_ = w + r;
@@ -46,7 +55,7 @@ __device__ __forceinline__ void fwd_warp(const DevPlan& P, const SubInfo& S, int
     const int rc = P.sn_r[gc];
     const double* U = ubuf + P.uofs[gc];
     const int* rl = P.rel + P.rel_off[gc];
-    for (int k = lane; k < rc; k += 32) v[rl[k]] += U[k];
+    for (int k = lane; k < rc; k += 32) v[rl[k]] += ld_upd<CL>(U + k);
     __syncwarp();
   }
   const int nq = (f_ + 31) / 32;  // warp-uniform
@@ -142,7 +151,7 @@ __device__ __forceinline__ void cta_sync(int team) {
 // 256 threads: forward step of a large supernode on the shared front vector.
 // 32 x 32 unit-lower diagonal blocks are staged in shared memory and solved
 // by warp 0; all threads apply the block's columns to the rest of the front.
-template <bool TEAM = false>
+template <bool TEAM = false, bool CL = false>
 __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int gs, const double* d2,
                                         double* ubuf, double* y, double* sf, double (*sm_blk)[kW + 1], int tid, int team = 0) {
   const int warp = tid / 32, lane = tid % 32;
@@ -155,7 +164,7 @@ __device__ __forceinline__ void fwd_cta(const DevPlan& P, const SubInfo& S, int 
     const int rc = P.sn_r[gc];
     const double* U = ubuf + P.uofs[gc];
     const int* rl = P.rel + P.rel_off[gc];
-    for (int k = tid; k < rc; k += kThreads) sf[rl[k]] += U[k];
+    for (int k = tid; k < rc; k += kThreads) sf[rl[k]] += ld_upd<CL>(U + k);
     cta_sync<TEAM>(team);
   }
   for (int kb = 0; kb < w; kb += kW) {
@@ -314,9 +323,14 @@ __device__ __forceinline__ void bwd_cta(const DevPlan& P, const SubInfo& S, int 
 // instructions are the scarce resource (64 clocks of a scheduler each): dot products run on eight lanes per column,
 // which needs three additions per four columns to reduce.  Supernodes of moderate size (kTeamF, kTeamW) spend most of
 // their time in chains of index loads, so the wide CTA's four teams of 256 threads take one each, side by side.
-// Measured per application (before: 256 threads per subdomain): 64 elasticity subdomains of 12^3 5.7 -> 2.7 ms, 125
-// uneven 3D heat subdomains 9.0 -> 4.75 ms (its largest subdomain sets it: two sweeps of 3.5 M entries on one SM's
-// FP64 pipe take 1.8 ms).
+// A cluster of 1 to 8 wide CTAs takes a subdomain: with fewer subdomains than SMs, or uneven ones, one SM's FP64 pipe
+// under the largest subdomain sets the time.  Each CTA has subtrees of its own (plan_solve_split), for which it needs
+// none of the others; the few supernodes above them are dealt out level by level, update vectors go through global
+// memory, and the columns that a shared supernode solves are stored into every CTA's vector.  Every front is computed as
+// by one CTA, so the results do not depend on the cluster size.
+// Measured per application (256 threads per subdomain -> one wide CTA -> the cluster of the dispatch's choice): 64
+// elasticity subdomains of 12^3 5.7 -> 2.7 -> 1.8 ms (2 CTAs), 27 of them 2.9 -> 1.2 (4), 125 uneven 3D heat subdomains
+// 9.0 -> 4.75 -> 2.1 ms (4; its largest subdomain's two sweeps of 3.5 M entries are 1.8 ms of one SM's FP64 pipe).
 constexpr int kWide = 1024;
 constexpr int kTeamF = 512, kTeamW = 64;  // largest front and width a team takes
 constexpr int kWR = 512;  // rows of an update pass (two per thread of a group)
@@ -338,6 +352,7 @@ __device__ __forceinline__ void wide_stage(const double* Ls, int f_, int kb, int
   }
 }
 
+template <bool CL>
 __device__ __forceinline__ void fwd_wide(const DevPlan& P, const SubInfo& S, int gs, const double* d2, double* ubuf,
                                          double* y, double* sf, double* part, WideSmem& ws, int tid) {
   const int warp = tid / 32, lane = tid % 32, g = tid / 256, t = tid % 256;
@@ -351,7 +366,7 @@ __device__ __forceinline__ void fwd_wide(const DevPlan& P, const SubInfo& S, int
     const int rc = P.sn_r[gc];
     const double* U = ubuf + P.uofs[gc];
     const int* rl = P.rel + P.rel_off[gc];
-    for (int k = tid; k < rc; k += kWide) sf[rl[k]] += U[k];
+    for (int k = tid; k < rc; k += kWide) sf[rl[k]] += ld_upd<CL>(U + k);
     __syncthreads();
   }
   // the own rows, block by block
@@ -532,11 +547,22 @@ __global__ void __launch_bounds__(128) inv_block_kernel(DevPlan P, int nsub) {
   }
 }
 
+// The rank of the cluster that writes column col of the solution: its piece's, 0 for the shared ones.
+__device__ __forceinline__ int col_owner(const DevPlan& P, const SubInfo& S, int col) {
+  int owner = 0;
+  for (int k = S.pc0; k < S.pc0 + S.npc; ++k) {
+    const int4 pc = P.pieces[k];
+    if (col >= pc.x && col < pc.y) owner = pc.z;
+  }
+  return owner;
+}
+
 // MODE 0: qi = B L^-T L^-1 P B^T p        (implicit apply, eq. 11)
 // MODE 1: qi = B K_reg^{-1} f             (d = B K^+ f - c, eq. 7)
 // MODE 2: u  = K_reg^{-1} (f - B^T lambda) (eq. 5 without R alpha)
-// NT: threads of the CTA (256, or the wide 1024).
-template <int MODE, int NT>
+// NT: threads of the CTA (256, or the wide 1024); CL: the wide CTAs of a cluster share a subdomain (an instantiation of
+// its own: the registers that it takes cost the small problems of single CTAs 15 us of 75).
+template <int MODE, int NT, bool CL>
 __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
     implicit_kernel(DevPlan P, const int* order, int nsub, int* queue, const double* p, const double* f, double* qi,
                     double* u, double* uws, int64_t ustride, int nmax, int maxf) {
@@ -549,9 +575,23 @@ __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
   double* sfront = y + nmax;
   double* wbuf = sfront + maxf;
   WideSmem& wsm = *reinterpret_cast<WideSmem*>(wbuf + NT / 32 * kWF);  // NT == kWide
-  double* ubuf = uws + (int64_t)blockIdx.x * ustride;
+  static_assert(!CL || NT == kWide, "clusters of wide CTAs");
+  const int rank = CL ? (int)cl_rank() : 0, C = CL ? (int)cl_size() : 1;
+  __shared__ int item_s;
+  double* ubuf = uws + (int64_t)(blockIdx.x / C) * ustride;
   for (;;) {
-    const int itx = pop_item_s(queue);
+    int itx;
+    if constexpr (CL) {
+      cl_barrier();
+      if (rank == 0 && tid == 0) {
+        const int it = atomicAdd(queue, 1);
+        for (int c = 0; c < C; ++c) cl_store(&item_s, c, it);
+      }
+      cl_barrier();
+      itx = item_s;
+    } else {
+      itx = pop_item_s(queue);
+    }
     if (itx >= nsub) return;
     const int si = order[itx];
     const SubInfo& S = P.sub[si];
@@ -573,50 +613,47 @@ __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
       }
     }
     __syncthreads();
-    // forward substitution L z = y, level by level from the leaves of the
+    // Forward substitution L z = y, level by level from the leaves of the
     // supernodal tree.  Supernodes of one level are independent: each one
     // assembles its front vector from its own columns of y and the update
     // vectors of its children (in fixed order, so the result is
     // deterministic), solves with its diagonal block and writes its own
     // update vector for the parent.  Small fronts take one warp each, large
-    // ones the whole CTA.
-    const int* lvo = P.lvl_off + S.lvl0;
+    // ones the whole CTA.  first, step: this CTA's share of the level [lo, hi).
     const int* lsn = P.lvl_sn;
-    for (int l = 0; l < S.nlev; ++l) {
-      const int lo = lvo[l], hi = lvo[l + 1];
-      for (int it = lo + warp; it < hi; it += NT / 32) {
+    auto forward = [&](int lo, int hi, int first, int step) {
+      for (int it = lo + first + step * warp; it < hi; it += step * (NT / 32)) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w > 32 || f_ > kWF) continue;
-        fwd_warp(P, S, gs, d2, ubuf, y, wbuf + warp * kWF, lane);
+        fwd_warp<CL>(P, S, gs, d2, ubuf, y, wbuf + warp * kWF, lane);
       }
       __syncthreads();
       if constexpr (NT == kWide) {
         double* tbuf = wbuf + (tid / 256) * (kTeamF + kW * (kW + 1));
         int q = 0;
-        for (int it = lo; it < hi; ++it) {
+        for (int it = lo + first; it < hi; it += step) {
           const int gs = S.sn0 + lsn[it];
           const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
           if ((w <= 32 && f_ <= kWF) || w > kTeamW || f_ > kTeamF) continue;
           if ((q++ & 3) != tid / 256) continue;
-          fwd_cta<true>(P, S, gs, d2, ubuf, y, tbuf, reinterpret_cast<double(*)[kW + 1]>(tbuf + kTeamF), tid % 256, tid / 256);
+          fwd_cta<true, CL>(P, S, gs, d2, ubuf, y, tbuf, reinterpret_cast<double(*)[kW + 1]>(tbuf + kTeamF), tid % 256, tid / 256);
         }
         __syncthreads();
       }
-      for (int it = lo; it < hi; ++it) {
+      for (int it = lo + first; it < hi; it += step) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w <= 32 && f_ <= kWF) continue;
         if (NT == kWide && w <= kTeamW && f_ <= kTeamF) continue;
-        if constexpr (NT == kWide) fwd_wide(P, S, gs, d2, ubuf, y, sfront, wbuf, wsm, tid);
+        if constexpr (NT == kWide) fwd_wide<CL>(P, S, gs, d2, ubuf, y, sfront, wbuf, wsm, tid);
         else fwd_cta(P, S, gs, d2, ubuf, y, sfront, sm_blk, tid);
       }
-    }
-    // backward substitution L^T x = z, level by level from the roots; every
-    // supernode reads only ancestors' entries of x and writes its own columns
-    for (int l = S.nlev - 1; l >= 0; --l) {
-      const int lo = lvo[l], hi = lvo[l + 1];
-      for (int it = lo + warp; it < hi; it += NT / 32) {
+    };
+    // Backward substitution L^T x = z, level by level from the roots; every
+    // supernode reads only ancestors' entries of x and writes its own columns.
+    auto backward = [&](int lo, int hi, int first, int step) {
+      for (int it = lo + first + step * warp; it < hi; it += step * (NT / 32)) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w > 32 || f_ > kWF) continue;
@@ -626,7 +663,7 @@ __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
       if constexpr (NT == kWide) {
         double* tbuf = wbuf + (tid / 256) * (kTeamF + kW * (kW + 1));
         int q = 0;
-        for (int it = lo; it < hi; ++it) {
+        for (int it = lo + first; it < hi; it += step) {
           const int gs = S.sn0 + lsn[it];
           const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
           if ((w <= 32 && f_ <= kWF) || w > kTeamW || f_ > kTeamF) continue;
@@ -635,7 +672,7 @@ __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
         }
         __syncthreads();
       }
-      for (int it = lo; it < hi; ++it) {
+      for (int it = lo + first; it < hi; it += step) {
         const int gs = S.sn0 + lsn[it];
         const int w = P.sn_w[gs], f_ = w + P.sn_r[gs];
         if (w <= 32 && f_ <= kWF) continue;
@@ -643,13 +680,55 @@ __global__ void __launch_bounds__(NT, NT == kWide ? 1 : 4)
         if constexpr (NT == kWide) bwd_wide(P, S, gs, y, sfront, wsm, tid);
         else bwd_cta(P, S, gs, y, sfront, sm_blk, tid);
       }
+    };
+    const int nl = S.nlev;
+    const int* lvo = P.lvl_off + S.lvl0;
+    if constexpr (CL) {
+      // own levels, then the shared ones with a barrier after each (one call site each way: the sweeps' code is long)
+      const int* lvt = lvo + (1 + C) * (nl + 1);
+      lvo += (1 + rank) * (nl + 1);
+      for (int q = 0; q < 2 * nl; ++q) {
+        const bool top = q >= nl;
+        const int* lv = top ? lvt + (q - nl) : lvo + q;
+        if (q == nl) cl_barrier();
+        const int lo = lv[0], hi = lv[1];
+        if (lo == hi) continue;
+        forward(lo, hi, top ? rank : 0, top ? C : 1);
+        if (top) cl_barrier();
+      }
+      for (int q = 2 * nl - 1; q >= 0; --q) {
+        const bool top = q >= nl;
+        const int* lv = top ? lvt + (q - nl) : lvo + q;
+        const int lo = lv[0], hi = lv[1];
+        if (lo == hi) continue;
+        backward(lo, hi, top ? rank : 0, top ? C : 1);
+        if (top) {
+          __syncthreads();
+          // the columns solved here to the other CTAs
+          for (int it = lo + rank; it < hi; it += C) {
+            const int gs = S.sn0 + lsn[it], c0 = P.sn_c0[gs], w = P.sn_w[gs];
+            for (int c = 1; c < C; ++c)
+              for (int i = tid; i < w; i += NT) cl_store(y + c0 + i, (rank + c) % C, y[c0 + i]);
+          }
+          cl_barrier();
+        }
+      }
+    } else {
+      for (int l = 0; l < nl; ++l) forward(lvo[l], lvo[l + 1], 0, 1);
+      for (int l = nl - 1; l >= 0; --l) backward(lvo[l], lvo[l + 1], 0, 1);
     }
     __syncthreads();
+    // every CTA has x in its own columns and the shared ones (which rank 0 writes)
     if (MODE == 0 || MODE == 1) {
-      for (int j = tid; j < S.m_pad; j += NT)
-        qi[S.qcol + j] = j < S.m ? P.qsign[S.qcol + j] * y[P.spos[S.col0 + j]] : 0.0;
+      for (int j = tid; j < S.m_pad; j += NT) {
+        const int col = j < S.m ? P.spos[S.col0 + j] : -1;
+        if (!CL || col_owner(P, S, col) == rank) qi[S.qcol + j] = col >= 0 ? P.qsign[S.qcol + j] * y[col] : 0.0;
+      }
     } else {
-      for (int k = tid; k < n; k += NT) u[S.dof + k] = y[P.iperm[S.diag0 + k]];
+      for (int k = tid; k < n; k += NT) {
+        const int col = P.iperm[S.diag0 + k];
+        if (!CL || col_owner(P, S, col) == rank) u[S.dof + k] = y[col];
+      }
     }
     __syncthreads();
   }
@@ -937,26 +1016,60 @@ bool implicit_wide(int nsub, int nsm, int nmax, int maxf) {
   return nsub <= nsm && implicit_smem(nmax, maxf, true) + 1024 <= 227 * 1024;
 }
 
+static cudaLaunchConfig_t cluster_launch(int ctas, int cluster, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(kWide);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  *at = {};
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)cluster;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 template <int MODE>
-static void launch_implicit_mode(bool wide, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
+static void launch_implicit_mode(int cluster, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
                                  const double* f, double* qi, double* u, double* uws, int64_t ustride, int nmax,
                                  int maxf, int grid, size_t smem, cudaStream_t st) {
-  if (wide) {
-    cudaFuncSetAttribute(implicit_kernel<MODE, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<MODE, kWide><<<grid, kWide, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax,
-                                                            maxf);
+  if (cluster > 1) {
+    auto kern = implicit_kernel<MODE, kWide, true>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t cfg = cluster_launch(grid * cluster, cluster, smem, st, &at);
+    cudaLaunchKernelEx(&cfg, kern, P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf);
+  } else if (cluster == 1) {
+    auto kern = implicit_kernel<MODE, kWide, false>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<grid, kWide, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf);
   } else {
-    cudaFuncSetAttribute(implicit_kernel<MODE, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    implicit_kernel<MODE, kThreads><<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride,
-                                                                  nmax, maxf);
+    auto kern = implicit_kernel<MODE, kThreads, false>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<grid, kThreads, smem, st>>>(P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf);
   }
 }
 
-void launch_implicit(int mode, bool wide, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
+void launch_implicit(int mode, int cluster, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
                      const double* f, double* qi, double* u, double* uws, int64_t ustride, int nmax, int maxf,
                      int grid, size_t smem, cudaStream_t st) {
   auto fn = mode == 0 ? launch_implicit_mode<0> : mode == 1 ? launch_implicit_mode<1> : launch_implicit_mode<2>;
-  fn(wide, P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf, grid, smem, st);
+  fn(cluster, P, order, nsub, queue, p, f, qi, u, uws, ustride, nmax, maxf, grid, smem, st);
+}
+
+int implicit_clusters(size_t smem, int cluster) {
+  auto kern = implicit_kernel<0, kWide, true>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = cluster_launch(64 * cluster, cluster, smem, 0, &at);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 void launch_inv_blocks(const DevPlan& P, int nsub, cudaStream_t st) {
@@ -969,11 +1082,10 @@ void launch_unit_scale(const DevPlan& P, int nsub, int nmax, double* d2, cudaStr
   unit_scale_kernel<<<dim3((unsigned)gx, (unsigned)std::min(nsub, 65535)), 256, 0, st>>>(P, nsub, d2);
 }
 
-int implicit_occupancy(size_t smem, bool wide) {
-  if (wide) return 1;
+int implicit_occupancy(size_t smem) {
   int nb = 0;
-  cudaFuncSetAttribute(implicit_kernel<0, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, implicit_kernel<0, kThreads>, kThreads, smem);
+  cudaFuncSetAttribute(implicit_kernel<0, kThreads, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, implicit_kernel<0, kThreads, false>, kThreads, smem);
   return std::max(nb, 1);
 }
 

@@ -93,11 +93,13 @@ void launch_gather_lambda(const int* c0, const int* c1, int nlam, const double* 
 // FP64 solve side: implicit operator (eq. 11), K_reg solves (eqs. 5, 7),
 // coarse problem and projector (eqs. 6-8), PCPG vectors (Algorithm 1)
 size_t implicit_smem(int nmax, int maxf, bool wide);
-bool implicit_wide(int nsub, int nsm, int nmax, int maxf);  // one 1024-thread CTA per subdomain
+bool implicit_wide(int nsub, int nsm, int nmax, int maxf);  // 1024-thread CTAs, one per SM
 void launch_inv_blocks(const DevPlan& P, int nsub, cudaStream_t st);  // for the wide solves, after launch_unit_scale
 void launch_unit_scale(const DevPlan& P, int nsub, int nmax, double* d2, cudaStream_t st);
-int implicit_occupancy(size_t smem, bool wide);
-void launch_implicit(int mode, bool wide, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
+int implicit_occupancy(size_t smem);  // 256-thread CTAs per SM
+int implicit_clusters(size_t smem, int cluster);  // clusters of wide CTAs that are resident at once
+// cluster: wide CTAs per subdomain, grid clusters of them; 0: grid 256-thread CTAs
+void launch_implicit(int mode, int cluster, const DevPlan& P, const int* order, int nsub, int* queue, const double* p,
                      const double* f, double* qi, double* u, double* uws, int64_t ustride, int nmax, int maxf,
                      int grid, size_t smem, cudaStream_t st);
 void launch_gather_minus_c(const int* c0, const int* c1, int nlam, const double* qi, const double* c, double* q,

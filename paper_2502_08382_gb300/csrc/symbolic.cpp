@@ -736,6 +736,87 @@ void plan_tasks(PatternPlan& P, double target, int big_f, double target_small) {
   }
 }
 
+SolveSplit plan_solve_split(const PatternPlan& P, int C) {
+  const int ns = P.nsn;
+  // panel entries (1.25 ns each, both sweeps), plus what a supernode costs besides them: a block step of a wide front
+  // takes about 2500 entries' time, a cluster barrier 1500, the latencies of a level 12000
+  constexpr double kStep = 2500, kTeam = 1500, kWarp = 300, kBarrier = 1500, kLevel = 12000;
+  std::vector<double> own(ns), sub(ns, 0.0);
+  for (int s = 0; s < ns; ++s) {
+    const double w = P.sn_w[s], r = P.sn_r[s];
+    own[s] = w * (0.5 * w + r) + (w <= 32 && w + r <= 128 ? kWarp : w <= 64 && w + r <= 512 ? kTeam : kStep * std::ceil(w / 32));
+    sub[s] += own[s];
+    if (P.sn_parent[s] >= 0) sub[P.sn_parent[s]] += sub[s];
+  }
+  std::vector<int> lvl(ns);
+  for (int l = 0; l < P.nlev; ++l)
+    for (int q = P.lvl_off[l]; q < P.lvl_off[l + 1]; ++q) lvl[P.lvl_sn[q]] = l;
+  std::vector<int> roots, top;
+  for (int s = 0; s < ns; ++s)
+    if (P.sn_parent[s] < 0) roots.push_back(s);
+  auto heavier = [&](int a, int b) { return sub[a] != sub[b] ? sub[a] > sub[b] : a < b; };
+  // heaviest first to the least loaded rank
+  auto deal = [&](const std::vector<int>& r, std::vector<int>* rank) {
+    std::vector<double> load(C, 0.0);
+    for (int s : r) {
+      const int k = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      load[k] += sub[s];
+      if (rank) rank->push_back(k);
+    }
+    return *std::max_element(load.begin(), load.end());
+  };
+  auto top_cost = [&] {
+    std::vector<std::vector<int>> at(P.nlev);
+    std::vector<int> t = top;
+    std::sort(t.begin(), t.end());
+    for (int s : t) at[lvl[s]].push_back(s);
+    double sum = C > 1 ? kBarrier : 0.0;
+    for (auto& v : at) {
+      std::vector<double> load(C, 0.0);
+      for (size_t q = 0; q < v.size(); ++q) load[q % C] += own[v[q]];
+      if (!v.empty()) sum += *std::max_element(load.begin(), load.end()) + kBarrier;
+    }
+    return sum;
+  };
+  // split the heaviest subtree again and again, keep the best state
+  std::sort(roots.begin(), roots.end(), heavier);
+  std::vector<int> best_roots = roots, best_top;
+  double best = deal(roots, nullptr) + top_cost();
+  for (int k = 0; C > 1 && k < 4 * C && !roots.empty(); ++k) {
+    const int s = roots.front();
+    if (P.ch_off[s + 1] == P.ch_off[s]) break;
+    roots.erase(roots.begin());
+    top.push_back(s);
+    for (int q = P.ch_off[s]; q < P.ch_off[s + 1]; ++q) roots.push_back(P.ch_list[q]);
+    std::sort(roots.begin(), roots.end(), heavier);
+    const double t = deal(roots, nullptr) + top_cost();
+    if (t < best) {
+      best = t;
+      best_roots = roots;
+      best_top = top;
+    }
+  }
+  SolveSplit S;
+  S.cost = best + kLevel * P.nlev;
+  std::vector<int> rank, list(ns, C);  // list of each supernode: a rank, or the top
+  deal(best_roots, &rank);
+  for (size_t k = 0; k < best_roots.size(); ++k) {
+    const int s = best_roots[k];
+    for (int q = P.sn_first_desc[s]; q <= s; ++q) list[q] = rank[k];
+    S.pieces.push_back({s, P.sn_c0[P.sn_first_desc[s]], P.sn_c0[s] + P.sn_w[s], rank[k]});
+  }
+  std::sort(S.pieces.begin(), S.pieces.end(), [](const auto& a, const auto& b) { return a.c0 < b.c0; });
+  S.own.resize(C + 1);
+  S.off.assign(C + 1, std::vector<int>(1, 0));
+  for (int l = 0; l < P.nlev; ++l) {
+    for (int q = P.lvl_off[l]; q < P.lvl_off[l + 1]; ++q) S.own[list[P.lvl_sn[q]]].push_back(P.lvl_sn[q]);
+    for (int k = 0; k <= C; ++k) S.off[k].push_back((int)S.own[k].size());
+  }
+  // the order that top_cost assumes
+  for (int l = 0; l < P.nlev; ++l) std::sort(S.own[C].begin() + S.off[C][l], S.own[C].begin() + S.off[C][l + 1]);
+  return S;
+}
+
 void plan_rhs(const PatternPlan& P, int m, const int32_t* B_dof, BPlan& Bp) {
   Bp = BPlan();
   Bp.m = m;

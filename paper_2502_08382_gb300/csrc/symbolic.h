@@ -83,6 +83,19 @@ struct PatternPlan {
 // large set.  Also lays the update blocks out anew (upd_stack_ofs).
 void plan_tasks(PatternPlan& P, double target, int big_f = 0, double target_small = 0);
 
+// A supernodal tree split over the C CTAs of a cluster for the substitutions: disjoint subtrees (pieces), each with one
+// owner, which need nothing of one another, and the supernodes above them (the top), whose levels all CTAs share.
+struct SolveSplit {
+  struct Piece {
+    int root, c0, c1, rank;  // columns [c0, c1)
+  };
+  std::vector<Piece> pieces;          // by column
+  std::vector<std::vector<int>> own;  // [C + 1] supernodes by level: the ranks' own, then the top
+  std::vector<std::vector<int>> off;  // [C + 1][nlev + 1]
+  double cost = 0;                    // estimate of one sweep (panel entries, and what a front costs besides)
+};
+SolveSplit plan_solve_split(const PatternPlan& P, int C);
+
 // First-fit places for blocks with a lifetime (take .. release), in one linear workspace.
 struct BlockPlaces {
   struct Block {
