@@ -471,7 +471,7 @@ void build(feti_ctx* c) {
   // ---- concatenate pattern tables
   std::vector<int> sn_c0, sn_w, sn_r, sn_parent, rows, ch_off, ch_list, rel, kmap_src, kmap_dst, diag_src, iperm;
   std::vector<int64_t> sn_rows, rel_off, Lofs, kmap_off, upd_ofs, uofs, usm_ofs;
-  std::vector<int> sn_small, sn_task, sn_big;
+  std::vector<int> sn_small, sn_task, sn_big, sn_back;
   std::vector<int64_t> sn_hoff, lh_ofs, di_ofs;
   // mixed precision: the fronts the large-front TRSM takes (a bottom block of 128 rows or more, or 256 own rows
   // or more) get a row-major bf16 hi/lo copy of their panel, pat_lh elements per pattern
@@ -506,6 +506,7 @@ void build(feti_ctx* c) {
       sn_task.push_back(P.sn_task[s]);
       sn_hoff.push_back(P.sn_hoff[s]);
       sn_big.push_back(P.sn_big[s]);
+      sn_back.push_back(P.sn_back[s]);
       lh_ofs.push_back(lh_big(P, s) ? pat_lh[p] : -1);
       di_ofs.push_back(lh_big(P, s) ? pat_di[p] : -1);
       if (lh_big(P, s)) {
@@ -515,8 +516,8 @@ void build(feti_ctx* c) {
       uofs.push_back(P.uofs[s]);
     }
     for (int s = 0; s < P.nsn; ++s) {
-      lt_ofs.push_back(P.sn_big[s] ? c->pat_lt[p] / 512 : -1);
-      for (int kB = 0; P.sn_big[s] && kB < P.sn_w[s]; kB += 128)
+      lt_ofs.push_back(P.sn_back[s] ? c->pat_lt[p] / 512 : -1);
+      for (int kB = 0; P.sn_back[s] && kB < P.sn_w[s]; kB += 128)
         c->pat_lt[p] += bsolve_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
     }
     if (!c->fp32) {
@@ -960,6 +961,7 @@ void build(feti_ctx* c) {
   D.usm_ofs = upload(c, usm_ofs);
   D.sn_task = upload(c, sn_task);
   D.sn_big = upload(c, sn_big);
+  D.sn_back = upload(c, sn_back);
   D.sn_hoff = upload(c, sn_hoff);
   D.lh_ofs = upload(c, lh_ofs);
   D.di_ofs = upload(c, di_ofs);

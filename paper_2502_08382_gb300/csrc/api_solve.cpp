@@ -688,11 +688,11 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
         const auto& pat = ctx->pats[ctx->subs[b[e].sub].pat];
         int64_t ofs = b[e].lt;
         for (int s = 0; s < pat.nsn; ++s)
-          for (int kB = 0; pat.sn_big[s] && kB < pat.sn_w[s]; kB += 128) {
+          for (int kB = 0; pat.sn_back[s] && kB < pat.sn_w[s]; kB += 128) {
             lv.push_back(make_int4(b[e].sub, s, kB, (int)(ofs / 512)));
             ofs += bsolve_oz_block_bytes(pat.sn_w[s], pat.sn_r[s], kB);
           }
-        if (pat.has_big)
+        if (pat.has_back)
           for (int cb = 0; cb < (b[e].m_pad + 127) / 128; ++cb) yv.push_back(make_int2(e, cb));
       }
       if ((int64_t)lv.size() > ctx->adj_lit_cap) {

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kAT) adj_bsolve_kernel(DevPlan P, const AdjBat
     const double* Lsub = P.L + S.L;
     for (int s = S.nsn - 1; s >= 0; --s) {
       const int gs = S.sn0 + s;
-      if (skip_big && P.sn_big[gs]) continue;  // bsolve_oz_kernel's
+      if (skip_big && P.sn_back[gs]) continue;  // bsolve_oz_kernel's
       const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs], f = w + r;
       const double* Ls = Lsub + P.Lofs[gs];
       const int* srow = P.rows + P.sn_rows[gs];

@@ -1,4 +1,4 @@
-// Backward solve V <- L_u^{-T} V of the large fronts (P.sn_big, the top of the tree) for the adjoint and the TRSM-path
+// Backward solve V <- L_u^{-T} V of the large fronts (P.sn_back, the top of the tree) for the adjoint and the TRSM-path
 // assembly, on the tensor cores by exact slicing; adj_bsolve_kernel then does the supernodes below them.
 //
 // One work item is a block of 128 columns of one subdomain's V (n x ld row-major, rows in the factor's numbering; the
@@ -8,6 +8,10 @@
 // runs against the digits of L^T; inside the block, in steps of 32 from the last, the step is multiplied by the inverse
 // of its unit-lower block and the block's earlier columns take its rank-32 update.  dig_lt_kernel cuts L^T once per
 // batch.  The tiles are those of oz_engine.cuh.
+//
+// What bounds it: the latency of a front's steps (cut, multiply, drain) on the narrow fronts; where the line to the
+// FP64 kernel lies and why, at kBackFront.  Measured, the backward solve of one adjoint of 8 elasticity subdomains of
+// 10^3: 60 ms with every front on the FP64 pipe -> 10.4 + 0.2 (digits) + 1.1 (the fronts below, FP64 pipe).
 #include <algorithm>
 #include <cuda_bf16.h>
 
@@ -25,9 +29,10 @@ constexpr int kTRows = 160;  // rows of the in-block digits: 128 and the overhan
 // Digit layout of one 128-column block (byte offsets; multiples of 512): inverses, in-block rows, groups of 128 below.
 struct LtBlock {
   int64_t inv, invex, in, inex, grp, end;
+  int64_t grpsz;       // bytes of a group: the digits, then 128 exponents
   int K, nck, nb, ng;  // own columns, chunks, rows below the block, groups of them
+  int bp;              // own columns padded to the 64 of a tile
 };
-constexpr int64_t kGroupBytes = (int64_t)kDig * 4 * 128 * 64 + 512;
 __host__ __device__ inline LtBlock lt_block(int w, int r, int kB) {
   LtBlock b;
   b.K = w - kB < 128 ? w - kB : 128;
@@ -39,7 +44,9 @@ __host__ __device__ inline LtBlock lt_block(int w, int r, int kB) {
   b.in = b.invex + 512;
   b.inex = b.in + (int64_t)kDig * b.nck * kTRows * 64;
   b.grp = b.inex + 1024;
-  b.end = b.grp + b.ng * kGroupBytes;
+  b.bp = (b.K + 63) / 64 * 64;
+  b.grpsz = (int64_t)kDig * 4 * b.bp * 64 + 512;
+  b.end = b.grp + b.ng * b.grpsz;
   return b;
 }
 
@@ -107,9 +114,9 @@ __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* item
                 reinterpret_cast<int*>(out + b.inex), warp - 4, 4);
   }
   for (int g = 0; g < b.ng; ++g) {
-    char* o = out + b.grp + g * kGroupBytes;
-    dig_rows<4>(PanelRow{Ls + (int64_t)kB * f + kE + 128 * g, f, false}, b.K, min(128, b.nb - 128 * g), 0, 128, o, 4,
-                128, reinterpret_cast<int*>(o + kGroupBytes - 512), warp, 8);
+    char* o = out + b.grp + g * b.grpsz;
+    dig_rows<4>(PanelRow{Ls + (int64_t)kB * f + kE + 128 * g, f, false}, b.K, min(128, b.nb - 128 * g), 0, b.bp, o,
+                4, b.bp, reinterpret_cast<int*>(o + b.grpsz - 512), warp, 8);
   }
 }
 
@@ -215,7 +222,7 @@ __global__ void __launch_bounds__(kCT, 1)
     double* V = work + E.v_ofs + 128 * items[it].y;
     for (int s = S.nsn - 1; s >= 0; --s) {
       const int gs = S.sn0 + s;
-      if (!P.sn_big[gs]) continue;
+      if (!P.sn_back[gs]) continue;
       const int c0 = P.sn_c0[gs], w = P.sn_w[gs], r = P.sn_r[gs];
       const int* srow = P.rows + P.sn_rows[gs];
       // the blocks' digits lie first block first
@@ -227,10 +234,10 @@ __global__ void __launch_bounds__(kCT, 1)
         const int kE = kB + b.K, ntn = (b.K + 63) / 64;
         for (int g = 0; g < b.ng; ++g) {
           const int K = min(128, b.nb - 128 * g);
-          const char* o = lt + b.grp + g * kGroupBytes;
+          const char* o = lt + b.grp + g * b.grpsz;
           dig_rows<4>(GatherRow{V, ld, srow, c0, w, kE + 128 * g}, n, K, 0, 128, SL, 4, 128, EX, warp, kCT / 32);
-          BackJob<false> bj{SL, o, EX, reinterpret_cast<const int*>(o + kGroupBytes - 512), (int64_t)4 * 128 * 64,
-                            (int64_t)4 * 128 * 64, (K + 31) / 32, n, 128, ntn, b.K, V + (int64_t)(c0 + kB) * ld, ld};
+          BackJob<false> bj{SL, o, EX, reinterpret_cast<const int*>(o + b.grpsz - 512), (int64_t)4 * 128 * 64,
+                            (int64_t)4 * b.bp * 64, (K + 31) / 32, n, b.bp, ntn, b.K, V + (int64_t)(c0 + kB) * ld, ld};
           dig_product(st, bj, 0, 1, ntn);
         }
         for (int sb = b.nck - 1; sb >= 0; --sb) {

@@ -673,6 +673,13 @@ void plan_tasks(PatternPlan& P, double target, int big_f, double target_small) {
     }
     for (int s = 0; s < ns; ++s) P.has_big = P.has_big || P.sn_big[s];
   }
+  P.sn_back = P.sn_big;
+  if (big_f > 0)
+    for (int s = 0; s < ns; ++s) {
+      if (P.sn_w[s] + P.sn_r[s] >= kBackFront) P.sn_back[s] = 1;
+      if (P.sn_back[s] && P.sn_parent[s] >= 0) P.sn_back[P.sn_parent[s]] = 1;
+    }
+  P.has_back = std::find(P.sn_back.begin(), P.sn_back.end(), 1) != P.sn_back.end();
   P.sn_task.assign(ns, 0);
   P.sn_hoff.assign(ns, -1);
   P.task_parent.assign(1, -1);

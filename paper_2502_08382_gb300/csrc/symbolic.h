@@ -19,6 +19,11 @@ constexpr int kTile = 64;  // F tile edge (apply and SYRK)
 // CTA in shared memory; larger ones by the tiled CTA path.
 constexpr int kSmallFront = 40;
 constexpr int kMidFront = 112;
+// The adjoint's backward solve takes fronts of this width (and their ancestors) on the tensor cores.  One adjoint with
+// 256 / 192 / 128 / 96 / 64 in milliseconds: 8 elasticity subdomains of 10^3 33.6 / 31.0 / 28.5 / 27.0 / 26.7; with
+// 256 / 96 / 64: 27 elasticity subdomains of 6^3 11.2 / 8.7 / 8.5, 27 heat subdomains of 12^3 23.4 / 18.8 / 19.1, 16 2D
+// heat subdomains of 40^2 3.09 / 3.08 / 3.17 (few fronts: the FP64 kernel is as good).
+constexpr int kBackFront = 96;
 
 // padded row length of a supernode X block (16-byte aligned rows)
 inline int xpad(int w) { return (w + 7) & ~7; }
@@ -69,6 +74,8 @@ struct PatternPlan {
   int64_t hsize = 0;               // doubles of all hand-over slots
   std::vector<int> sn_big;         // 1: a front at least big_f wide or an ancestor of one
   bool has_big = false;
+  std::vector<int> sn_back;        // 1: the backward solve's large set (kBackFront) or an ancestor of one
+  bool has_back = false;
   std::vector<int> task_big;       // 1: the task's supernodes are large (the tensor-core Cholesky's)
   std::vector<int> task_nbig;      // large child tasks
   // doubles of workspace for the update blocks outside and inside the large set (neither handed over nor small)
