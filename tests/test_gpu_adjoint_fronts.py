@@ -14,7 +14,7 @@ CASES = [
     (3, "elasticity", [[5, 2]] * 3),
     (3, "elasticity", [[7, 4]] * 3),
     (3, "heat", [[9, 5]] * 3),
-    (2, "heat", [[45, 7], [40, 9]]),
+    (2, "heat", [[45, 7], [40, 12]]),
 ]
 
 
