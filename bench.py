@@ -160,7 +160,7 @@ def other_rooflines(st, impl_ms, hbm):
                               "algorithmic_flops": st["chol_flops"], "ms": st["t_chol_ms"],
                               "tc_kernel_ms": st.get("t_chol_tc_ms", 0.0),
                               "note": "FP64 flops of the factorisation over both Cholesky kernels; the rank-32 and "
-                                      "rank-128 updates of the fronts at least 384 wide run on the tensor cores "
+                                      "rank-128 updates of the fronts at least 256 wide run on the tensor cores "
                                       "(exact bf16 slicing, chol_tc_kernel), so frac is against the FP64 pipe only"}
     if st["t_trsm_ms"] > 0:
         a = st["trsm_flops"] / (st["t_trsm_ms"] * 1e-3) / 1e12

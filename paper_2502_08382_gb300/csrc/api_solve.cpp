@@ -134,7 +134,7 @@ void enqueue_precond(feti_ctx* c, int mode, cudaStream_t st) {
 }
 
 // One PCPG iteration (Algorithm 1) on the device: five launches with M = I,
-// nine with the lumped preconditioner; every kernel returns at once if the
+// eleven with the lumped preconditioner; every kernel returns at once if the
 // control block says the iteration has stopped.
 // ev (4 events or null): before the tile kernel, around it, after the gather.
 void enqueue_iteration(feti_ctx* c, double* lam, const cudaEvent_t* ev, cudaStream_t st, bool capture, bool last = false) {

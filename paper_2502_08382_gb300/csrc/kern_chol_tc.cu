@@ -15,9 +15,9 @@
 // shared data is in global memory).  C is as large as keeps the CTAs within the SMs (chol_tc_cluster).
 //
 // Measured (the kernel alone; before: 9 slices of 7 bits, 45 MMAs of N = 32 per 16-deep step, one CTA per front, the
-// panel on the FP64 pipe, updates copied to the stack): 64 uneven 3D heat subdomains 50.3 -> 13.7 ms (C = 2), 27
-// elasticity subdomains of 12^3 59.0 -> 9.5 ms (C = 4), 64 of them 66.0 -> 15.4 ms (C = 2), 125 uneven 3D heat
-// subdomains 40.8 -> 9.7 ms (C = 1; these fronts were partly chol_kernel's before).  Of this, forming the bottom block
+// panel on the FP64 pipe, updates copied to the stack): 64 uneven 3D heat subdomains 50.3 -> 13.2 ms (C = 2), 27
+// elasticity subdomains of 12^3 59.0 -> 9.4 ms (C = 4), 64 of them 66.0 -> 15.0 ms (C = 2), 125 uneven 3D heat
+// subdomains 40.8 -> 9.3 ms (C = 1; these fronts were partly chol_kernel's before).  Of this, forming the bottom block
 // in place and assembling by columns took 64 elasticity subdomains from 20.7 to 15.4 ms (assembly and copy were 36%).
 // What bounds it now: on wide fronts the staging of the digits (96 KB from L2 per 2304 clocks of MMA), on fronts of a
 // few hundred rows the pivot blocks (16 k clocks of FP64 work for 32 columns) and the barriers between the phases.
