@@ -278,8 +278,9 @@ bool reserve_syrk_oz(feti_ctx* c) {
   return false;
 }
 
-// Buffers and work lists of the FP64 forward solve of the large fronts on the tensor cores; false where there are no
-// such fronts or the digits take more than a third of the free memory (trsm_kernel then solves everything).
+// Buffers and work lists of the FP64 forward solve of the large fronts on the tensor cores, in batches of consecutive
+// subdomains whose digits of L fit 16 GB and, with the hand-over blocks, a third of the free memory; false where there
+// are no such fronts or not even one subdomain fits (trsm_kernel then solves everything).
 bool reserve_trsm_oz(feti_ctx* c) {
   if (c->tx_planned && (!c->tx_on || c->d_LD)) return c->tx_on;
   size_t free_b = 0, total_b = 0;
@@ -287,9 +288,23 @@ bool reserve_trsm_oz(feti_ctx* c) {
   const bool first = !c->tx_planned;
   c->tx_planned = true;
   c->tx_on = false;
-  if (c->ld_bytes == 0 || c->ld_bytes + c->th_bytes > free_b / 3) return false;
+  if (c->ld_bytes == 0 || c->th_bytes > free_b / 3) return false;
   try {
     if (first) {
+      const size_t budget = std::min<size_t>((size_t)16 << 30, free_b / 3 - c->th_bytes);
+      auto ld_end = [&](int i) { return i + 1 < c->nsub ? (size_t)c->info[i + 1].ld : c->ld_bytes; };
+      c->tx_ld_bytes = 0;
+      for (int i = 0; i < c->nsub;) {
+        feti_ctx::TxBatch b;
+        b.sub0 = i;
+        b.ld0 = c->info[i].ld;
+        do ++i;
+        while (i < c->nsub && ld_end(i) - (size_t)b.ld0 <= budget);
+        b.sub1 = i;
+        c->tx_ld_bytes = std::max(c->tx_ld_bytes, ld_end(i - 1) - (size_t)b.ld0);
+        c->tx_batches.push_back(b);
+      }
+      if (c->tx_ld_bytes > budget) return false;
       std::vector<int4> di;
       int64_t n256 = 0;
       for (int i = 0; i < c->nsub; ++i) {
@@ -306,19 +321,26 @@ bool reserve_trsm_oz(feti_ctx* c) {
         if (P.has_big) n256 += (c->subs[i].m + 255) / 256;
       }
       c->tx_cw = n256 >= 2 * (int64_t)c->nsm ? 256 : 128;
-      std::vector<int> order;
-      for (int i = 0; i < c->nsub; ++i)
-        if (c->pats[c->subs[i].pat].has_big && c->subs[i].m > 0) order.push_back(i);
-      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return c->bps[c->subs[a].bp].trsm_flops > c->bps[c->subs[b].bp].trsm_flops;
-      });
       std::vector<int2> it;
-      for (int i : order)
-        for (int ca = 0; ca < c->subs[i].m; ca += c->tx_cw) it.push_back(make_int2(i, ca));
-      c->n_tx_ditems = (int)di.size();
-      c->n_tx_items = (int)it.size();
+      size_t most = 0, dk = 0;
+      for (auto& b : c->tx_batches) {
+        std::vector<int> order;
+        for (int i = b.sub0; i < b.sub1; ++i)
+          if (c->pats[c->subs[i].pat].has_big && c->subs[i].m > 0) order.push_back(i);
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b2) {
+          return c->bps[c->subs[a].bp].trsm_flops > c->bps[c->subs[b2].bp].trsm_flops;
+        });
+        b.item0 = (int)it.size();
+        for (int i : order)
+          for (int ca = 0; ca < c->subs[i].m; ca += c->tx_cw) it.push_back(make_int2(i, ca));
+        b.nitems = (int)it.size() - b.item0;
+        b.ditem0 = (int)dk;  // di is in the order of the subdomains
+        while (dk < di.size() && di[dk].x < b.sub1) ++dk;
+        b.nditems = (int)dk - b.ditem0;
+        most = std::max(most, (size_t)b.nitems);
+      }
       if (it.empty() || di.empty()) return false;
-      c->tx_grid = std::min(c->nsm, c->n_tx_items);
+      c->tx_grid = (int)std::min<size_t>(c->nsm, most);
       c->d_tx_ditems = upload(c, di);
       c->d_tx_items = upload(c, it);
       c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * std::max<int64_t>(c->tx_stack, 8) * c->tx_cw * 8);
@@ -326,7 +348,7 @@ bool reserve_trsm_oz(feti_ctx* c) {
       CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
     }
     if (!c->d_txscr) return false;
-    c->d_LD = dalloc(c, c->ld_bytes);
+    c->d_LD = dalloc(c, c->tx_ld_bytes);
     c->d_th = (double*)dalloc(c, std::max<size_t>(c->th_bytes, 8));
     c->tx_on = true;
   } catch (std::bad_alloc&) {
@@ -1404,7 +1426,6 @@ feti_status feti_assemble(feti_ctx* ctx) {
       launch_l32(ctx->P.L, ctx->d_L32, ctx->stats.L_doubles, ctx->nsm * 8, s2);
       launch_l16(ctx->P, ctx->d_l16_items, ctx->n_l16, ctx->d_L32, ctx->P.LH, ctx->P.DI, ctx->nsm * 6, s2);
     }
-    if (tx) launch_dig_l(ctx->P, ctx->d_tx_ditems, ctx->n_tx_ditems, ctx->d_LD, s2);
     if (!ctx->trsm_tuned) {
       // autotuner: time every work split of the TRSM on this problem (X is the same bitwise for all)
       for (auto& tc : ctx->trsm_cands) {
@@ -1424,9 +1445,13 @@ feti_status feti_assemble(feti_ctx* ctx) {
       CK(cudaEventRecord(ctx->ev[1], s2));
     }
     run_trsm(ctx->trsm_cands[ctx->trsm_pick], s2);
-    if (tx) {
+    for (size_t k = 0; tx && k < ctx->tx_batches.size(); ++k) {
+      const auto& b = ctx->tx_batches[k];
+      if (b.nitems == 0) continue;
+      char* LD = (char*)ctx->d_LD - b.ld0;  // the subdomains' offsets count from the first subdomain's
+      launch_dig_l(ctx->P, ctx->d_tx_ditems + b.ditem0, b.nditems, LD, s2);
       CK(cudaMemsetAsync(ctx->d_queue + 17, 0, sizeof(int), s2));
-      launch_trsm_oz(ctx->P, ctx->d_tx_items, ctx->n_tx_items, ctx->tx_cw, ctx->d_queue + 17, ctx->d_LD, ctx->d_th,
+      launch_trsm_oz(ctx->P, ctx->d_tx_items + b.item0, b.nitems, ctx->tx_cw, ctx->d_queue + 17, LD, ctx->d_th,
                      (double*)ctx->d_X, ctx->d_txws, std::max<int64_t>(ctx->tx_stack, 8) * ctx->tx_cw, ctx->d_txscr, trsm_oz_scratch(ctx->tx_cw), ctx->tx_grid,
                      ctx->d_status, s2);
     }
@@ -1478,7 +1503,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
   };
   // Cholesky, pruned TRSM, unit-lower scaling, SYRK (+ lumped values, or the Dirichlet factorisation and tiles)
   ctx->stats.launches += 4 + (ctx->precond_kind == 1 ? 1 : ctx->precond_kind == 2 ? 2 : 0);
-  if (tx) ctx->stats.launches += 2;
+  if (tx)
+    for (const auto& b : ctx->tx_batches) ctx->stats.launches += b.nitems > 0 ? 2 : 0;
   if (oz) ctx->stats.launches += 3 * (int64_t)ctx->oz_batches.size() - 1;
   const int want = ctx->opt.assembly_route;
   if (want == 2 || (want == 3 && ctx->route_tuned && ctx->route == 2)) {

@@ -107,7 +107,14 @@ struct feti_ctx {
   bool tx_planned = false, tx_on = false;
   int4* d_tx_ditems = nullptr;       // 128-column blocks of the large panels to cut
   int2* d_tx_items = nullptr;        // (subdomain, first column) of the solve
-  int n_tx_ditems = 0, n_tx_items = 0, tx_cw = 128, tx_grid = 0;
+  // batches of consecutive subdomains whose digits of L are cut and used in turn
+  struct TxBatch {
+    int sub0 = 0, sub1 = 0, ditem0 = 0, nditems = 0, item0 = 0, nitems = 0;
+    int64_t ld0 = 0;
+  };
+  std::vector<TxBatch> tx_batches;
+  size_t tx_ld_bytes = 0;
+  int tx_cw = 128, tx_grid = 0;
   size_t ld_bytes = 0, th_bytes = 0;
   int64_t tx_stack = 0;  // doubles per column
   void* d_LD = nullptr;              // digits of the large panels
