@@ -135,6 +135,12 @@ typedef struct {
   int32_t chol_tc_front;      /* with chol_tc = 0: the narrowest front (w + r) taken by the tensor-core kernel,
                                  with all its ancestors (0 = 256, within 3% of the fastest measured on 3D
                                  elasticity and uneven 3D heat; values below 128 act as 128) */
+  int32_t apply_kernel;       /* F-streaming kernel of the explicit apply: 0 = autotuned at the first
+                                 feti_assemble; k = feti_stats.apply_variant k - 1 (7: FP64 tiles only) */
+  int32_t implicit_cluster;   /* CTAs per subdomain of the implicit solves: 0 = chosen from the plans; -1 = one
+                                 of 256 threads; 1, 2, 4, 8 = that many of 1024 threads, as a cluster
+                                 (FETI_ERR_ARG where the subdomains do not fit their shared memory).  The
+                                 results are the same bit for bit for 1, 2, 4 and 8 */
 } feti_options;
 
 typedef struct {
@@ -179,6 +185,7 @@ typedef struct {
                                  and two CTAs per SM) */
   int32_t assembly_route;     /* route of the last feti_assemble (0 SYRK path, 1 Schur complement, 2 TRSM path) */
   double route_ms[3];         /* route 3: time of the TRSM + SYRK (0) and of the TRSM path (2) at the first call */
+  int32_t implicit_cluster;   /* CTAs per subdomain of the implicit solves (-1: one of 256 threads) */
 } feti_stats;
 
 typedef struct feti_ctx feti_ctx;

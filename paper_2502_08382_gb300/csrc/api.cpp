@@ -458,10 +458,16 @@ void build(feti_ctx* c) {
     int nmax = 0, maxf = 0;
     for (auto& sh : c->subs) nmax = std::max(nmax, sh.n);
     for (auto& P : c->pats) maxf = std::max(maxf, P.max_f);
-    c->impl_wide = implicit_wide(ns, nsm, nmax, maxf);
+    const int force = c->opt.implicit_cluster;
+    if (force != 0 && force != -1 && force != 1 && force != 2 && force != 4 && force != 8)
+      throw ArgError("bad implicit_cluster (0 auto, -1 one 256-thread CTA, or 1, 2, 4, 8)");
+    c->impl_wide = force > 0 || (force == 0 && implicit_wide(ns, nsm, nmax, maxf));
+    if (force > 0 && (!implicit_wide(1, nsm, nmax, maxf) ||
+                      (force > 1 && implicit_clusters(implicit_smem(nmax, maxf, true), force) < 1)))
+      throw ArgError("implicit_cluster: the subdomains do not fit the shared memory of such a cluster");
     if (c->impl_wide) {
       double best = 0;
-      for (int C = 1; C <= 8; C *= 2) {
+      for (int C = force > 0 ? force : 1; C <= (force > 0 ? force : 8); C *= 2) {
         const int ncl = C == 1 ? nsm : implicit_clusters(implicit_smem(nmax, maxf, true), C);
         if (ncl < 1) break;
         std::vector<SolveSplit> sp;
@@ -478,7 +484,7 @@ void build(feti_ctx* c) {
           load.push(y);
           t = std::max(t, y);
         }
-        if (C == 1 || t < 0.95 * best) {
+        if (force > 0 || C == 1 || t < 0.95 * best) {
           best = t;
           c->impl_cluster = C;
           c->solve_splits = std::move(sp);
@@ -1194,6 +1200,18 @@ void build(feti_ctx* c) {
     }
     if (c->apply_cands.empty()) throw CudaError("no launchable configuration of the apply kernel");
     c->apply_pick = (int)c->apply_cands.size() - 1;
+    if (c->opt.apply_kernel < 0 || c->opt.apply_kernel > apply_variants())
+      throw ArgError("bad apply_kernel (0 auto, else feti_stats.apply_variant + 1)");
+    if (c->opt.apply_kernel > 0) {
+      for (size_t k = 0; k < c->apply_cands.size(); ++k)
+        if (c->apply_cands[k].variant == c->opt.apply_kernel - 1) {
+          c->apply_pick = (int)k;
+          c->apply_tuned = true;
+        }
+      if (!c->apply_tuned) throw ArgError("apply_kernel: not for this precision");
+      c->stats.apply_variant = c->apply_cands[c->apply_pick].variant;
+      c->stats.apply_grid = c->apply_cands[c->apply_pick].grid;
+    }
   }
   c->d_syrk2_items = upload(c, sy2i);
   c->d_blocks = upload(c, blocks);
@@ -1232,6 +1250,7 @@ void build(feti_ctx* c) {
   CK(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->st));
   CK(cudaMemsetAsync(c->d_tpart, 0, (size_t)std::max<int64_t>(tpo, 1) * 8, c->st));
   c->stats.workspace_bytes = (int64_t)gw * c->ws_stride * 8;
+  c->stats.implicit_cluster = c->impl_wide ? c->impl_cluster : -1;
   for (auto& e : c->ev) CK(cudaEventCreate(&e));
   CK(cudaStreamSynchronize(c->st));
   c->stats.device_bytes = (int64_t)c->device_bytes;

@@ -51,7 +51,8 @@ class FetiOptions(C.Structure):
                 ("alloc_ctx", C.c_void_p), ("stream", C.c_void_p), ("leaf_dofs", C.c_int32),
                 ("use_coords", C.c_int32), ("refine_drop", C.c_double), ("refine_restart", C.c_int32),
                 ("precond", C.c_int32), ("adjoint_work_bytes", C.c_int64), ("assembly_route", C.c_int32),
-                ("chol_split", C.c_int32), ("syrk_kernel", C.c_int32), ("chol_tc", C.c_int32), ("chol_tc_front", C.c_int32)]
+                ("chol_split", C.c_int32), ("syrk_kernel", C.c_int32), ("chol_tc", C.c_int32), ("chol_tc_front", C.c_int32),
+                ("apply_kernel", C.c_int32), ("implicit_cluster", C.c_int32)]
 
 
 class FetiSolveInfo(C.Structure):
@@ -72,7 +73,7 @@ class FetiStats(C.Structure):
                 ("apply_tiles_ms", C.c_double), ("implicit_calls", C.c_int64), ("implicit_ms", C.c_double),
                 ("apply_variant", C.c_int32), ("apply_grid", C.c_int32), ("trsm_cols", C.c_int32),
                 ("trsm_grid", C.c_int32), ("chol_tasks", C.c_int32), ("syrk_variant", C.c_int32), ("assembly_route", C.c_int32),
-                ("route_ms", C.c_double * 3)]
+                ("route_ms", C.c_double * 3), ("implicit_cluster", C.c_int32)]
 
     def as_dict(self):
         d = {k: getattr(self, k) for k, _ in self._fields_}
@@ -238,7 +239,9 @@ class FetiOperator:
     place of K_i; needs route="schur"); chol_split: "auto" (autotuned), "whole"
     (one subdomain per CTA) or "tasks" (heavy subtrees on CTAs of their own); syrk_kernel: -1 (autotuned)
     or the split-bf16 SYRK kernel 0, 1, 2 to use; chol_tc: the large fronts' updates on
-    the tensor cores (exact bf16 slicing) or all of the Cholesky on the FP64 pipe."""
+    the tensor cores (exact bf16 slicing) or all of the Cholesky on the FP64 pipe;
+    apply_kernel: -1 (autotuned) or the apply's tile kernel (feti_stats.apply_variant) to use;
+    implicit_cluster: 0 (chosen from the plans), -1 (one 256-thread CTA per subdomain) or 1, 2, 4, 8 wide CTAs."""
 
     def __init__(self, problem, prec: str = "fp64", tol: float = 1e-10, maxit: int = 2000,
                  refine_every: int = 0, refine_drop: float = 0.0, refine_restart: bool = False,
@@ -246,7 +249,8 @@ class FetiOperator:
                  with_elements: bool = False, unit_scale: bool = False, per_element: bool = False,
                  recompute_X: bool = False, adjoint_work_bytes: int = 0, route: str = "syrk",
                  chol_split: str = "auto", syrk_kernel: int = -1, chol_tc: bool = True,
-                 chol_tc_front: int = 0, torch_alloc: bool = True):
+                 chol_tc_front: int = 0, apply_kernel: int = -1, implicit_cluster: int = 0,
+                 torch_alloc: bool = True):
         import torch
         self.torch = torch
         self.lib = load_library()
@@ -276,6 +280,8 @@ class FetiOperator:
         opt.syrk_kernel = 0 if syrk_kernel < 0 else syrk_kernel + 1
         opt.chol_tc = 0 if chol_tc else 1
         opt.chol_tc_front = int(chol_tc_front)
+        opt.apply_kernel = 0 if apply_kernel < 0 else apply_kernel + 1
+        opt.implicit_cluster = int(implicit_cluster)
         self._cb = None
         if torch_alloc:
             dev = self.device.index
