@@ -52,6 +52,7 @@ __host__ __device__ inline LtBlock lt_block(int w, int r, int kB) {
 
 // row b = column b of the panel, entries k below it; strict: only those below the (unit) diagonal
 struct PanelRow {
+  static constexpr bool kShift = false;
   const double* A;
   int64_t ld;
   bool strict;
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* item
 
 // row c = column c of V (from the item's first), entry k = front row i0 + k (own rows from c0, then the row list)
 struct GatherRow {
+  static constexpr bool kShift = false;
   const double* V;
   int64_t ld;
   const int* srow;

@@ -3,7 +3,8 @@
 //
 // A front's w own columns go in blocks of 128, and inside a block in steps of 32:
 //   pivot   the 32 x 32 block's factor L_bb and inverse on the FP64 pipe (eight warps);
-//   panel   the rows below, X = A L_bb^{-T}, on the tensor cores (K = 32, N = 32);
+//   panel   the rows below, X = A L_bb^{-T}, on the tensor cores (K = 32, N = 32), A's columns and those of the inverse
+//           cut with opposite shifts of half the diagonal's exponents (oz.cuh);
 //   block   the block's later columns, C -= X X^T, on the tensor cores (K = 32);
 // after the block the rest of the front takes C -= X X^T with K = 128.  All products run by exact slicing of FP64
 // into bf16 digits (oz.cuh); a product costs one FP64 addition per entry of C, the rest of the epilogue (sums of the
@@ -178,25 +179,26 @@ __device__ __forceinline__ void pivot_block(PivotSmem& sm, int nbk, int* bad) {
   }
 }
 
-// The digits of L_bb^{-1} (rows j < 32, K = 32) into the panel's B operand in shared memory, and its row exponents.
-__device__ __forceinline__ void dig_inverse(const PivotSmem& sm, uint8_t* bpan, int* EXB) {
+// The digits of L_bb^{-1} (rows j < 32, K = 32, shifts -es) into the panel's B operand in shared memory, and its row
+// exponents.
+__device__ __forceinline__ void dig_inverse(const PivotSmem& sm, const int* es, uint8_t* bpan, int* EXB) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, q = lane & 3;
   if (warp >= 4) return;
   const int i = warp * 8 + (lane >> 2);
   double v[8];
-  uint32_t mx = 0;
+  int mx = kKeyZero;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
     v[e] = sm.M[i][q * 8 + e];
-    mx = max(mx, (uint32_t)__double2hiint(v[e]) & 0x7fffffffu);
+    mx = max(mx, dig_key(v[e], -es[q * 8 + e]));
   }
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  const int ex = dig_exponent(mx);
+  const int ex = dig_key_exponent(mx);
   if (q == 0) EXB[i] = ex;
   uint64_t w[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[e], ex);
+  for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[e], ex - es[q * 8 + e]);
 #pragma unroll
   for (int p = 0; p < kDig; ++p)
     *reinterpret_cast<uint4*>(bpan + p * kCB + i * 64 + ((q ^ ((i >> 1) & 3)) << 4)) =
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(kCT, 1)
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
   __shared__ int bad, item_s;
-  __shared__ __align__(16) int EXB[kNB];
+  __shared__ __align__(16) int EXB[kNB], es[kNB];  // es: the shifts of a 32-column step
   __shared__ double red[kCT / 32];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int rank = (int)cl_rank(), C = (int)cl_size(), cluster = blockIdx.x / C;
@@ -372,17 +374,19 @@ __global__ void __launch_bounds__(kCT, 1)
             // the pivot block (every CTA), and the digits of this CTA's panel rows
             for (int idx = tid; idx < kNB * kNB; idx += kCT) {
               const int i = idx % kNB, j = idx / kNB;
-              sm.D[i][j] = (i < nbk && j <= i) ? __ldcg(Ls + (int64_t)(kb + j) * f + kb + i) : 0.0;
+              const double a = (i < nbk && j <= i) ? __ldcg(Ls + (int64_t)(kb + j) * f + kb + i) : 0.0;
+              sm.D[i][j] = a;
+              if (i == j) es[j] = dig_half_exponent(a);
             }
             __syncthreads();
             pivot_block(sm, nbk, &bad);
             // warps 8-11 start on the panel rows while the others factor the block
             if (warp >= 8)
               for (int tm = rank; tm < ntm; tm += C)
-                dig_rows<1>(ColMajor{Ls + (int64_t)kb * f + ke, f}, n, nbk, tm * kCM, tm * kCM + kCM, S1, 1, npad, EX1,
-                            warp - 8, 4);
+                dig_rows<1>(Shifted<ColMajor, false>{{Ls + (int64_t)kb * f + ke, f}, es}, n, nbk, tm * kCM,
+                            tm * kCM + kCM, S1, 1, npad, EX1, warp - 8, 4);
             __syncthreads();
-            dig_inverse(sm, st.bpan, EXB);
+            dig_inverse(sm, es, st.bpan, EXB);
             double lb[3];
             for (int u = 0; u < 3; ++u) {
               const int idx = tid + u * kCT;

@@ -12,6 +12,12 @@
 // Rounding to 62 bits costs 2^-63 of the largest entry and the dropped pairs (p + q >= 8) about as much per
 // product, far below one FP64 rounding of the same sum.
 //
+// A vector's entries share one exponent, so an entry far below the largest one keeps fewer than 53 bits.  Where the
+// scales of a product's inner index are opposite on its two sides (a factor's inverse and a right-hand side: the one
+// grows with the unknown's stiffness, the other falls), that would lose bits that FP64 keeps.  There both sides are
+// cut with a shift s_k per inner index, x_k 2^-s_k and y_k 2^s_k (dig_key), which balances them; the shifts follow the
+// unknowns' scales, so that the result is as independent of a power-of-two scaling of the unknowns as FP64's.
+//
 // All right-hand digits of one column block are stacked as the N rows of one operand (digit 0 first), so the MMA
 // of left digit p with the stacked digits 0 .. 7 - p adds into the accumulators p .. 7, which lie side by side in
 // TMEM: eight MMAs of N = 8 - p column blocks do all 36 products.
@@ -34,7 +40,22 @@ __device__ __forceinline__ int dig_exponent(uint32_t hi_max) {
   return be == 0x7FF ? kExpBad : max(be - 1022, kExpMin);
 }
 
-// the digits of x (|x| < 2^e) as signed bytes, digit 0 in the top byte
+// key of x 2^-s: its biased exponent minus s; the largest key of a vector gives its exponent
+constexpr int kKeyZero = -(1 << 20), kKeyBad = 1 << 20;
+__device__ __forceinline__ int dig_key(double x, int s) {
+  const int be = (__double2hiint(x) >> 20) & 0x7FF;
+  return be == 0 ? kKeyZero : be == 0x7FF ? kKeyBad : be - s;
+}
+__device__ __forceinline__ int dig_key_exponent(int key) {
+  return key >= kKeyBad ? kExpBad : max(key - 1022, kExpMin);
+}
+// half the exponent of a positive normal x (a shift of about sqrt(x)), 0 otherwise
+__device__ __forceinline__ int dig_half_exponent(double x) {
+  const int be = __double2hiint(x) >> 20;
+  return be <= 0 || be >= 0x7FF ? 0 : (be - 1023) >> 1;
+}
+
+// the digits of x (|x| < 2^e; |x| 2^-s < 2^e: cut with e + s) as signed bytes, digit 0 in the top byte
 __device__ __forceinline__ uint64_t dig_cut(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int be = (int)((b >> 52) & 0x7FF);

@@ -52,6 +52,7 @@ __device__ __forceinline__ void st4(double* p, double a, double b, double c, dou
 // Eight entries of a row (columns k .. k + 7, zero from K on): of a column-major matrix, and of a row-major one of this
 // CTA whose rows are 32-byte aligned and padded to a multiple of 8.
 struct ColMajor {
+  static constexpr bool kShift = false;
   const double* A;
   int64_t ld;
   __device__ __forceinline__ void get(int i, int k, int K, double (&v)[8]) const {
@@ -60,6 +61,7 @@ struct ColMajor {
   }
 };
 struct RowMajor {
+  static constexpr bool kShift = false;
   const double* A;
   int64_t ld;
   __device__ __forceinline__ void get(int i, int k, int K, double (&v)[8]) const {
@@ -72,9 +74,23 @@ struct RowMajor {
     for (int e = 0; e < 8; ++e) v[e] = k + e < K ? v[e] : 0.0;
   }
 };
+// SRC with the shift sh[k] (NEG: -sh[k]) of column k; sh holds whole chunks of 32, 16-byte aligned
+template <class SRC, bool NEG>
+struct Shifted {
+  static constexpr bool kShift = true;
+  SRC src;
+  const int* sh;
+  __device__ __forceinline__ void get(int i, int k, int K, double (&v)[8]) const { src.get(i, k, K, v); }
+  __device__ __forceinline__ void shifts(int k, int (&s)[8]) const {
+    const int4 a = *reinterpret_cast<const int4*>(sh + k), b = *reinterpret_cast<const int4*>(sh + k + 4);
+    s[0] = a.x, s[1] = a.y, s[2] = a.z, s[3] = a.w, s[4] = b.x, s[5] = b.y, s[6] = b.z, s[7] = b.w;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s[e] = NEG ? -s[e] : s[e];
+  }
+};
 
-// Digits of the rows [r0, r1) (multiples of 8) of A (K <= 128 columns): row exponents EX and the digits in the layout
-// above (npad rows; rows >= n are zero).  Four lanes per row, eight of its columns each.
+// Digits of the rows [r0, r1) (multiples of 8) of A (K <= 128 columns; with A's shifts where it has some): row exponents
+// EX and the digits in the layout above (npad rows; rows >= n are zero).  Four lanes per row, eight of its columns each.
 template <int NCK, class SRC>
 __device__ __forceinline__ void dig_rows(const SRC& A, int n, int K, int r0, int r1, char* SL, int nck,
                                          int npad, int* EX, int warp, int nwarps) {
@@ -82,7 +98,7 @@ __device__ __forceinline__ void dig_rows(const SRC& A, int n, int K, int r0, int
   for (int rb = r0 + warp * 8; rb < r1; rb += nwarps * 8) {
     const int i = rb + (lane >> 2);
     double v[NCK][8];
-    uint32_t mx = 0;
+    int mx = SRC::kShift ? kKeyZero : 0;
 #pragma unroll
     for (int c = 0; c < NCK; ++c) {
       if (i < n) {
@@ -91,20 +107,34 @@ __device__ __forceinline__ void dig_rows(const SRC& A, int n, int K, int r0, int
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[c][e] = 0.0;
       }
+      if constexpr (SRC::kShift) {
+        int s[8];
+        A.shifts(c * 32 + q * 8, s);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) mx = max(mx, (uint32_t)__double2hiint(v[c][e]) & 0x7fffffffu);
+        for (int e = 0; e < 8; ++e) mx = max(mx, dig_key(v[c][e], s[e]));
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) mx = max(mx, __double2hiint(v[c][e]) & 0x7fffffff);
+      }
     }
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const int ex = dig_exponent(mx);
+    const int ex = SRC::kShift ? dig_key_exponent(mx) : dig_exponent((uint32_t)mx);
     if (q == 0) EX[i] = ex;
     const int64_t o = (int64_t)i * 64 + ((q ^ ((i >> 1) & 3)) << 4);
 #pragma unroll
     for (int c = 0; c < NCK; ++c) {
       if (c >= nck) break;
       uint64_t w[8];
+      if constexpr (SRC::kShift) {
+        int s[8];
+        A.shifts(c * 32 + q * 8, s);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[c][e], ex);
+        for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[c][e], ex + s[e]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) w[e] = dig_cut(v[c][e], ex);
+      }
 #pragma unroll
       for (int p = 0; p < kDig; ++p)
         *reinterpret_cast<uint4*>(SL + ((int64_t)(p * nck + c) * npad) * 64 + o) =

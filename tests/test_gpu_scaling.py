@@ -1,0 +1,66 @@
+"""Unknowns of very different stiffness: K -> S K S with S a diagonal of powers of two (exponents -20 .. 20, so entries of
+K over 24 decades).  FP64 arithmetic commutes with such a scaling: every result, its scaling undone, is that of the
+unscaled problem to the last bit.  The products by digits cut whole vectors at one exponent, so they have to follow the
+unknowns' scales to be as accurate; each test here holds the scaled problem, its scaling undone (exactly), to the bar of
+the unscaled one.
+
+The subdomains are made regular (K_reg in place of K, no kernel), because the penalty rho = max diag K does not scale.
+chol_tc_front = 128 brings the tensor-core kernels to these small problems."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import feti_oracle as O
+from paper_2502_08382_gb300 import feti
+from paper_2502_08382_gb300.problems import make_problem, make_W, seeded_vector
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    (3, "elasticity", [[6, 5]] * 3),
+    (3, "heat", [[11, 9]] * 3),
+    (2, "heat", [[60, 50]] * 2),
+]
+
+
+def scaled(P, seed, reach=20):
+    """P with regular subdomains, the same scaled by S, S per global DOF and per multiplier."""
+    g = np.exp2(np.random.default_rng([seed, 9]).integers(-reach, reach + 1, size=P.n_global_dofs).astype(np.float64))
+    lam = np.ones(P.n_lambda)
+    plain, scal = [], []
+    for s in P.subs:
+        K = O.K_reg(s)
+        S = g[s.l2g]
+        rows = np.repeat(np.arange(s.n), np.diff(s.K_rowptr))
+        val = K[rows, s.K_col]
+        none = dict(R=np.zeros((s.n, 0)), fix_dofs=np.zeros(0, np.int32))
+        plain.append(dataclasses.replace(s, K_val=val, **none))
+        scal.append(dataclasses.replace(s, K_val=val * S[rows] * S[s.K_col], f=s.f * S, **none))
+        lam[s.B_lambda] = S[s.B_dof]
+    return dataclasses.replace(P, subs=plain), dataclasses.replace(P, subs=scal), g, lam
+
+
+def problem(dim, physics, cuts, seed=1):
+    return scaled(make_problem(dim=dim, physics=physics, cuts=cuts, material="lognormal", sigma=0.5, seed=seed), seed)
+
+
+@pytest.mark.parametrize("dim,physics,cuts", CASES)
+def test_factor(dim, physics, cuts):
+    """The Cholesky, seen through the implicit operator (FP64 substitutions); the bar is that of its own test."""
+    P, Q, _, lam = problem(dim, physics, cuts)
+    p = seeded_vector(P.n_lambda, 6)
+    op = feti.FetiOperator(Q, prec="fp64", chol_tc_front=128)
+    op.assemble()
+    q = op.apply_implicit(torch.from_numpy(p * lam).cuda()).cpu().numpy() * lam
+    op.close()
+    ref, size, kappa = np.zeros_like(q), 0.0, 0.0
+    for s in P.subs:
+        l = np.asarray(s.B_lambda, dtype=np.int64)
+        K = O.K_dense(s)
+        part = O.local_F(s, K) @ p[l]
+        ref[l] += part
+        size += np.linalg.norm(part)
+        kappa = max(kappa, np.linalg.cond(K, 1))
+    assert np.linalg.norm(q - ref) <= 8 * 2.0 ** -53 * kappa * size
