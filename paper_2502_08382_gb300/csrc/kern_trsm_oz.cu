@@ -5,7 +5,8 @@
 // diagonal blocks, the block's own rows and the rows below it.  trsm_oz_kernel then takes one block of 128 or 256
 // sorted columns of one subdomain per work item (the columns are independent) up the tree of its large fronts.  The
 // right-hand sides of a front are rows here, X^T (J x w): per 128 columns of the front, in steps of 32,
-//   X^T_b <- A L_bb^{-T}              (K = 32, the explicit inverse, as the FP64-pipe solve uses it),
+//   X^T_b <- A L_bb^{-T}              (K = 32, the explicit inverse, as the FP64-pipe solve uses it; cut with opposite
+//                                      shifts of L's pivots' exponents, oz.cuh),
 //   the block's later columns         -= X^T_b L^T (K = 32),
 // and after the block the later columns of the front and its update block -= X^T L^T with K = 128.  The tiles are
 // those of oz_engine.cuh.
@@ -30,7 +31,7 @@ constexpr int kInRows = 160;  // rows of the in-block digits: 128 and the overha
 
 // Digit layout of one 128-column block of a large panel (byte offsets within the block; all multiples of 512).
 struct LdBlock {
-  int64_t inv, invex, in, inex, bel, belex, end;
+  int64_t inv, invex, in, inex, piv, bel, belex, end;  // piv: the shifts of the block's columns
   int K, nck, own, ownp, botp;  // columns, chunks, own rows below the block (padded to 64), bottom rows padded to 64
 };
 __host__ __device__ inline LdBlock ld_block(int w, int r, int kB) {
@@ -44,7 +45,8 @@ __host__ __device__ inline LdBlock ld_block(int w, int r, int kB) {
   b.invex = 4 * kDig * kCB;
   b.in = b.invex + 512;
   b.inex = b.in + (int64_t)kDig * b.nck * kInRows * 64;
-  b.bel = b.inex + 1024;
+  b.piv = b.inex + 1024;
+  b.bel = b.piv + 512;
   b.belex = b.bel + (int64_t)kDig * b.nck * (b.ownp + b.botp) * 64;
   b.end = (b.belex + (int64_t)(b.ownp + b.botp) * 4 + 511) / 512 * 512;
   return b;
@@ -65,6 +67,8 @@ __global__ void __launch_bounds__(256) dig_l_kernel(DevPlan P, const int4* items
     // the inverse of diagonal block `warp`, lane = column
     const int k0 = kB + 32 * warp, nb = min(32, kE - k0);
     double(*d)[kNB + 1] = D[warp];
+    const int es = lane < nb ? dig_pivot_shift(Ls[(int64_t)(k0 + lane) * f + k0 + lane]) : 0;
+    reinterpret_cast<int*>(out + b.piv)[32 * warp + lane] = es;
     for (int k = 0; k < kNB; ++k)
       d[lane][k] = (lane < nb && k <= lane && k < nb) ? Ls[(int64_t)(k0 + k) * f + k0 + lane] : (lane == k ? 1.0 : 0.0);
     __syncwarp();
@@ -83,19 +87,20 @@ __global__ void __launch_bounds__(256) dig_l_kernel(DevPlan P, const int4* items
     for (int i0 = 0; i0 < kNB; i0 += 8) {
       const int i = i0 + (lane >> 2), q = lane & 3;
       double v[8];
-      uint32_t mx = 0;
+      int sh[8], mx = kKeyZero;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         v[e] = d[i][q * 8 + e];
-        mx = max(mx, (uint32_t)__double2hiint(v[e]) & 0x7fffffffu);
+        sh[e] = -__shfl_sync(0xffffffffu, es, q * 8 + e);
+        mx = max(mx, dig_key(v[e], sh[e]));
       }
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      const int ex = dig_exponent(mx);
+      const int ex = dig_key_exponent(mx);
       if (q == 0) reinterpret_cast<int*>(out + b.invex)[32 * warp + i] = ex;
       uint64_t c[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) c[e] = dig_cut(v[e], ex);
+      for (int e = 0; e < 8; ++e) c[e] = dig_cut(v[e], ex + sh[e]);
 #pragma unroll
       for (int p = 0; p < kDig; ++p)
         *reinterpret_cast<uint4*>(out + b.inv + (warp * kDig + p) * kCB + i * 64 + ((q ^ ((i >> 1) & 3)) << 4)) =
@@ -306,7 +311,8 @@ __global__ void __launch_bounds__(kCT, 1)
         const int kE = kB + b.K;
         for (int kb = kB, sb = 0; kb < kE; kb += 32, ++sb) {
           const int ke = min(kE, kb + 32), nbk = ke - kb;
-          dig_rows<1>(RowMajor{Xs + kb, wp}, J, nbk, 0, npad, SL, 1, npad, EX1, warp, kCT / 32);
+          dig_rows<1>(Shifted<RowMajor, false>{{Xs + kb, wp}, reinterpret_cast<const int*>(ld + b.piv) + 32 * sb}, J,
+                      nbk, 0, npad, SL, 1, npad, EX1, warp, kCT / 32);
           SolveJob sj{SL, ld + b.inv + sb * kDig * kCB, EX1, reinterpret_cast<const int*>(ld + b.invex) + 32 * sb,
                       (int64_t)npad * 64, kCB, 1, J, nbk, Xs + kb, wp};
           dig_product(st, sj, 0, 1, ntm);

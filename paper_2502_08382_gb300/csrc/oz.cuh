@@ -49,10 +49,13 @@ __device__ __forceinline__ int dig_key(double x, int s) {
 __device__ __forceinline__ int dig_key_exponent(int key) {
   return key >= kKeyBad ? kExpBad : max(key - 1022, kExpMin);
 }
-// half the exponent of a positive normal x (a shift of about sqrt(x)), 0 otherwise
-__device__ __forceinline__ int dig_half_exponent(double x) {
+// shift of a pivot x: its exponent if it is positive and normal, 0 otherwise; and half of it (for x a square)
+__device__ __forceinline__ int dig_pivot_shift(double x) {
   const int be = __double2hiint(x) >> 20;
-  return be <= 0 || be >= 0x7FF ? 0 : (be - 1023) >> 1;
+  return be <= 0 || be >= 0x7FF ? 0 : be - 1023;
+}
+__device__ __forceinline__ int dig_half_exponent(double x) {
+  return dig_pivot_shift(x) >> 1;
 }
 
 // the digits of x (|x| < 2^e; |x| 2^-s < 2^e: cut with e + s) as signed bytes, digit 0 in the top byte

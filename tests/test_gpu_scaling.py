@@ -64,3 +64,17 @@ def test_factor(dim, physics, cuts):
         size += np.linalg.norm(part)
         kappa = max(kappa, np.linalg.cond(K, 1))
     assert np.linalg.norm(q - ref) <= 8 * 2.0 ** -53 * kappa * size
+
+
+@pytest.mark.parametrize("dim,physics,cuts", CASES)
+def test_F(dim, physics, cuts):
+    """The forward solve and the SYRK, at the FP64 parity bar."""
+    P, Q, _, lam = problem(dim, physics, cuts)
+    op = feti.FetiOperator(Q, prec="fp64", chol_tc_front=128)
+    op.assemble()
+    for i, s in enumerate(P.subs):
+        l = lam[s.B_lambda]
+        F = op.get_F(i) * l[:, None] * l[None, :]
+        Fo = O.local_F(s, O.K_dense(s))
+        assert np.linalg.norm(F - Fo) <= 1e-12 * np.linalg.norm(Fo)
+    op.close()
