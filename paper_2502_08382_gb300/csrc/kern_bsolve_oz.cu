@@ -7,7 +7,8 @@
 //   V^T_b -= V^T_below L_below,b        (K = 128)
 // runs against the digits of L^T; inside the block, in steps of 32 from the last, the step is multiplied by the inverse
 // of its unit-lower block and the block's earlier columns take its rank-32 update.  dig_lt_kernel cuts L^T once per
-// batch.  The tiles are those of oz_engine.cuh.
+// batch.  The tiles are those of oz_engine.cuh.  Row i of V falls with unknown i's stiffness and row i of L_u grows with
+// it: the two are cut with opposite shifts of the pivot L_ii's exponent (oz.cuh), kept with the digits.
 //
 // What bounds it: the latency of a front's steps (cut, multiply, drain) on the narrow fronts; where the line to the
 // FP64 kernel lies and why, at kBackFront.  Measured, the backward solve of one adjoint of 8 elasticity subdomains of
@@ -26,12 +27,13 @@ namespace {
 constexpr int kYDyn = 1024 + kCStages * kCStage;
 constexpr int kTRows = 160;  // rows of the in-block digits: 128 and the overhang of a 64-column tile
 
-// Digit layout of one 128-column block (byte offsets; multiples of 512): inverses, in-block rows, groups of 128 below.
+// Digit layout of one 128-column block (byte offsets; multiples of 512): inverses, in-block rows, groups of 128 below,
+// each with its exponents and the shifts of its inner index.
 struct LtBlock {
-  int64_t inv, invex, in, inex, grp, end;
-  int64_t grpsz;       // bytes of a group: the digits, then 128 exponents
-  int K, nck, nb, ng;  // own columns, chunks, rows below the block, groups of them
-  int bp;              // own columns padded to the 64 of a tile
+  int64_t inv, invex, in, inex, piv, grp, end;
+  int64_t grpex, grpsz;  // of a group: its 128 exponents (after the digits; then the 128 shifts), its bytes
+  int K, nck, nb, ng;    // own columns, chunks, rows below the block, groups of them
+  int bp;                // own columns padded to the 64 of a tile
 };
 __host__ __device__ inline LtBlock lt_block(int w, int r, int kB) {
   LtBlock b;
@@ -43,9 +45,11 @@ __host__ __device__ inline LtBlock lt_block(int w, int r, int kB) {
   b.invex = 4 * kDig * kCB;
   b.in = b.invex + 512;
   b.inex = b.in + (int64_t)kDig * b.nck * kTRows * 64;
-  b.grp = b.inex + 1024;
+  b.piv = b.inex + 1024;
+  b.grp = b.piv + 512;
   b.bp = (b.K + 63) / 64 * 64;
-  b.grpsz = (int64_t)kDig * 4 * b.bp * 64 + 512;
+  b.grpex = (int64_t)kDig * 4 * b.bp * 64;
+  b.grpsz = b.grpex + 1024;
   b.end = b.grp + b.ng * b.grpsz;
   return b;
 }
@@ -65,6 +69,7 @@ struct PanelRow {
 // items: (subdomain, supernode, first column of the block, byte offset / 512 of the block); base: per item's subdomain
 __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* items, char* LT) {
   __shared__ double D[4][kNB][kNB + 1];
+  __shared__ __align__(16) int es[128];
   const int4 it = items[blockIdx.x];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const SubInfo& S = P.sub[it.x];
@@ -73,6 +78,13 @@ __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* item
   const LtBlock b = lt_block(w, r, kB);
   char* out = LT + (int64_t)it.w * 512;
   const int kE = kB + b.K;
+  const double* d2 = P.dinv + S.dof;  // 1 / L_ii^2
+  auto shift = [&](int col) { return -(dig_pivot_shift(d2[col]) >> 1); };  // about the exponent of L_ii
+  if (tid < 128) {
+    es[tid] = tid < b.K ? shift(P.sn_c0[gs] + kB + tid) : 0;
+    reinterpret_cast<int*>(out + b.piv)[tid] = es[tid];
+  }
+  __syncthreads();
   if (warp < 4) {
     // the inverse of the unit-lower diagonal block `warp`: lane = column k, m[i] = Linv[i][k]; row k of the operand
     const int k0 = kB + 32 * warp, nb = min(32, kE - k0);
@@ -94,16 +106,17 @@ __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* item
     __syncwarp();
     for (int i0 = 0; i0 < kNB; i0 += 8) {
       const int i = i0 + (lane >> 2), q = lane & 3;
-      uint32_t mx = 0;
+      const int* sh = es + 32 * warp + q * 8;
+      int mx = kKeyZero;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) mx = max(mx, (uint32_t)__double2hiint(d[i][q * 8 + e]) & 0x7fffffffu);
+      for (int e = 0; e < 8; ++e) mx = max(mx, dig_key(d[i][q * 8 + e], sh[e]));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      const int ex = dig_exponent(mx);
+      const int ex = dig_key_exponent(mx);
       if (q == 0) reinterpret_cast<int*>(out + b.invex)[32 * warp + i] = ex;
       uint64_t c[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) c[e] = dig_cut(d[i][q * 8 + e], ex);
+      for (int e = 0; e < 8; ++e) c[e] = dig_cut(d[i][q * 8 + e], ex + sh[e]);
 #pragma unroll
       for (int p = 0; p < kDig; ++p)
         *reinterpret_cast<uint4*>(out + b.inv + (warp * kDig + p) * kCB + i * 64 + ((q ^ ((i >> 1) & 3)) << 4)) =
@@ -111,13 +124,20 @@ __global__ void __launch_bounds__(256) dig_lt_kernel(DevPlan P, const int4* item
                        dig_pair(c[6], c[7], p));
     }
   } else {
-    dig_rows<4>(PanelRow{Ls + (int64_t)kB * f + kB, f, true}, b.K, b.K, 0, 128, out + b.in, b.nck, kTRows,
-                reinterpret_cast<int*>(out + b.inex), warp - 4, 4);
+    dig_rows<4>(Shifted<PanelRow, false>{{Ls + (int64_t)kB * f + kB, f, true}, es}, b.K, b.K, 0, 128, out + b.in, b.nck,
+                kTRows, reinterpret_cast<int*>(out + b.inex), warp - 4, 4);
   }
   for (int g = 0; g < b.ng; ++g) {
     char* o = out + b.grp + g * b.grpsz;
-    dig_rows<4>(PanelRow{Ls + (int64_t)kB * f + kE + 128 * g, f, false}, b.K, min(128, b.nb - 128 * g), 0, b.bp, o,
-                4, b.bp, reinterpret_cast<int*>(o + b.grpsz - 512), warp, 8);
+    __syncthreads();
+    if (tid < 128) {
+      const int i = kE + 128 * g + tid;  // row of the front
+      es[tid] = 128 * g + tid < b.nb ? shift(i < w ? P.sn_c0[gs] + i : P.rows[P.sn_rows[gs] + i - w]) : 0;
+      reinterpret_cast<int*>(o + b.grpex)[128 + tid] = es[tid];
+    }
+    __syncthreads();
+    dig_rows<4>(Shifted<PanelRow, false>{{Ls + (int64_t)kB * f + kE + 128 * g, f, false}, es}, b.K,
+                min(128, b.nb - 128 * g), 0, b.bp, o, 4, b.bp, reinterpret_cast<int*>(o + b.grpex), warp, 8);
   }
 }
 
@@ -237,19 +257,23 @@ __global__ void __launch_bounds__(kCT, 1)
         for (int g = 0; g < b.ng; ++g) {
           const int K = min(128, b.nb - 128 * g);
           const char* o = lt + b.grp + g * b.grpsz;
-          dig_rows<4>(GatherRow{V, ld, srow, c0, w, kE + 128 * g}, n, K, 0, 128, SL, 4, 128, EX, warp, kCT / 32);
-          BackJob<false> bj{SL, o, EX, reinterpret_cast<const int*>(o + b.grpsz - 512), (int64_t)4 * 128 * 64,
+          const int* ex = reinterpret_cast<const int*>(o + b.grpex);
+          dig_rows<4>(Shifted<GatherRow, true>{{V, ld, srow, c0, w, kE + 128 * g}, ex + 128}, n, K, 0, 128, SL, 4, 128,
+                      EX, warp, kCT / 32);
+          BackJob<false> bj{SL, o, EX, ex, (int64_t)4 * 128 * 64,
                             (int64_t)4 * b.bp * 64, (K + 31) / 32, n, b.bp, ntn, b.K, V + (int64_t)(c0 + kB) * ld, ld};
           dig_product(st, bj, 0, 1, ntn);
         }
         for (int sb = b.nck - 1; sb >= 0; --sb) {
           const int k0 = kB + 32 * sb, nbk = min(32, kE - k0);
-          dig_rows<1>(GatherRow{V, ld, srow, c0, w, k0}, n, nbk, 0, 128, SL, 1, 128, EX, warp, kCT / 32);
+          const Shifted<GatherRow, true> own{{V, ld, srow, c0, w, k0},
+                                             reinterpret_cast<const int*>(lt + b.piv) + 32 * sb};
+          dig_rows<1>(own, n, nbk, 0, 128, SL, 1, 128, EX, warp, kCT / 32);
           BackJob<true> sj{SL, lt + b.inv + sb * kDig * kCB, EX, reinterpret_cast<const int*>(lt + b.invex) + 32 * sb,
                            (int64_t)128 * 64, kCB, 1, n, 0, 1, nbk, V + (int64_t)(c0 + k0) * ld, ld};
           dig_product(st, sj, 0, 1, 1);
           if (sb > 0) {
-            dig_rows<1>(GatherRow{V, ld, srow, c0, w, k0}, n, nbk, 0, 128, SL, 1, 128, EX, warp, kCT / 32);
+            dig_rows<1>(own, n, nbk, 0, 128, SL, 1, 128, EX, warp, kCT / 32);
             const int nt = (32 * sb + 63) / 64;
             BackJob<false> uj{SL, lt + b.in + (int64_t)sb * kTRows * 64, EX, reinterpret_cast<const int*>(lt + b.inex),
                               (int64_t)128 * 64, (int64_t)b.nck * kTRows * 64, 1, n, kTRows, nt, 32 * sb,

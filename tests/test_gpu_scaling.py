@@ -78,3 +78,17 @@ def test_F(dim, physics, cuts):
         Fo = O.local_F(s, O.K_dense(s))
         assert np.linalg.norm(F - Fo) <= 1e-12 * np.linalg.norm(Fo)
     op.close()
+
+
+@pytest.mark.parametrize("dim,physics,cuts", CASES)
+def test_backward(dim, physics, cuts):
+    """The backward solve: F_i of the TRSM-path assembly, at the FP64 parity bar."""
+    P, Q, _, lam = problem(dim, physics, cuts)
+    op = feti.FetiOperator(Q, prec="fp64", chol_tc_front=128, route="trsm")
+    op.assemble()
+    for i, s in enumerate(P.subs):
+        l = lam[s.B_lambda]
+        F = op.get_F(i) * l[:, None] * l[None, :]
+        Fo = O.local_F(s, O.K_dense(s))
+        assert np.linalg.norm(F - Fo) <= 1e-12 * np.linalg.norm(Fo)
+    op.close()
