@@ -440,9 +440,9 @@ void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t 
     keep_it.push_back(items);
     CKS(cudaMemcpyAsync(ctx->d_adj_ent, keep_ent.back().data(), ents.size() * sizeof(DenseEnt), cudaMemcpyHostToDevice, st));
     CKS(cudaMemcpyAsync(ctx->d_adj_dit, keep_it.back().data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-    launch_dense_oz(ctx->d_adj_ent, (int)ents.size(), ctx->d_adj_dit, (int)items.size(), ctx->d_adj_work, ctx->d_adj_dig,
-                    ctx->d_adj_dex, ctx->d_adj_work, ctx->nsm, ctx->d_status, st);
-    ctx->stats.launches += 3;
+    launch_dense_oz(ctx->d_adj_ent, (int)ents.size(), ctx->d_adj_dit, (int)items.size(), ctx->P.spos, ctx->d_adj_work,
+                    ctx->d_adj_dig, ctx->d_adj_dex, ctx->d_adj_work, ctx->nsm, ctx->d_status, st);
+    ctx->stats.launches += 4;
     ents.clear();
     items.clear();
     bytes = nex = 0;
@@ -467,6 +467,9 @@ void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t 
       d.b = bytes + rows * rb;
       d.exa = nex;
       d.exb = nex + rows;
+      d.exs = d.exb + e.m;
+      d.z = e.v_ofs;
+      d.col0 = ctx->info[e.sub].col0;
       d.ld = ld;
       d.ldb = e.m_pad;
       d.rows = rows;
@@ -478,7 +481,7 @@ void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t 
           items.push_back(make_int4((int)ents.size(), bi | bj << 16, (int)((q + 3) / 4), 0));
       ents.push_back(d);
       bytes += wb + rows * rb;
-      nex += rows + e.m;
+      nex += rows + 2 * e.m;
       r0 += rows;
     }
   }

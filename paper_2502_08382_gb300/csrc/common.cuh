@@ -252,10 +252,13 @@ struct OzBatch {
 };
 
 // One dense FP64 product out = A B by exact slicing (launch_dense_oz): A rows x K (ld), B K x cols (ldb), row-major;
-// out has A's ld.  Offsets in doubles of A, B (source) and out, bytes of the digits, entries of the exponents.
+// out has A's ld.  Offsets in doubles of A, B (source) and out, bytes of the digits, entries of the exponents (exs: the K
+// shifts of the inner index).  The products are Z W of the adjoint: Z's rows start at `z`, its column a belongs to the
+// row spos[col0 + a], whose entry there is F_aa.
 struct DenseEnt {
   int64_t src_a, src_b, out, a, b;
-  int64_t exa, exb, ld, ldb;
+  int64_t exa, exb, exs, ld, ldb;
+  int64_t z, col0;
   int rows, cols, K, pieces;
 };
 

@@ -373,22 +373,41 @@ __global__ void __launch_bounds__(kOThreads, 1)
 
 // Row exponents and digits of the dense products' operands: A (rows x K, row-major, ld) and B^T (K x cols, row-major:
 // B's row c is its column c).  blockIdx.y = product.
+//
+// Shifts of the inner index a (oz.cuh), A's column a 2^-s_a against B's row a 2^s_a: column a of Z falls with the
+// stiffness of its multiplier's unknown as sqrt(F_aa) does, W is the caller's, so s_a takes half the difference of the
+// exponents of sqrt(F_aa) and of W's largest entry in row a.  (Not of Z's own largest entry: that would depend on how
+// many rows go together.)  One warp per a.
+__global__ void __launch_bounds__(256) dense_shift_kernel(const DenseEnt* ents, const int* spos, const double* src, int* EX) {
+  const DenseEnt e = ents[blockIdx.y];
+  const int lane = threadIdx.x % 32;
+  for (int a = (blockIdx.x * 256 + threadIdx.x) / 32; a < e.K; a += gridDim.x * 8) {
+    const double* b = src + e.src_b + (int64_t)a * e.ldb;
+    uint32_t mx = 0;
+    for (int j = lane; j < e.cols; j += 32) mx = max(mx, (uint32_t)__double2hiint(b[j]) & 0x7fffffffu);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) {
+      const double f = fabs(src[e.z + (int64_t)spos[e.col0 + a] * e.ld + a]);
+      EX[e.exs + a] = ((dig_pivot_shift(f) >> 1) - dig_pivot_shift(__hiloint2double((int)mx, 0))) >> 1;
+    }
+  }
+}
 __global__ void __launch_bounds__(256) dense_exp_kernel(const DenseEnt* ents, const double* src, int* EX) {
   const DenseEnt e = ents[blockIdx.y];
   const int lane = threadIdx.x % 32;
   for (int i = (blockIdx.x * 256 + threadIdx.x) / 32; i < e.rows; i += gridDim.x * 8) {
     const double* a = src + e.src_a + (int64_t)i * e.ld;
-    uint32_t mx = 0;
-    for (int k = lane; k < e.K; k += 32) mx = max(mx, (uint32_t)__double2hiint(a[k]) & 0x7fffffffu);
+    int mx = kKeyZero;
+    for (int k = lane; k < e.K; k += 32) mx = max(mx, dig_key(a[k], EX[e.exs + k]));
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) EX[e.exa + i] = dig_exponent(mx);
+    if (lane == 0) EX[e.exa + i] = dig_key_exponent(mx);
   }
   for (int c = blockIdx.x * 256 + threadIdx.x; c < e.cols; c += gridDim.x * 256) {
     const double* b = src + e.src_b + c;
-    uint32_t mx = 0;
+    int mx = kKeyZero;
 #pragma unroll 8
-    for (int k = 0; k < e.K; ++k) mx = max(mx, (uint32_t)__double2hiint(b[(int64_t)k * e.ldb]) & 0x7fffffffu);
-    EX[e.exb + c] = dig_exponent(mx);
+    for (int k = 0; k < e.K; ++k) mx = max(mx, dig_key(b[(int64_t)k * e.ldb], -EX[e.exs + k]));
+    EX[e.exb + c] = dig_key_exponent(mx);
   }
 }
 
@@ -408,14 +427,15 @@ __global__ void __launch_bounds__(256) dense_cut_kernel(const DenseEnt* ents, co
       const int i = (int)(u / e.pieces), q = (int)(u - (int64_t)i * e.pieces), ex = EX[e.exa + i];
       const double* a = src + e.src_a + (int64_t)i * e.ld + 8 * q;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) c[k] = dig_cut(8 * q + k < e.K ? a[k] : 0.0, ex);
+      for (int k = 0; k < 8; ++k) c[k] = 8 * q + k < e.K ? dig_cut(a[k], ex + EX[e.exs + 8 * q + k]) : 0;
       store_digits(reinterpret_cast<uint4*>(XD + e.a + ((int64_t)q * e.rows + i) * 128), c);
     } else {  // column fastest
       const int64_t v = u - na;
       const int q = (int)(v / e.cols), j = (int)(v - (int64_t)q * e.cols), ex = EX[e.exb + j];
       const double* b = src + e.src_b + (int64_t)8 * q * e.ldb + j;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) c[k] = dig_cut(8 * q + k < e.K ? b[(int64_t)k * e.ldb] : 0.0, ex);
+      for (int k = 0; k < 8; ++k)
+        c[k] = 8 * q + k < e.K ? dig_cut(b[(int64_t)k * e.ldb], ex - EX[e.exs + 8 * q + k]) : 0;
       store_digits(reinterpret_cast<uint4*>(XD + e.b + ((int64_t)q * e.cols + j) * 128), c);
     }
   }
@@ -436,10 +456,11 @@ void launch_syrk_oz(const DevPlan& P, const double* X, const OzBatch& b, const i
                                                                           (const char*)XD, b.x0, EX, F, status);
 }
 
-void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const double* src, void* XD, int* EX,
-                     double* out, int nsm, int* status, cudaStream_t st) {
+void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const int* spos, const double* src,
+                     void* XD, int* EX, double* out, int nsm, int* status, cudaStream_t st) {
   if (nent <= 0 || nitems <= 0) return;
   const dim3 g((unsigned)std::max(1, nsm * 16 / nent), (unsigned)nent);
+  dense_shift_kernel<<<g, 256, 0, st>>>(ents, spos, src, EX);
   dense_exp_kernel<<<g, 256, 0, st>>>(ents, src, EX);
   dense_cut_kernel<<<g, 256, 0, st>>>(ents, src, EX, (char*)XD);
   cudaFuncSetAttribute(syrk_oz_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kODyn);

@@ -57,8 +57,8 @@ void launch_dig_lt(const DevPlan& P, const int4* items, int nitems, void* LT, cu
 void launch_bsolve_oz(const DevPlan& P, const AdjBatch* B, const int2* items, int nitems, int* queue, const void* LT,
                       double* work, void* scratch, int grid, int* status, cudaStream_t st);
 // dense FP64 products by the same tiles; items (product, 128-row block | 64-column block << 16, 32-deep chunks, 0)
-void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const double* src, void* XD, int* EX,
-                     double* out, int nsm, int* status, cudaStream_t st);
+void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nitems, const int* spos, const double* src,
+                     void* XD, int* EX, double* out, int nsm, int* status, cudaStream_t st);
 // FP64 forward solve of the large fronts on the tensor cores (kern_trsm_oz.cu): digits of the large panels (items:
 // subdomain, supernode, first column of the 128-column block, its offset / 512), then, after launch_trsm with `hand`,
 // blocks of cw sorted columns (items: subdomain, first column); ws: per CTA front_sz + stack doubles

@@ -92,3 +92,21 @@ def test_backward(dim, physics, cuts):
         Fo = O.local_F(s, O.K_dense(s))
         assert np.linalg.norm(F - Fo) <= 1e-12 * np.linalg.norm(Fo)
     op.close()
+
+
+@pytest.mark.parametrize("physics,elems", [("elasticity", 7), ("heat", 13)])
+def test_adjoint(physics, elems):
+    """One subdomain with element matrices and weights scaled along, at the adjoint's parity bar (the gradient does not
+    change under the scaling)."""
+    P, Q, g, lam = problem(3, physics, [[elems]] * 3)
+    s, S = P.subs[0], g[P.subs[0].l2g]
+    W = make_W(P, seed=0)[0]
+    Se = S[s.elem_dofs]
+    Q = dataclasses.replace(Q, K_ref=np.asarray(P.K_ref)[None] * Se[:, :, None] * Se[:, None, :])
+    op = feti.FetiOperator(Q, prec="fp64", chol_tc_front=128, with_elements=True, per_element=True)
+    op.assemble()
+    l = lam[s.B_lambda]
+    grad = op.adjoint([W * l[:, None] * l[None, :]]).cpu().numpy()
+    op.close()
+    go = O.gradient_sub(s, W, P.K_ref, Kr=O.K_dense(s))
+    assert np.linalg.norm(grad - go) <= 1e-10 * np.linalg.norm(go)
