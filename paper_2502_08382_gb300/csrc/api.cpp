@@ -1191,6 +1191,10 @@ void build(feti_ctx* c) {
     // the apply deals tiles to warps round-robin; candidates of the autotuner:
     // every variant of the tile kernel at its full occupancy (capped at one tile per warp)
     c->d_tdesc = upload(c, tdesc);
+    if (!c->fp32) {
+      c->d_fscale = (int*)dalloc(c, (size_t)std::max<int64_t>(c->ncols, 1) * sizeof(int));
+      if (c->precond_kind == 2) c->d_mscale = (int*)dalloc(c, (size_t)std::max<int64_t>(c->ncols, 1) * sizeof(int));
+    }
     for (int v = 0; v < apply_variants(); ++v) {
       const int wpc = apply_warps_per_cta(v);
       const int occ = apply_max_ctas_per_sm(c->fp32, v);
@@ -1585,6 +1589,12 @@ feti_status feti_assemble(feti_ctx* ctx) {
       ctx->asm_th = ctx->d_th;
     }
   }
+  if (!ctx->fp32) {
+    launch_tile_scales(ctx->P, ctx->nsub, ctx->m_max, (const double*)ctx->d_F, ctx->d_fscale, st);
+    if (ctx->precond_kind == 2)
+      launch_tile_scales(ctx->P, ctx->nsub, ctx->m_max, (const double*)ctx->d_M, ctx->d_mscale, st);
+    ctx->stats.launches += ctx->precond_kind == 2 ? 2 : 1;
+  }
   CK(cudaGetLastError());
   ctx->stats.assembly_route = ctx->route;
   for (int k = 0; k < 3; ++k) ctx->stats.route_ms[k] = ctx->route_ms[k];
@@ -1638,7 +1648,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
         if (rep == 2) CK(cudaEventRecord(ctx->ev[5], st));
         launch_apply(ctx->P, ctx->fp32, ctx->d_tdesc, ctx->napply, ctx->d_F, ctx->P.qmap, ctx->ncols, pz,
                      ctx->d_pg, ctx->d_rowpart, ctx->d_tpart, ctx->d_blocks, ctx->nblocks, ctx->d_qi, ctx->d_c0,
-                     ctx->d_c1, ctx->nlam, qz, c2.grid, c2.variant, ctx->d_status, st);
+                     ctx->d_c1, ctx->nlam, qz, c2.grid, c2.variant, ctx->d_fscale, ctx->d_status, st);
       }
       CK(cudaEventRecord(ctx->ev[6], st));
       CK(cudaEventSynchronize(ctx->ev[6]));
@@ -1677,7 +1687,7 @@ feti_status feti_apply(feti_ctx* ctx, const double* p_dev, double* q_dev) {
   }
   launch_apply(ctx->P, ctx->fp32, ctx->d_tdesc, ctx->napply, ctx->d_F, ctx->P.qmap, ctx->ncols, p_dev, ctx->d_pg,
                ctx->d_rowpart, ctx->d_tpart, ctx->d_blocks, ctx->nblocks, ctx->d_qi, ctx->d_c0, ctx->d_c1, ctx->nlam,
-               q_dev, grid, cand.variant, ctx->d_status, st, ev.b, ev.c);
+               q_dev, grid, cand.variant, ctx->d_fscale, ctx->d_status, st, ev.b, ev.c);
   ctx->stats.launches += 3;
   ctx->stats.apply_calls += 1;
   if (ctx->prof) {

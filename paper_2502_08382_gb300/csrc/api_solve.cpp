@@ -118,7 +118,7 @@ void enqueue_precond(feti_ctx* c, int mode, cudaStream_t st) {
     const auto& cand = c->apply_cands[c->apply_pick];
     launch_dir_pre(c->fp32, n, c->d_w_off, c->d_w_col, c->d_w_val, w, c->d_c0, c->d_c1, c->d_pg2, ctrl, iter, st);
     launch_apply_core(c->fp32, c->d_tdesc, c->napply, c->d_M, c->d_pg2, c->d_rowpart, c->d_tpart, cand.grid,
-                      cand.variant, iter ? active_dev(c) : nullptr, c->d_status, st);
+                      cand.variant, c->d_mscale, iter ? active_dev(c) : nullptr, c->d_status, st);
     launch_dir_mid(c->fp32, c->d_lamcol, n, c->d_rowpart, c->d_tpart, vec(c, V_U), ctrl, iter, st);
     launch_dir_post(n, c->d_w_off, c->d_w_col, c->d_w_val, vec(c, V_U), v, ctrl, iter, st);
   } else {
@@ -147,7 +147,7 @@ void enqueue_iteration(feti_ctx* c, double* lam, const cudaEvent_t* ev, cudaStre
   const auto& cand = c->apply_cands[c->apply_pick];
   if (ev) CKS(cudaEventRecordWithFlags(ev[0], st, evf));
   launch_apply_core(c->fp32, c->d_tdesc, c->napply, c->d_F, c->d_pg, c->d_rowpart, c->d_tpart, cand.grid,
-                    cand.variant, active_dev(c), c->d_status, st, ev ? ev[1] : nullptr, ev ? ev[2] : nullptr, capture);
+                    cand.variant, c->d_fscale, active_dev(c), c->d_status, st, ev ? ev[1] : nullptr, ev ? ev[2] : nullptr, capture);
   launch_pcg_gather_dot(c->fp32, c->d_lamcol, c->d_c0, c->d_c1, n, c->d_rowpart, c->d_tpart, p, y, qk, c->d_qcol,
                         c->d_part, ctrl, st);
   if (ev) CKS(cudaEventRecordWithFlags(ev[3], st, evf));

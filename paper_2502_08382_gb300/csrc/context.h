@@ -129,6 +129,7 @@ struct feti_ctx {
   size_t xd_bytes = 0;
   int* d_oz_ex = nullptr;
   feti::TileDesc* d_tdesc = nullptr;
+  int *d_fscale = nullptr, *d_mscale = nullptr;  // FP64: scales of the F tiles (and of the Dirichlet M tiles)
   struct ApplyCand {
     int variant, grid;  // tile-kernel variant (load batch) and grid
     double ms;

@@ -543,7 +543,8 @@ void launch_ring(int grid, cudaStream_t st, const TileDesc* desc, int ntiles, co
 
 template <typename TF>
 void launch_tiles(int variant, int grid, cudaStream_t st, const TileDesc* desc, int ntiles, const TF* F,
-                  const TF* pg, TF* rowpart, TF* colpart, const int* active = nullptr, int* status = nullptr) {
+                  const TF* pg, TF* rowpart, TF* colpart, const int* active = nullptr, int* status = nullptr,
+                  const int* scale = nullptr) {
   if (ntiles <= 0) return;
   switch (variant) {
     case 0:
@@ -562,7 +563,7 @@ void launch_tiles(int variant, int grid, cudaStream_t st, const TileDesc* desc, 
     case 4: launch_ring<TF, 8, 3>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
     case 5: launch_ring<TF, 2, 6>(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status); break;
     default:
-      if constexpr (sizeof(TF) == 8) launch_apply_dig(grid, st, desc, ntiles, F, pg, rowpart, colpart, active, status);
+      if constexpr (sizeof(TF) == 8) launch_apply_dig(grid, st, desc, ntiles, F, pg, scale, rowpart, colpart, active, status);
       break;
   }
 }
@@ -580,12 +581,12 @@ template <typename TF>
 static void launch_apply_t(const DevPlan& P, const TileDesc* desc, int ntiles, const void* F, const int* qmap,
                            int64_t ncols, const double* p, void* pg, void* rowpart, void* colpart, const int2* blocks,
                            int nblocks, double* qi, const int* c0, const int* c1, int nlam, double* q, int grid,
-                           int variant, int* status, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
+                           int variant, const int* scale, int* status, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
   const int sg = (int)std::max<int64_t>(1, std::min<int64_t>((ncols + 255) / 256, 152 * 8));
   scatter_kernel<TF><<<sg, 256, 0, st>>>(qmap, ncols, p, (TF*)pg);
   if (e0) cudaEventRecord(e0, st);
   launch_tiles<TF>(variant, grid, st, desc, ntiles, (const TF*)F, (const TF*)pg, (TF*)rowpart, (TF*)colpart, nullptr,
-                   status);
+                   status, scale);
   if (e1) cudaEventRecord(e1, st);
   const int gg = std::max(1, std::min((nlam + 255) / 256, 152 * 8));
   gather_tiles_kernel<TF><<<gg, 256, 0, st>>>(P, P.colsub, c0, c1, nlam, (const TF*)rowpart, (const TF*)colpart, q);
@@ -599,13 +600,13 @@ void launch_gather_lambda(const int* c0, const int* c1, int nlam, const double* 
 void launch_apply(const DevPlan& P, bool fp32, const TileDesc* desc, int ntiles, const void* F, const int* qmap,
                   int64_t ncols, const double* p, void* pg, void* rowpart, void* colpart, const int2* blocks,
                   int nblocks, double* qi, const int* c0, const int* c1, int nlam, double* q, int grid, int variant,
-                  int* status, cudaStream_t st, cudaEvent_t ev_tiles0, cudaEvent_t ev_tiles1) {
+                  const int* scale, int* status, cudaStream_t st, cudaEvent_t ev_tiles0, cudaEvent_t ev_tiles1) {
   if (fp32)
     launch_apply_t<float>(P, desc, ntiles, F, qmap, ncols, p, pg, rowpart, colpart, blocks, nblocks, qi, c0, c1,
-                          nlam, q, grid, variant, status, st, ev_tiles0, ev_tiles1);
+                          nlam, q, grid, variant, scale, status, st, ev_tiles0, ev_tiles1);
   else
     launch_apply_t<double>(P, desc, ntiles, F, qmap, ncols, p, pg, rowpart, colpart, blocks, nblocks, qi, c0, c1,
-                           nlam, q, grid, variant, status, st, ev_tiles0, ev_tiles1);
+                           nlam, q, grid, variant, scale, status, st, ev_tiles0, ev_tiles1);
 }
 
 // The F-streaming part of the apply for the projected CG, whose scatter and
@@ -613,7 +614,8 @@ void launch_apply(const DevPlan& P, bool fp32, const TileDesc* desc, int ntiles,
 // partials itself); skipped when *active == 0 (an iteration enqueued after
 // the solve has stopped).
 void launch_apply_core(bool fp32, const TileDesc* desc, int ntiles, const void* F, const void* pg, void* rowpart,
-                       void* colpart, int grid, int variant, const int* active, int* status, cudaStream_t st,
+                       void* colpart, int grid, int variant, const int* scale, const int* active, int* status,
+                       cudaStream_t st,
                        cudaEvent_t ev_tiles0, cudaEvent_t ev_tiles1, bool ev_external) {
   // under stream capture only an external record becomes a timed event-record node
   const unsigned evf = ev_external ? cudaEventRecordExternal : cudaEventRecordDefault;
@@ -624,7 +626,7 @@ void launch_apply_core(bool fp32, const TileDesc* desc, int ntiles, const void* 
     if (ev_tiles1) cudaEventRecordWithFlags(ev_tiles1, st, evf);
   } else {
     launch_tiles<double>(variant, grid, st, desc, ntiles, (const double*)F, (const double*)pg, (double*)rowpart,
-                         (double*)colpart, active, status);
+                         (double*)colpart, active, status, scale);
     if (ev_tiles1) cudaEventRecordWithFlags(ev_tiles1, st, evf);
   }
 }

@@ -20,7 +20,14 @@
 //            accumulator per 16 columns collects digit sums d = p + q <= 7 (at most 8 16 2^14 = 2^21, exact); the four
 //            strips' partials are added in FP64 in a fixed order.
 // Strips or vectors that hold an infinity or NaN take plain FP64 FMAs (slow_strip), so those propagate as before.
+//
+// Scales.  F_ij is at most sqrt(F_ii F_jj), which may differ by many decades between the rows of a strip (a stiff and a
+// soft material), so the tile is cut as F_ij 2^-(s_i + s_j) with s_i half the exponent of F_ii (tile_scales_kernel,
+// once per assembly) and p as p_j 2^s_j: 62 bits below the largest scaled entry are then far below what FP64 can know of
+// F_ij itself, u sqrt(F_ii F_jj).  The scales only enter the exponents of the cut and of the results.
 #include <cuda_fp16.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -33,10 +40,27 @@ constexpr int kDT = 128;
 constexpr int kTileBytes = kT * kT * 8;
 constexpr int kDDyn = 2 * kTileBytes + 128;  // two tile buffers
 
-// exponent e with |x| < 2^e; kExpBad for infinities, NaN, and values too small for the cut below
-__device__ __forceinline__ int strip_exponent(uint32_t hi_max) {
-  const int be = (int)(hi_max >> 20);
-  return be == 0x7FF || (be < 72 && hi_max) ? kExpBad : max(be - 1022, -950);
+// Exponent e of a strip or vector from its largest key (biased exponent less the scales, which are within kMaxScale
+// each): 0 if all entries are zero, kExpBad for infinities, NaN, and entries too small or too large for the cut below.
+constexpr int kMaxScale = 400;
+__device__ __forceinline__ int scaled_exponent(int key, int least, int bad, bool zero) {
+  return key >= least && key < bad ? key - 1022 : key < least && zero ? 0 : kExpBad;
+}
+constexpr int kBadF = 2047 - 2 * kMaxScale, kLeastF = 923, kLeastP = 522;  // least: so that e + s_i + s_j and e - s_j are at least -950 (zeros shift out)
+
+// s_j of every sorted column from the diagonal of the FP64 tiles (0 for padding and for entries not positive)
+__global__ void __launch_bounds__(256) tile_scales_kernel(DevPlan P, int nsub, const double* F, int* scale) {
+  for (int si = blockIdx.y; si < nsub; si += gridDim.y) {
+    const SubInfo& S = P.sub[si];
+    for (int j = blockIdx.x * 256 + threadIdx.x; j < S.m_pad; j += gridDim.x * 256) {
+      int s = 0;
+      if (j < S.m) {
+        const int b = j / kT, r = j % kT;
+        s = dig_pivot_shift(F[S.F + tile_offset<8>(S.nb, S.vr, b, b) + diag_pos<8>(r, r)]) >> 1;
+      }
+      scale[S.qcol + j] = max(-kMaxScale, min(kMaxScale, s));
+    }
+  }
 }
 
 // The digits of x (|x| < 2^e, e >= -950) plus 128 as bytes, digit 0 in the top byte: x cut (not rounded) to 62
@@ -94,13 +118,15 @@ __device__ void slow_strip(const TileDesc& d, const double* F, const double* pg,
 
 __global__ void __launch_bounds__(kDT, 3)
     apply_dig_kernel(const TileDesc* __restrict__ desc, int ntiles, const double* __restrict__ F,
-                     const double* __restrict__ pg, double* rowpart, double* colpart, const int* active, int* status) {
+                     const double* __restrict__ pg, const int* __restrict__ scale, double* rowpart, double* colpart,
+                     const int* active, int* status) {
   if (active && *active == 0) return;  // the iteration this launch belongs to has stopped
   extern __shared__ uint8_t ad_raw[];
   // bytes 8 .. 15: the digits of p (column block, then row block) plus 128; bytes 0 .. 7: 128 (a zero digit)
   __shared__ __align__(16) uint8_t pd[2 * kT][16];
   __shared__ double cs[4][kT], dgs[kT];
-  __shared__ uint32_t mx_s[4];
+  __shared__ int mx_s[4];
+  __shared__ __align__(16) int sx[2 * kT];  // scales of the column block, then of the row block
   __shared__ uint64_t full[2];
   uint8_t* buf = ad_raw + ((128u - (smem_u32(ad_raw) & 127u)) & 127u);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane / 4, t = lane % 4;
@@ -130,20 +156,27 @@ __global__ void __launch_bounds__(kDT, 3)
     fetch(blockIdx.x, 0);
     if (blockIdx.x + gridDim.x < ntiles) fetch(blockIdx.x + gridDim.x, 1);
   }
+  auto sval = [&](const TileDesc& d) {
+    return tid < kT ? scale[d.pcol + tid] : (tid - kT < d.rows ? scale[d.prow + tid - kT] : 0);
+  };
   TileDesc dn = desc[blockIdx.x];
   double pn = pval(dn);
+  int sn = sval(dn);
   int it = 0;
   bool ok_all = true;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
     const TileDesc d = dn;
     const double pv = pn;
+    const int sv = sn;
     if (tile + (int)gridDim.x < ntiles) {
       dn = desc[tile + gridDim.x];
       pn = pval(dn);
+      sn = sval(dn);
     }
     const bool diag = (d.flags & kTileDiag) != 0;
-    const uint32_t pm = __reduce_max_sync(0xffffffffu, (uint32_t)__double2hiint(pv) & 0x7fffffffu);
+    const int pm = __reduce_max_sync(0xffffffffu, dig_key(pv, -sv));
     if (lane == 0) mx_s[warp] = pm;
+    sx[tid] = sv;
     const double* Ft = reinterpret_cast<const double*>(buf + (it & 1) * kTileBytes);
     // every lane waits, so that each one sees the copied bytes
     ok_all = ok_all && mbar_wait(smem_u32(&full[it & 1]), (it >> 1) & 1);
@@ -169,20 +202,38 @@ __global__ void __launch_bounds__(kDT, 3)
           f[kb][j] = v;
         }
     }
+    if (diag && tid < kT && tid < d.rows) dgs[tid] = Ft[diag_row_off<8>(tid) + tid];
+    __syncthreads();
+    const int si[2] = {sx[kT + r0], sx[kT + r0 + 8]};
+    // the largest scaled entry: high words less the scales, 1024 exponents up so that they stay positive
     uint32_t fm = 0;
 #pragma unroll
     for (int kb = 0; kb < 4; ++kb)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        fm = max(fm, max((uint32_t)__double2hiint(f[kb][j].x) & 0x7fffffffu,
-                         (uint32_t)__double2hiint(f[kb][j].y) & 0x7fffffffu));
-    if (diag && tid < kT && tid < d.rows) dgs[tid] = Ft[diag_row_off<8>(tid) + tid];
-    const int ef = strip_exponent(__reduce_max_sync(0xffffffffu, fm));
-    __syncthreads();
-    const int epc = strip_exponent(max(mx_s[0], mx_s[1])), epr = strip_exponent(max(mx_s[2], mx_s[3]));
+      for (int j = 0; j < 4; ++j) {
+        const int2 sj = *reinterpret_cast<const int2*>(&sx[16 * kb + 2 * t + 8 * (j >> 1)]);
+        const uint32_t c = (uint32_t)(1024 - si[j & 1]) << 20;
+        fm = max(fm, max(((uint32_t)__double2hiint(f[kb][j].x) & 0x7fffffffu) + c - ((uint32_t)sj.x << 20),
+                         ((uint32_t)__double2hiint(f[kb][j].y) & 0x7fffffffu) + c - ((uint32_t)sj.y << 20)));
+      }
+    const int fkey = (int)(__reduce_max_sync(0xffffffffu, fm) >> 20) - 1024;
+    bool fzero = false;
+    if (fkey < kLeastF) {  // all zero, or tiny against the diagonal
+      uint32_t z = 0;
+#pragma unroll
+      for (int kb = 0; kb < 4; ++kb)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          z |= ((uint32_t)__double2hiint(f[kb][j].x) | (uint32_t)__double2hiint(f[kb][j].y)) & 0x7fffffffu;
+      fzero = __reduce_or_sync(0xffffffffu, z) == 0;
+    }
+    const int ef = scaled_exponent(fkey, kLeastF, kBadF, fzero);
+    const int kpc = max(mx_s[0], mx_s[1]), kpr = max(mx_s[2], mx_s[3]);
+    const int epc = scaled_exponent(kpc, kLeastP, kKeyBad, kpc == kKeyZero);
+    const int epr = scaled_exponent(kpr, kLeastP, kKeyBad, kpr == kKeyZero);
     {
       const int e = tid < kT ? epc : epr;
-      const uint64_t w = e == kExpBad ? 0 : dig_bytes(pv, e);
+      const uint64_t w = e == kExpBad ? 0 : dig_bytes(pv, e - sv);
       const uint32_t hi = (uint32_t)(w >> 32), lo = (uint32_t)w;
       *reinterpret_cast<uint4*>(pd[tid]) = make_uint4(0x80808080u, 0x80808080u, __byte_perm(hi, 0, 0x0123),
                                                       __byte_perm(lo, 0, 0x0123));
@@ -213,8 +264,9 @@ __global__ void __launch_bounds__(kDT, 3)
         uint64_t wx[4], wy[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          wx[j] = dig_bytes(f[kb][j].x, ef);
-          wy[j] = dig_bytes(f[kb][j].y, ef);
+          const int2 sj = *reinterpret_cast<const int2*>(&sx[16 * kb + 2 * t + 8 * (j >> 1)]);
+          wx[j] = dig_bytes(f[kb][j].x, ef + si[j & 1] + sj.x);
+          wy[j] = dig_bytes(f[kb][j].y, ef + si[j & 1] + sj.y);
         }
         float ca[4] = {};
 #pragma unroll
@@ -243,7 +295,8 @@ __global__ void __launch_bounds__(kDT, 3)
         const int got = __shfl_xor_sync(0xffffffffu, give, 1);
         const long long pr = (t & 1) ? (long long)got * 65536 + mine : (long long)mine * 65536 + got;
         const long long ot = __shfl_xor_sync(0xffffffffu, pr, 2);
-        const double yv = dig_value((t & 2) ? ot : pr, (t & 2) ? pr : ot, ef + epr - 68);
+        const double yv = dig_value((t & 2) ? ot : pr, (t & 2) ? pr : ot,
+                                    ef + epr - 68 + sx[16 * kb + g + 8 * (t & 1)]);
         if (t < 2) cs[warp][16 * kb + g + 8 * (t & 1)] = yv;
       }
       // rows g (acc[p][0], [1]) and g + 8 (acc[p][2], [3]): digit columns q = 2 t and 2 t + 1
@@ -256,7 +309,7 @@ __global__ void __launch_bounds__(kDT, 3)
           u[j] = (j < 8 ? __float2int_rn(acc[j][2 * h]) : 0) + (j > 0 ? __float2int_rn(acc[j - 1][2 * h + 1]) : 0);
         const long long hi = ((long long)(u[0] * 256 + u[1]) * 65536 + (u[2] * 256 + u[3])) * 256 + u[4];
         const long long lo = (long long)(u[5] * 256 + u[6]) * 65536 + (u[7] * 256 + u[8]);
-        rs[h] = dig_value(hi, lo, ef + epc - 76 - 16 * t);
+        rs[h] = dig_value(hi, lo, ef + epc - 76 - 16 * t + si[h]);
       }
       // lanes t = 0, 2 add up row g, t = 1, 3 row g + 8
       double s = (t & 1) ? rs[1] : rs[0];
@@ -279,9 +332,14 @@ __global__ void __launch_bounds__(kDT, 3)
 }  // namespace
 
 void launch_apply_dig(int grid, cudaStream_t st, const TileDesc* desc, int ntiles, const double* F, const double* pg,
-                      double* rowpart, double* colpart, const int* active, int* status) {
+                      const int* scale, double* rowpart, double* colpart, const int* active, int* status) {
   cudaFuncSetAttribute(apply_dig_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDDyn);
-  apply_dig_kernel<<<grid, kDT, kDDyn, st>>>(desc, ntiles, F, pg, rowpart, colpart, active, status);
+  apply_dig_kernel<<<grid, kDT, kDDyn, st>>>(desc, ntiles, F, pg, scale, rowpart, colpart, active, status);
+}
+
+void launch_tile_scales(const DevPlan& P, int nsub, int m_max, const double* F, int* scale, cudaStream_t st) {
+  const dim3 g((unsigned)std::max(1, std::min((m_max + kT + 255) / 256, 64)), (unsigned)std::max(1, std::min(nsub, 32768)));
+  tile_scales_kernel<<<g, 256, 0, st>>>(P, nsub, F, scale);
 }
 
 int apply_dig_occupancy() {

@@ -71,16 +71,18 @@ void launch_trsm_oz(const DevPlan& P, const int2* items, int nitems, int cw, int
 // chunks of the tile whose contributing supernodes have np[0 .. n) 8-row pieces (the loaders' batching)
 int syrk_oz_chunks(const int* np, int n);
 
-// ev_tiles0/1: optional events recorded just before / after the F-streaming kernel
+// scale: of the FP64 tiles (launch_tile_scales); ev_tiles0/1: optional events recorded just before / after the F-streaming kernel
 void launch_apply(const DevPlan& P, bool fp32, const TileDesc* desc, int ntiles, const void* F, const int* qmap,
                   int64_t ncols, const double* p, void* pg, void* rowpart, void* colpart, const int2* blocks,
                   int nblocks, double* qi, const int* c0, const int* c1, int nlam, double* q, int grid, int variant,
-                  int* status, cudaStream_t st, cudaEvent_t ev_tiles0 = nullptr, cudaEvent_t ev_tiles1 = nullptr);
+                  const int* scale, int* status, cudaStream_t st, cudaEvent_t ev_tiles0 = nullptr, cudaEvent_t ev_tiles1 = nullptr);
 void launch_apply_core(bool fp32, const TileDesc* desc, int ntiles, const void* F, const void* pg, void* rowpart,
-                       void* colpart, int grid, int variant, const int* active, int* status, cudaStream_t st,
-                       cudaEvent_t ev_tiles0 = nullptr, cudaEvent_t ev_tiles1 = nullptr, bool ev_external = false);
+                       void* colpart, int grid, int variant, const int* scale, const int* active, int* status,
+                       cudaStream_t st, cudaEvent_t ev_tiles0 = nullptr, cudaEvent_t ev_tiles1 = nullptr, bool ev_external = false);
 void launch_apply_dig(int grid, cudaStream_t st, const TileDesc* desc, int ntiles, const double* F, const double* pg,
-                      double* rowpart, double* colpart, const int* active, int* status);
+                      const int* scale, double* rowpart, double* colpart, const int* active, int* status);
+// the scales of the FP64 tiles' rows and columns (variant 6), whenever the tiles are new
+void launch_tile_scales(const DevPlan& P, int nsub, int m_max, const double* F, int* scale, cudaStream_t st);
 int apply_dig_occupancy();
 int apply_variants();
 int apply_max_ctas_per_sm(bool fp32, int variant);

@@ -110,3 +110,49 @@ def test_adjoint(physics, elems):
     op.close()
     go = O.gradient_sub(s, W, P.K_ref, Kr=O.K_dense(s))
     assert np.linalg.norm(grad - go) <= 1e-10 * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("kernel", [0, 6])
+@pytest.mark.parametrize("dim,physics,cuts", CASES + [(2, "heat", [[31, 34], [34, 31]])])
+def test_apply(dim, physics, cuts, kernel):
+    """The explicit apply against its own F_i.  Bar: n 2^-52 (|F| |p|)_l for FP64 sums in any order; the tile kernel by
+    digits has F_ij / (s_i s_j) below 4 and p_j s_j below sqrt(F_jj) |p_j| (s_j = 2^floor(log2 F_jj / 2)), each cut to
+    within 2^-62 of the next power of two above its largest and multiplied without the pairs p + q >= 8 (7.1 2^-62 at
+    most): below 2^-55 sqrt(F_ll) max_j sqrt(F_jj) |p_j| a product."""
+    P, Q, _, lam = problem(dim, physics, cuts)
+    op = feti.FetiOperator(Q, prec="fp64", apply_kernel=kernel)
+    op.assemble()
+    Fs = [op.get_F(i) * lam[s.B_lambda][:, None] * lam[s.B_lambda] for i, s in enumerate(P.subs)]
+    rng = np.random.default_rng(4)
+    for k in range(3):
+        p = rng.normal(size=P.n_lambda)
+        if k == 1:
+            p *= np.exp2(rng.integers(-30, 30, size=P.n_lambda))
+        if k == 2:
+            p[rng.random(P.n_lambda) < 0.95] = 0.0
+        q = op.apply(torch.from_numpy(p * lam).cuda()).cpu().numpy() * lam
+        ref, bar = np.zeros_like(q), np.zeros_like(q)
+        for s, F in zip(P.subs, Fs):
+            l = np.asarray(s.B_lambda, dtype=np.int64)
+            ref[l] += F @ p[l]
+            d = np.sqrt(np.diag(F))
+            bar[l] += (s.m + 8) * (2.0 ** -52 * (np.abs(F) @ np.abs(p[l])) + 2.0 ** -55 * d * (d * np.abs(p[l])).max())
+        assert np.all(np.abs(q - ref) <= bar)
+    op.close()
+
+
+def test_dirichlet_tiles():
+    """The Dirichlet preconditioner's tiles by either tile kernel: the same solution at the solve's tolerance."""
+    P = make_problem(dim=2, physics="heat", cuts=[[12, 9], [9, 12]], material="lognormal", sigma=1.0, seed=2)
+    um = O.monolithic_solve(P)
+    for kernel in (0, 6):
+        op = feti.FetiOperator(P, prec="fp64", route="schur", precond="dirichlet", apply_kernel=kernel, tol=1e-12)
+        op.assemble()
+        u, info = op.solve()[2:]
+        u = u.cpu().numpy()
+        op.close()
+        assert info["converged"]
+        off = 0
+        for s in P.subs:
+            assert np.abs(u[off:off + s.n] - um[s.l2g]).max() <= 1e-10 * np.abs(um).max()
+            off += s.n
