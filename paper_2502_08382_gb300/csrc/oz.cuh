@@ -112,8 +112,8 @@ __device__ __forceinline__ double dig_value(long long hi, long long lo, int ex) 
   const unsigned long long mant = (m >> 11) + ((m >> 10) & 1);  // 53 bits, 2^52 <= mant <= 2^53
   const int e = 95 - lz + ex;                                   // value = mant 2^(e - 52)
   unsigned long long b = ((unsigned long long)(e + 1022) << 52) + mant;
-  if (h == 0 || e < -1021) b = 0;
-  if (h != 0 && e > 1022) b = 0x7FF0000000000000ULL;
+  if (h == 0 || e < -1022) b = 0;  // subnormal results are flushed
+  if (h != 0 && e > 1023) b = 0x7FF0000000000000ULL;  // (e = 1023 rounds up to infinity by itself)
   return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ULL : 0ULL)));
 }
 

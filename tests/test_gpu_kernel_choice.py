@@ -96,3 +96,23 @@ def test_refused_options():
     for kw in ({"implicit_cluster": 3}, {"implicit_cluster": 16}, {"apply_kernel": 7}, {"apply_kernel": 6, "prec": "tf32"}):
         with pytest.raises(feti.FetiError):
             feti.FetiOperator(P, **kw)
+
+
+@pytest.mark.parametrize("kernel", [0, 6])
+def test_apply_top_binade(kernel):
+    """Results between 2^1023 and the largest FP64 number are finite: column j of F, scaled by a power of two that takes
+    its largest off-diagonal entry there (one product an entry: exact up to the tiles' cut, 2^-55 max |F|)."""
+    P = make_problem(dim=2, physics="heat", cuts=[[30], [30]], material="lognormal", sigma=0.5)
+    op = feti.FetiOperator(P, prec="fp64", apply_kernel=kernel)
+    op.assemble()
+    F, j = op.get_F(0), P.n_lambda // 2
+    off = np.delete(F[:, j], j)
+    k = 1023 - int(np.floor(np.log2(np.abs(off).max())))
+    p = np.zeros(P.n_lambda)
+    p[j] = 2.0 ** k if k < 1024 else 2.0 ** 1023
+    q = np.delete(op.apply(torch.from_numpy(p).cuda()).cpu().numpy(), j)
+    op.close()
+    assert np.isfinite(q).all()
+    assert np.abs(q / p[j] - off).max() <= 2.0 ** -55 * np.abs(F).max()
+    if k < 1024:
+        assert np.abs(q).max() >= 2.0 ** 1023
