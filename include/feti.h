@@ -186,6 +186,9 @@ typedef struct {
   int32_t assembly_route;     /* route of the last feti_assemble (0 SYRK path, 1 Schur complement, 2 TRSM path) */
   double route_ms[3];         /* route 3: time of the TRSM + SYRK (0) and of the TRSM path (2) at the first call */
   int32_t implicit_cluster;   /* CTAs per subdomain of the implicit solves (-1: one of 256 threads) */
+  int32_t digit_kernels;      /* FP64: kernels of the last feti_assemble that ran by exact slicing on the tensor
+                                 cores: 1 the SYRK, 2 the large fronts' forward solve (where their digits find
+                                 no memory, or there are no large fronts, the FP64 pipe does the work) */
 } feti_stats;
 
 typedef struct feti_ctx feti_ctx;

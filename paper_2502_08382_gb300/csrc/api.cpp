@@ -247,34 +247,45 @@ void plan_syrk_oz(feti_ctx* c, size_t budget) {
   c->xd_bytes = most;
 }
 
-// The digit buffer: as many subdomains at a time as a fifth of the free memory holds (16 GB at most), fewer if the
-// allocator refuses; false when not even one subdomain fits (the FP64-pipe kernel takes over).
+// The digit buffer: as many subdomains at a time as a fifth of the free memory holds (16 GB at most), one at a time if
+// the allocator refuses that; false when not even one subdomain fits (the FP64-pipe kernel takes over).  The memory comes
+// first and the plan after it, so a refusal leaves the plan and the recorded assembly as they are; it is not asked for
+// again before that much more memory is free (recompute_X: asked for at every assembly, as X is).
 bool reserve_syrk_oz(feti_ctx* c) {
   if (c->d_XD) return true;
-  if (!c->oz_batches.empty()) {  // released after the previous assembly (recompute_X)
-    try {
-      c->d_XD = dalloc(c, c->xd_bytes);
-      return true;
-    } catch (std::bad_alloc&) {
-    }
-  }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  size_t want = 0;
-  for (int i = 0; i < c->nsub; ++i) want += 16 * (size_t)c->bps[c->subs[i].bp].Xsize;
-  const size_t budget = std::min(want, std::min<size_t>((size_t)16 << 30, free_b / 5));
-  for (size_t b : {budget, (size_t)0}) {
-    try {
-      plan_syrk_oz(c, b);
-      c->d_XD = dalloc(c, c->xd_bytes);
-      if (!c->d_oz_ex) c->d_oz_ex = (int*)dalloc(c, (size_t)std::max<int64_t>(c->ncols, 1) * sizeof(int));
-      return true;
-    } catch (std::bad_alloc&) {
-      dfree(c, c->d_XD);
-      c->d_XD = nullptr;
-      c->oz_batches.clear();  // planned anew by the next assembly
-    }
+  size_t want = 0, least = 0;
+  for (int i = 0; i < c->nsub; ++i) {
+    const size_t x = 16 * (size_t)c->bps[c->subs[i].bp].Xsize;
+    want += x;
+    least = std::max(least, x);
   }
+  if (!c->opt.recompute_X && c->xd_refused > 0 && free_b < c->xd_refused + least) return false;
+  auto take = [&](size_t bytes) {
+    try {
+      c->d_XD = dalloc(c, bytes);
+    } catch (std::bad_alloc&) {
+      c->d_XD = nullptr;
+    }
+    return c->d_XD != nullptr;
+  };
+  try {
+    if (!c->d_oz_ex) c->d_oz_ex = (int*)dalloc(c, (size_t)std::max<int64_t>(c->ncols, 1) * sizeof(int));
+    // the plan at hand first (its buffer was released by recompute_X)
+    if (!c->oz_batches.empty() && take(c->xd_bytes)) return true;
+    const size_t budget = std::min(want, std::min<size_t>((size_t)16 << 30, free_b / 5));
+    for (size_t b : {budget, (size_t)0})
+      if (take(std::max(b, least))) {
+        plan_syrk_oz(c, b);
+        return true;
+      }
+  } catch (std::bad_alloc&) {  // of the small lists
+    dfree(c, c->d_XD);
+    c->d_XD = nullptr;
+    c->oz_batches.clear();
+  }
+  c->xd_refused = std::max<size_t>(free_b, 1);
   return false;
 }
 
@@ -1529,6 +1540,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
   if (tx)
     for (const auto& b : ctx->tx_batches) ctx->stats.launches += b.nitems > 0 ? 2 : 0;
   if (oz) ctx->stats.launches += 3 * (int64_t)ctx->oz_batches.size() - 1;
+  ctx->stats.digit_kernels = (oz ? 1 : 0) | (tx ? 2 : 0);
   const int want = ctx->opt.assembly_route;
   if (want == 2 || (want == 3 && ctx->route_tuned && ctx->route == 2)) {
     ctx->route = 2;

@@ -126,7 +126,8 @@ struct feti_ctx {
   int4* d_oz_items = nullptr;
   int4* d_oz_ditems = nullptr;
   void* d_XD = nullptr;
-  size_t xd_bytes = 0;
+  size_t xd_bytes = 0;       // of the plan's largest batch
+  size_t xd_refused = 0;     // free memory when the digits were last refused (0: never)
   int* d_oz_ex = nullptr;
   feti::TileDesc* d_tdesc = nullptr;
   int *d_fscale = nullptr, *d_mscale = nullptr;  // FP64: scales of the F tiles (and of the Dirichlet M tiles)

@@ -73,7 +73,7 @@ class FetiStats(C.Structure):
                 ("apply_tiles_ms", C.c_double), ("implicit_calls", C.c_int64), ("implicit_ms", C.c_double),
                 ("apply_variant", C.c_int32), ("apply_grid", C.c_int32), ("trsm_cols", C.c_int32),
                 ("trsm_grid", C.c_int32), ("chol_tasks", C.c_int32), ("syrk_variant", C.c_int32), ("assembly_route", C.c_int32),
-                ("route_ms", C.c_double * 3), ("implicit_cluster", C.c_int32)]
+                ("route_ms", C.c_double * 3), ("implicit_cluster", C.c_int32), ("digit_kernels", C.c_int32)]
 
     def as_dict(self):
         d = {k: getattr(self, k) for k, _ in self._fields_}

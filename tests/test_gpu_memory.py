@@ -1,0 +1,77 @@
+"""Short device memory: buffers that the allocator refuses, when they are asked for again, and what feti_stats says
+about it.  Bars: the FP64 parity bar 1e-12 between two assemblies of the same problem, twice for both sides."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2502_08382_gb300 import feti
+from paper_2502_08382_gb300.problems import make_problem
+
+pytestmark = pytest.mark.gpu
+
+
+class Refuser:
+    """torch's allocator, refusing the requests that `rule(nbytes)` picks while it is armed; counts them."""
+
+    def __init__(self, monkeypatch):
+        self.rule, self.refused, self.real = None, 0, torch.cuda.caching_allocator_alloc
+        monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", self)
+
+    def __call__(self, nbytes, *a, **k):
+        if self.rule and self.rule(nbytes):
+            self.refused += 1
+            raise torch.cuda.OutOfMemoryError("refused by the test")
+        return self.real(nbytes, *a, **k)
+
+
+@pytest.fixture
+def ref():
+    P = make_problem(dim=3, physics="elasticity", cuts=[[6, 5]] * 3, material="lognormal", sigma=0.5)
+    op = feti.FetiOperator(P, prec="fp64")
+    op.assemble()
+    F = [op.get_F(i) for i in range(P.nsub)]
+    op.close()
+    return P, F
+
+
+def check(op, F):
+    for i, f in enumerate(F):
+        assert np.linalg.norm(op.get_F(i) - f) <= 2e-12 * np.linalg.norm(f)
+
+
+def test_syrk_refused(monkeypatch, ref):
+    """A refused digit buffer is not asked for again while no more memory is free; the FP64-pipe kernel does the SYRK."""
+    P, F = ref
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64")
+    r.rule = lambda n: n > 1 << 20
+    for _ in range(4):
+        op.assemble()
+        check(op, F)
+    assert r.refused == 2  # all subdomains, then one at a time, in the first assembly only
+    assert op.stats()["digit_kernels"] == 0
+    op.close()
+
+
+def test_syrk_passing_shortage(monkeypatch, ref):
+    """With recompute_X the buffer is asked for at every assembly, so a passing shortage passes."""
+    P, F = ref
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", recompute_X=True)
+    x = 8 * op.stats()["X_elems"]
+    for short in (False, True, False):
+        r.rule = (lambda n: n > x + 256) if short else None  # X itself is granted
+        op.assemble()
+        r.rule = None
+        check(op, F)
+        # one subdomain at a time fits
+        assert op.stats()["digit_kernels"] == 1
+    r.rule = lambda n: n != (x + 255) // 256 * 256 and n > 1 << 20
+    op.assemble()
+    r.rule = None
+    check(op, F)
+    assert op.stats()["digit_kernels"] == 0
+    op.assemble()
+    check(op, F)
+    assert op.stats()["digit_kernels"] == 1
+    op.close()
