@@ -289,84 +289,118 @@ bool reserve_syrk_oz(feti_ctx* c) {
   return false;
 }
 
-// Buffers and work lists of the FP64 forward solve of the large fronts on the tensor cores, in batches of consecutive
-// subdomains whose digits of L fit 16 GB and, with the hand-over blocks, a third of the free memory; false where there
-// are no such fronts or not even one subdomain fits (trsm_kernel then solves everything).
+// Work lists of the FP64 forward solve of the large fronts on the tensor cores, in batches of consecutive subdomains
+// whose digits of L fit `budget` bytes (one subdomain at least), and the CTAs' workspaces.
+void plan_trsm_oz(feti_ctx* c, size_t budget) {
+  c->tx_planned = false;
+  c->tx_batches.clear();
+  auto ld_end = [&](int i) { return i + 1 < c->nsub ? (size_t)c->info[i + 1].ld : c->ld_bytes; };
+  for (int i = 0; i < c->nsub;) {
+    feti_ctx::TxBatch b;
+    b.sub0 = i;
+    b.ld0 = c->info[i].ld;
+    do ++i;
+    while (i < c->nsub && ld_end(i) - (size_t)b.ld0 <= budget);
+    b.sub1 = i;
+    c->tx_batches.push_back(b);
+  }
+  std::vector<int4> di;
+  int64_t n256 = 0;
+  for (int i = 0; i < c->nsub; ++i) {
+    auto& P = c->pats[c->subs[i].pat];
+    auto& B = c->bps[c->subs[i].bp];
+    int64_t ofs = 0;
+    for (int s = 0; s < P.nsn; ++s) {
+      if (!P.sn_big[s]) continue;
+      for (int kB = 0; kB < P.sn_w[s]; kB += 128) {
+        if (B.je[s] > B.jb[s]) di.push_back(make_int4(i, s, kB, (int)(ofs / 512)));
+        ofs += trsm_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
+      }
+    }
+    if (P.has_big) n256 += (c->subs[i].m + 255) / 256;
+  }
+  c->tx_cw = n256 >= 2 * (int64_t)c->nsm ? 256 : 128;
+  std::vector<int2> it;
+  size_t most = 0, dk = 0;
+  for (auto& b : c->tx_batches) {
+    std::vector<int> order;
+    for (int i = b.sub0; i < b.sub1; ++i)
+      if (c->pats[c->subs[i].pat].has_big && c->subs[i].m > 0) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b2) {
+      return c->bps[c->subs[a].bp].trsm_flops > c->bps[c->subs[b2].bp].trsm_flops;
+    });
+    b.item0 = (int)it.size();
+    for (int i : order)
+      for (int ca = 0; ca < c->subs[i].m; ca += c->tx_cw) it.push_back(make_int2(i, ca));
+    b.nitems = (int)it.size() - b.item0;
+    b.ditem0 = (int)dk;  // di is in the order of the subdomains
+    while (dk < di.size() && di[dk].x < b.sub1) ++dk;
+    b.nditems = (int)dk - b.ditem0;
+    most = std::max(most, (size_t)b.nitems);
+  }
+  c->tx_grid = (int)std::min<size_t>(c->nsm, std::max<size_t>(most, 1));
+  // a recorded assembly holds the old lists
+  if (c->asm_exec) CK(cudaGraphExecDestroy(c->asm_exec));
+  c->asm_exec = nullptr;
+  for (void** p : {(void**)&c->d_tx_ditems, (void**)&c->d_tx_items, (void**)&c->d_txws, (void**)&c->d_txscr}) {
+    dfree(c, *p);
+    *p = nullptr;
+  }
+  c->d_tx_ditems = upload(c, di);
+  c->d_tx_items = upload(c, it);
+  c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * std::max<int64_t>(c->tx_stack, 8) * c->tx_cw * 8);
+  c->d_txscr = (char*)dalloc(c, (size_t)c->tx_grid * trsm_oz_scratch(c->tx_cw));
+  CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
+  c->tx_none = it.empty() || di.empty();
+  c->tx_planned = true;
+}
+
+// The buffers of that solve: the hand-over blocks, and the digits of as many subdomains at a time as 16 GB and, with the
+// hand-over blocks, a third of the free memory hold, one at a time if the allocator refuses that; false where there are
+// no large fronts or not even one subdomain fits (trsm_kernel then solves everything).  Memory first, as in
+// reserve_syrk_oz, and asked for again by the same rule.
 bool reserve_trsm_oz(feti_ctx* c) {
-  if (c->tx_planned && (!c->tx_on || c->d_LD)) return c->tx_on;
+  if (c->ld_bytes == 0 || (c->tx_planned && c->tx_none)) return false;
+  if (c->d_LD) return true;
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  const bool first = !c->tx_planned;
-  c->tx_planned = true;
-  c->tx_on = false;
-  if (c->ld_bytes == 0 || c->th_bytes > free_b / 3) return false;
-  try {
-    if (first) {
-      const size_t budget = std::min<size_t>((size_t)16 << 30, free_b / 3 - c->th_bytes);
-      auto ld_end = [&](int i) { return i + 1 < c->nsub ? (size_t)c->info[i + 1].ld : c->ld_bytes; };
-      c->tx_ld_bytes = 0;
-      for (int i = 0; i < c->nsub;) {
-        feti_ctx::TxBatch b;
-        b.sub0 = i;
-        b.ld0 = c->info[i].ld;
-        do ++i;
-        while (i < c->nsub && ld_end(i) - (size_t)b.ld0 <= budget);
-        b.sub1 = i;
-        c->tx_ld_bytes = std::max(c->tx_ld_bytes, ld_end(i - 1) - (size_t)b.ld0);
-        c->tx_batches.push_back(b);
-      }
-      if (c->tx_ld_bytes > budget) return false;
-      std::vector<int4> di;
-      int64_t n256 = 0;
-      for (int i = 0; i < c->nsub; ++i) {
-        auto& P = c->pats[c->subs[i].pat];
-        auto& B = c->bps[c->subs[i].bp];
-        int64_t ofs = 0;
-        for (int s = 0; s < P.nsn; ++s) {
-          if (!P.sn_big[s]) continue;
-          for (int kB = 0; kB < P.sn_w[s]; kB += 128) {
-            if (B.je[s] > B.jb[s]) di.push_back(make_int4(i, s, kB, (int)(ofs / 512)));
-            ofs += trsm_oz_block_bytes(P.sn_w[s], P.sn_r[s], kB);
-          }
-        }
-        if (P.has_big) n256 += (c->subs[i].m + 255) / 256;
-      }
-      c->tx_cw = n256 >= 2 * (int64_t)c->nsm ? 256 : 128;
-      std::vector<int2> it;
-      size_t most = 0, dk = 0;
-      for (auto& b : c->tx_batches) {
-        std::vector<int> order;
-        for (int i = b.sub0; i < b.sub1; ++i)
-          if (c->pats[c->subs[i].pat].has_big && c->subs[i].m > 0) order.push_back(i);
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b2) {
-          return c->bps[c->subs[a].bp].trsm_flops > c->bps[c->subs[b2].bp].trsm_flops;
-        });
-        b.item0 = (int)it.size();
-        for (int i : order)
-          for (int ca = 0; ca < c->subs[i].m; ca += c->tx_cw) it.push_back(make_int2(i, ca));
-        b.nitems = (int)it.size() - b.item0;
-        b.ditem0 = (int)dk;  // di is in the order of the subdomains
-        while (dk < di.size() && di[dk].x < b.sub1) ++dk;
-        b.nditems = (int)dk - b.ditem0;
-        most = std::max(most, (size_t)b.nitems);
-      }
-      if (it.empty() || di.empty()) return false;
-      c->tx_grid = (int)std::min<size_t>(c->nsm, most);
-      c->d_tx_ditems = upload(c, di);
-      c->d_tx_items = upload(c, it);
-      c->d_txws = (double*)dalloc(c, (size_t)c->tx_grid * std::max<int64_t>(c->tx_stack, 8) * c->tx_cw * 8);
-      c->d_txscr = (char*)dalloc(c, (size_t)c->tx_grid * trsm_oz_scratch(c->tx_cw));
-      CK(cudaStreamSynchronize(c->st));  // the host arrays go out of scope
+  size_t least = 0;
+  for (int i = 0; i < c->nsub; ++i)
+    least = std::max(least, (i + 1 < c->nsub ? (size_t)c->info[i + 1].ld : c->ld_bytes) - (size_t)c->info[i].ld);
+  if (!c->opt.recompute_X && c->tx_refused > 0 && free_b < c->tx_refused + least + c->th_bytes) return false;
+  auto take = [&](size_t bytes) {
+    try {
+      c->d_LD = dalloc(c, bytes);
+      c->d_th = (double*)dalloc(c, std::max<size_t>(c->th_bytes, 8));
+      return true;
+    } catch (std::bad_alloc&) {
+      dfree(c, c->d_LD);
+      c->d_LD = nullptr;
+      return false;
     }
-    if (!c->d_txscr) return false;
-    c->d_LD = dalloc(c, c->tx_ld_bytes);
-    c->d_th = (double*)dalloc(c, std::max<size_t>(c->th_bytes, 8));
-    c->tx_on = true;
-  } catch (std::bad_alloc&) {
-    dfree(c, c->d_LD);
-    c->d_LD = nullptr;
+  };
+  try {
+    // the plan at hand first (its buffers were released by recompute_X)
+    if (c->tx_planned && take(c->tx_ld_bytes)) return true;
+    if (c->th_bytes + least <= free_b / 3) {
+      const size_t budget = std::min(c->ld_bytes, std::min<size_t>((size_t)16 << 30, free_b / 3 - c->th_bytes));
+      for (size_t b : {budget, (size_t)0}) {
+        const size_t bytes = std::max(b, least);
+        if (!take(bytes)) continue;
+        plan_trsm_oz(c, b);
+        c->tx_ld_bytes = bytes;
+        if (!c->tx_none) return true;
+        break;
+      }
+    }
+  } catch (std::bad_alloc&) {  // of the lists or the workspaces
   }
-  return c->tx_on;
+  dfree(c, c->d_LD);
+  c->d_LD = nullptr;
+  dfree(c, c->d_th);
+  c->d_th = nullptr;
+  c->tx_refused = std::max<size_t>(free_b, 1);
+  return false;
 }
 
 void build(feti_ctx* c) {

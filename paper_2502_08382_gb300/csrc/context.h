@@ -104,7 +104,8 @@ struct feti_ctx {
   int* d_impl_order = nullptr;
   int2* d_syrk_items = nullptr;
   // FP64 forward solve of the large fronts on the tensor cores
-  bool tx_planned = false, tx_on = false;
+  bool tx_planned = false, tx_none = false;  // tx_none: no items
+  size_t tx_refused = 0;             // free memory when the digits of L were last refused (0: never)
   int4* d_tx_ditems = nullptr;       // 128-column blocks of the large panels to cut
   int2* d_tx_items = nullptr;        // (subdomain, first column) of the solve
   // batches of consecutive subdomains whose digits of L are cut and used in turn

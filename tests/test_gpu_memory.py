@@ -75,3 +75,49 @@ def test_syrk_passing_shortage(monkeypatch, ref):
     check(op, F)
     assert op.stats()["digit_kernels"] == 1
     op.close()
+
+
+@pytest.mark.parametrize("recompute", [False, True])
+def test_trsm_refused_once(monkeypatch, ref, recompute):
+    """The digits of L are refused for all subdomains together and granted one subdomain at a time."""
+    P, F = ref
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", chol_tc_front=128, recompute_X=recompute)
+    r.rule = lambda n: n > 1 << 20 and r.refused == 0
+    for _ in range(3):
+        op.assemble()
+        check(op, F)
+        assert op.stats()["digit_kernels"] == 3
+    assert r.refused == 1
+    op.close()
+
+
+def test_trsm_passing_shortage(monkeypatch, ref):
+    """With recompute_X a shortage at one assembly does not keep the next ones from the digits."""
+    P, F = ref
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", chol_tc_front=128, recompute_X=True)
+    x = (8 * op.stats()["X_elems"] + 255) // 256 * 256
+    for short in (True, False, True, False):
+        r.rule = (lambda n: n != x and n > 1 << 20) if short else None  # X itself is granted
+        op.assemble()
+        r.rule = None
+        check(op, F)
+        assert op.stats()["digit_kernels"] == (0 if short else 3)
+    op.close()
+
+
+def test_trsm_refused(monkeypatch, ref):
+    """Refused for good, the digits are not asked for again while no more memory is free."""
+    P, F = ref
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", chol_tc_front=128)
+    r.rule = lambda n: n > 1 << 20
+    op.assemble()
+    first = r.refused
+    for _ in range(3):
+        op.assemble()
+        check(op, F)
+    assert first == 4 and r.refused == first  # L and X, all subdomains and then one at a time
+    assert op.stats()["digit_kernels"] == 0
+    op.close()
