@@ -53,7 +53,7 @@ __global__ void wsort_kernel(const AdjBatch* B, int nb, const double* W, const i
 // column group cg of kBuildCols columns):
 //   V_Z[c0 + k][jb + j] = d2[c0 + k] X_s[j][k]            (j < J_s; written by column group 0)
 //   V_Y[c0 + k][c]      = d2[c0 + k] sum_j X_s[j][k] Ws[jb + j][c]   (zcols = 0)
-// scaled: the X given is the assembly's X = D^{-1} X_u, so V_Z = D^{-1} X.
+// scaled: the X given is the assembly's X = D^{-1} X_u, so both take D^{-1} instead of d2.
 // computed in 64 x 64 output tiles (4 x 4 per thread) over 32-deep chunks of j.
 __global__ void __launch_bounds__(kAT) adj_build_kernel(DevPlan P, const AdjBatch* B, const int4* items, int nitems,
                                                        int* queue, const double* Xu, int scaled, int zcols,
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kAT) adj_build_kernel(DevPlan P, const AdjBatc
       for (int u = 0; u < 4; ++u) {
         const int k = ty + 16 * u;
         if (k >= nk) continue;
-        const double sc = d2[c0 + k0 + k];
+        const double dk = d2[c0 + k0 + k], sc = scaled ? sqrt(dk) : dk;
         double* row = V + (int64_t)(c0 + k0 + k) * ld + mp + cb;
 #pragma unroll
         for (int v = 0; v < 4; ++v) row[tx + 16 * v] = sc * acc[u][v];

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from paper_2502_08382_gb300 import feti
-from paper_2502_08382_gb300.problems import make_problem
+from paper_2502_08382_gb300.problems import make_problem, make_W
 
 pytestmark = pytest.mark.gpu
 
@@ -121,3 +121,29 @@ def test_trsm_refused(monkeypatch, ref):
     assert first == 4 and r.refused == first  # L and X, all subdomains and then one at a time
     assert op.stats()["digit_kernels"] == 0
     op.close()
+
+
+def elast(axis=2, elems=6):
+    return make_problem(dim=3, physics="elasticity", cuts=[[elems] * axis] * 3, material="density", seed=3)
+
+
+@pytest.mark.parametrize("recompute", [False, True])
+def test_adjoint_dense_refused(monkeypatch, recompute):
+    """The dense product's digits refused, Y comes from X W, with the assembly's X or with X_u solved for again: the same
+    gradient at the parity bar 1e-10."""
+    P = elast()
+    Ws = make_W(P, seed=0)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    g = op.adjoint(Ws).cpu().numpy()
+    op.close()
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True, recompute_X=recompute)
+    op.assemble()
+    W = op._W_dev(Ws)
+    x = (8 * op.stats()["X_elems"] + 255) // 256 * 256
+    r.rule = lambda n: n != x and n > 4096 and r.refused == 0
+    h = op.adjoint(W).cpu().numpy()
+    op.close()
+    assert r.refused == 1
+    assert np.linalg.norm(h - g) <= 1e-10 * np.linalg.norm(g)
