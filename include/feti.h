@@ -104,8 +104,10 @@ typedef struct {
   int32_t precond;            /* PCPG preconditioner M of Algorithm 1 (the paper leaves it open):
                                  0 = none (M = I); 1 = lumped, M = W (sum_i B_i K_i B_i^T) W with
                                  W = (B B^T)^{-1}, rebuilt from K at every feti_assemble */
-  int64_t adjoint_work_bytes; /* device work budget of one feti_adjoint batch (dense n_i x 2 m_i arrays
-                                 of the subdomains in the batch); 0 = min(24 GiB, 45% of free memory) */
+  int64_t adjoint_work_bytes; /* device work budget of one feti_adjoint batch: the dense n_i x 2 m_i arrays and
+                                 W_i of its subdomains, their large fronts' digits of L^T, and the digits of
+                                 Z and W (at most half of it), besides about 40 MB of fixed scratch; one
+                                 subdomain at least.  0 = min(24 GiB, 45% of free memory) */
   int32_t assembly_route;     /* how F_i is formed (Sec. III-IV):
                                  0 = the SYRK path: nested-dissection ordering, pruned TRSM
                                      X_i = L_i^{-1} P B_i^T, F_i = X_i^T X_i;

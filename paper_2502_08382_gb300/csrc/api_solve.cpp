@@ -491,8 +491,9 @@ void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t 
 // Z_i = P^T L_u^{-T} D^{-2} X_u (and, for the adjoint, Y_i = Z_i W_i) over batches of subdomains whose
 // dense work arrays fit the budget, from X_u = L_u^{-1} P B^T recomputed in FP64 by the pruned forward
 // solve with the unit-lower factor.  W_dev != null: the adjoint, dtheta_e = -sum (dK_e)_ab Y[b,:] . Z[a,:]
-// into dtheta; W_dev == null: the TRSM-path assembly, F_i = B_i Z_i into the F tiles.  Synchronises.
-void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStream_t st) {
+// into dtheta; W_dev == null: the TRSM-path assembly, F_i = B_i Z_i into the F tiles.  digits: with the products on the
+// tensor cores.  Synchronises.
+void z_batches_once(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, bool digits, cudaStream_t st) {
   const bool adjoint = W_dev != nullptr;
   const int ns = ctx->nsub;
   // the FP64 assembly's X = L^{-1} P B^T is X_u up to the pivots (X_u = D X); where it is not kept (mixed precision,
@@ -512,11 +513,12 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
   CKS(cudaMemGetInfo(&free_b, &total_b));
   const double cap = ctx->opt.adjoint_work_bytes > 0
                          ? (double)ctx->opt.adjoint_work_bytes
-                         : std::min<double>(24.0 * (1 << 30), 0.45 * (double)(free_b + ctx->adj_work_bytes));
+                         : std::min<double>(24.0 * (1 << 30), 0.45 * (double)(free_b + ctx->adj_work_bytes +
+                                                                              ctx->adj_dig_bytes + ctx->adj_lt_bytes));
   // the adjoint's Y = Z W by digit products on the tensor cores: the digits of W and of as many rows of Z as half the
   // cap holds (8 GiB at most, the largest subdomain's W and 128 rows at least; the rows' results do not depend on how
   // many go together); where the allocator refuses, Y is formed as X_u W and solved for with Z
-  bool dense = adjoint;
+  bool dense = adjoint && digits;
   if (dense) {
     int64_t want = 0, least = 0;
     for (int i = 0; i < ns; ++i) {
@@ -538,13 +540,15 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
       }
     }
   }
+  // the large fronts' part of the backward solve on the tensor cores; a batch's digits of L^T count in its budget
+  bool boz = dense || (!adjoint && digits);
   const int64_t budget = std::max<int64_t>((int64_t)(cap / 8) - (dense ? ctx->adj_dig_bytes / 8 : 0), 1);
   std::vector<int64_t> woff(ns + 1, 0);
   for (int i = 0; i < ns; ++i) woff[i + 1] = woff[i] + (int64_t)ctx->subs[i].m * ctx->subs[i].m;
   std::vector<std::vector<AdjBatch>> batches;
   {
     std::vector<AdjBatch> cur;
-    int64_t used = 0;
+    int64_t used = 0, lt = 0;
     for (int i = 0; i < ns; ++i) {
       const auto& s = ctx->subs[i];
       if (adjoint && s.nelem == 0) continue;
@@ -555,10 +559,11 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
       const auto& I = ctx->info[i];
       const int64_t vlen = (int64_t)s.n * (adjoint ? 2 : 1) * I.m_pad;
       const int64_t need = vlen + (adjoint ? (int64_t)I.m_pad * I.m_pad : 0);
-      if (!cur.empty() && used + need > budget) {
+      const int64_t lt_need = boz ? ctx->pat_lt[s.pat] : 0;
+      if (!cur.empty() && used + need + (lt + lt_need) / 8 > budget) {
         batches.push_back(cur);
         cur.clear();
-        used = 0;
+        used = lt = 0;
       }
       AdjBatch e{};
       e.sub = i;
@@ -571,12 +576,14 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
       e.w_src = woff[i];
       e.v_ofs = used;
       e.ws_ofs = used + vlen;
+      e.lt = lt;
       e.el_dofs = adjoint ? ctx->elem_dofs_ofs[i] : 0;
       e.el_dk = adjoint ? ctx->elem_dk_ofs[i] : 0;
       e.el_out = adjoint ? ctx->elem_ofs[i] : 0;
       e.dk_stride = s.dk_stride;
       cur.push_back(e);
       used += need;
+      lt += lt_need;
     }
     if (!cur.empty()) batches.push_back(cur);
   }
@@ -598,18 +605,9 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
     ctx->d_adj_batch = (AdjBatch*)dalloc(ctx, (size_t)max_nb * sizeof(AdjBatch));
     ctx->adj_batch_cap = max_nb;
   }
-  // the large fronts' part of the backward solve on the tensor cores, unless their digits find no memory
-  bool boz = dense || !adjoint;
-  if (boz) {
+  if (boz) {  // unless the digits find no memory
     int64_t want = 0;
-    for (auto& b : batches) {
-      int64_t t = 0;
-      for (auto& e : b) {
-        e.lt = t;
-        t += ctx->pat_lt[ctx->subs[e.sub].pat];
-      }
-      want = std::max(want, t);
-    }
+    for (auto& b : batches) want = std::max(want, b.back().lt + ctx->pat_lt[ctx->subs[b.back().sub].pat]);
     boz = want > 0;
     try {
       if (want > ctx->adj_lt_bytes) {
@@ -733,6 +731,32 @@ void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStrea
     CKS(cudaStreamSynchronize(st));
   }
   CKS(cudaStreamSynchronize(st));
+}
+
+// z_batches_once; where it finds no memory, again without the digits that an FP64 assembly keeps between calls (the next
+// one asks for them anew), then without digits of its own.
+void z_batches(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, cudaStream_t st) {
+  auto drop = [&](auto*& p) {
+    dfree(ctx, p);
+    p = nullptr;
+  };
+  for (int attempt = W_dev ? 0 : 1;; ++attempt) {
+    try {
+      return z_batches_once(ctx, W_dev, dtheta_dev, attempt < 2, st);
+    } catch (std::bad_alloc&) {
+      if (attempt == 2) throw;
+      CKS(cudaStreamSynchronize(st));
+      if (attempt == 0) {
+        drop(ctx->d_XD);
+        drop(ctx->d_LD);
+        drop(ctx->d_th);
+      } else {
+        drop(ctx->d_adj_dig);
+        drop(ctx->d_adj_lt);
+        ctx->adj_dig_bytes = ctx->adj_lt_bytes = 0;
+      }
+    }
+  }
 }
 
 }  // namespace

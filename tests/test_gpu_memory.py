@@ -147,3 +147,90 @@ def test_adjoint_dense_refused(monkeypatch, recompute):
     op.close()
     assert r.refused == 1
     assert np.linalg.norm(h - g) <= 1e-10 * np.linalg.norm(g)
+
+
+def test_adjoint_budget():
+    """adjoint_work_bytes caps what feti_adjoint takes, its digits included, besides the fixed scratch."""
+    P = elast()
+    Ws = make_W(P, seed=0)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    g = op.adjoint(Ws).cpu().numpy()
+    op.close()
+    cap = 60 << 20
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True, adjoint_work_bytes=cap)
+    op.assemble()
+    before = torch.cuda.memory_allocated()
+    assert np.array_equal(op.adjoint(Ws).cpu().numpy(), g)
+    scratch = torch.cuda.get_device_properties(0).multi_processor_count * 128 * (2048 + 4)
+    assert torch.cuda.memory_allocated() - before <= cap + scratch + (1 << 20)  # and a few small lists
+    op.close()
+
+
+def test_adjoint_short_memory():
+    """Later calls do as many subdomains at a time as the first, whose buffers they take over (700 MB are left free)."""
+    P = elast(axis=3)
+    Ws = make_W(P, seed=0)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True, torch_alloc=False)
+    op.assemble()
+    W = op._W_dev(Ws)
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (700 << 20), dtype=torch.uint8, device="cuda")
+    counts, grads = [], []
+    for _ in range(3):
+        n = op.stats()["launches"]
+        grads.append(op.adjoint(W))
+        counts.append(op.stats()["launches"] - n)
+    del hog
+    torch.cuda.empty_cache()
+    op.close()
+    assert torch.equal(grads[0], grads[1]) and torch.equal(grads[0], grads[2])
+    assert max(counts) <= 1.5 * counts[0], counts
+
+
+def test_adjoint_refused(monkeypatch):
+    """Where nothing large is granted beyond the work array, the FP64-pipe kernels do the adjoint (the parity bar 1e-10)."""
+    P = elast()
+    Ws = make_W(P, seed=0)
+    r = Refuser(monkeypatch)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    g = op.adjoint(Ws).cpu().numpy()
+    op.close()
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    W = op._W_dev(Ws)
+    # digits and work array, with and without the assembly's digits held; then the work array is granted
+    r.rule = lambda n: n > 4096 and r.refused < 4
+    h = op.adjoint(W).cpu().numpy()
+    r.rule = None
+    assert r.refused == 4
+    assert np.linalg.norm(h - g) <= 1e-10 * np.linalg.norm(g)
+    op.assemble()
+    assert op.stats()["digit_kernels"] & 1
+    assert np.linalg.norm(op.adjoint(W).cpu().numpy() - g) <= 1e-10 * np.linalg.norm(g)
+    op.close()
+
+
+def test_adjoint_backward_refused(monkeypatch):
+    """The digits of L^T refused, the FP64-pipe kernel does the whole backward solve."""
+    P = elast()
+    Ws = make_W(P, seed=0)
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    g = op.adjoint(Ws).cpu().numpy()
+    op.close()
+    r, big = Refuser(monkeypatch), [0]
+    op = feti.FetiOperator(P, prec="fp64", with_elements=True)
+    op.assemble()
+    W = op._W_dev(Ws)
+
+    def third(n):  # after the dense digits and the work array
+        big[0] += n > 4096
+        return big[0] == 3 and n > 4096
+
+    r.rule = third
+    h = op.adjoint(W).cpu().numpy()
+    op.close()
+    assert r.refused == 1
+    assert np.linalg.norm(h - g) <= 1e-10 * np.linalg.norm(g)
