@@ -7,6 +7,7 @@
 #include <vector>
 #include <stdexcept>
 #include <string>
+#include <type_traits>
 
 #include "context.h"
 #include "kernels.h"
@@ -413,6 +414,21 @@ feti_status solve_impl(feti_ctx* ctx, double* lambda_dev, double* alpha_dev, dou
   }
 }
 
+// A work buffer of `need` elements at least.  The stream is waited for before the old one is given back: launches may
+// still use it, and dev_free may hand its memory on at once.
+template <typename T>
+void grow(feti_ctx* ctx, T*& p, int64_t& cap, int64_t need) {
+  if (need <= cap) return;
+  if (p) {
+    CKS(cudaStreamSynchronize(ctx->st));
+    dfree(ctx, p);
+  }
+  p = nullptr;
+  cap = 0;
+  p = (T*)dalloc(ctx, (size_t)need * (std::is_void_v<T> ? 1 : sizeof(std::conditional_t<std::is_void_v<T>, char, T>)));
+  cap = need;
+}
+
 // Y = Z W of every entry of an adjoint batch by digit products: groups of (entry, rows) whose digits fit the buffer.
 void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t st,
                     std::vector<std::vector<DenseEnt>>& keep_ent, std::vector<std::vector<int4>>& keep_it) {
@@ -421,21 +437,9 @@ void dense_products(feti_ctx* ctx, const std::vector<AdjBatch>& b, cudaStream_t 
   int64_t bytes = 0, nex = 0;
   auto flush = [&]() {
     if (ents.empty()) return;
-    if ((int64_t)ents.size() > ctx->adj_ent_cap) {
-      dfree(ctx, ctx->d_adj_ent);
-      ctx->d_adj_ent = (DenseEnt*)dalloc(ctx, ents.size() * sizeof(DenseEnt));
-      ctx->adj_ent_cap = (int64_t)ents.size();
-    }
-    if ((int64_t)items.size() > ctx->adj_dit_cap) {
-      dfree(ctx, ctx->d_adj_dit);
-      ctx->d_adj_dit = (int4*)dalloc(ctx, items.size() * sizeof(int4));
-      ctx->adj_dit_cap = (int64_t)items.size();
-    }
-    if (nex > ctx->adj_dex_cap) {
-      dfree(ctx, ctx->d_adj_dex);
-      ctx->d_adj_dex = (int*)dalloc(ctx, (size_t)nex * sizeof(int));
-      ctx->adj_dex_cap = nex;
-    }
+    grow(ctx, ctx->d_adj_ent, ctx->adj_ent_cap, (int64_t)ents.size());
+    grow(ctx, ctx->d_adj_dit, ctx->adj_dit_cap, (int64_t)items.size());
+    grow(ctx, ctx->d_adj_dex, ctx->adj_dex_cap, nex);
     keep_ent.push_back(ents);
     keep_it.push_back(items);
     CKS(cudaMemcpyAsync(ctx->d_adj_ent, keep_ent.back().data(), ents.size() * sizeof(DenseEnt), cudaMemcpyHostToDevice, st));
@@ -528,16 +532,10 @@ void z_batches_once(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, bool
       least = std::max(least, (m + 128) * q * 128);
     }
     want = std::max(least, std::min(want, (int64_t)std::min(0.5 * cap, 8.0 * (1 << 30))));
-    if (want > ctx->adj_dig_bytes) {
-      dfree(ctx, ctx->d_adj_dig);
-      ctx->d_adj_dig = nullptr;
-      ctx->adj_dig_bytes = 0;
-      try {
-        ctx->d_adj_dig = dalloc(ctx, (size_t)want);
-        ctx->adj_dig_bytes = want;
-      } catch (std::bad_alloc&) {
-        dense = false;
-      }
+    try {
+      grow(ctx, ctx->d_adj_dig, ctx->adj_dig_bytes, want);
+    } catch (std::bad_alloc&) {
+      dense = false;
     }
   }
   // the large fronts' part of the backward solve on the tensor cores; a batch's digits of L^T count in its budget
@@ -593,30 +591,17 @@ void z_batches_once(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, bool
     max_used = std::max<int64_t>(max_used, l.ws_ofs + (adjoint ? (int64_t)l.m_pad * l.m_pad : 0));
     max_nb = std::max<int64_t>(max_nb, (int64_t)b.size());
   }
-  if (max_used * 8 > ctx->adj_work_bytes) {
-    dfree(ctx, ctx->d_adj_work);
-    ctx->d_adj_work = nullptr;
-    ctx->adj_work_bytes = 0;
-    ctx->d_adj_work = (double*)dalloc(ctx, (size_t)max_used * 8);
-    ctx->adj_work_bytes = max_used * 8;
-  }
-  if (max_nb > ctx->adj_batch_cap) {
-    dfree(ctx, ctx->d_adj_batch);
-    ctx->d_adj_batch = (AdjBatch*)dalloc(ctx, (size_t)max_nb * sizeof(AdjBatch));
-    ctx->adj_batch_cap = max_nb;
-  }
+  int64_t work = ctx->adj_work_bytes / 8;  // in doubles
+  ctx->adj_work_bytes = 0;
+  grow(ctx, ctx->d_adj_work, work, max_used);
+  ctx->adj_work_bytes = work * 8;
+  grow(ctx, ctx->d_adj_batch, ctx->adj_batch_cap, max_nb);
   if (boz) {  // unless the digits find no memory
     int64_t want = 0;
     for (auto& b : batches) want = std::max(want, b.back().lt + ctx->pat_lt[ctx->subs[b.back().sub].pat]);
     boz = want > 0;
     try {
-      if (want > ctx->adj_lt_bytes) {
-        dfree(ctx, ctx->d_adj_lt);
-        ctx->d_adj_lt = nullptr;
-        ctx->adj_lt_bytes = 0;
-        ctx->d_adj_lt = dalloc(ctx, (size_t)want);
-        ctx->adj_lt_bytes = want;
-      }
+      grow(ctx, ctx->d_adj_lt, ctx->adj_lt_bytes, want);
       if (boz && !ctx->d_adj_bscr) ctx->d_adj_bscr = (char*)dalloc(ctx, (size_t)ctx->nsm * bsolve_oz_scratch());
     } catch (std::bad_alloc&) {
       boz = false;
@@ -660,16 +645,8 @@ void z_batches_once(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, bool
     sv.reserve(si.size());
     for (auto& x : bi) bv.push_back(x.second);
     for (auto& x : si) sv.push_back(x.second);
-    if ((int64_t)bv.size() > ctx->adj_items4_cap) {
-      dfree(ctx, ctx->d_adj_items4);
-      ctx->d_adj_items4 = (int4*)dalloc(ctx, bv.size() * sizeof(int4));
-      ctx->adj_items4_cap = (int64_t)bv.size();
-    }
-    if ((int64_t)sv.size() > ctx->adj_items2_cap) {
-      dfree(ctx, ctx->d_adj_items2);
-      ctx->d_adj_items2 = (int2*)dalloc(ctx, sv.size() * sizeof(int2));
-      ctx->adj_items2_cap = (int64_t)sv.size();
-    }
+    grow(ctx, ctx->d_adj_items4, ctx->adj_items4_cap, (int64_t)bv.size());
+    grow(ctx, ctx->d_adj_items2, ctx->adj_items2_cap, (int64_t)sv.size());
     // the host vectors outlive the copies: the stream is synchronised at the end of each batch
     CKS(cudaMemcpyAsync(ctx->d_adj_batch, b.data(), nb * sizeof(AdjBatch), cudaMemcpyHostToDevice, st));
     if (!bv.empty())
@@ -696,16 +673,8 @@ void z_batches_once(feti_ctx* ctx, const double* W_dev, double* dtheta_dev, bool
         if (pat.has_back)
           for (int cb = 0; cb < (b[e].m_pad + 127) / 128; ++cb) yv.push_back(make_int2(e, cb));
       }
-      if ((int64_t)lv.size() > ctx->adj_lit_cap) {
-        dfree(ctx, ctx->d_adj_lit);
-        ctx->d_adj_lit = (int4*)dalloc(ctx, lv.size() * sizeof(int4));
-        ctx->adj_lit_cap = (int64_t)lv.size();
-      }
-      if ((int64_t)yv.size() > ctx->adj_bit_cap) {
-        dfree(ctx, ctx->d_adj_bit);
-        ctx->d_adj_bit = (int2*)dalloc(ctx, yv.size() * sizeof(int2));
-        ctx->adj_bit_cap = (int64_t)yv.size();
-      }
+      grow(ctx, ctx->d_adj_lit, ctx->adj_lit_cap, (int64_t)lv.size());
+      grow(ctx, ctx->d_adj_bit, ctx->adj_bit_cap, (int64_t)yv.size());
       if (!yv.empty()) {
         CKS(cudaMemcpyAsync(ctx->d_adj_lit, lv.data(), lv.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
         CKS(cudaMemcpyAsync(ctx->d_adj_bit, yv.data(), yv.size() * sizeof(int2), cudaMemcpyHostToDevice, st));

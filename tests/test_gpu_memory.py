@@ -234,3 +234,24 @@ def test_adjoint_backward_refused(monkeypatch):
     op.close()
     assert r.refused == 1
     assert np.linalg.norm(h - g) <= 1e-10 * np.linalg.norm(g)
+
+
+def test_adjoint_frees_idle_buffers(monkeypatch):
+    """A buffer goes back to dev_free only when no launch uses it any more (a caller's allocator may hand it on)."""
+    P = make_problem(dim=3, physics="elasticity", cuts=[[7, 4, 6]] * 3, material="density", seed=3)
+    Ws = make_W(P, seed=0)
+    idle, real = [], torch.cuda.caching_allocator_delete
+
+    def delete(p):
+        idle.append(torch.cuda.current_stream().query())
+        real(p)
+
+    for cap in (20, 40, 60, 100):
+        op = feti.FetiOperator(P, prec="fp64", with_elements=True, adjoint_work_bytes=cap << 20)
+        op.assemble()
+        W = op._W_dev(Ws)
+        with monkeypatch.context() as mp:
+            mp.setattr(torch.cuda, "caching_allocator_delete", delete)
+            op.adjoint(W)
+        op.close()
+    assert len(idle) > 0 and all(idle), (len(idle), sum(idle))
