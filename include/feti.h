@@ -91,7 +91,8 @@ typedef struct {
                                  intermediate of the assembly) nor the FP64 X_i of feti_adjoint after that
                                  call: both are released and recomputed from L_i when next needed, for
                                  problems where HBM is short; 0 = keep both buffers for reuse */
-  void* (*dev_alloc)(size_t bytes, void* ctx);  /* optional device allocator (NULL: cudaMalloc) */
+  void* (*dev_alloc)(size_t bytes, void* ctx);  /* optional device allocator (NULL: cudaMalloc); where it aligns to
+                                 less than 256 bytes it is asked for 256 more */
   void (*dev_free)(void* ptr, void* ctx);
   void* alloc_ctx;
   void* stream;               /* cudaStream_t; NULL = legacy default stream */

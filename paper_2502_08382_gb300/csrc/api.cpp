@@ -33,14 +33,24 @@ feti_status set_error(feti_ctx* c, feti_status s, const std::string& msg) {
 void* dalloc(feti_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 16;
   bytes = (bytes + 255) & ~size_t(255);
-  void* p = nullptr;
+  void *p = nullptr, *base = nullptr;
   if (c->opt.dev_alloc) {
-    p = c->opt.dev_alloc(bytes, c->opt.alloc_ctx);
+    // the kernels' widest accesses are of 32 bytes, their bulk copies of 16: a caller's allocator that aligns to less
+    // than 256 bytes is asked for as much more
+    constexpr size_t kAlign = 256;
+    base = p = c->opt.dev_alloc(bytes, c->opt.alloc_ctx);
+    if (p && (uintptr_t)p % kAlign != 0) {
+      if (c->opt.dev_free) c->opt.dev_free(p, c->opt.alloc_ctx);
+      bytes += kAlign;
+      base = c->opt.dev_alloc(bytes, c->opt.alloc_ctx);
+      p = base ? (void*)(((uintptr_t)base + kAlign - 1) / kAlign * kAlign) : nullptr;
+    }
   } else {
     if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+    base = p;
   }
   if (!p) throw std::bad_alloc();
-  c->bufs.push_back({p, bytes});
+  c->bufs.push_back({p, bytes, base});
   c->device_bytes += bytes;
   return p;
 }
@@ -49,7 +59,7 @@ void dfree(feti_ctx* c, void* p) {
   if (!p) return;
   for (size_t k = 0; k < c->bufs.size(); ++k)
     if (c->bufs[k].p == p) {
-      if (c->opt.dev_free) c->opt.dev_free(p, c->opt.alloc_ctx);
+      if (c->opt.dev_free) c->opt.dev_free(c->bufs[k].base, c->opt.alloc_ctx);
       else if (!c->opt.dev_alloc) cudaFree(p);
       c->device_bytes -= c->bufs[k].bytes;
       c->bufs.erase(c->bufs.begin() + (long)k);
@@ -1831,7 +1841,7 @@ void feti_destroy(feti_ctx* ctx) {
     if (e) cudaEventDestroy(e);
   if (ctx->cap_st) cudaStreamDestroy(ctx->cap_st);
   for (auto& b : ctx->bufs) {
-    if (ctx->opt.dev_free) ctx->opt.dev_free(b.p, ctx->opt.alloc_ctx);
+    if (ctx->opt.dev_free) ctx->opt.dev_free(b.base, ctx->opt.alloc_ctx);
     else if (!ctx->opt.dev_alloc) cudaFree(b.p);
   }
   delete ctx;

@@ -31,6 +31,7 @@ struct SubHost {
 struct DBuf {
   void* p = nullptr;
   size_t bytes = 0;
+  void* base = nullptr;  // what the allocator returned
 };
 
 }  // namespace feti

@@ -255,3 +255,34 @@ def test_adjoint_frees_idle_buffers(monkeypatch):
             op.adjoint(W)
         op.close()
     assert len(idle) > 0 and all(idle), (len(idle), sum(idle))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "split_bf16"])
+def test_allocator_alignment(monkeypatch, prec):
+    """An allocator that aligns to 16 bytes only: every buffer is aligned by the library, and goes back as it came."""
+    P = elast(elems=4)
+    Ws = make_W(P, seed=0)
+    op = feti.FetiOperator(P, prec=prec, with_elements=True, chol_tc_front=128)
+    op.assemble()
+    g, F = op.adjoint(Ws).cpu().numpy(), op.get_F(0)
+    op.close()
+    alloc, delete, live = torch.cuda.caching_allocator_alloc, torch.cuda.caching_allocator_delete, set()
+
+    def odd_alloc(nbytes, *a, **k):
+        p = alloc(nbytes + 16, *a, **k) + 16
+        live.add(p)
+        return p
+
+    def odd_delete(p):
+        live.remove(p)
+        delete(p - 16)
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", odd_alloc)
+    monkeypatch.setattr(torch.cuda, "caching_allocator_delete", odd_delete)
+    op = feti.FetiOperator(P, prec=prec, with_elements=True, chol_tc_front=128, recompute_X=True)
+    op.assemble()
+    assert np.linalg.norm(op.adjoint(Ws).cpu().numpy() - g) <= 1e-10 * np.linalg.norm(g)
+    if prec == "fp64":
+        assert np.linalg.norm(op.get_F(0) - F) <= 2e-12 * np.linalg.norm(F)
+    op.close()
+    assert not live
