@@ -705,7 +705,7 @@ void build(feti_ctx* c) {
   int fixo = 0, alo = 0;
   double chol = 0, trsm = 0, syrk = 0, syrke = 0, implb = 0;
   int64_t sub_chol = 0, big_chol = 0;
-  int64_t max_chol = 0, max_rhs = 0, max_cf = 0, max_rf = 0, max_usm = 0;
+  int64_t max_rhs = 0, max_rf = 0, max_usm = 0, ntasks = 0;
   size_t esz = c->fp32 ? 4 : 8;
   double apply_bytes = 0, stored_bytes = 0;
   c->colperm_ofs.resize(ns);
@@ -810,9 +810,8 @@ void build(feti_ctx* c) {
     syrk += B.syrk_flops;
     syrke += B.syrk_exec_flops;
     implb += 2.0 * 8.0 * P.nnzL;
-    max_chol = std::max(max_chol, P.chol_stack);
+    ntasks += P.ntask;
     max_usm = std::max(max_usm, P.usm_size);
-    max_cf = std::max(max_cf, P.chol_front);
     sub_chol = std::max(sub_chol, P.sub_stack);
     big_chol = std::max(big_chol, P.big_stack);
     max_rhs = std::max(max_rhs, B.rhs_stack);
@@ -997,26 +996,27 @@ void build(feti_ctx* c) {
     c->grid_trsm32 = (int)std::min<int64_t>(c->grid_trsm, (int64_t)c->nsm * trsm_ctas_per_sm(true, 2));
   }
   c->rhs_front = max_rf;
-  c->ws_stride = std::max(std::max(max_cf + max_chol, sub_chol) + max_usm, std::max(big_chol, max_rf + max_rhs));
-  c->ws_stride = (c->ws_stride + 31) / 32 * 32;
+  // one buffer for three kernels that run one after another: the TRSM's fronts and stacks per CTA or the tensor-core
+  // Cholesky's update blocks per cluster (ws_stride), or chol_kernel's update blocks per CTA (sub_stride)
+  c->ws_stride = std::max<int64_t>((std::max(big_chol, max_rf + max_rhs) + 31) / 32 * 32, 32);
+  c->sub_stack = sub_chol;
+  c->sub_stride = std::max<int64_t>((sub_chol + max_usm + 31) / 32 * 32, 32);
   {
-    // the per-CTA workspace (fronts and update stacks) of all persistent CTAs may take at most 40% of the
-    // free device memory: large fronts (the Schur-complement route's dense root) get fewer CTAs
+    // it may take at most 40% of the free device memory: large fronts (the Schur-complement route's dense root) get
+    // fewer CTAs
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
     const int64_t cap = std::max<int64_t>(1, (int64_t)(0.4 * (double)free_b) / (c->ws_stride * 8));
-    c->grid_chol = (int)std::max<int64_t>(1, std::min<int64_t>(c->grid_chol, cap));
+    c->grid_ws = (int)std::max<int64_t>(1, std::min<int64_t>(c->grid_chol, cap));
     c->grid_trsm = (int)std::max<int64_t>(1, std::min<int64_t>(c->grid_trsm, cap));
     c->grid_trsm32 = std::max(1, std::min(c->grid_trsm32, c->grid_trsm));
+    c->grid_ws = std::max(c->grid_ws, c->grid_trsm);
+    // chol_kernel's tasks outnumber the subdomains (with one CTA per subdomain 64 subdomains left half the SMs idle)
+    const int64_t cap_c = std::max<int64_t>(1, (int64_t)(0.4 * (double)free_b) / (c->sub_stride * 8));
+    c->grid_chol = (int)std::min<int64_t>(std::min<int64_t>((int64_t)c->nsm * chol_ctas_per_sm(), cap_c),
+                                          std::max<int64_t>(ntasks, 1));
   }
-  int gw = std::max(c->grid_chol, c->grid_trsm);
-  c->grid_ws = gw;
-  // chol_kernel needs the update blocks outside the large set only: as many CTAs as fit the same workspace (its
-  // tasks outnumber the subdomains; with one CTA per subdomain 64 subdomains left half the SMs idle)
-  c->sub_stack = sub_chol;
-  c->sub_stride = std::max<int64_t>((sub_chol + max_usm + 31) / 32 * 32, 32);
-  c->grid_chol = (int)std::max<int64_t>(
-      c->grid_chol, std::min<int64_t>((int64_t)c->nsm * chol_ctas_per_sm(), (int64_t)gw * c->ws_stride / c->sub_stride));
+  const int64_t ws_doubles = std::max((int64_t)c->grid_ws * c->ws_stride, (int64_t)c->grid_chol * c->sub_stride);
 
   // ---- device uploads
   DevPlan& D = c->P;
@@ -1110,7 +1110,7 @@ void build(feti_ctx* c) {
   D.rho = (double*)dalloc(c, (size_t)ns * 8);
   c->d_X = dalloc(c, (size_t)Xo * esz);
   c->d_F = dalloc(c, (size_t)Fo * esz);
-  c->d_ws = (double*)dalloc(c, (size_t)gw * c->ws_stride * 8);
+  c->d_ws = (double*)dalloc(c, (size_t)ws_doubles * 8);
   c->d_trow = (double*)dalloc(c, (size_t)qo * 8);
   c->d_tpart = (double*)dalloc(c, (size_t)std::max<int64_t>(tpo, 1) * 8);
   c->d_rowpart = dalloc(c, (size_t)std::max<int64_t>(tpo, 1) * 8);
@@ -1308,7 +1308,7 @@ void build(feti_ctx* c) {
   }
   CK(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->st));
   CK(cudaMemsetAsync(c->d_tpart, 0, (size_t)std::max<int64_t>(tpo, 1) * 8, c->st));
-  c->stats.workspace_bytes = (int64_t)gw * c->ws_stride * 8;
+  c->stats.workspace_bytes = ws_doubles * 8;
   c->stats.implicit_cluster = c->impl_wide ? c->impl_cluster : -1;
   for (auto& e : c->ev) CK(cudaEventCreate(&e));
   CK(cudaStreamSynchronize(c->st));

@@ -286,3 +286,16 @@ def test_allocator_alignment(monkeypatch, prec):
         assert np.linalg.norm(op.get_F(0) - F) <= 2e-12 * np.linalg.norm(F)
     op.close()
     assert not live
+
+
+def test_workspace_size():
+    """The workspace holds what the kernels use: with few multipliers the TRSM needs little, and no Cholesky kernel keeps a
+    stack of whole fronts per CTA any more (chol_stack doubles, per CTA of the TRSM)."""
+    P = make_problem(dim=3, physics="elasticity", cuts=[[8, 8]] * 3)
+    op = feti.FetiOperator(P, prec="fp64", route="schur")
+    st = op.stats()
+    stack = max(feti.analyse(s, route="schur")["chol_stack"] for s in P.subs)
+    op.assemble()
+    ctas = op.stats()["trsm_grid"]
+    op.close()
+    assert st["workspace_bytes"] < 8 * ctas * stack
