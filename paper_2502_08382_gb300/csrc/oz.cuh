@@ -9,8 +9,9 @@
 // accumulation is exact.  With hi = sum_{d <= 3} acc_d 2^(8 (3 - d)) and lo = sum_{d >= 4} acc_d 2^(8 (7 - d)) in
 // 64-bit integers,
 //   sum_k x_k y_k = 2^(e_x + e_y - 68) (2^32 hi + lo).
-// Rounding to 62 bits costs 2^-63 of the largest entry and the dropped pairs (p + q >= 8) about as much per
-// product, far below one FP64 rounding of the same sum.
+// Rounding to 62 bits costs 2^-63 of the largest entry in either factor, the dropped pairs (seven with p + q = 8, of at
+// most 2^14 2^48 2^-124 each, and fewer beyond) at most 7.1 2^-62: a product of K entries lies within K 2^-58 2^(e_x + e_y)
+// of the exact sum, against K 2^-53 for FP64 where all terms are of that size.
 //
 // A vector's entries share one exponent, so an entry far below the largest one keeps fewer than 53 bits.  Where the
 // scales of a product's inner index are opposite on its two sides (a factor's inverse and a right-hand side: the one
