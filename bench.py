@@ -159,8 +159,8 @@ def other_rooflines(st, impl_ms, hbm):
                               "frac": a / FP64_PEAK_TFLOPS, "peak_kind": "derived FP64",
                               "algorithmic_flops": st["chol_flops"], "ms": st["t_chol_ms"],
                               "tc_kernel_ms": st.get("t_chol_tc_ms", 0.0),
-                              "note": "FP64 flops of the factorisation over both Cholesky kernels; the rank-32 and "
-                                      "rank-128 updates of the fronts at least 256 wide run on the tensor cores "
+                              "note": "FP64 flops of the factorisation over both Cholesky kernels; the panels and the "
+                                      "rank-32 and rank-128 updates of the fronts at least 256 wide run on the tensor cores "
                                       "(exact bf16 slicing, chol_tc_kernel), so frac is against the FP64 pipe only"}
     if st["t_trsm_ms"] > 0:
         a = st["trsm_flops"] / (st["t_trsm_ms"] * 1e-3) / 1e12
@@ -395,7 +395,7 @@ def main():
         b.record(st)
         b.synchronize()
         adjoint = {"ms": a.elapsed_time(b), "elements": int(g.numel()),
-                   "what": "feti_adjoint over all 216 subdomains (FP64 X_u recomputed, Z and Y by backward solves, "
+                   "what": "feti_adjoint over all 216 subdomains (FP64 X_u recomputed, Z by the backward solve, Y = Z W, "
                            "element contraction), one call"}
         del Wd, g
 

@@ -43,7 +43,11 @@ typedef enum {
 } feti_status;
 
 typedef enum {
-  FETI_PREC_FP64 = 0,       /* FP64 everywhere; F_i stored as FP64 tiles */
+  FETI_PREC_FP64 = 0,       /* FP64 everywhere; F_i stored as FP64 tiles.  The large contractions (Cholesky and
+                               forward solve of large fronts, SYRK, the apply where it is the fastest, the
+                               adjoint's) run on the tensor cores by exact slicing: operands rounded to 62 bits
+                               below the largest entry of a vector, scaled with the unknowns, and summed
+                               exactly, so that errors are FP64's or less relative to the largest terms */
   FETI_PREC_TF32 = 1,       /* TRSM updates / SYRK on tensor cores in TF32, F_i as FP32 tiles */
   FETI_PREC_SPLIT_BF16 = 2  /* as TF32 but each FP32 operand split into two bf16 halves */
 } feti_precision;
@@ -90,7 +94,10 @@ typedef struct {
   int32_t recompute_X;        /* 1 = do not keep X_i = L_i^{-1} P B_i^T after feti_assemble (it is an
                                  intermediate of the assembly) nor the FP64 X_i of feti_adjoint after that
                                  call: both are released and recomputed from L_i when next needed, for
-                                 problems where HBM is short; 0 = keep both buffers for reuse */
+                                 problems where HBM is short; 0 = keep both buffers for reuse.  The same
+                                 holds for what an FP64 context needs to slice X and L: digits of at most
+                                 16 GB each (and a fifth and a third of the free memory), and the update
+                                 blocks between the two parts of the forward solve */
   void* (*dev_alloc)(size_t bytes, void* ctx);  /* optional device allocator (NULL: cudaMalloc); where it aligns to
                                  less than 256 bytes it is asked for 256 more */
   void (*dev_free)(void* ptr, void* ctx);
@@ -131,13 +138,16 @@ typedef struct {
                                  SMs.  The factor is the same bit for bit either way */
   int32_t syrk_kernel;        /* split-bf16 SYRK kernel: 0 = autotuned at the first feti_assemble; 1, 2, 3 =
                                  feti_stats.syrk_variant 0, 1, 2 (the same F bit for bit) */
-  int32_t chol_tc;            /* 0 = the rank-32 and rank-128 updates of the fronts at least 256 wide run on
-                                 the tensor cores by exact slicing of FP64 into bf16 integers (integer partial
-                                 sums exact in FP32; error below FP64's own normwise bound); 1 = all of the
-                                 Cholesky on the FP64 pipe */
+  int32_t chol_tc;            /* 0 = the panels and the rank-32 and rank-128 updates of the fronts at least
+                                 256 wide run on the tensor cores by exact slicing of FP64 into bf16 integers
+                                 (integer partial sums exact in FP32; error below FP64's own normwise bound,
+                                 see FETI_PREC_FP64); 1 = all of the Cholesky on the FP64 pipe, and with it
+                                 these fronts' part of the FP64 forward solve and of the backward solve of
+                                 feti_adjoint and assembly_route 2 */
   int32_t chol_tc_front;      /* with chol_tc = 0: the narrowest front (w + r) taken by the tensor-core kernel,
-                                 with all its ancestors (0 = 256, within 3% of the fastest measured on 3D
-                                 elasticity and uneven 3D heat; values below 128 act as 128) */
+                                 with all its ancestors (0 = 256; values below 128 act as 128).  Of 192, 256
+                                 and 384, 256 is the fastest on most 3D problems measured; on 64 uneven 3D
+                                 heat subdomains 192 takes 23.6 ms against 27.3 */
   int32_t apply_kernel;       /* F-streaming kernel of the explicit apply: 0 = autotuned at the first
                                  feti_assemble; k = feti_stats.apply_variant k - 1 (7: FP64 tiles only) */
   int32_t implicit_cluster;   /* CTAs per subdomain of the implicit solves: 0 = chosen from the plans; -1 = one
@@ -249,9 +259,11 @@ feti_status feti_solve_warm(feti_ctx* ctx, double* lambda_dev, double* alpha_dev
 /* Adjoint of L = sum_i <W_i, F_i>: dtheta[e] = -<Z_i^T dK_e Z_i, W_i> with
  * Z_i = K_reg,i^{-1} B_i^T (derivative of the inverse, rho held fixed), in
  * FP64.  With K_reg = P^T L L^T P and L = L_u D (unit lower L_u):
- * Z_i = P^T L_u^{-T} D^{-2} X_u and Y_i = Z_i W_i = P^T L_u^{-T} D^{-2} (X_u W_i)
- * with X_u = L_u^{-1} P B_i^T from the pruned forward solve (recomputed here in
- * FP64 from L), and dtheta_e = -sum_{a,b in e} (dK_e)_ab Y_i[b,:] . Z_i[a,:].
+ * Z_i = P^T L_u^{-T} D^{-2} X_u with X_u = L_u^{-1} P B_i^T (the assembly's X_i
+ * times D in an FP64 context that keeps it, otherwise solved for in FP64 from L),
+ * Y_i = Z_i W_i (where the digits of that product find no memory,
+ * P^T L_u^{-T} D^{-2} (X_u W_i)), and
+ * dtheta_e = -sum_{a,b in e} (dK_e)_ab Y_i[b,:] . Z_i[a,:].
  * Subdomains are processed in batches whose dense n_i x 2 m_i work arrays fit
  * a device budget.  W_dev: per subdomain m_i x m_i row-major FP64 in B-row
  * order, concatenated (W_i symmetric); dtheta_dev: [sum nelem_i] device FP64.

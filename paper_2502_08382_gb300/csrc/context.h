@@ -190,7 +190,7 @@ struct feti_ctx {
   int64_t* d_mc_kidx = nullptr;
   double* d_mc_sign = nullptr;
   int64_t m_nnz = 0;
-  double* d_vec = nullptr;     // PCPG vectors (11 x n_lambda)
+  double* d_vec = nullptr;     // PCPG vectors (12 x n_lambda)
   double* d_cv = nullptr;      // coarse vectors (7 x D)
   double* d_sc = nullptr;      // scalars
   double* d_part = nullptr;    // block partials of the PCPG reductions (2 x kPcgMaxBlocks)

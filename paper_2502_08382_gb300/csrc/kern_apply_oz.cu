@@ -1,15 +1,15 @@
 // The F-streaming part of the explicit apply for FP64 tiles (see kern_apply.cu) by exact slicing on mma.sync.
 //
-// With FMAs an FP64 tile costs two FP64 FMAs and half an addition per entry (row and column partial), and the FP64
-// pipe of this GPU does two a clock and SM: it bounds the stream at 1.5 TB/s.  Here every entry is cut into eight
+// With FMAs an FP64 tile costs two FP64 FMAs per entry (row and column partial) and some additions, and the FP64 pipe of
+// this GPU does two a clock and SM: it bounds the stream at 2.4 TB/s (those kernels reach 1.2 to 1.75).  Here every entry is cut into eight
 // balanced base-256 digits (oz.cuh; 62 bits below the largest entry of its 16 x 64 strip), the digits go as f16
 // integers through mma.sync.m16n8k16 against the digits of p (N = 8: the eight digits of one vector), and the exact
 // integer sums are put together in 64-bit integers; about forty FP64 instructions per tile are left.  The operands
 // come out of registers and are used once, so tcgen05 (operands through shared memory, N at least 8 of one vector)
-// has nothing to gain: the cutting, about 25 integer instructions an entry, sets the pace (ncu: integer ALU 49%,
-// issue slots 53%, HMMA 13%, FP64 7%, twelve warps per SM).  Measured: 0.57 GB of FP64 tiles (125 uneven 3D heat
-// subdomains) 361 us with the register-batch kernel -> 262 us; 48 small tiles (16 subdomains of 16^2), where one warp
-// per tile was a long chain of FP64 instructions, 20 -> 5.5 us.  The other variants stay for the autotuner: they win
+// has nothing to gain: the cutting, about 25 integer instructions an entry, sets the pace (ncu: integer ALU 50%,
+// HMMA 12%, FP64 7%, twelve warps per SM).  Measured: 0.57 GB of FP64 tiles (125 uneven 3D heat subdomains) 361 us with
+// the register-batch kernel -> 272 us (262 before the scales below); 48 small tiles (16 subdomains of 16^2), where one
+// warp per tile is a long chain of FP64 instructions, 25 us with the fastest of the others -> 9.5 (launch included).  The other variants stay for the autotuner: they win
 // where few tiles leave the stream latency-bound and for FP32 tiles.
 //
 // One CTA of four warps per tile at a time, its tiles copied two ahead into shared memory (one bulk copy each); warp v

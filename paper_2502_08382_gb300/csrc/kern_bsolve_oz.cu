@@ -12,7 +12,7 @@
 //
 // What bounds it: the latency of a front's steps (cut, multiply, drain) on the narrow fronts; where the line to the
 // FP64 kernel lies and why, at kBackFront.  Measured, the backward solve of one adjoint of 8 elasticity subdomains of
-// 10^3: 60 ms with every front on the FP64 pipe -> 10.4 + 0.2 (digits) + 1.1 (the fronts below, FP64 pipe).
+// 10^3: 60 ms with every front on the FP64 pipe -> 11.1 + 0.4 (digits) + 1.1 (the fronts below, FP64 pipe).
 #include <algorithm>
 #include <cuda_bf16.h>
 

@@ -1010,8 +1010,12 @@ size_t implicit_smem(int nmax, int maxf, bool wide) {
   return ((size_t)nmax + maxf + (wide ? kWideBuf : kThreads / 32 * kWF)) * 8;
 }
 
-// The wide CTA takes one subdomain per SM; with more subdomains than SMs several 256-thread CTAs per SM hide one
-// another's latency better.
+// The wide CTA takes one subdomain per SM.  With more subdomains than SMs several 256-thread CTAs per SM hide one
+// another's latency better on 2D fronts, not on large 3D ones; the line at the SM count is a simple one and not the best
+// (options.implicit_cluster overrides it).  Milliseconds with 256 threads / 1 / 2 / 4 wide CTAs: 576 2D heat subdomains
+// of 64^2 1.34 / 2.68 / 3.56 / 5.48, 169 of them 0.94 / 1.31 / 1.33 / 1.66; 125 elasticity subdomains of 12^3 5.68 / 2.72 /
+// 3.35 / 4.54, 216 of them 6.43 / 5.40 / 5.00 / 7.02; 216 uneven 3D heat subdomains 8.2 / 4.4 / 2.7 / 3.2, 512 of them 8.2 /
+// 4.5 / 5.9 / 8.8.
 bool implicit_wide(int nsub, int nsm, int nmax, int maxf) {
   return nsub <= nsm && implicit_smem(nmax, maxf, true) + 1024 <= 227 * 1024;
 }

@@ -61,7 +61,8 @@ void launch_dense_oz(const DenseEnt* ents, int nent, const int4* items, int nite
                      void* XD, int* EX, double* out, int nsm, int* status, cudaStream_t st);
 // FP64 forward solve of the large fronts on the tensor cores (kern_trsm_oz.cu): digits of the large panels (items:
 // subdomain, supernode, first column of the 128-column block, its offset / 512), then, after launch_trsm with `hand`,
-// blocks of cw sorted columns (items: subdomain, first column); ws: per CTA front_sz + stack doubles
+// blocks of cw sorted columns (items: subdomain, first column); ws: per CTA the update blocks of the large fronts,
+// ws_stride doubles
 int64_t trsm_oz_block_bytes(int w, int r, int kB);
 int64_t trsm_oz_scratch(int cw);
 void launch_dig_l(const DevPlan& P, const int4* items, int nitems, void* LD, cudaStream_t st);

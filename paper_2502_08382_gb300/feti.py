@@ -241,7 +241,8 @@ class FetiOperator:
     or the split-bf16 SYRK kernel 0, 1, 2 to use; chol_tc: the large fronts' updates on
     the tensor cores (exact bf16 slicing) or all of the Cholesky on the FP64 pipe;
     apply_kernel: -1 (autotuned) or the apply's tile kernel (feti_stats.apply_variant) to use;
-    implicit_cluster: 0 (chosen from the plans), -1 (one 256-thread CTA per subdomain) or 1, 2, 4, 8 wide CTAs."""
+    implicit_cluster: 0 (chosen from the plans), -1 (one 256-thread CTA per subdomain) or 1, 2, 4, 8 wide CTAs per
+    subdomain."""
 
     def __init__(self, problem, prec: str = "fp64", tol: float = 1e-10, maxit: int = 2000,
                  refine_every: int = 0, refine_drop: float = 0.0, refine_restart: bool = False,
@@ -418,8 +419,7 @@ def _feti_weighted_trace():
         forward sets the CSR values of K_i from the element coefficients
         (finite-element assembly of the inputs), runs feti_assemble and forms
         L on the device (feti_weighted_trace); backward maps dL/dF_i = W_i to
-        dL/dcoef_e with the FP64 adjoint kernel (feti_adjoint, X_i recomputed
-        from L_i).  The operator must be created with with_elements=True and
+        dL/dcoef_e with the FP64 adjoint (feti_adjoint).  The operator must be created with with_elements=True and
         unit_scale=True (dK_e/dcoef_e = K_ref)."""
 
         @staticmethod
