@@ -174,7 +174,10 @@ __global__ void __launch_bounds__(kDT, 3)
       sn = sval(dn);
     }
     const bool diag = (d.flags & kTileDiag) != 0;
-    const int pm = __reduce_max_sync(0xffffffffu, dig_key(pv, -sv));
+    // (subnormal entries, which the cut below would drop, go the slow way)
+    const uint32_t ph = (uint32_t)__double2hiint(pv) & 0x7fffffffu;
+    const bool tiny = ph < 0x00100000u && (ph | (uint32_t)__double2loint(pv)) != 0;
+    const int pm = __reduce_max_sync(0xffffffffu, tiny ? kKeyBad : dig_key(pv, -sv));
     if (lane == 0) mx_s[warp] = pm;
     sx[tid] = sv;
     const double* Ft = reinterpret_cast<const double*>(buf + (it & 1) * kTileBytes);
@@ -224,7 +227,8 @@ __global__ void __launch_bounds__(kDT, 3)
       for (int kb = 0; kb < 4; ++kb)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          z |= ((uint32_t)__double2hiint(f[kb][j].x) | (uint32_t)__double2hiint(f[kb][j].y)) & 0x7fffffffu;
+          z |= (((uint32_t)__double2hiint(f[kb][j].x) | (uint32_t)__double2hiint(f[kb][j].y)) & 0x7fffffffu) |
+               (uint32_t)__double2loint(f[kb][j].x) | (uint32_t)__double2loint(f[kb][j].y);
       fzero = __reduce_or_sync(0xffffffffu, z) == 0;
     }
     const int ef = scaled_exponent(fkey, kLeastF, kBadF, fzero);

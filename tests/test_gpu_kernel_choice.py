@@ -116,3 +116,23 @@ def test_apply_top_binade(kernel):
     assert np.abs(q / p[j] - off).max() <= 2.0 ** -55 * np.abs(F).max()
     if k < 1024:
         assert np.abs(q).max() >= 2.0 ** 1023
+
+
+@pytest.mark.parametrize("kernel", range(7))
+def test_apply_subnormal(kernel):
+    """p of subnormal numbers (and one of a single smallest one): products and sums are multiples of 2^-1074, each rounded
+    to within half of it, so m + 8 of them are off by as many at most."""
+    P = make_problem(dim=2, physics="heat", cuts=[[30], [30]], material="lognormal", sigma=0.5)
+    op = feti.FetiOperator(P, prec="fp64", apply_kernel=kernel)
+    op.assemble()
+    F = op.get_F(0)
+    rng = np.random.default_rng(5)
+    k = rng.integers(-2 ** 40, 2 ** 40, size=P.n_lambda)
+    for ints in (k, np.eye(1, P.n_lambda, P.n_lambda // 2, dtype=np.int64)[0]):
+        p = ints.astype(np.float64) * 2.0 ** -1074
+        q = op.apply(torch.from_numpy(p).cuda()).cpu().numpy()
+        ref = F @ ints  # in units of 2^-1074
+        got = np.ldexp(q, 600) * 2.0 ** 474
+        assert np.abs(got - ref).max() <= P.n_lambda + 8 + 2.0 ** -40 * np.abs(ref).max()
+        assert np.abs(got).max() > 0
+    op.close()
