@@ -1435,8 +1435,9 @@ feti_status feti_assemble(feti_ctx* ctx) {
   // error is that of its SYRK alone; in the TF32 mode X_i is rounded to TF32 for that SYRK
   const int tcmode = ctx->fp32 ? 2 : 0;
   const int tf32_out = ctx->fp32 && ctx->opt.prec == FETI_PREC_TF32 ? 1 : 0;
-  // FP64: the forward solve of the large fronts by exact slicing on the tensor cores
-  const bool tx = !ctx->fp32 && ctx->opt.assembly_route != 2 && reserve_trsm_oz(ctx);
+  // FP64: the forward solve of the large fronts by exact slicing on the tensor cores (not on the TRSM path)
+  const bool path2 = ctx->opt.assembly_route == 2 || (ctx->opt.assembly_route == 3 && ctx->route_tuned && ctx->route == 2);
+  const bool tx = !ctx->fp32 && !path2 && reserve_trsm_oz(ctx);
   ctx->stats.trsm_grid = ctx->fp32 ? ctx->grid_trsm32 : ctx->grid_trsm;
   auto run_trsm = [&](const feti_ctx::TrsmCand& tc, cudaStream_t s2) {
     CK(cudaMemsetAsync(ctx->d_queue + 16, 0, sizeof(int), s2));
@@ -1446,7 +1447,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
                 ctx->d_status, s2, 0, ctx->d_X2, ctx->d_L32, split ? 1 : 0, tx ? ctx->d_th : nullptr);
   };
   // FP64: the SYRK by exact slicing on the tensor cores
-  const bool oz = !ctx->fp32 && ctx->opt.assembly_route != 2 && ctx->stats.syrk_flops > 0 && reserve_syrk_oz(ctx);
+  const bool oz = !ctx->fp32 && !path2 && ctx->stats.syrk_flops > 0 && reserve_syrk_oz(ctx);
   // the numeric phase as one sequence of launches (recorded once into a CUDA graph, see below); r2: the
   // TRSM-path route (F_i = B_i P^T L^{-T} X_i in host-driven batches, not captured)
   auto enqueue = [&](cudaStream_t s2, unsigned evf, bool r2) {
@@ -1584,9 +1585,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
   if (tx)
     for (const auto& b : ctx->tx_batches) ctx->stats.launches += b.nitems > 0 ? 2 : 0;
   if (oz) ctx->stats.launches += 3 * (int64_t)ctx->oz_batches.size() - 1;
-  ctx->stats.digit_kernels = (oz ? 1 : 0) | (tx ? 2 : 0);
   const int want = ctx->opt.assembly_route;
-  if (want == 2 || (want == 3 && ctx->route_tuned && ctx->route == 2)) {
+  if (path2) {
     ctx->route = 2;
     if (!ctx->trsm_tuned) {  // the unit-lower TRSM of this route takes whole subdomains
       ctx->trsm_pick = 0;
@@ -1653,6 +1653,7 @@ feti_status feti_assemble(feti_ctx* ctx) {
   }
   CK(cudaGetLastError());
   ctx->stats.assembly_route = ctx->route;
+  ctx->stats.digit_kernels = ctx->route == 2 ? 0 : (oz ? 1 : 0) | (tx ? 2 : 0);
   for (int k = 0; k < 3; ++k) ctx->stats.route_ms[k] = ctx->route_ms[k];
   if (!ctx->coarse_ready) {
     // G = B R does not depend on the values of K: the coarse problem is set up once
@@ -1667,6 +1668,8 @@ feti_status feti_assemble(feti_ctx* ctx) {
     ctx->d_X = nullptr;
     dfree(ctx, ctx->d_X2);
     ctx->d_X2 = nullptr;
+  }
+  if (ctx->opt.recompute_X || ctx->route == 2) {  // (the TRSM path has no use for the digits its rival was timed with)
     dfree(ctx, ctx->d_XD);
     ctx->d_XD = nullptr;
     dfree(ctx, ctx->d_LD);

@@ -299,3 +299,21 @@ def test_workspace_size():
     ctas = op.stats()["trsm_grid"]
     op.close()
     assert st["workspace_bytes"] < 8 * ctas * stack
+
+
+@pytest.mark.parametrize("cuts", [[[1], [1]], [[2], [2]], [[1, 1], [1, 1]], [[2, 2], [2, 2]]])
+def test_trsm_path_holds_no_digits(monkeypatch, cuts):
+    """Where the autotuner keeps the TRSM path, no digits of X and L are kept or asked for (on tiny problems the two routes
+    take about the same time, so some of these keep it)."""
+    P = make_problem(dim=2, physics="heat", cuts=cuts)
+    op = feti.FetiOperator(P, prec="fp64", route="auto")
+    op.assemble()
+    r = Refuser(monkeypatch)
+    r.rule = lambda n: True
+    op.assemble()
+    st = op.stats()
+    op.close()
+    if st["assembly_route"] == 2:
+        assert st["digit_kernels"] == 0 and r.refused == 0
+    else:
+        assert st["digit_kernels"] == 1
